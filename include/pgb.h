@@ -70,7 +70,8 @@ typedef struct pgb_params {
     double theta;         /* multipole acceptance criterion; 0 = direct sum */
     int32_t leaf_size;    /* N_crit: max panels per octree leaf, 1..1024 */
     int32_t group_size;   /* targets per interaction list: 32 (one warp) */
-    int32_t p2p_item;     /* P2P work item: at most this many 32-point tiles of one group, 1..4096 (0 = 64) */
+    int32_t p2p_item;     /* P2P work item: the panels of at most this many runs of 32 quadrature points of one
+                             group, at least one panel, 1..4096 (0 = 64) */
     int32_t m2p_item;     /* M2P work item: at most this many far nodes of one group, 1..4096 (0 = 64) */
     int32_t precond;      /* GMRES preconditioner: 0 none (the paper's solver), 1 block-diagonal: per
                              panel, the inverse of the 2x2 (molecule) or 1x1 (surface) block of its own
@@ -200,7 +201,7 @@ int pgb_tree_build(struct pgb_ctx* ctx);
 int pgb_tree_stats(struct pgb_ctx* ctx, pgb_tree_info* info);
 
 /* Recompute what the current poses change -- world geometry, node and group
- * centres, the offsets of the list entries and P2P tiles, cross-body
+ * centres, the offsets of the list entries and P2P columns, cross-body
  * near-field entries -- while keeping the near/far interaction lists (and the
  * work items) of the last pgb_tree_build.  The product is then the treecode
  * with those lists at the new poses: a small pose change (finite differences

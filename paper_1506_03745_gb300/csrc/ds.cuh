@@ -83,30 +83,52 @@ __device__ __forceinline__ ds mul_f(ds a, float b) {
 }
 __device__ __forceinline__ bool operator>(ds a, ds b) { return a.hi > b.hi || (a.hi == b.hi && a.lo > b.lo); }
 
+// The same operations without the closing renormalisation (3 fewer each): the
+// result's lo may reach a few ulps of its hi.  They take such operands
+// themselves, as long as no cancellation has made lo large beside hi: products
+// drop lo * lo, a few 2^-46 of the result.
+__device__ __forceinline__ ds ds_mul_u(ds a, ds b) {
+    const float p = __fmul_rn(a.hi, b.hi);
+    float e = __fmaf_rn(a.hi, b.hi, -p);
+    e = __fmaf_rn(a.hi, b.lo, e);
+    return ds(p, __fmaf_rn(a.lo, b.hi, e));
+}
+__device__ __forceinline__ ds ds_add_u(ds a, ds b) {
+    const ds s = two_sum(a.hi, b.hi);
+    return ds(s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo)));
+}
+__device__ __forceinline__ ds ds_fma_u(ds a, ds b, ds c) {
+    const ds p = ds_mul_u(a, b);
+    const ds s = two_sum(p.hi, c.hi);
+    return ds(s.hi, __fadd_rn(s.lo, __fadd_rn(p.lo, c.lo)));
+}
+__device__ __forceinline__ ds ds_norm(ds a) { return fast_two_sum(a.hi, a.lo); }
+
 // 1/sqrt(x), x > 0 (x = 0 gives a non-finite value; callers mask it): the
-// SFU estimate y of 1/sqrt(x.hi) (relative error below 2^-22) and one Newton
-// step y + (y/2)(1 - x y^2) with the residual 1 - x y^2 formed in
-// double-single; the step leaves a relative error of about 1.5 d^2 < 3e-14.
+// SFU estimate y of 1/sqrt(x.hi) (relative error below 2^-22) and one step of
+// Halley's form y + y e (1/2 + 3/8 e), e = 1 - x y^2.  x.hi y = p + q exactly,
+// and 1 - p y, of size 2^-21, loses only its own rounding (2^-45) in one fused
+// operation, so e costs six operations instead of a double-single chain of 23.
 __device__ __forceinline__ ds ds_rsqrt(ds x) {
     float y;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x.hi));
-    const ds e = ds(1) - mul_f(mul_f(x, y), y);
-    return two_sum(y, __fmul_rn(__fmul_rn(0.5f, y), e.hi));
+    const float p = __fmul_rn(x.hi, y);
+    const float q = __fmaf_rn(x.hi, y, -p);
+    float e = __fmaf_rn(-p, y, 1.f);
+    e = __fmaf_rn(-q, y, e);
+    e = __fmaf_rn(-__fmul_rn(x.lo, y), y, e);
+    return fast_two_sum(y, __fmul_rn(__fmul_rn(y, e), __fmaf_rn(0.375f, e, 0.5f)));
 }
 
 // 2^t for t < 127 (results below 2^-126 are returned as 0), table-driven
 // (Tang's reduction, ACM TOMS 15, 1989): t = m / 64 + f with m = rint(64 t.hi)
-// and |f| <= 1/128 (t.hi - m/64 is exact), so 2^t = 2^(m >> 6) 2^(j/64) 2^f
-// with j = m & 63.  2^(j/64) comes from a 64-entry double-single table
-// computed at compile time from the exponential series; 2^f from its Taylor
-// series sum_k (ln 2)^k f^k / k!: the terms k = 3..5 in FP32 (they are below
-// 2.7e-8 in all, so FP32 leaves them an error below 2e-15), k = 0..2 by
-// Horner steps in double-single; the truncation after k = 5 is below
-// 0.0055^6 / 720 < 4e-17.  Then 2^(m >> 6) is applied to both parts (exact).
-template <int K>
-struct DsCoef {
-    static constexpr ds v = ds_const(Exp2Coef<K>::v);
-};
+// and |f| <= 1/128 (t.hi - m/64 is exact), so 2^t = 2^(m >> 6) 2^(j/64) e^s
+// with j = m & 63 and s = f ln 2, |s| < 0.0055.  2^(j/64) comes from a 64-entry
+// double-single table computed at compile time from the exponential series.
+// e^s - 1 = s + s^2/2 + s^3 (1/6 + s/24 + s^2/120): s and s^2 with their error
+// terms, the cubic tail (below 2.8e-8) in FP32, whose rounding is below 2e-15
+// of the result; the truncation is below 4e-17.  35 FP32 operations (the
+// Horner form with double-single steps took 75).
 // e^x by its series, for the compile-time table (|x| < 1: 30 terms reach
 // double rounding)
 __host__ __device__ constexpr double exp_series(double x) {
@@ -126,22 +148,33 @@ struct Exp2Table {
 __device__ const Exp2Table kExp2Table = Exp2Table();
 
 __device__ __forceinline__ ds ds_exp2(ds t) {
+    constexpr ds ln2 = ds_const(PGB_LN2);
     const float mf = rintf(__fmul_rn(t.hi, 64.f));
     const int m = (int)mf;
-    const ds f = two_sum(__fsub_rn(t.hi, __fmul_rn(mf, 0.015625f)), t.lo);
-    // tail k = 3..5 in FP32 (Horner), as the coefficient of f^3
-    float q = (float)Exp2Coef<5>::v;
-    q = __fmaf_rn(q, f.hi, (float)Exp2Coef<4>::v);
-    q = __fmaf_rn(q, f.hi, (float)Exp2Coef<3>::v);
-    ds p = DsCoef<2>::v + mul_f(f, q);
-    p = ds_fma(p, f, DsCoef<1>::v);
-    p = ds_fma(p, f, ds(1));
+    const float fe = __fmaf_rn(mf, -0.015625f, t.hi);  // exact; 0 or at least an ulp of t.hi
+    const ds f = fast_two_sum(fe, t.lo);
+    const float s = __fmul_rn(f.hi, ln2.hi);
+    float sl = __fmaf_rn(f.hi, ln2.hi, -s);
+    sl = __fmaf_rn(f.hi, ln2.lo, sl);
+    sl = __fmaf_rn(f.lo, ln2.hi, sl);
+    const float q = __fmul_rn(s, s);
+    const float ql = __fmaf_rn(s, s, -q);  // s^2 = q + ql + 2 s sl
+    float tail = __fmaf_rn(s, 1.f / 120.f, 1.f / 24.f);
+    tail = __fmul_rn(__fmaf_rn(tail, s, 1.f / 6.f), __fmul_rn(s, q));
+    const float a = __fmaf_rn(0.5f, q, s);
+    float lo = __fmaf_rn(0.5f, q, -__fsub_rn(a, s));
+    lo = __fadd_rn(__fadd_rn(lo, tail), __fmaf_rn(0.5f, ql, __fmaf_rn(s, sl, sl)));
     const float2 tv = __ldg(reinterpret_cast<const float2*>(&kExp2Table.v[m & 63]));
-    p = p * ds(tv.x, tv.y);
+    const float p = __fmul_rn(tv.x, a);
+    float pe = __fmaf_rn(tv.x, a, -p);
+    pe = __fmaf_rn(tv.x, lo, pe);
+    pe = __fmaf_rn(tv.y, a, pe);
+    const float h = __fadd_rn(tv.x, p);  // |p| < |tv.x|
+    const float l = __fadd_rn(__fsub_rn(p, __fsub_rn(h, tv.x)), __fadd_rn(pe, tv.y));
     const int n = m >> 6;  // floor(m / 64)
     if (n < -126) return ds(0);
     const float sc = __int_as_float((127 + n) << 23);
-    return ds(__fmul_rn(p.hi, sc), __fmul_rn(p.lo, sc));
+    return ds(__fmul_rn(h, sc), __fmul_rn(l, sc));
 }
 
 // e^x = 2^(x log2 e)

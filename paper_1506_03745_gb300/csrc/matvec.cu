@@ -29,7 +29,7 @@ static inline int nblk(int64_t n, int t) { return (int)std::max<int64_t>(1, (n +
 template <typename real>
 __global__ void k_src_prep(Geo g, BodyDev bd, const double* __restrict__ x, int mode,
                            const typename V4<real>::t* __restrict__ yrel, typename V4<real>::t* __restrict__ src,
-                           real* __restrict__ dens, double eps_out) {
+                           typename V4<real>::t* __restrict__ pd, real* __restrict__ dens, double eps_out) {
     const bool known = mode == 1;
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= g.n_pan) return;
@@ -63,6 +63,13 @@ __global__ void k_src_prep(Geo g, BodyDev bd, const double* __restrict__ x, int 
     dens[3 * i] = rL;
     dens[3 * i + 1] = rY;
     dens[3 * i + 2] = rp;
+    const real area = (real)g.A[i];
+    typename V4<real>::t pv;
+    pv.x = area * rL;
+    pv.y = area * rY;
+    pv.z = area * rp;
+    pv.w = 0;
+    pd[i] = pv;
     const real nx = (real)g.n[3 * i], ny = (real)g.n[3 * i + 1], nz = (real)g.n[3 * i + 2];
     for (int m = 0; m < g.K; ++m) {
         const int64_t p = i * g.K + m;
@@ -200,7 +207,7 @@ __global__ void k_rows_init(Geo g, BodyDev bd, const double* x, int mode, double
 template <typename real>
 __global__ void k_src_region(Geo g, BodyDev bd, RegionDev rd, const double* __restrict__ x, int mode,
                              const typename V4<real>::t* __restrict__ yrel, typename V4<real>::t* __restrict__ src,
-                             real* __restrict__ dens) {
+                             typename V4<real>::t* __restrict__ pd, real* __restrict__ dens) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= g.n_pan) return;
     const int b = g.pbody[i];
@@ -230,6 +237,13 @@ __global__ void k_src_region(Geo g, BodyDev bd, RegionDev rd, const double* __re
     dens[3 * i] = 0;
     dens[3 * i + 1] = rY;
     dens[3 * i + 2] = rp;
+    const real area = (real)g.A[i];
+    typename V4<real>::t pv;
+    pv.x = 0;
+    pv.y = area * rY;
+    pv.z = area * rp;
+    pv.w = 0;
+    pd[i] = pv;
     const real nx = (real)g.n[3 * i], ny = (real)g.n[3 * i + 1], nz = (real)g.n[3 * i + 2];
     for (int m = 0; m < g.K; ++m) {
         const int64_t p = i * g.K + m;
@@ -392,11 +406,14 @@ void reserve_product(pgb_ctx* c, int precision) {
     const int TP = n_terms_pad(c->p.P);
     if (pi == 0) {
         c->d_src32.resize(2 * nsrc);
+        c->d_pd32.resize(c->n_pan);
         c->d_mom32.resize((size_t)c->n_nodes * 2 * T);
         c->d_far32.resize((size_t)c->n_nodes * 2 * TP);
     } else {
         c->d_src64.resize(2 * nsrc);
         c->d_src_ds.resize(2 * nsrc);
+        c->d_pd64.resize(c->n_pan);
+        c->d_pd_ds.resize(c->n_pan);
         c->d_mom64.resize((size_t)c->n_nodes * 2 * T);
         c->d_far64.resize((size_t)c->n_nodes * 2 * TP);
         c->d_mom_ds.resize((size_t)c->n_nodes * 2 * T);
@@ -480,16 +497,19 @@ void apply_mode(pgb_ctx* c, const double* x, double* y, int precision, int mode,
     ev.g_hi = c->shard_g[0] >= 0 ? c->shard_g[1] : c->n_groups;
     ev.near4 = c->d_near4;
     ev.far4 = c->d_far4;
-    ev.tile_off = c->d_tile_off;
-    ev.tile_d = c->d_tile_d;
-    ev.tile_m = c->d_tile_m;
+    ev.col_off = c->d_col_off;
+    ev.col = c->d_col;
+    ev.pnode = c->d_pnode;
+    ev.pbody = c->d_pbody;
+    ev.rule = far_rule(c->p.K);
+    ev.src_mask = 0;
+    for (size_t b = 0; b < c->bodies.size(); ++b) ev.src_mask |= (unsigned long long)(ev.src_active[b] != 0) << b;
     ev.n_pitems = c->n_pitems;
     ev.n_fitems = c->n_fitems;
     ev.pitem_off = c->d_pitem_off;
     ev.fitem_off = c->d_fitem_off;
     ev.pitem_group = c->d_pitem_group;
     ev.fitem_group = c->d_fitem_group;
-    ev.p2p_item = c->p.p2p_item;
     ev.m2p_item = c->p.m2p_item;
     ev.Up = Up;
     ev.Uf = Uf;
@@ -506,19 +526,28 @@ void apply_mode(pgb_ctx* c, const double* x, double* y, int precision, int mode,
     const int TP = n_terms_pad(P);
     if (f32) {
         c->d_src32.resize(2 * nsrc);
+        c->d_pd32.resize(c->n_pan);
         c->d_mom32.resize((size_t)c->n_nodes * 2 * T);
         c->d_far32.resize((size_t)c->n_nodes * 2 * TP);
         up.far = c->d_far32.p;
+        ev.pg = c->d_pg32.p;
+        ev.pd = c->d_pd32.p;
     } else {
         c->d_src64.resize(2 * nsrc);
+        c->d_pd64.resize(c->n_pan);
         c->d_mom64.resize((size_t)c->n_nodes * 2 * T);
         c->d_far64.resize((size_t)c->n_nodes * 2 * TP);
         up.far = c->d_far64.p;
+        ev.pg = c->d_pg64.p;
+        ev.pd = c->d_pd64.p;
         if (precision == PGB_FP64_DS) {
             c->d_src_ds.resize(2 * nsrc);
+            c->d_pd_ds.resize(c->n_pan);
             c->d_mom_ds.resize((size_t)c->n_nodes * 2 * T);
             c->d_far_ds.resize((size_t)c->n_nodes * 2 * TP);
             up.far = c->d_far_ds.p;
+            ev.pg = c->d_pg_ds.p;
+            ev.pd = c->d_pd_ds.p;
         }
     }
     const bool dsp = precision == PGB_FP64_DS;
@@ -543,22 +572,29 @@ void apply_mode(pgb_ctx* c, const double* x, double* y, int precision, int mode,
                 PGB_CUDA(cudaMemsetAsync(c->d_work.p, 0, 16, s));
             ev.all_active = 1;
             ev.tgt_mask = 0;
+            ev.src_mask = 0;
             for (size_t b = 0; b < c->bodies.size(); ++b) {
                 ev.src_active[b] = up.src_active[b] = rd.sign[b] != 0 && !c->body_off[b];
                 ev.all_active &= ev.src_active[b];
-                if (ev.src_active[b]) ev.tgt_mask |= 1ull << b;  // only the region's own rows
+                if (ev.src_active[b]) {  // only the region's own rows
+                    ev.tgt_mask |= 1ull << b;
+                    ev.src_mask |= 1ull << b;
+                }
             }
             {
                 StageTimer tm(c, PGB_STAGE_SOURCES + (f32 ? 0 : PGB_STAGE_FP64));
                 if (f32)
-                    k_src_region<float><<<nblk(c->n_pan, 128), 128, 0, s>>>(g, bd, rd, x, mode, c->d_y32, c->d_src32,
+                    k_src_region<float><<<nblk(c->n_pan, 128), 128, 0, s>>>(g, bd, rd, x, mode, c->d_y32, c->d_src32, c->d_pd32,
                                                                              (float*)dens.p);
                 else
                     k_src_region<double><<<nblk(c->n_pan, 128), 128, 0, s>>>(g, bd, rd, x, mode, c->d_y64,
-                                                                              c->d_src64, dens.p);
-                if (precision == PGB_FP64_DS) convert_src_ds(c->d_src64, c->d_src_ds, 2 * nsrc, s);
+                                                                              c->d_src64, c->d_pd64, dens.p);
+                if (precision == PGB_FP64_DS) {
+                    convert_src_ds(c->d_src64, c->d_src_ds, 2 * nsrc, s);
+                    convert_src_ds(c->d_pd64, c->d_pd_ds, c->n_pan, s);
+                }
                 PGB_CUDA(cudaGetLastError());
-                PGB_LAUNCHED(c, precision == PGB_FP64_DS ? 2 : 1);
+                PGB_LAUNCHED(c, precision == PGB_FP64_DS ? 3 : 1);
             }
             for (int stage : {PGB_STAGE_UPWARD, PGB_STAGE_P2P, PGB_STAGE_M2P}) {
                 StageTimer tm(c, stage + (f32 ? 0 : PGB_STAGE_FP64));
@@ -593,14 +629,17 @@ void apply_mode(pgb_ctx* c, const double* x, double* y, int precision, int mode,
     {
         StageTimer tm(c, PGB_STAGE_SOURCES + (f32 ? 0 : PGB_STAGE_FP64));
         if (f32)
-            k_src_prep<float><<<nblk(c->n_pan, 128), 128, 0, s>>>(g, bd, x, mode, c->d_y32, c->d_src32,
+            k_src_prep<float><<<nblk(c->n_pan, 128), 128, 0, s>>>(g, bd, x, mode, c->d_y32, c->d_src32, c->d_pd32,
                                                                   (float*)dens.p, c->eps_out);
         else
-            k_src_prep<double><<<nblk(c->n_pan, 128), 128, 0, s>>>(g, bd, x, mode, c->d_y64, c->d_src64,
+            k_src_prep<double><<<nblk(c->n_pan, 128), 128, 0, s>>>(g, bd, x, mode, c->d_y64, c->d_src64, c->d_pd64,
                                                                    dens.p, c->eps_out);
-        if (precision == PGB_FP64_DS) convert_src_ds(c->d_src64, c->d_src_ds, 2 * nsrc, s);
+        if (precision == PGB_FP64_DS) {
+            convert_src_ds(c->d_src64, c->d_src_ds, 2 * nsrc, s);
+            convert_src_ds(c->d_pd64, c->d_pd_ds, c->n_pan, s);
+        }
         PGB_CUDA(cudaGetLastError());
-        PGB_LAUNCHED(c, precision == PGB_FP64_DS ? 2 : 1);
+        PGB_LAUNCHED(c, precision == PGB_FP64_DS ? 3 : 1);
     }
     // the upward pass on its own stream, beside P2P (which does not read the
     // moments); M2P waits for it

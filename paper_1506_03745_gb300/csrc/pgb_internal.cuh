@@ -100,6 +100,17 @@ struct DBuf {  // owning device buffer
 // Taylor term count of total degree <= P in three variables.
 __host__ __device__ constexpr int n_terms(int P) { return (P + 1) * (P + 2) * (P + 3) / 6; }
 
+// Columns of a P2P work item: the panels of p2p_item runs of 32 quadrature points.
+inline int p2p_item_cols(int p2p_item, int K) { return p2p_item * 32 / K > 0 ? p2p_item * 32 / K : 1; }
+
+// The far rule (Section 3.1) as its symmetric orbits: the centroid (w[0], 0
+// without one) and up to two orbits of three points c - 3 alpha (v_k - c);
+// a[o] = 3 alpha, w[1 + o] the weight of each of the orbit's points.
+struct FarRule {
+    double a[2], w[3];
+};
+FarRule far_rule(int K);
+
 // Far-field coefficient tables (farfield.cu) of one Taylor order and
 // screening: moments -> the coefficients the M2P kernels evaluate.
 struct FarTab {
@@ -231,12 +242,16 @@ struct pgb_ctx {
     pgb::DBuf<int32_t> d_near, d_far;
     pgb::DBuf<float4> d_near4, d_far4;   // FP32 entry offsets (node centre - group centre), node id
     pgb::DBuf<int32_t> d_list_tmp;       // entries kept by the counting traversal (fixed rows per group)
-    int64_t n_tiles = 0;                 // P2P tiles (<= 32 points of one near leaf) over all groups
-    pgb::DBuf<int64_t> d_tile_off;
-    pgb::DBuf<float4> d_tile_d;
-    pgb::DBuf<int4> d_tile_m;
-    // work items: a group's P2P tiles and its far entries in runs of at most
-    // p.p2p_item / p.m2p_item, one block each, so that no block carries a
+    int64_t n_cols = 0;                  // P2P columns (panels of a group's near leaves) over all groups
+    pgb::DBuf<int64_t> d_col_off;        // per group (+ total)
+    pgb::DBuf<float4> d_col;             // leaf centre - group centre, panel
+    pgb::DBuf<int32_t> d_pnode;          // leaf node of every panel
+    pgb::DBuf<float> d_pg32;             // panel geometry of the P2P kernels, 16 values each
+    pgb::DBuf<double> d_pg64, d_pg_ds;   // in FP64 and as double-single pairs (8 bytes a value)
+    pgb::DBuf<float4> d_pd32;            // panel densities times area: psiL, psiY, phi
+    pgb::DBuf<pgb::dbl4> d_pd64, d_pd_ds;
+    // work items: a group's P2P columns and its far entries in even runs of at most
+    // p2p_item_cols(p.p2p_item) / p.m2p_item, one block each, so that no block carries a
     // whole heavy group; each item leaves 32 (L) + 32 (Y) partial sums
     int64_t n_pitems = 0, n_fitems = 0;
     pgb::DBuf<int64_t> d_pitem_off, d_fitem_off;  // per group (+ total)

@@ -121,20 +121,20 @@ void shard_partition(const double* work, int64_t ng, int world, int64_t* bounds)
     bounds[world] = ng;
 }
 
-// Work of each target group (P2P tiles and far entries, weighted by their
-// operation counts: a tile of 32 points for 32 targets against a far node
-// for 32 targets, about 3 : 1 at P = 6) and the rank's group and row range.
+// Work of each target group (P2P columns and far entries, weighted by their
+// operation counts for 32 targets: 32 quadrature points against a far node,
+// about 3 : 1 at P = 6) and the rank's group and row range.
 static void shard_ranges(pgb_ctx* c, int world, std::vector<int64_t>& gb, std::vector<int64_t>& rb) {
     const int64_t ng = c->n_groups;
     std::vector<int64_t> toff(ng + 1), foff(ng + 1);
     std::vector<int32_t> gs(ng);
     cudaStream_t s = c->stream;
-    PGB_CUDA(cudaMemcpyAsync(toff.data(), c->d_tile_off.p, 8 * (ng + 1), cudaMemcpyDeviceToHost, s));
+    PGB_CUDA(cudaMemcpyAsync(toff.data(), c->d_col_off.p, 8 * (ng + 1), cudaMemcpyDeviceToHost, s));
     PGB_CUDA(cudaMemcpyAsync(foff.data(), c->d_far_off.p, 8 * (ng + 1), cudaMemcpyDeviceToHost, s));
     PGB_CUDA(cudaMemcpyAsync(gs.data(), c->d_group_start.p, 4 * ng, cudaMemcpyDeviceToHost, s));
     PGB_CUDA(cudaStreamSynchronize(s));
     std::vector<double> work(ng);
-    for (int64_t g = 0; g < ng; ++g) work[g] = 3.0 * (toff[g + 1] - toff[g]) + (foff[g + 1] - foff[g]) + 1.0;
+    for (int64_t g = 0; g < ng; ++g) work[g] = 3.0 * c->p.K / 32.0 * (toff[g + 1] - toff[g]) + (foff[g + 1] - foff[g]) + 1.0;
     gb.assign(world + 1, 0);
     shard_partition(work.data(), ng, world, gb.data());
     // sharded row of the first panel of a group: the body's unknown offset

@@ -56,6 +56,20 @@ Rules make_rules(int K, int Kn, int ne) {
     return r;
 }
 
+FarRule far_rule(int K) {
+    const Rules r = make_rules(K, 19, 9);
+    FarRule f = {{0, 0}, {0, 0, 0}};
+    const int o = K == 3 ? 0 : 1;  // the first orbit's first point
+    if (K != 3) f.w[0] = r.w[0];
+    for (int k = 0; k < 2 && o + 3 * k < K; ++k) {
+        // of (alpha, alpha, -2 alpha) in some order, the value that occurs twice
+        const double* m = r.mu[o + 3 * k];
+        f.a[k] = 3.0 * (fabs(m[0] - m[1]) < 1e-9 ? m[0] : m[2]);
+        f.w[1 + k] = r.w[o + 3 * k];
+    }
+    return f;
+}
+
 static inline int nblk(int64_t n, int t) { return (int)std::max<int64_t>(1, (n + t - 1) / t); }
 
 // ---------------------------------------------------------------- scan
@@ -815,6 +829,40 @@ __global__ void k_rel_sources(const int32_t* pan_leaf, const int32_t* leaf_node,
     y64[p] = dbl4{dx, dy, dz, W[p]};
 }
 
+// Panel geometry of the P2P kernels, 16 values per panel relative to its leaf
+// centre (PanelGeo in treecode.cuh): the centroid c, the vectors 2 (v_0 - c)
+// and 2 (v_1 - c), the normal, and g_k = |v_k - c|^2; in FP32, FP64 and split
+// into double-single.
+__global__ void k_panel_geo(const int32_t* pan_leaf, const int32_t* leaf_node, const double* ncen, int64_t n,
+                            const double* V, const double* C, const double* Nn, int32_t* pnode, float* g32,
+                            double* g64, ds* gds) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int nd = leaf_node[pan_leaf[i]];
+    pnode[i] = nd;
+    double o[16], s[3][3], gk[3];
+    for (int k = 0; k < 3; ++k) {
+        gk[k] = 0;
+        for (int a = 0; a < 3; ++a) {
+            s[k][a] = V[9 * i + 3 * k + a] - C[3 * i + a];
+            gk[k] += s[k][a] * s[k][a];
+        }
+    }
+    for (int a = 0; a < 3; ++a) {
+        o[a] = C[3 * i + a] - ncen[3 * nd + a];
+        o[4 + a] = 2.0 * s[0][a];
+        o[8 + a] = 2.0 * s[1][a];
+        o[12 + a] = Nn[3 * i + a];
+        o[3 + 4 * a] = gk[a];
+    }
+    o[15] = 0.0;
+    for (int q = 0; q < 16; ++q) {
+        g32[16 * i + q] = (float)o[q];
+        g64[16 * i + q] = o[q];
+        gds[16 * i + q] = ds_from_double(o[q]);
+    }
+}
+
 void build_geometry(pgb_ctx* c) {
     cudaStream_t s = c->stream;
     int64_t n = c->n_pan;
@@ -909,6 +957,12 @@ void build_geometry(pgb_ctx* c) {
     c->d_y64.resize(n * K);
     k_rel_sources<<<nblk(n * K, 256), 256, 0, s>>>(c->d_pan_leaf, c->d_leaf_node, c->d_node_center, n, K, c->d_y,
                                                    c->d_w, c->d_y32, c->d_y64);
+    c->d_pnode.resize(n);
+    c->d_pg32.resize(16 * n);
+    c->d_pg64.resize(16 * n);
+    c->d_pg_ds.resize(16 * n);
+    k_panel_geo<<<nblk(n, 128), 128, 0, s>>>(c->d_pan_leaf, c->d_leaf_node, c->d_node_center, n, c->d_v, c->d_c,
+                                             c->d_n, c->d_pnode, c->d_pg32, c->d_pg64, (ds*)c->d_pg_ds.p);
     PGB_CUDA(cudaGetLastError());
     PGB_CUDA(cudaStreamSynchronize(s));
 }
@@ -1056,66 +1110,35 @@ __global__ void k_list_offsets(int64_t ng, const int64_t* off, const int32_t* id
     }
 }
 
-// P2P tiles: every near leaf of a group cut into runs of at most 32
-// quadrature points; descriptor = (leaf centre - group centre in FP32, first
-// point) and (leaf, count, flags: 1 Laplace pair, 2 leaf holds group targets, body).
-// One warp per group; the lanes take its near entries 32 at a time.
-__global__ void k_tile_count(int64_t ng, const int64_t* noff, const int32_t* nearl, const int32_t* nstart,
-                             const int32_t* nend, int K, int64_t* cnt) {
+// P2P columns: the panels of a group's near leaves one after another, in list
+// order; descriptor = (leaf centre - group centre in FP32, panel).  One warp
+// per group; the lanes take its near entries 32 at a time.
+__global__ void k_col_count(int64_t ng, const int64_t* noff, const int32_t* nearl, const int32_t* nstart,
+                            const int32_t* nend, int64_t* cnt) {
     const int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (g >= ng) return;
     int64_t c = 0;
-    for (int64_t e = noff[g] + lane; e < noff[g + 1]; e += 32) {
-        const int nd = nearl[e];
-        c += ((int64_t)(nend[nd] - nstart[nd]) * K + 31) / 32;
-    }
+    for (int64_t e = noff[g] + lane; e < noff[g + 1]; e += 32) c += nend[nearl[e]] - nstart[nearl[e]];
     for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
     if (lane == 0) cnt[g] = c;
 }
-// Tiles in entry order: a warp scan of the lanes' tile counts places each
-// entry's run after those of the entries before it.
-__global__ void k_tile_fill(int64_t ng, const int64_t* noff, const int32_t* nearl, const float4* near4,
-                            const int32_t* nstart, const int32_t* nend, const int32_t* nbody, const int32_t* gstart,
-                            const int32_t* gend, const int32_t* gbody, BodyDev bd, int K, const int64_t* toff,
-                            float4* td, int4* tm) {
+// The entries one after another, each entry's panels written by the warp.
+__global__ void k_col_fill(int64_t ng, const int64_t* noff, const int32_t* nearl, const float4* near4,
+                           const int32_t* nstart, const int32_t* nend, const int64_t* coff, float4* col) {
     const int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (g >= ng) return;
-    int64_t w = toff[g];
-    const int gb = gbody[g];
-    const int64_t e1 = noff[g + 1];
-    for (int64_t e0 = noff[g]; e0 < e1; e0 += 32) {
-        const int64_t e = e0 + lane;
-        int nd = 0;
-        int64_t s0 = 0, s1 = 0, nt = 0;
-        if (e < e1) {
-            nd = nearl[e];
-            s0 = (int64_t)nstart[nd] * K;
-            s1 = (int64_t)nend[nd] * K;
-            nt = (s1 - s0 + 31) / 32;
-        }
-        int64_t incl = nt;  // inclusive scan over the lanes
-        for (int o = 1; o < 32; o <<= 1) {
-            const int64_t v = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += v;
-        }
-        if (e < e1) {
-            const int nb = nbody[nd];
-            const int flags = ((nb == gb && bd.kind[gb] == PGB_DIELECTRIC) ? 1 : 0) |
-                              ((nstart[nd] < gend[g] && nend[nd] > gstart[g]) ? 2 : 0);
-            const float4 o = near4[e];
-            int64_t t = w + incl - nt;
-            for (int64_t q = s0; q < s1; q += 32, ++t) {
-                td[t] = make_float4(o.x, o.y, o.z, __int_as_float((int)q));
-                tm[t] = make_int4(nd, (int)min((int64_t)32, s1 - q), flags, nb);
-            }
-        }
-        w += __shfl_sync(0xffffffffu, incl, 31);
+    int64_t w = coff[g];
+    for (int64_t e = noff[g]; e < noff[g + 1]; ++e) {
+        const float4 o = near4[e];
+        const int s = nstart[nearl[e]], n = nend[nearl[e]] - s;
+        for (int q = lane; q < n; q += 32) col[w + q] = make_float4(o.x, o.y, o.z, __int_as_float(s + q));
+        w += n;
     }
 }
 
-// Work items per group: ceil(tiles / p2p_item) for P2P and
+// Work items per group: ceil(columns / pi) for P2P and
 // ceil(far entries / m2p_item) for M2P.
 __global__ void k_item_count(int64_t ng, const int64_t* toff, const int64_t* foff, int pi, int fi, int64_t* pc,
                              int64_t* fc) {
@@ -1207,19 +1230,16 @@ void build_lists(pgb_ctx* c) {
     {
         DBuf<int64_t> tc;
         tc.resize(ng);
-        c->d_tile_off.resize(ng + 1);
-        k_tile_count<<<nblk(32 * ng, 128), 128, 0, s>>>(ng, c->d_near_off, c->d_near, c->d_node_start, c->d_node_end,
-                                                   c->p.K, tc);
+        c->d_col_off.resize(ng + 1);
+        k_col_count<<<nblk(32 * ng, 128), 128, 0, s>>>(ng, c->d_near_off, c->d_near, c->d_node_start, c->d_node_end,
+                                                       tc);
         int64_t nt = 0;
-        exclusive_scan_i64(tc, c->d_tile_off, ng, s, &nt);
-        PGB_CUDA(cudaMemcpyAsync(c->d_tile_off.p + ng, &nt, 8, cudaMemcpyHostToDevice, s));
-        c->n_tiles = nt;
-        c->d_tile_d.resize(nt);
-        c->d_tile_m.resize(nt);
-        k_tile_fill<<<nblk(32 * ng, 128), 128, 0, s>>>(ng, c->d_near_off, c->d_near, c->d_near4, c->d_node_start,
-                                                  c->d_node_end, c->d_node_body, c->d_group_start, c->d_group_end,
-                                                  c->d_group_body, body_dev(c), c->p.K, c->d_tile_off, c->d_tile_d,
-                                                  c->d_tile_m);
+        exclusive_scan_i64(tc, c->d_col_off, ng, s, &nt);
+        PGB_CUDA(cudaMemcpyAsync(c->d_col_off.p + ng, &nt, 8, cudaMemcpyHostToDevice, s));
+        c->n_cols = nt;
+        c->d_col.resize(nt);
+        k_col_fill<<<nblk(32 * ng, 128), 128, 0, s>>>(ng, c->d_near_off, c->d_near, c->d_near4, c->d_node_start,
+                                                      c->d_node_end, c->d_col_off, c->d_col);
         PGB_CUDA(cudaGetLastError());
     }
     {
@@ -1228,8 +1248,8 @@ void build_lists(pgb_ctx* c) {
         fc.resize(ng);
         c->d_pitem_off.resize(ng + 1);
         c->d_fitem_off.resize(ng + 1);
-        k_item_count<<<nblk(ng, 128), 128, 0, s>>>(ng, c->d_tile_off, c->d_far_off, c->p.p2p_item, c->p.m2p_item,
-                                                   pc, fc);
+        k_item_count<<<nblk(ng, 128), 128, 0, s>>>(ng, c->d_col_off, c->d_far_off, p2p_item_cols(c->p.p2p_item, c->p.K),
+                                                   c->p.m2p_item, pc, fc);
         int64_t np = 0, nf = 0;
         exclusive_scan_i64(pc, c->d_pitem_off, ng, s, &np);
         exclusive_scan_i64(fc, c->d_fitem_off, ng, s, &nf);
@@ -1249,8 +1269,8 @@ void build_lists(pgb_ctx* c) {
     c->lists_valid = true;
 }
 
-// Offsets of the kept list entries and P2P tiles after the node and group
-// centres moved (pgb_tree_refresh): entries, tiles and work items stay.
+// Offsets of the kept list entries and P2P columns after the node and group
+// centres moved (pgb_tree_refresh): entries, columns and work items stay.
 void refresh_lists(pgb_ctx* c) {
     cudaStream_t s = c->stream;
     const int64_t ng = c->n_groups;
@@ -1259,10 +1279,8 @@ void refresh_lists(pgb_ctx* c) {
                                                c->d_near4);
     k_list_offsets<<<(unsigned)ng, 64, 0, s>>>(ng, c->d_far_off, c->d_far, c->d_node_center, c->d_group_center,
                                                c->d_far4);
-    k_tile_fill<<<nblk(32 * ng, 128), 128, 0, s>>>(ng, c->d_near_off, c->d_near, c->d_near4, c->d_node_start,
-                                                   c->d_node_end, c->d_node_body, c->d_group_start, c->d_group_end,
-                                                   c->d_group_body, body_dev(c), c->p.K, c->d_tile_off, c->d_tile_d,
-                                                   c->d_tile_m);
+    k_col_fill<<<nblk(32 * ng, 128), 128, 0, s>>>(ng, c->d_near_off, c->d_near, c->d_near4, c->d_node_start,
+                                                  c->d_node_end, c->d_col_off, c->d_col);
     PGB_CUDA(cudaGetLastError());
     PGB_CUDA(cudaStreamSynchronize(s));
     PGB_LAUNCHED(c, 3);

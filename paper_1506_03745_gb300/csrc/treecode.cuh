@@ -76,6 +76,16 @@ __device__ __forceinline__ ds4 cvt4<ds>(const dbl4& v) {
 __device__ __forceinline__ double to_dbl(float v) { return (double)v; }
 __device__ __forceinline__ double to_dbl(double v) { return v; }
 __device__ __forceinline__ double to_dbl(ds v) { return ds_to_double(v); }
+// a double in the arithmetic type
+template <typename real>
+__device__ __forceinline__ real from_dbl(double v) {
+    return (real)v;
+}
+template <>
+__device__ __forceinline__ ds from_dbl<ds>(double v) {
+    return ds_from_double(v);
+}
+
 // a double literal in the arithmetic type (split at compile time for ds)
 template <typename C>
 __device__ __forceinline__ C lit(double d) {
@@ -230,14 +240,19 @@ struct EvalArgs {
     const unsigned long long* bmask = nullptr;
     const float4* near4;           // per near entry: leaf centre - group centre, node id bits
     const float4* far4;            // per far entry: node centre - group centre, node id bits
-    const int64_t* tile_off;       // per group: its P2P tiles [tile_off[g], tile_off[g+1])
-    const float4* tile_d;          // per tile: leaf centre - group centre (FP32), first point (int bits)
-    const int4* tile_m;            // per tile: leaf node, point count, flags (1 Laplace, 2 own panel), body
-    // work items (a group's tiles / far entries in runs of p2p_item / m2p_item)
+    const int64_t* col_off;        // per group: its P2P columns [col_off[g], col_off[g+1])
+    const float4* col;             // per column: leaf centre - group centre (FP32), panel (int bits)
+    const int32_t* pnode;          // leaf node of a panel (FP64 and double-single offsets)
+    const int32_t* pbody;          // body of a panel
+    const void* pg;                // panel geometry (PanelGeo) in the kernel's arithmetic
+    const void* pd;                // panel densities x area, same arithmetic: {psiL, psiY, phi, unused}
+    FarRule rule;
+    unsigned long long src_mask;   // bit b: src_active[b]
+    // work items (a group's columns in even runs, its far entries in runs of m2p_item)
     int64_t n_pitems, n_fitems;
     const int64_t *pitem_off, *fitem_off;  // per group
     const int32_t *pitem_group, *fitem_group;
-    int p2p_item, m2p_item;
+    int m2p_item;
     double *Up, *Uf;               // per item: 32 Laplace then 32 Yukawa partial sums (one per lane)
     // persistent launch: a grid smaller than the item count whose blocks take
     // items from these counters (zero before the launch); nullptr: one item per block
@@ -376,56 +391,116 @@ __device__ __forceinline__ void far_eval(real Rx, real Ry, real Rz, real kappa, 
     uL = LAP ? aL * ri : real(0);
 }
 
-// K-point sums of one tile of source points for one target (relative position
-// r0 = target - leaf centre).  With OWN, points of the target's own panel
-// (indices [own_lo, own_hi)) are skipped.
-template <typename real, bool LAP, bool OWN>
-__device__ __forceinline__ void p2p_tile(const typename V4<real>::t* sA, const typename V4<real>::t* sB, int cnt,
-                                         int64_t t, int64_t own_lo, int64_t own_hi, real r0x, real r0y, real r0z,
-                                         real kappa, real& sumL, real& sumY) {
-    using v4 = typename V4<real>::t;
-    const real nkl = -kappa * lit<real>(1.4426950408889634);  // -kappa log2(e)
-    real sL2 = 0, sY2 = 0;  // second accumulator pair: two independent chains
-#pragma unroll 4
-    for (int j = 0; j < cnt; ++j) {
-        const v4 A = sA[j], B = sB[j];
-        const real dx = r0x - A.x, dy = r0y - A.y, dz = r0z - A.z;
-        real r2;
-        if constexpr (is_ds<real>) r2 = madd(dx, dx, madd(dy, dy, dz * dz));
-        else r2 = dx * dx + dy * dy + dz * dz;
-        // a quadrature node of another panel never coincides with a target
-        // centroid on a valid (non-overlapping) mesh; only the target's own
-        // panel, in the leaf that holds the group, needs the exclusion
-        real ri = rsqrt_fast(r2);
-        if (OWN) ri = (r2 > real(0) && !(t + j >= own_lo && t + j < own_hi)) ? ri : real(0);
-        real pd;
-        if constexpr (is_ds<real>) pd = madd(B.x, dx, madd(B.y, dy, B.z * dz));
-        else pd = B.x * dx + B.y * dy + B.z * dz;
-        const real tt = pd * (ri * ri);
-        const real r = r2 * ri;
-        const real ex = exp2_(nkl * r);
-        if constexpr (is_ds<real>) {
-            const ds yw = madd(-madd(kappa, r, ds(1)), tt, B.w);  // B.w - (kappa r + 1) tt
-            if (j & 1) {
-                if (LAP) sL2 = madd(ri, A.w - tt, sL2);
-                sY2 = madd(ex * ri, yw, sY2);
-            } else {
-                if (LAP) sumL = madd(ri, A.w - tt, sumL);
-                sumY = madd(ex * ri, yw, sumY);
+// Arithmetic of the P2P sums: the compiler's contracted forms in FP32 and
+// FP64, double-single without renormalisation where no cancellation follows.
+__device__ __forceinline__ float mul_(float a, float b) { return a * b; }
+__device__ __forceinline__ double mul_(double a, double b) { return a * b; }
+__device__ __forceinline__ ds mul_(ds a, ds b) { return ds_mul_u(a, b); }
+__device__ __forceinline__ float add_(float a, float b) { return a + b; }
+__device__ __forceinline__ double add_(double a, double b) { return a + b; }
+__device__ __forceinline__ ds add_(ds a, ds b) { return ds_add_u(a, b); }
+__device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ ds fma_(ds a, ds b, ds c) { return ds_fma_u(a, b, c); }
+__device__ __forceinline__ float norm_(float a) { return a; }
+__device__ __forceinline__ double norm_(double a) { return a; }
+__device__ __forceinline__ ds norm_(ds a) { return ds_norm(a); }
+// 1/sqrt of a squared distance formed with a cancellation: a value rounded
+// below zero is taken by its magnitude (FP32; the others keep 50 bits more
+// than the distances that occur)
+__device__ __forceinline__ float rsqrt_abs(float x) { return rsqrt_fast(fabsf(x)); }
+__device__ __forceinline__ double rsqrt_abs(double x) { return rsqrt_fast(x); }
+__device__ __forceinline__ ds rsqrt_abs(ds x) { return ds_rsqrt(x); }
+
+// One panel staged for the P2P sums: the centroid relative to the group's
+// centre (PanelGeo holds it relative to the leaf's), 2 (v_0 - c), 2 (v_1 - c),
+// the unit normal, g_k = |v_k - c|^2, and the densities times the area:
+// {psi_L, psi_Y, phi of the Laplace pair, phi}; the Laplace two are zero
+// unless the panel and the group share a dielectric body.
+template <typename real>
+struct __align__(16) PanelS {
+    real cx, cy, cz, g0;
+    real ux, uy, uz, g1;
+    real vx, vy, vz, g2;
+    real nx, ny, nz, qL;
+    real qY, pL, pY, pad;
+};
+
+// Sums over the far rule's points of one panel for one target at X (relative
+// to the group's centre).  The rule's points are c and c - 3 alpha s_k, s_k =
+// v_k - c, so with d = X - c and a = 3 alpha
+//   |X - y|^2 = |d|^2 + a (2 d.s_k + a |s_k|^2),
+// two operations a point instead of six, and n.(X - y) = n.d is the panel's:
+//   V = sum w / r, K = n.d sum w / r^3 (Laplace), with e^{-kappa r} and
+//   (1 + kappa r) e^{-kappa r} for Yukawa; U += q V - p K.
+// The densities and the normal product are met once per panel.  In FP32 a
+// point costs 15 FMA-pipe operations with the panel's share (19 point by
+// point) and 2 MUFU (16 cycles a warp), and a panel five 16-byte shared loads
+// instead of 14; in double-single 185 operations (320).  The squared distance
+// loses a factor |d|^2 / r^2 of relative accuracy, below ten on shape-regular
+// panels, of the order of what the FP32 coordinates leave.
+template <typename real, int K, bool LAP, bool OWN>
+__device__ __forceinline__ void p2p_panel(const PanelS<real>& q, bool own, real X, real Y, real Z, real kappa,
+                                          real nkl, const real (&ra)[2], const real (&rw)[3], real& UL, real& UY) {
+    const real dx = X - q.cx, dy = Y - q.cy, dz = Z - q.cz;
+    const real D2 = norm_(fma_(dz, dz, fma_(dy, dy, mul_(dx, dx))));
+    const real h = fma_(q.nz, dz, fma_(q.ny, dy, mul_(q.nx, dx)));
+    const real one = real(1);
+    real VL = real(0), KL = real(0), VY = real(0), KY = real(0);
+    auto point = [&](const real r2, real& sV, real& sK, real& sW, real& sM, bool first) {
+        const real ri = rsqrt_abs(r2);
+        const real i2 = mul_(ri, ri);
+        const real r = mul_(r2, ri);
+        const real e = mul_(exp2_(mul_(nkl, r)), ri);
+        const real gg = fma_(kappa, r, one);
+        const real e2 = mul_(e, i2);
+        if (first) {
+            if (LAP) {
+                sV = ri;
+                sK = mul_(ri, i2);
             }
+            sW = e;
+            sM = mul_(e2, gg);
         } else {
-            const real gg = kappa * r + real(1);
-            if (j & 1) {
-                if (LAP) sL2 += ri * (A.w - tt);
-                sY2 += (ex * ri) * (B.w - gg * tt);
-            } else {
-                if (LAP) sumL += ri * (A.w - tt);
-                sumY += (ex * ri) * (B.w - gg * tt);
+            if (LAP) {
+                sV = add_(sV, ri);
+                sK = fma_(ri, i2, sK);
             }
+            sW = add_(sW, e);
+            sM = fma_(e2, gg, sM);
+        }
+    };
+    if (K != 3) {
+        real sV, sK, sW, sM;
+        point(D2, sV, sK, sW, sM, true);
+        if (LAP) {
+            VL = mul_(rw[0], sV);
+            KL = mul_(rw[0], sK);
+        }
+        VY = mul_(rw[0], sW);
+        KY = mul_(rw[0], sM);
+    }
+    if (K >= 3) {
+        const real p0 = norm_(fma_(q.uz, dz, fma_(q.uy, dy, mul_(q.ux, dx))));
+        const real p1 = norm_(fma_(q.vz, dz, fma_(q.vy, dy, mul_(q.vx, dx))));
+        const real p2 = -norm_(add_(p0, p1));
+#pragma unroll
+        for (int o = 0; o < (K == 7 ? 2 : 1); ++o) {
+            real sV, sK, sW, sM;
+            point(norm_(fma_(ra[o], fma_(ra[o], q.g0, p0), D2)), sV, sK, sW, sM, true);
+            point(norm_(fma_(ra[o], fma_(ra[o], q.g1, p1), D2)), sV, sK, sW, sM, false);
+            point(norm_(fma_(ra[o], fma_(ra[o], q.g2, p2), D2)), sV, sK, sW, sM, false);
+            if (LAP) {
+                VL = fma_(rw[1 + o], sV, VL);
+                KL = fma_(rw[1 + o], sK, KL);
+            }
+            VY = fma_(rw[1 + o], sW, VY);
+            KY = fma_(rw[1 + o], sM, KY);
         }
     }
-    sumL += sL2;
-    sumY += sY2;
+    if (OWN && own) VL = KL = VY = KY = real(0);  // the panel's own integral is a near-field correction
+    if (LAP) UL = fma_(q.qL, VL, fma_(mul_(-q.pL, h), KL, UL));
+    UY = fma_(q.qY, VY, fma_(mul_(-q.pY, h), KY, UY));
 }
 
 // One block of NW warps per target group (32 targets, one per lane): the
@@ -475,98 +550,140 @@ __device__ __forceinline__ void store_item(real (*red)[4][32], int w, int lane, 
     }
 }
 
-// P2P: one block of NW warps per work item, i.e. up to p2p_item source tiles
-// (up to 32 quadrature points of one near leaf each) of one target group (32
-// targets, one per lane); the tiles are dealt round robin to the warps, the
-// next tile prefetched into registers.  The item's partial sums go to Up.
-// The source terms come in the arithmetic type (for double-single, split
-// once per product by k_src_to_ds); the targets in the storage type.
-template <typename real, int NW>
-__global__ void __launch_bounds__(NW * 32) k_p2p(EvalArgs a, const typename V4<real>::t* __restrict__ src,
-                                                 const typename V4<typename Store<real>::S>::t* __restrict__ xrel) {
-    using S = typename Store<real>::S;  // storage type of the inputs
-    using v4 = typename V4<real>::t;
-    using s4 = typename V4<S>::t;
-    __shared__ v4 sA[NW][32], sB[NW][32];
+// Offset of a column's leaf centre from the group's centre: from the column in
+// FP32, formed in FP64 from the centres otherwise.
+template <typename real>
+__device__ __forceinline__ void col_offset(const EvalArgs& a, const float4& c, int j, int64_t g, real& ox, real& oy,
+                                           real& oz) {
+    if constexpr (sizeof(real) == sizeof(float)) {
+        ox = c.x;
+        oy = c.y;
+        oz = c.z;
+    } else {
+        const int nd = a.pnode[j];
+        ox = from_dbl<real>(a.ncenter[3 * nd] - a.gcenter[3 * g]);
+        oy = from_dbl<real>(a.ncenter[3 * nd + 1] - a.gcenter[3 * g + 1]);
+        oz = from_dbl<real>(a.ncenter[3 * nd + 2] - a.gcenter[3 * g + 2]);
+    }
+}
+
+// P2P: one block of NW warps per work item, i.e. an even share of the columns
+// (panels of the near leaves) of one target group (32 targets, one per lane).
+// The item's columns go to the warps in NW even runs; a warp stages up to 32
+// panels at a time, one per lane, moved to the group's frame, and every lane
+// then sums them for its target (p2p_panel).  The panels of several leaves
+// share a stage, so a warp's steps are full whatever the leaf sizes.  The
+// item's partial sums go to Up.
+template <typename real, int K, int NW>
+__global__ void __launch_bounds__(NW * 32) k_p2p(EvalArgs a, const typename V4<typename Store<real>::S>::t* __restrict__ xrel) {
+    using S = typename Store<real>::S;  // storage type of the targets
+    __shared__ __align__(16) PanelS<real> sP[NW][32];
     __shared__ real red[NW][4][32];
     __shared__ int64_t s_item;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const unsigned long long dm = body_mask(a.bmask);
-    for (int64_t it = next_item(a.p2p_work, -1, &s_item); it < a.n_pitems; it = next_item(a.p2p_work, it, &s_item)) {
-    const int64_t g = a.pitem_group[it];
-    if (!(((a.tgt_mask & dm) >> a.gbody[g]) & 1ull) || g < a.g_lo || g >= a.g_hi) continue;  // rows not used (block-uniform)
-    const int64_t p0 = a.gstart[g], p1 = a.gend[g];
-    const int64_t p = p0 + lane;
-    const bool active = p < p1;
-    const s4 xr = active ? xrel[p] : xrel[p0];
-    const double gc0 = a.gcenter[3 * g], gc1 = a.gcenter[3 * g + 1], gc2 = a.gcenter[3 * g + 2];
+    const unsigned long long dm = body_mask(a.bmask), act = a.src_mask & dm;
     const real kappa = to_c<real>((S)a.kappa);
-    const int64_t own_lo = p * a.K, own_hi = own_lo + a.K;
-    real UL = 0, cL = 0, UY = 0, cY = 0;
-    const int64_t tb = a.tile_off[g] + (it - a.pitem_off[g]) * a.p2p_item;
-    const int64_t t1 = min(a.tile_off[g + 1], tb + a.p2p_item);
-    int64_t t = tb + w;
-    v4 pa = v4(), pb = v4();
-    int4 m = make_int4(0, 0, 0, 0);
-    float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (t < t1) {
-        d = a.tile_d[t];
-        m = a.tile_m[t];
-        if (lane < m.y) {
-            const int64_t q = (int64_t)__float_as_int(d.w) + lane;
-            pa = src[2 * q];
-            pb = src[2 * q + 1];
-        }
-    }
-    while (t < t1) {
-        const int cnt = m.y, flags = m.z | (a.src_active[m.w] && ((dm >> m.w) & 1ull) ? 0 : 4);
-        const int64_t first = (int64_t)__float_as_int(d.w);
-        // target relative to the leaf centre: FP32 from the tile's offset,
-        // else formed in FP64 (and split for double-single)
-        real r0x, r0y, r0z;
-        if constexpr (sizeof(real) == sizeof(float)) {
-            r0x = xr.x - (real)d.x;
-            r0y = xr.y - (real)d.y;
-            r0z = xr.z - (real)d.z;
-        } else {
-            const int nd = m.x;
-            const S ox = (S)(a.ncenter[3 * nd] - gc0);
-            const S oy = (S)(a.ncenter[3 * nd + 1] - gc1);
-            const S oz = (S)(a.ncenter[3 * nd + 2] - gc2);
-            r0x = to_c<real>(xr.x - ox);
-            r0y = to_c<real>(xr.y - oy);
-            r0z = to_c<real>(xr.z - oz);
-        }
-        __syncwarp();
-        if (lane < cnt) {
-            sA[w][lane] = pa;
-            sB[w][lane] = pb;
-        }
-        __syncwarp();
-        t += NW;
-        if (t < t1) {  // prefetch this warp's next tile
-            d = a.tile_d[t];
-            m = a.tile_m[t];
-            if (lane < m.y) {
-                const int64_t q = (int64_t)__float_as_int(d.w) + lane;
-                pa = src[2 * q];
-                pb = src[2 * q + 1];
+    const real nkl = -kappa * lit<real>(1.4426950408889634);  // -kappa log2(e)
+    const real ra[2] = {from_dbl<real>(a.rule.a[0]), from_dbl<real>(a.rule.a[1])};
+    const real rw[3] = {from_dbl<real>(a.rule.w[0]), from_dbl<real>(a.rule.w[1]), from_dbl<real>(a.rule.w[2])};
+    const real* __restrict__ pg = (const real*)a.pg;
+    const real* __restrict__ pd = (const real*)a.pd;
+    for (int64_t it = next_item(a.p2p_work, -1, &s_item); it < a.n_pitems; it = next_item(a.p2p_work, it, &s_item)) {
+        const int64_t g = a.pitem_group[it];
+        const int gb = a.gbody[g];
+        if (!(((a.tgt_mask & dm) >> gb) & 1ull) || g < a.g_lo || g >= a.g_hi) continue;  // rows not used (block-uniform)
+        const int p0 = a.gstart[g], p1 = a.gend[g];
+        const int p = p0 + lane;
+        const typename V4<S>::t xr = xrel[p < p1 ? p : p0];
+        const real X = to_c<real>(xr.x), Y = to_c<real>(xr.y), Z = to_c<real>(xr.z);
+        const bool glap = a.lap_body[gb];
+        real UL = 0, cL = 0, UY = 0, cY = 0;
+        // the item's columns, then this warp's
+        const int64_t i0 = a.pitem_off[g], c0 = a.col_off[g], nc = a.col_off[g + 1] - c0;
+        const int64_t per = (nc + a.pitem_off[g + 1] - i0 - 1) / (a.pitem_off[g + 1] - i0);
+        const int64_t b0 = c0 + (it - i0) * per, b1 = min(c0 + nc, b0 + per);
+        const int64_t wper = b1 > b0 ? (b1 - b0 + NW - 1) / NW : 0;
+        const int64_t w1 = min(b1, b0 + (w + 1) * wper);
+        for (int64_t e = b0 + w * wper; e < w1; e += 32) {
+            const int cnt = (int)min((int64_t)32, w1 - e);
+            bool lap = false, has_own = false;
+            int own = -1;  // the stage's slot of this lane's own panel
+            __syncwarp();
+            int j = -1;
+            if (lane < cnt) {
+                const float4 c = a.col[e + lane];
+                j = __float_as_int(c.w);
+                const int b = a.pbody[j];
+                lap = glap && b == gb;
+                has_own = j >= p0 && j < p1;
+                real ox, oy, oz;
+                col_offset<real>(a, c, j, g, ox, oy, oz);
+                PanelS<real>& q = sP[w][lane];
+                const PanelS<real>& v = *reinterpret_cast<const PanelS<real>*>(pg + 16 * (int64_t)j);  // its first 15 values
+                q.cx = v.cx + ox;
+                q.cy = v.cy + oy;
+                q.cz = v.cz + oz;
+                q.g0 = v.g0;
+                q.ux = v.ux;
+                q.uy = v.uy;
+                q.uz = v.uz;
+                q.g1 = v.g1;
+                q.vx = v.vx;
+                q.vy = v.vy;
+                q.vz = v.vz;
+                q.g2 = v.g2;
+                q.nx = v.nx;
+                q.ny = v.ny;
+                q.nz = v.nz;
+                const bool on = (act >> b) & 1ull;  // a body without density in this product adds nothing
+                const real z = real(0);
+                q.qL = on && lap ? pd[4 * (int64_t)j] : z;
+                q.qY = on ? pd[4 * (int64_t)j + 1] : z;
+                const real ph = on ? pd[4 * (int64_t)j + 2] : z;
+                q.pL = lap ? ph : z;
+                q.pY = ph;
             }
+            lap = __any_sync(0xffffffffu, lap);
+            has_own = __any_sync(0xffffffffu, has_own);
+            if (has_own)
+                for (int k = 0; k < cnt; ++k)
+                    if (__shfl_sync(0xffffffffu, j, k) == p) own = k;
+            __syncwarp();
+            real sumL = 0, sumY = 0;
+            if (has_own) {
+                if (lap)
+                    for (int k = 0; k < cnt; ++k)
+                        p2p_panel<real, K, true, true>(sP[w][k], k == own, X, Y, Z, kappa, nkl, ra, rw, sumL, sumY);
+                else
+                    for (int k = 0; k < cnt; ++k)
+                        p2p_panel<real, K, false, true>(sP[w][k], k == own, X, Y, Z, kappa, nkl, ra, rw, sumL, sumY);
+            } else if (lap) {
+                for (int k = 0; k < cnt; ++k)
+                    p2p_panel<real, K, true, false>(sP[w][k], false, X, Y, Z, kappa, nkl, ra, rw, sumL, sumY);
+            } else {
+                for (int k = 0; k < cnt; ++k)
+                    p2p_panel<real, K, false, false>(sP[w][k], false, X, Y, Z, kappa, nkl, ra, rw, sumL, sumY);
+            }
+            kadd(UL, cL, sumL);
+            kadd(UY, cY, sumY);
         }
-        real sumL = 0, sumY = 0;
-        if (flags & 4) {
-            // source body without density in this product (imposed-boundary terms)
-        } else if (flags & 2) {
-            if (flags & 1) p2p_tile<real, true, true>(sA[w], sB[w], cnt, first, own_lo, own_hi, r0x, r0y, r0z, kappa, sumL, sumY);
-            else p2p_tile<real, false, true>(sA[w], sB[w], cnt, first, own_lo, own_hi, r0x, r0y, r0z, kappa, sumL, sumY);
-        } else {
-            if (flags & 1) p2p_tile<real, true, false>(sA[w], sB[w], cnt, first, own_lo, own_hi, r0x, r0y, r0z, kappa, sumL, sumY);
-            else p2p_tile<real, false, false>(sA[w], sB[w], cnt, first, own_lo, own_hi, r0x, r0y, r0z, kappa, sumL, sumY);
-        }
-        kadd(UL, cL, sumL);
-        kadd(UY, cY, sumY);
+        store_item<real, NW>(red, w, lane, UL, cL, UY, cY, a.Up + 64 * it);
     }
-    store_item<real, NW>(red, w, lane, UL, cL, UY, cY, a.Up + 64 * it);
+}
+
+// The P2P launch for the context's far rule.
+template <typename real>
+void launch_p2p(const EvalArgs& ev, int K, const void* xrel, cudaStream_t s) {
+    constexpr int NW = 8;  // warps per block
+    using x4 = typename V4<typename Store<real>::S>::t;
+    if (ev.n_pitems <= 0) return;
+    const unsigned grid = (unsigned)(ev.p2p_work ? ev.persist_blocks : ev.n_pitems);
+    switch (K) {
+        case 1: k_p2p<real, 1, NW><<<grid, NW * 32, 0, s>>>(ev, (const x4*)xrel); break;
+        case 3: k_p2p<real, 3, NW><<<grid, NW * 32, 0, s>>>(ev, (const x4*)xrel); break;
+        case 4: k_p2p<real, 4, NW><<<grid, NW * 32, 0, s>>>(ev, (const x4*)xrel); break;
+        case 7: k_p2p<real, 7, NW><<<grid, NW * 32, 0, s>>>(ev, (const x4*)xrel); break;
+        default: fail(PGB_EINVAL, "K must be 1, 3, 4 or 7");
     }
 }
 
@@ -941,16 +1058,6 @@ __device__ __forceinline__ ds ld_cg(const ds* p) {
     const float2 v = __ldcg(reinterpret_cast<const float2*>(p));
     return ds(v.x, v.y);
 }
-// a double in the arithmetic type
-template <typename real>
-__device__ __forceinline__ real from_dbl(double v) {
-    return (real)v;
-}
-template <>
-__device__ __forceinline__ ds from_dbl<ds>(double v) {
-    return ds_from_double(v);
-}
-
 // P2M of node nd (a leaf) into mom[nd]: the moments about its centre,
 // u = c - y, one thread per multi-index k (two when T > 128).  The
 // double-layer part is split off:

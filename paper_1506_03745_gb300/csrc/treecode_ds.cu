@@ -7,7 +7,7 @@
 namespace pgb {
 
 // FP64 source terms split into double-single once per product, so that the
-// P2P tiles stage them without conversion.
+// P2P and P2M stage them without conversion.
 __global__ void k_src_to_ds(const dbl4* __restrict__ in, ds4* __restrict__ out, int64_t n) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i < n) out[i] = cvt4<ds>(in[i]);
