@@ -467,7 +467,7 @@ int solve_seg(pgb_ctx* c, int mode, double tol, int max_iter, int restart, doubl
     std::vector<int> its(B);
     if (mode != PGB_FP32_REFINE) {
         const int prec = mode == PGB_FP64 ? PGB_FP64 : PGB_FP32;
-        for (int p = 0; p < B; ++p) tolv[p] = tol * bn[p];
+        for (int p = 0; p < B; ++p) tolv[p] = (prec == PGB_FP32 ? PGB_FP32_STOP : 1.0) * tol * bn[p];
         int mv = 0;
         gmres_seg(c, prec, c->d_b, x, tolv.data(), max_iter, restart, &mv, its.data(), est.data(), true);
         apply_operator(c, x, c->d_r, prec, false);

@@ -22,7 +22,7 @@
 // (2^j j! (2d-1)!!).  (Lap^m (|s|^{2m} h) = 2^m m! prod_i (2i + 2d + 1) h for
 // harmonic h of degree d, and the other parts of mu_n project to zero.)
 //
-// Table layout (T = (P+1)(P+2)(P+3)/6): rows = output coefficients in the
+// The table of pgb_far_table (T = (P+1)(P+2)(P+3)/6): rows = output coefficients in the
 // evaluation order (a = 0..P, b = 0..P-a, c = 0..P-a-b for S^(a,b,c)), columns
 // = moments in the graded order of the upward pass (degree, then kx and ky
 // descending); the Yukawa table (T x T) then the Laplace table (T x T).
@@ -138,64 +138,107 @@ void far_tables(int P, double kappa, std::vector<double>& tab) {
     }
 }
 
-// Device copy of the tables for the context's P and the screening kappa
-// (one per kappa: the solvent, and each region of a nested system), in FP64,
-// double-single and FP32 (transposed dense, and packed for orders above 8).
+// The kernels evaluate E_p in a basis of the harmonic polynomials of degree p
+// (2p + 1 coefficients instead of (p + 1)(p + 2)/2 monomial ones):
+//   B_{l,m} = q_{l,m} Re (x + i y)^m and q_{l,m} Im (x + i y)^m, m = 0..l,
+//   q_{m,m} = 1,  q_{l+1,m} = z q_{l,m} - c_{l,m} |s|^2 q_{l-1,m},
+//   c_{l,m} = (l^2 - m^2) / (4 l^2 - 1)
+// (the z-polynomials of the associated Legendre functions, leading
+// coefficient 1).  In the inner product <s^a, s^b> = a! delta_ab (Fischer) the
+// multiples of |s|^2 are orthogonal to the harmonics and |s|^2 is adjoint to
+// the Laplacian, so the coefficient of B in h_{n,j}, n = l + 2j, for the
+// moment M_k (|k| = n, mu_n = s^k / k!) is
+//   [coefficient of s^k in |s|^{2j} B] / (norm_j <B, B>),
+// norm_j = 2^j j! prod_{i=1..j} (2l + 2i + 1) as above.
+//
+// Device layout: the Yukawa then the Laplace table, each transposed, tab[k][j]:
+// k the moment, rows of far_cols(P) columns, j = l^2 (m = 0), l^2 + 2m - 1
+// (Re, m > 0) or l^2 + 2m (Im); zero where degree |k| < l or of other parity
+// (Yukawa), or |k| != l (Laplace).
+static void far_harmonics(int P, double kappa, std::vector<double>& tab) {
+    const int T = n_terms(P), TR = far_cols(P);
+    tab.assign(2 * (size_t)T * TR, 0.0);
+    auto times_z = [](int d, const Poly& f) {
+        Poly out(n_deg(d + 1), 0.0);
+        for (int a = 0; a <= d; ++a)
+            for (int b = 0; b <= d - a; ++b) out[pos(d + 1, a, b)] = f[pos(d, a, b)];
+        return out;
+    };
+    Poly re(1, 1.0), im(1, 0.0);  // (x + i y)^m
+    for (int m = 0; m <= P; ++m) {
+        for (int s = 0; s < (m ? 2 : 1); ++s) {
+            Poly prev, cur = s ? im : re;
+            for (int l = m; l <= P; ++l) {
+                const int j = l * l + (m ? 2 * m - 1 + s : 0);
+                double bb = 0;
+                for (int a = 0; a <= l; ++a)
+                    for (int b = 0; b <= l - a; ++b) {
+                        const double v = cur[pos(l, a, b)];
+                        bb += v * v * fact(a) * fact(b) * fact(l - a - b);
+                    }
+                Poly f = cur;
+                double norm = bb;
+                for (int i = 0; l + 2 * i <= P; ++i) {
+                    const int n = l + 2 * i;
+                    if (i > 0) {
+                        f = times_r2(n - 2, f);
+                        norm *= 2.0 * i * (2 * l + 2 * i + 1);
+                    }
+                    const int k0 = n == 0 ? 0 : n_terms(n - 1);
+                    for (int k = 0; k < n_deg(n); ++k) {
+                        tab[(size_t)(k0 + k) * TR + j] = pow(kappa, 2 * i) * f[k] / norm;
+                        if (i == 0)
+                            tab[(size_t)(T + k0 + k) * TR + j] =
+                                ((l & 1) ? -1.0 : 1.0) * dfact(2 * l - 1) * f[k] / norm;
+                    }
+                }
+                const double c = (double)(l * l - m * m) / (4.0 * l * l - 1.0);
+                Poly next = times_z(l, cur);
+                if (l > m) {
+                    const Poly r = times_r2(l - 1, prev);
+                    for (size_t q = 0; q < next.size(); ++q) next[q] -= c * r[q];
+                }
+                prev = cur;
+                cur = next;
+            }
+        }
+        Poly nre(n_deg(m + 1), 0.0), nim(n_deg(m + 1), 0.0);
+        for (int a = 0; a <= m; ++a)
+            for (int b = 0; b <= m - a; ++b) {
+                const double u = re[pos(m, a, b)], v = im[pos(m, a, b)];
+                nre[pos(m + 1, a + 1, b)] += u;
+                nim[pos(m + 1, a, b + 1)] += u;
+                nre[pos(m + 1, a, b + 1)] -= v;
+                nim[pos(m + 1, a + 1, b)] += v;
+            }
+        re = nre;
+        im = nim;
+    }
+}
+
+// Device copy of the harmonic tables for the context's P and the screening
+// kappa (one per kappa: the solvent, and each region of a nested system), in
+// FP64, double-single and FP32.
 const FarTab& far_table(pgb_ctx* c, double kappa) {
     for (const auto& t : c->far_tabs)
         if (t->P == c->p.P && t->kappa == kappa) return *t;
-    std::vector<double> rowmajor;
-    far_tables(c->p.P, kappa, rowmajor);
-    // device layout: packed rows in the graded order of the moments, per row
-    // the Yukawa entries over the moment degrees p, p + 2, ..., P then the
-    // Laplace entries over degree p (k_far_coef)
-    const int P = c->p.P, T = n_terms(P);
-    std::vector<int> ev((P + 1) * (P + 1) * (P + 1), -1);
-    {
-        int e = 0;
-        for (int a = 0; a <= P; ++a)
-            for (int b = 0; b <= P - a; ++b)
-                for (int cc = 0; cc <= P - a - b; ++cc) ev[(a * (P + 1) + b) * (P + 1) + cc] = e++;
-    }
     std::vector<double> h;
-    for (int n = 0; n <= P; ++n)
-        for (int a = n; a >= 0; --a)
-            for (int b = n - a; b >= 0; --b) {
-                const int row = ev[(a * (P + 1) + b) * (P + 1) + (n - a - b)];
-                for (int q = n; q <= P; q += 2)
-                    for (int k = (q > 0 ? n_terms(q - 1) : 0); k < n_terms(q); ++k)
-                        h.push_back(rowmajor[(size_t)row * T + k]);
-                for (int k = (n > 0 ? n_terms(n - 1) : 0); k < n_terms(n); ++k)
-                    h.push_back(rowmajor[(size_t)T * T + (size_t)row * T + k]);
-            }
-    // FP32 layout: each table transposed, tab[k][j] with rows of far_tr(P)
-    // columns (k_far_f32), Yukawa then Laplace
-    const int TR = (((T + 3) & ~3) + 31) & ~31;
-    std::vector<float> hf(2 * (size_t)T * TR, 0.f);
-    for (int q = 0; q < 2; ++q)
-        for (int j = 0; j < T; ++j)
-            for (int k = 0; k < T; ++k)
-                hf[(size_t)q * T * TR + (size_t)k * TR + j] = (float)rowmajor[(size_t)q * T * T + (size_t)j * T + k];
+    far_harmonics(c->p.P, kappa, h);
     auto t = std::make_unique<FarTab>();
     t->P = c->p.P;
     t->kappa = kappa;
     // double-single: hi = the FP32 rounding, lo = the FP32 rounding of the rest
-    std::vector<float> hds(2 * h.size());
+    std::vector<float> hf(h.size()), hds(2 * h.size());
     for (size_t q = 0; q < h.size(); ++q) {
-        const float hi = (float)h[q];
-        hds[2 * q] = hi;
-        hds[2 * q + 1] = (float)(h[q] - (double)hi);
+        hf[q] = hds[2 * q] = (float)h[q];
+        hds[2 * q + 1] = (float)(h[q] - (double)hf[q]);
     }
-    std::vector<float> hp(h.size());
-    for (size_t q = 0; q < h.size(); ++q) hp[q] = (float)h[q];
     t->t64.resize(h.size());
     t->t32.resize(hf.size());
     t->tds.resize(h.size());
-    t->t32p.resize(hp.size());
     PGB_CUDA(cudaMemcpyAsync(t->t64.p, h.data(), 8 * h.size(), cudaMemcpyHostToDevice, c->stream));
     PGB_CUDA(cudaMemcpyAsync(t->t32.p, hf.data(), 4 * hf.size(), cudaMemcpyHostToDevice, c->stream));
     PGB_CUDA(cudaMemcpyAsync(t->tds.p, hds.data(), 4 * hds.size(), cudaMemcpyHostToDevice, c->stream));
-    PGB_CUDA(cudaMemcpyAsync(t->t32p.p, hp.data(), 4 * hp.size(), cudaMemcpyHostToDevice, c->stream));
     PGB_CUDA(cudaStreamSynchronize(c->stream));
     c->far_tabs.push_back(std::move(t));
     return *c->far_tabs.back();

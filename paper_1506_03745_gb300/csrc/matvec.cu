@@ -21,6 +21,7 @@ static inline int nblk(int64_t n, int t) { return (int)std::max<int64_t>(1, (n +
 // A = {y - c_leaf, w psi_L}, B = {w phi n, w psi_Y}.
 //   dielectric: psi_L = dphi, psi_Y = (eps_in/eps_out) dphi, phi = phi
 //   imposed potential: psi_Y = u; imposed charge: phi = u
+// pd: the panel densities times the area (and wcorr, far_rule_f32_scale, in FP32).
 // known == true builds the imposed-boundary densities instead: phi0 as the
 // double-layer density of an imposed-potential surface, dphi = -sigma0/eps_out
 // as the single layer of an imposed-charge surface, zero on molecules.
@@ -29,7 +30,8 @@ static inline int nblk(int64_t n, int t) { return (int)std::max<int64_t>(1, (n +
 template <typename real>
 __global__ void k_src_prep(Geo g, BodyDev bd, const double* __restrict__ x, int mode,
                            const typename V4<real>::t* __restrict__ yrel, typename V4<real>::t* __restrict__ src,
-                           typename V4<real>::t* __restrict__ pd, real* __restrict__ dens, double eps_out) {
+                           typename V4<real>::t* __restrict__ pd, real* __restrict__ dens, double eps_out,
+                           double wcorr) {
     const bool known = mode == 1;
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= g.n_pan) return;
@@ -63,7 +65,7 @@ __global__ void k_src_prep(Geo g, BodyDev bd, const double* __restrict__ x, int 
     dens[3 * i] = rL;
     dens[3 * i + 1] = rY;
     dens[3 * i + 2] = rp;
-    const real area = (real)g.A[i];
+    const real area = (real)(g.A[i] * wcorr);
     typename V4<real>::t pv;
     pv.x = area * rL;
     pv.y = area * rY;
@@ -207,7 +209,7 @@ __global__ void k_rows_init(Geo g, BodyDev bd, const double* x, int mode, double
 template <typename real>
 __global__ void k_src_region(Geo g, BodyDev bd, RegionDev rd, const double* __restrict__ x, int mode,
                              const typename V4<real>::t* __restrict__ yrel, typename V4<real>::t* __restrict__ src,
-                             typename V4<real>::t* __restrict__ pd, real* __restrict__ dens) {
+                             typename V4<real>::t* __restrict__ pd, real* __restrict__ dens, double wcorr) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= g.n_pan) return;
     const int b = g.pbody[i];
@@ -237,7 +239,7 @@ __global__ void k_src_region(Geo g, BodyDev bd, RegionDev rd, const double* __re
     dens[3 * i] = 0;
     dens[3 * i + 1] = rY;
     dens[3 * i + 2] = rp;
-    const real area = (real)g.A[i];
+    const real area = (real)(g.A[i] * wcorr);
     typename V4<real>::t pv;
     pv.x = 0;
     pv.y = area * rY;
@@ -403,7 +405,7 @@ void reserve_product(pgb_ctx* c, int precision) {
     c->d_Up[pi].resize(64 * std::max<int64_t>(c->n_pitems, 1));
     c->d_Uf[pi].resize(64 * std::max<int64_t>(c->n_fitems, 1));
     c->d_work.resize(2);
-    const int TP = n_terms_pad(c->p.P);
+    const int TP = n_far_pad(c->p.P);
     if (pi == 0) {
         c->d_src32.resize(2 * nsrc);
         c->d_pd32.resize(c->n_pan);
@@ -510,7 +512,6 @@ void apply_mode(pgb_ctx* c, const double* x, double* y, int precision, int mode,
     ev.fitem_off = c->d_fitem_off;
     ev.pitem_group = c->d_pitem_group;
     ev.fitem_group = c->d_fitem_group;
-    ev.m2p_item = c->p.m2p_item;
     ev.Up = Up;
     ev.Uf = Uf;
     ev.p2p_work = ev.m2p_work = nullptr;
@@ -523,7 +524,8 @@ void apply_mode(pgb_ctx* c, const double* x, double* y, int precision, int mode,
         ev.persist_blocks = c->persist_blocks;
     }
     const bool f32 = precision == PGB_FP32;
-    const int TP = n_terms_pad(P);
+    const double wcorr = f32 ? far_rule_f32_scale(c->p.K) : 1.0;
+    const int TP = n_far_pad(P);
     if (f32) {
         c->d_src32.resize(2 * nsrc);
         c->d_pd32.resize(c->n_pan);
@@ -553,7 +555,7 @@ void apply_mode(pgb_ctx* c, const double* x, double* y, int precision, int mode,
     const bool dsp = precision == PGB_FP64_DS;
     auto tab_for = [&](double kappa) -> const void* {
         const FarTab& t = far_table(c, kappa);
-        if (f32) return P > 8 ? (const void*)t.t32p.p : (const void*)t.t32.p;
+        if (f32) return t.t32.p;
         return dsp ? (const void*)t.tds.p : (const void*)t.t64.p;
     };
     up.far_tab = tab_for(c->kappa);
@@ -585,10 +587,10 @@ void apply_mode(pgb_ctx* c, const double* x, double* y, int precision, int mode,
                 StageTimer tm(c, PGB_STAGE_SOURCES + (f32 ? 0 : PGB_STAGE_FP64));
                 if (f32)
                     k_src_region<float><<<nblk(c->n_pan, 128), 128, 0, s>>>(g, bd, rd, x, mode, c->d_y32, c->d_src32, c->d_pd32,
-                                                                             (float*)dens.p);
+                                                                             (float*)dens.p, wcorr);
                 else
                     k_src_region<double><<<nblk(c->n_pan, 128), 128, 0, s>>>(g, bd, rd, x, mode, c->d_y64,
-                                                                              c->d_src64, c->d_pd64, dens.p);
+                                                                              c->d_src64, c->d_pd64, dens.p, wcorr);
                 if (precision == PGB_FP64_DS) {
                     convert_src_ds(c->d_src64, c->d_src_ds, 2 * nsrc, s);
                     convert_src_ds(c->d_pd64, c->d_pd_ds, c->n_pan, s);
@@ -630,10 +632,10 @@ void apply_mode(pgb_ctx* c, const double* x, double* y, int precision, int mode,
         StageTimer tm(c, PGB_STAGE_SOURCES + (f32 ? 0 : PGB_STAGE_FP64));
         if (f32)
             k_src_prep<float><<<nblk(c->n_pan, 128), 128, 0, s>>>(g, bd, x, mode, c->d_y32, c->d_src32, c->d_pd32,
-                                                                  (float*)dens.p, c->eps_out);
+                                                                  (float*)dens.p, c->eps_out, wcorr);
         else
             k_src_prep<double><<<nblk(c->n_pan, 128), 128, 0, s>>>(g, bd, x, mode, c->d_y64, c->d_src64, c->d_pd64,
-                                                                   dens.p, c->eps_out);
+                                                                   dens.p, c->eps_out, wcorr);
         if (precision == PGB_FP64_DS) {
             convert_src_ds(c->d_src64, c->d_src_ds, 2 * nsrc, s);
             convert_src_ds(c->d_pd64, c->d_pd_ds, c->n_pan, s);

@@ -15,6 +15,12 @@ inline bool p_supported(int P) { return (P >= 0 && P <= 8) || P == 10 || P == 12
 #define PGB_MAX_BODIES 64
 #define PGB_LIST_STACK 96
 
+// PGB_FP32 solves stop their iteration at this part of the tolerance: the
+// residual that decides the status comes from one more FP32 product, which is
+// off the Arnoldi estimate by that product's rounding (2e-3 of the tolerance at
+// tol 1e-6), and an estimate a hair below the tolerance must not miss it then.
+#define PGB_FP32_STOP 0.99
+
 namespace pgb {
 
 struct __align__(32) dbl4 {
@@ -110,6 +116,7 @@ struct FarRule {
     double a[2], w[3];
 };
 FarRule far_rule(int K);
+double far_rule_f32_scale(int K);
 
 // Far-field coefficient tables (farfield.cu) of one Taylor order and
 // screening: moments -> the coefficients the M2P kernels evaluate.
@@ -119,10 +126,12 @@ struct FarTab {
     DBuf<double> t64;
     DBuf<float> t32;
     DBuf<double> tds;  // the FP64 table split into double-single pairs (8 bytes each)
-    DBuf<float> t32p;  // the packed layout of t64 rounded to FP32 (orders above 8)
 };
-// padded coefficient count per kernel: rows of 16 bytes for vector loads
-__host__ __device__ constexpr int n_terms_pad(int P) { return (n_terms(P) + 3) & ~3; }
+// far-field coefficients per kernel (2p + 1 per degree p), padded to whole
+// 16-byte vectors, and the tables' columns
+__host__ __device__ constexpr int n_far(int P) { return (P + 1) * (P + 1); }
+__host__ __device__ constexpr int n_far_pad(int P) { return (n_far(P) + 3) & ~3; }
+__host__ __device__ constexpr int far_cols(int P) { return (n_far(P) + 31) & ~31; }
 void far_tables(int P, double kappa, std::vector<double>& tab);
 
 struct Body {
@@ -244,7 +253,7 @@ struct pgb_ctx {
     pgb::DBuf<int32_t> d_list_tmp;       // entries kept by the counting traversal (fixed rows per group)
     int64_t n_cols = 0;                  // P2P columns (panels of a group's near leaves) over all groups
     pgb::DBuf<int64_t> d_col_off;        // per group (+ total)
-    pgb::DBuf<float4> d_col;             // leaf centre - group centre, panel
+    pgb::DBuf<float4> d_col;             // panel centroid - group centre, panel
     pgb::DBuf<int32_t> d_pnode;          // leaf node of every panel
     pgb::DBuf<float> d_pg32;             // panel geometry of the P2P kernels, 16 values each
     pgb::DBuf<double> d_pg64, d_pg_ds;   // in FP64 and as double-single pairs (8 bytes a value)
@@ -298,7 +307,7 @@ struct pgb_ctx {
     pgb::DBuf<double> d_mom64;
     pgb::DBuf<int> d_arrive[2];          // upward pass: children finished per node, per precision
     uint64_t arrive_gen[2] = {~0ull, ~0ull};  // tree_gen the counters were zeroed for
-    pgb::DBuf<float> d_far32;            // far-field coefficients: 2 * n_terms_pad(P) per node
+    pgb::DBuf<float> d_far32;            // far-field coefficients: 2 * n_far_pad(P) per node
     pgb::DBuf<double> d_far64;
     pgb::DBuf<double> d_mom_ds, d_far_ds;  // moments and coefficients of the double-single product (8 bytes each)
     std::vector<std::unique_ptr<pgb::FarTab>> far_tabs;  // per (P, kappa)

@@ -1023,7 +1023,8 @@ int solve(pgb_ctx* c, int mode, double tol, int max_iter, int restart, double* x
         // FP32 operator throughout, FP64 Arnoldi/Givens; the reported residual
         // uses the same FP32 operator
         int mv = 0;
-        z.iterations = gmres(c, PGB_FP32, c->d_b, x, tol * bnorm, max_iter, restart, &mv, nullptr, true);
+        z.iterations =
+            gmres(c, PGB_FP32, c->d_b, x, PGB_FP32_STOP * tol * bnorm, max_iter, restart, &mv, nullptr, true);
         z.matvecs += mv;
         z.outer_steps = 1;
         apply_operator(c, x, c->d_r, PGB_FP32, false);

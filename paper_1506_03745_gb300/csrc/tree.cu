@@ -70,6 +70,15 @@ FarRule far_rule(int K) {
     return f;
 }
 
+// The rule's weights rounded to FP32 no longer sum to one, an error that all
+// panels share; the FP32 densities take its reciprocal.
+double far_rule_f32_scale(int K) {
+    const FarRule f = far_rule(K);
+    double s = (double)(float)f.w[0];
+    for (int o = 0; o < 2; ++o) s += 3.0 * (double)(float)f.w[1 + o];
+    return 1.0 / s;
+}
+
 static inline int nblk(int64_t n, int t) { return (int)std::max<int64_t>(1, (n + t - 1) / t); }
 
 // ---------------------------------------------------------------- scan
@@ -1111,8 +1120,9 @@ __global__ void k_list_offsets(int64_t ng, const int64_t* off, const int32_t* id
 }
 
 // P2P columns: the panels of a group's near leaves one after another, in list
-// order; descriptor = (leaf centre - group centre in FP32, panel).  One warp
-// per group; the lanes take its near entries 32 at a time.
+// order; descriptor = (panel centroid - group centre, formed in FP64 and
+// rounded once to FP32, panel).  One warp per group; the lanes take its near
+// entries 32 at a time.
 __global__ void k_col_count(int64_t ng, const int64_t* noff, const int32_t* nearl, const int32_t* nstart,
                             const int32_t* nend, int64_t* cnt) {
     const int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
@@ -1124,16 +1134,21 @@ __global__ void k_col_count(int64_t ng, const int64_t* noff, const int32_t* near
     if (lane == 0) cnt[g] = c;
 }
 // The entries one after another, each entry's panels written by the warp.
-__global__ void k_col_fill(int64_t ng, const int64_t* noff, const int32_t* nearl, const float4* near4,
-                           const int32_t* nstart, const int32_t* nend, const int64_t* coff, float4* col) {
+__global__ void k_col_fill(int64_t ng, const int64_t* noff, const int32_t* nearl, const int32_t* nstart,
+                           const int32_t* nend, const double* C, const double* gcen, const int64_t* coff,
+                           float4* col) {
     const int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (g >= ng) return;
+    const double g0 = gcen[3 * g], g1 = gcen[3 * g + 1], g2 = gcen[3 * g + 2];
     int64_t w = coff[g];
     for (int64_t e = noff[g]; e < noff[g + 1]; ++e) {
-        const float4 o = near4[e];
         const int s = nstart[nearl[e]], n = nend[nearl[e]] - s;
-        for (int q = lane; q < n; q += 32) col[w + q] = make_float4(o.x, o.y, o.z, __int_as_float(s + q));
+        for (int q = lane; q < n; q += 32) {
+            const int64_t j = s + q;
+            col[w + q] = make_float4((float)(C[3 * j] - g0), (float)(C[3 * j + 1] - g1), (float)(C[3 * j + 2] - g2),
+                                     __int_as_float(s + q));
+        }
         w += n;
     }
 }
@@ -1238,8 +1253,9 @@ void build_lists(pgb_ctx* c) {
         PGB_CUDA(cudaMemcpyAsync(c->d_col_off.p + ng, &nt, 8, cudaMemcpyHostToDevice, s));
         c->n_cols = nt;
         c->d_col.resize(nt);
-        k_col_fill<<<nblk(32 * ng, 128), 128, 0, s>>>(ng, c->d_near_off, c->d_near, c->d_near4, c->d_node_start,
-                                                      c->d_node_end, c->d_col_off, c->d_col);
+        k_col_fill<<<nblk(32 * ng, 128), 128, 0, s>>>(ng, c->d_near_off, c->d_near, c->d_node_start,
+                                                      c->d_node_end, c->d_c, c->d_group_center, c->d_col_off,
+                                                      c->d_col);
         PGB_CUDA(cudaGetLastError());
     }
     {
@@ -1279,8 +1295,8 @@ void refresh_lists(pgb_ctx* c) {
                                                c->d_near4);
     k_list_offsets<<<(unsigned)ng, 64, 0, s>>>(ng, c->d_far_off, c->d_far, c->d_node_center, c->d_group_center,
                                                c->d_far4);
-    k_col_fill<<<nblk(32 * ng, 128), 128, 0, s>>>(ng, c->d_near_off, c->d_near, c->d_near4, c->d_node_start,
-                                                  c->d_node_end, c->d_col_off, c->d_col);
+    k_col_fill<<<nblk(32 * ng, 128), 128, 0, s>>>(ng, c->d_near_off, c->d_near, c->d_node_start, c->d_node_end,
+                                                  c->d_c, c->d_group_center, c->d_col_off, c->d_col);
     PGB_CUDA(cudaGetLastError());
     PGB_CUDA(cudaStreamSynchronize(s));
     PGB_LAUNCHED(c, 3);

@@ -154,6 +154,65 @@ constexpr bool is_ds = false;
 template <>
 constexpr bool is_ds<ds> = true;
 
+// Arithmetic of the P2P and M2P sums: fused forms in FP32 and FP64,
+// double-single without renormalisation where no cancellation follows.
+__device__ __forceinline__ float mul_(float a, float b) { return a * b; }
+__device__ __forceinline__ double mul_(double a, double b) { return a * b; }
+__device__ __forceinline__ ds mul_(ds a, ds b) { return ds_mul_u(a, b); }
+__device__ __forceinline__ float add_(float a, float b) { return a + b; }
+__device__ __forceinline__ double add_(double a, double b) { return a + b; }
+__device__ __forceinline__ ds add_(ds a, ds b) { return ds_add_u(a, b); }
+__device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ ds fma_(ds a, ds b, ds c) { return ds_fma_u(a, b, c); }
+__device__ __forceinline__ float norm_(float a) { return a; }
+__device__ __forceinline__ double norm_(double a) { return a; }
+__device__ __forceinline__ ds norm_(ds a) { return ds_norm(a); }
+// Two FP32 values in one 64-bit register pair: Blackwell's packed FP32
+// arithmetic does both with one instruction.  The FMA pipe takes as long as
+// for two scalar ones (measured: 113-118 lane FMAs per clock and SM either
+// way); what halves is the issue slots.
+struct __align__(8) f2 {
+    float a, b;
+};
+__device__ __forceinline__ unsigned long long f2_bits(f2 x) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x.a), "f"(x.b));
+    return r;
+}
+__device__ __forceinline__ f2 f2_from(unsigned long long v) {
+    f2 x;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x.a), "=f"(x.b) : "l"(v));
+    return x;
+}
+__device__ __forceinline__ f2 mul_(f2 x, f2 y) {
+    unsigned long long r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_bits(x)), "l"(f2_bits(y)));
+    return f2_from(r);
+}
+__device__ __forceinline__ f2 add_(f2 x, f2 y) {
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_bits(x)), "l"(f2_bits(y)));
+    return f2_from(r);
+}
+__device__ __forceinline__ f2 fma_(f2 x, f2 y, f2 z) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(f2_bits(x)), "l"(f2_bits(y)), "l"(f2_bits(z)));
+    return f2_from(r);
+}
+__device__ __forceinline__ f2 operator-(f2 x) { return f2{-x.a, -x.b}; }
+__device__ __forceinline__ f2 rsqrt_(f2 x) { return f2{rsqrt_(x.a), rsqrt_(x.b)}; }
+__device__ __forceinline__ f2 exp_(f2 x) { return f2{exp_(x.a), exp_(x.b)}; }
+// a constant in the arithmetic type
+template <typename V>
+__device__ __forceinline__ V cst(double d) {
+    return (V)d;
+}
+template <>
+__device__ __forceinline__ f2 cst<f2>(double d) {
+    return f2{(float)d, (float)d};
+}
+
 // Multi-indices of total degree <= P: graded, and within a degree kx
 // descending then ky descending.
 template <int P>
@@ -241,7 +300,7 @@ struct EvalArgs {
     const float4* near4;           // per near entry: leaf centre - group centre, node id bits
     const float4* far4;            // per far entry: node centre - group centre, node id bits
     const int64_t* col_off;        // per group: its P2P columns [col_off[g], col_off[g+1])
-    const float4* col;             // per column: leaf centre - group centre (FP32), panel (int bits)
+    const float4* col;             // per column: panel centroid - group centre (FP32), panel (int bits)
     const int32_t* pnode;          // leaf node of a panel (FP64 and double-single offsets)
     const int32_t* pbody;          // body of a panel
     const void* pg;                // panel geometry (PanelGeo) in the kernel's arithmetic
@@ -252,7 +311,6 @@ struct EvalArgs {
     int64_t n_pitems, n_fitems;
     const int64_t *pitem_off, *fitem_off;  // per group
     const int32_t *pitem_group, *fitem_group;
-    int m2p_item;
     double *Up, *Uf;               // per item: 32 Laplace then 32 Yukawa partial sums (one per lane)
     // persistent launch: a grid smaller than the item count whose blocks take
     // items from these counters (zero before the launch); nullptr: one item per block
@@ -279,14 +337,6 @@ struct alignas(16) Vec16 {
     real v[N];
 };
 
-// Far field of one node at R = target - node centre from its coefficients in
-// the evaluation order (a = 0..P, b = 0..P-a, c = 0..P-a-b for S^(a,b,c)),
-// S = R / r^2 and x = kappa r (the tables of farfield.cu):
-//   U_Y = (e^{-x} / r) sum_p g_p(x) sum_{a+b+c=p} cY_abc S^(a,b,c),
-//   U_L = (1 / r) sum_abc cL_abc S^(a,b,c),
-// g_0 = 1, g_1 = -(1 + x), g_p = x^2 g_{p-2} - (2p - 1) g_{p-1}.  The monomials
-// are formed in nested order, one product each, and summed per degree, so
-// that a term costs one product and one multiply-add per kernel.
 // Compile-time loop: f(std::integral_constant<int, I>) for I = B .. E-1, so
 // that array indices formed from I are constants whatever the trip count
 // (a plain unrolled loop nest is left partly rolled by the compiler at the
@@ -298,113 +348,178 @@ __device__ __forceinline__ void static_for(F&& f) {
         static_for<B + 1, E>(f);
     }
 }
-// index of S^(a,b,0) in the evaluation order of order P
-__host__ __device__ constexpr int eval_index(int P, int a, int b) {
-    int o = 0;
-    for (int q = 0; q < a; ++q) o += (P - q + 1) * (P - q + 2) / 2;
-    for (int q = 0; q < b; ++q) o += P - a - q + 1;
-    return o;
+// Position of the coefficient (l, m, s) among a node's: m = 0 first, then per
+// m the (Re, Im) pairs of l = m..P.
+__host__ __device__ constexpr int far_pos(int P, int l, int m, int s) {
+    return m == 0 ? l : (P + 1) + 2 * ((m - 1) * (P + 1) - (m - 1) * m / 2) + 2 * (l - m) + s;
 }
+// c_{l,m} of the q recurrence
+__host__ __device__ constexpr double far_c(int l, int m) { return (double)(l * l - m * m) / (4.0 * l * l - 1.0); }
 
-template <typename real, int P, bool LAP>
-__device__ __forceinline__ void far_eval(real Rx, real Ry, real Rz, real kappa, const real* __restrict__ cL,
-                                         const real* __restrict__ cY, real& uL, real& uY) {
-    using V = Vec16<real>;
-    constexpr int VN = V::N;
-    real r2;
-    if constexpr (is_ds<real>) r2 = madd(Rx, Rx, madd(Ry, Ry, Rz * Rz));
-    else r2 = Rx * Rx + Ry * Ry + Rz * Rz;
-    const real ri = rsqrt_(r2);
-    const real i2 = ri * ri;
-    const real sx = Rx * i2, sy = Ry * i2, sz = Rz * i2;
-    real acc[P + 1];
-#pragma unroll
-    for (int p = 0; p <= P; ++p) acc[p] = real(0);
-    real aL = real(0);
-    V qy, ql;
-    real xa = real(1);
-    if constexpr (is_ds<real> && P > 8) {
-        // double-single above order 8: loops the compiler unrolls as it sees
-        // fit (the full unroll of these long double-single bodies takes the
-        // compiler minutes); the FP64-class residual product runs a few times
-        // per solve
-        int idx = 0;
-#pragma unroll
-        for (int a = 0; a <= P; ++a) {
-            real xy = xa;
-#pragma unroll
-            for (int b = 0; b <= P - a; ++b) {
-                real t = xy;
-#pragma unroll
-                for (int c = 0; c <= P - a - b; ++c) {
-                    if (idx % VN == 0) {
-                        qy = *reinterpret_cast<const V*>(cY + idx);
-                        if (LAP) ql = *reinterpret_cast<const V*>(cL + idx);
-                    }
-                    acc[a + b + c] = madd(qy.v[idx % VN], t, acc[a + b + c]);
-                    if (LAP) aL = madd(ql.v[idx % VN], t, aL);
-                    ++idx;
-                    if (c < P - a - b) t = t * sz;
-                }
-                if (b < P - a) xy = xy * sy;
-            }
-            if (a < P) xa = xa * sx;
-        }
-    } else {
-    static_for<0, P + 1>([&](auto A) {
-        constexpr int a = decltype(A)::value;
-        real xy = xa;
-        static_for<0, P - a + 1>([&](auto Bc) {
-            constexpr int b = decltype(Bc)::value;
-            constexpr int i0 = eval_index(P, a, b);
-            real t = xy;
-            static_for<0, P - a - b + 1>([&](auto Cc) {
-                constexpr int c = decltype(Cc)::value;
-                constexpr int idx = i0 + c;
-                if constexpr (idx % VN == 0) {
-                    qy = *reinterpret_cast<const V*>(cY + idx);
-                    if constexpr (LAP) ql = *reinterpret_cast<const V*>(cL + idx);
-                }
-                acc[a + b + c] = madd(qy.v[idx % VN], t, acc[a + b + c]);
-                if constexpr (LAP) aL = madd(ql.v[idx % VN], t, aL);
-                if constexpr (c < P - a - b) t = t * sz;
-            });
-            if constexpr (b < P - a) xy = xy * sy;
-        });
-        if constexpr (a < P) xa = xa * sx;
+// Far field of one node at R = target - node centre from its harmonic
+// coefficients (farfield.cu), n = R / r, x = kappa r:
+//   U_Y = (e^{-x} / r) sum_l h_l sum_m q_{l,m}(n_z) (a Re + b Im)(n_x + i n_y)^m,
+//   U_L = (1 / r) sum_l r^{-l} sum_m ...,
+// h_l = g_l(x) r^{-l}: h_0 = 1, h_1 = -(1 + x) / r, h_l = kappa^2 h_{l-2} -
+// (2l - 1) h_{l-1} / r.  Unrolled at compile time, so that the radial factors
+// stay in registers.  V: the arithmetic (f2: two targets); C: the stored
+// constants' type, the recurrence constants -c_{l,m} at ctab[l (P + 1) + m] for
+// f2 (packed instructions take no immediates), immediate otherwise.
+template <typename V, int P, bool LAP>
+__device__ __forceinline__ void far_eval(V Rx, V Ry, V Rz, V kappa, const V* __restrict__ cL,
+                                         const V* __restrict__ cY, const V* __restrict__ ctab, V& uL, V& uY) {
+    using W = Vec16<V>;
+    constexpr int VN = W::N;
+    constexpr bool PACKED = std::is_same<V, f2>::value;
+    V hY[P + 1], hL[P + 1];
+    const V r2 = fma_(Rz, Rz, fma_(Ry, Ry, mul_(Rx, Rx)));
+    const V ri = rsqrt_(r2);
+    const V nx = mul_(Rx, ri), ny = mul_(Ry, ri), nz = mul_(Rz, ri);
+    const V ex = mul_(exp_(mul_(-kappa, mul_(r2, ri))), ri);
+    const V k2 = mul_(kappa, kappa);
+    hY[0] = hL[0] = cst<V>(1);
+    if constexpr (P >= 1) {
+        hY[1] = -add_(ri, kappa);  // -(1 + x) / r
+        hL[1] = ri;
+    }
+    V lr = ri;  // (2l - 1) / r
+    const V twice = add_(ri, ri);
+    static_for<2, P + 1>([&](auto Lc) {
+        constexpr int l = decltype(Lc)::value;
+        lr = add_(lr, twice);
+        hY[l] = fma_(-lr, hY[l - 1], mul_(k2, hY[l - 2]));
+        if constexpr (LAP) hL[l] = mul_(hL[l - 1], ri);
     });
-    }
-    const real r = r2 * ri;
-    const real x = kappa * r;
-    const real x2 = x * x;
-    real u = acc[0];
-    real gm2 = real(1), gm1 = -(x + real(1));
-    if (P >= 1) u = madd(gm1, acc[P >= 1 ? 1 : 0], u);
-#pragma unroll
-    for (int p = 2; p <= P; ++p) {
-        const real g = madd(x2, gm2, -(real(2 * p - 1) * gm1));
-        u = madd(g, acc[p], u);
-        gm2 = gm1;
-        gm1 = g;
-    }
-    uY = (exp_(-x) * ri) * u;
-    uL = LAP ? aL * ri : real(0);
+    V X = cst<V>(1), Y = cst<V>(0);
+    uL = uY = cst<V>(0);
+    W qy, ql;
+    static_for<0, P + 1>([&](auto M) {
+        constexpr int m = decltype(M)::value;
+        V q0 = cst<V>(1), q1 = cst<V>(0);  // q_{l,m}, q_{l-1,m}
+        V aY, bY, aL, bL;                  // the sums over l
+        static_for<m, P + 1>([&](auto Lc) {
+            constexpr int l = decltype(Lc)::value;
+            if constexpr (l > m) {
+                V q;
+                if constexpr (l == m + 1) q = nz;
+                else if constexpr (PACKED) q = fma_(nz, q0, mul_(ctab[(l - 1) * (P + 1) + m], q1));
+                else q = fma_(nz, q0, mul_(cst<V>(-far_c(l - 1, m)), q1));
+                q1 = q0;
+                q0 = q;
+            }
+            V w, v;
+            if constexpr (l > m) {
+                w = mul_(hY[l], q0);
+                if constexpr (LAP) v = mul_(hL[l], q0);
+            } else {
+                w = hY[l];
+                if constexpr (LAP) v = hL[l];
+            }
+            static_for<0, (m == 0 ? 1 : 2)>([&](auto Sc) {
+                constexpr int s = decltype(Sc)::value;
+                constexpr int i = far_pos(P, l, m, s);
+                if constexpr (i % VN == 0) {
+                    qy = *reinterpret_cast<const W*>(cY + i);
+                    if constexpr (LAP) ql = *reinterpret_cast<const W*>(cL + i);
+                }
+                V& sy = s == 0 ? aY : bY;
+                if constexpr (l == m) sy = mul_(w, qy.v[i % VN]);
+                else sy = fma_(w, qy.v[i % VN], sy);
+                if constexpr (LAP) {
+                    V& sl = s == 0 ? aL : bL;
+                    if constexpr (l == m) sl = mul_(v, ql.v[i % VN]);
+                    else sl = fma_(v, ql.v[i % VN], sl);
+                }
+            });
+        });
+        if constexpr (m == 0) {
+            uY = aY;
+            if constexpr (LAP) uL = aL;
+            X = nx;
+            Y = ny;
+        } else {
+            uY = fma_(X, aY, fma_(Y, bY, uY));
+            if constexpr (LAP) uL = fma_(X, aL, fma_(Y, bL, uL));
+            if constexpr (m < P) {
+                const V xn = fma_(nx, X, -mul_(ny, Y));
+                Y = fma_(nx, Y, mul_(ny, X));
+                X = xn;
+            }
+        }
+    });
+    uY = mul_(ex, uY);
+    if constexpr (LAP) uL = mul_(ri, uL);
 }
 
-// Arithmetic of the P2P sums: the compiler's contracted forms in FP32 and
-// FP64, double-single without renormalisation where no cancellation follows.
-__device__ __forceinline__ float mul_(float a, float b) { return a * b; }
-__device__ __forceinline__ double mul_(double a, double b) { return a * b; }
-__device__ __forceinline__ ds mul_(ds a, ds b) { return ds_mul_u(a, b); }
-__device__ __forceinline__ float add_(float a, float b) { return a + b; }
-__device__ __forceinline__ double add_(double a, double b) { return a + b; }
-__device__ __forceinline__ ds add_(ds a, ds b) { return ds_add_u(a, b); }
-__device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
-__device__ __forceinline__ ds fma_(ds a, ds b, ds c) { return ds_fma_u(a, b, c); }
-__device__ __forceinline__ float norm_(float a) { return a; }
-__device__ __forceinline__ double norm_(double a) { return a; }
-__device__ __forceinline__ ds norm_(ds a) { return ds_norm(a); }
+// c_{l,m} in double-single for the rolled form below
+struct FarC {
+    ds v[PGB_MAX_P + 1][PGB_MAX_P + 1];  // [m][l]
+    __host__ __device__ constexpr FarC() : v() {
+        for (int m = 0; m <= PGB_MAX_P; ++m)
+            for (int l = 1; l <= PGB_MAX_P; ++l) v[m][l] = ds_const(far_c(l, m));
+    }
+};
+__device__ __constant__ const FarC kFarC = FarC();
+
+// The same in double-single, as loops: unrolled, a pair's 2500 operations
+// overflow the instruction caches (the kernel waited for instructions more
+// than for anything else).  rad: the thread's radial factors in shared memory,
+// (h_l, r^{-l}) at rad[l * stride].
+template <int P, bool LAP>
+__device__ __forceinline__ void far_eval_ds(ds Rx, ds Ry, ds Rz, ds kappa, const ds* __restrict__ cL,
+                                            const ds* __restrict__ cY, float4* rad, int stride, ds& uL, ds& uY) {
+    const ds r2 = ds_norm(ds_fma_u(Rx, Rx, ds_fma_u(Ry, Ry, ds_mul_u(Rz, Rz))));
+    const ds ri = ds_rsqrt(r2);
+    const ds nx = Rx * ri, ny = Ry * ri, nz = Rz * ri;
+    const ds ex = ds_mul_u(ds_exp(-(kappa * (r2 * ri))), ri);
+    {
+        const ds k2 = kappa * kappa;
+        ds h0 = ds(1), h1 = -(ri + kappa), p = ds(1);
+        rad[0] = make_float4(1.f, 0.f, 1.f, 0.f);
+#pragma unroll 1
+        for (int l = 1; l <= P; ++l) {
+            if (l > 1) {
+                // both terms carry the sign (-1)^l: no cancellation
+                const ds h = ds_norm(ds_fma_u(k2, h0, ds_mul_u(mul_f(ri, -(float)(2 * l - 1)), h1)));
+                h0 = h1;
+                h1 = h;
+            }
+            p = p * ri;
+            rad[l * stride] = make_float4(h1.hi, h1.lo, p.hi, p.lo);
+        }
+    }
+    ds X = ds(1), Y = ds(0);
+    ds sY = ds(0), sL = ds(0);
+    int i = 0;
+#pragma unroll 1
+    for (int m = 0; m <= P; ++m) {
+        ds q0 = ds(1), q1 = ds(0), aY = ds(0), bY = ds(0), aL = ds(0), bL = ds(0);
+#pragma unroll 1
+        for (int l = m; l <= P; ++l) {
+            const float4 h = rad[l * stride];
+            const ds w = ds_mul_u(ds(h.x, h.y), q0);
+            aY = ds_fma_u(w, cY[i], aY);
+            if (m) bY = ds_fma_u(w, cY[i + 1], bY);
+            if (LAP) {
+                const ds v = ds_mul_u(ds(h.z, h.w), q0);
+                aL = ds_fma_u(v, cL[i], aL);
+                if (m) bL = ds_fma_u(v, cL[i + 1], bL);
+            }
+            i += m ? 2 : 1;
+            const ds q = nz * q0 - kFarC.v[m][l] * q1;  // c_{m,m} = 0
+            q1 = q0;
+            q0 = q;
+        }
+        sY = ds_fma_u(X, ds_norm(aY), ds_fma_u(Y, ds_norm(bY), sY));
+        if (LAP) sL = ds_fma_u(X, ds_norm(aL), ds_fma_u(Y, ds_norm(bL), sL));
+        const ds xn = nx * X - ny * Y;
+        Y = nx * Y + ny * X;
+        X = xn;
+    }
+    uY = ex * ds_norm(sY);
+    uL = LAP ? ri * ds_norm(sL) : ds(0);
+}
+
 // 1/sqrt of a squared distance formed with a cancellation: a value rounded
 // below zero is taken by its magnitude (FP32; the others keep 50 bits more
 // than the distances that occur)
@@ -503,30 +618,6 @@ __device__ __forceinline__ void p2p_panel(const PanelS<real>& q, bool own, real 
     UY = fma_(q.qY, VY, fma_(mul_(-q.pY, h), KY, UY));
 }
 
-// One block of NW warps per target group (32 targets, one per lane): the
-// warps share out the near leaves (P2P) and far nodes (M2P) of the group's
-// lists round robin, and their partial sums are combined in warp order.
-template <typename real>
-__device__ __forceinline__ void entry_offset(const EvalArgs& a, int64_t e, bool is_far, double gc0, double gc1,
-                                             double gc2, int& nd, real& ox, real& oy, real& oz);
-template <>
-__device__ __forceinline__ void entry_offset<float>(const EvalArgs& a, int64_t e, bool is_far, double, double, double,
-                                                    int& nd, float& ox, float& oy, float& oz) {
-    const float4 q = is_far ? a.far4[e] : a.near4[e];
-    nd = __float_as_int(q.w);
-    ox = q.x;
-    oy = q.y;
-    oz = q.z;
-}
-template <>
-__device__ __forceinline__ void entry_offset<double>(const EvalArgs& a, int64_t e, bool is_far, double gc0, double gc1,
-                                                     double gc2, int& nd, double& ox, double& oy, double& oz) {
-    nd = is_far ? a.far_l[e] : a.near_l[e];
-    ox = a.ncenter[3 * nd] - gc0;
-    oy = a.ncenter[3 * nd + 1] - gc1;
-    oz = a.ncenter[3 * nd + 2] - gc2;
-}
-
 // Partial sums of the NW warps of a block combined in warp order (each warp
 // carries a compensated pair per kernel) and stored per lane for the item.
 template <typename real, int NW>
@@ -550,22 +641,28 @@ __device__ __forceinline__ void store_item(real (*red)[4][32], int w, int lane, 
     }
 }
 
-// Offset of a column's leaf centre from the group's centre: from the column in
-// FP32, formed in FP64 from the centres otherwise.
+// Centroid of a column's panel relative to the group's centre: in FP32 from the
+// column (one rounding of the FP64 difference), otherwise the centroid
+// relative to its leaf's centre plus the FP64 difference of the centres.
 template <typename real>
-__device__ __forceinline__ void col_offset(const EvalArgs& a, const float4& c, int j, int64_t g, real& ox, real& oy,
-                                           real& oz) {
+__device__ __forceinline__ void col_centroid(const EvalArgs& a, const float4& c, int j, int64_t g,
+                                             const real* __restrict__ v, real& x, real& y, real& z) {
     if constexpr (sizeof(real) == sizeof(float)) {
-        ox = c.x;
-        oy = c.y;
-        oz = c.z;
+        x = c.x;
+        y = c.y;
+        z = c.z;
     } else {
         const int nd = a.pnode[j];
-        ox = from_dbl<real>(a.ncenter[3 * nd] - a.gcenter[3 * g]);
-        oy = from_dbl<real>(a.ncenter[3 * nd + 1] - a.gcenter[3 * g + 1]);
-        oz = from_dbl<real>(a.ncenter[3 * nd + 2] - a.gcenter[3 * g + 2]);
+        x = v[0] + from_dbl<real>(a.ncenter[3 * nd] - a.gcenter[3 * g]);
+        y = v[1] + from_dbl<real>(a.ncenter[3 * nd + 1] - a.gcenter[3 * g + 1]);
+        z = v[2] + from_dbl<real>(a.ncenter[3 * nd + 2] - a.gcenter[3 * g + 2]);
     }
 }
+
+// Panels summed plainly before they join the compensated sums: about the 32
+// points of rounding growth that the FP32 product's accuracy rests on.  (All
+// 32 panels of a stage in one plain sum: 10-20 % more error against FP64.)
+#define P2P_RUN 4
 
 // P2P: one block of NW warps per work item, i.e. an even share of the columns
 // (panels of the near leaves) of one target group (32 targets, one per lane).
@@ -616,13 +713,10 @@ __global__ void __launch_bounds__(NW * 32) k_p2p(EvalArgs a, const typename V4<t
                 const int b = a.pbody[j];
                 lap = glap && b == gb;
                 has_own = j >= p0 && j < p1;
-                real ox, oy, oz;
-                col_offset<real>(a, c, j, g, ox, oy, oz);
                 PanelS<real>& q = sP[w][lane];
-                const PanelS<real>& v = *reinterpret_cast<const PanelS<real>*>(pg + 16 * (int64_t)j);  // its first 15 values
-                q.cx = v.cx + ox;
-                q.cy = v.cy + oy;
-                q.cz = v.cz + oz;
+                // the first 15 values of a staged panel, relative to the leaf
+                const PanelS<real>& v = *reinterpret_cast<const PanelS<real>*>(pg + 16 * (int64_t)j);
+                col_centroid<real>(a, c, j, g, &v.cx, q.cx, q.cy, q.cz);
                 q.g0 = v.g0;
                 q.ux = v.ux;
                 q.uy = v.uy;
@@ -649,23 +743,25 @@ __global__ void __launch_bounds__(NW * 32) k_p2p(EvalArgs a, const typename V4<t
                 for (int k = 0; k < cnt; ++k)
                     if (__shfl_sync(0xffffffffu, j, k) == p) own = k;
             __syncwarp();
-            real sumL = 0, sumY = 0;
+            // a few panels in plain sums, then into the compensated ones
+            auto sums = [&](auto LAPc, auto OWNc) {
+                for (int k0 = 0; k0 < cnt; k0 += P2P_RUN) {
+                    real sumL = 0, sumY = 0;
+                    const int k1 = min(cnt, k0 + P2P_RUN);
+                    for (int k = k0; k < k1; ++k)
+                        p2p_panel<real, K, decltype(LAPc)::value, decltype(OWNc)::value>(
+                            sP[w][k], k == own, X, Y, Z, kappa, nkl, ra, rw, sumL, sumY);
+                    if (decltype(LAPc)::value) kadd(UL, cL, sumL);
+                    kadd(UY, cY, sumY);
+                }
+            };
             if (has_own) {
-                if (lap)
-                    for (int k = 0; k < cnt; ++k)
-                        p2p_panel<real, K, true, true>(sP[w][k], k == own, X, Y, Z, kappa, nkl, ra, rw, sumL, sumY);
-                else
-                    for (int k = 0; k < cnt; ++k)
-                        p2p_panel<real, K, false, true>(sP[w][k], k == own, X, Y, Z, kappa, nkl, ra, rw, sumL, sumY);
-            } else if (lap) {
-                for (int k = 0; k < cnt; ++k)
-                    p2p_panel<real, K, true, false>(sP[w][k], false, X, Y, Z, kappa, nkl, ra, rw, sumL, sumY);
+                if (lap) sums(std::true_type(), std::true_type());
+                else sums(std::false_type(), std::true_type());
             } else {
-                for (int k = 0; k < cnt; ++k)
-                    p2p_panel<real, K, false, false>(sP[w][k], false, X, Y, Z, kappa, nkl, ra, rw, sumL, sumY);
+                if (lap) sums(std::true_type(), std::false_type());
+                else sums(std::false_type(), std::false_type());
             }
-            kadd(UL, cL, sumL);
-            kadd(UY, cY, sumY);
         }
         store_item<real, NW>(red, w, lane, UL, cL, UY, cY, a.Up + 64 * it);
     }
@@ -688,96 +784,176 @@ void launch_p2p(const EvalArgs& ev, int K, const void* xrel, cudaStream_t s) {
 }
 
 // M2P: one block of NW warps per work item, i.e. up to m2p_item far entries of
-// one target group; the nodes go round robin to the warps with the next
-// node's far-field coefficients (k_far_coef) prefetched.  The item's partial
-// sums go to Uf.
+// one target group; the nodes go round robin to the warps, their far-field
+// coefficients (k_far) staged in shared memory.  The item's partial sums go to
+// Uf.  next_entry: the first entry from e on, in steps, whose source body is
+// used in this product.
+template <typename S>
+__device__ __forceinline__ int64_t next_entry(const EvalArgs& a, int64_t e, int64_t f1, int step,
+                                              unsigned long long dm) {
+    if (a.all_active) return e;
+    while (e < f1) {
+        const int nd = sizeof(S) == sizeof(float) ? __float_as_int(a.far4[e].w) : a.far_l[e];
+        const int b = a.nbody[nd];
+        if (a.src_active[b] && ((dm >> b) & 1ull)) return e;
+        e += step;
+    }
+    return e;
+}
+
+// FP32: a half warp takes a node, each of its 16 lanes two of the group's
+// targets as the halves of packed values.  A target per lane in scalar
+// arithmetic issued 384 instructions per (node, 32 targets) with monomials and
+// 314 in the harmonic basis, at 56-64 % of the issue rate; packed, they halve
+// and the FMA pipe is the bound.  The coefficients lie in shared memory twice
+// over (c, c), ready as packed operands, and so do the recurrence constants.
+template <int P, int NW>
+__global__ void __launch_bounds__(NW * 32) k_m2p_f32(EvalArgs a, const float4* __restrict__ xrel,
+                                                     const float* __restrict__ far) {
+    constexpr int NC = n_far_pad(P), NV = 2 * NC / 4;  // 16-byte vectors of a node's coefficients
+    constexpr int ML = (NV + 15) / 16;
+    constexpr bool PRE = P <= 8;  // the next node's coefficients wait in registers
+    __shared__ __align__(16) f2 sM[NW][2][2 * NC];
+    __shared__ f2 sC[(P + 1) * (P + 1)];
+    __shared__ float red[NW][4][32];
+    __shared__ int64_t s_item;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, half = lane >> 4, hl = lane & 15;
+    for (int k = threadIdx.x; k < (P + 1) * (P + 1); k += NW * 32) {
+        const int l = k / (P + 1), m = k - l * (P + 1);
+        const float c = l > 0 ? (float)(l * l - m * m) / (float)(4 * l * l - 1) : 0.f;
+        sC[k] = f2{-c, -c};
+    }
+    __syncthreads();
+    const unsigned long long dm = body_mask(a.bmask);
+    const float4* __restrict__ farv = (const float4*)far;
+    for (int64_t it = next_item(a.m2p_work, -1, &s_item); it < a.n_fitems; it = next_item(a.m2p_work, it, &s_item)) {
+        const int64_t g = a.fitem_group[it];
+        const int gb = a.gbody[g];
+        if (!(((a.tgt_mask & dm) >> gb) & 1ull) || g < a.g_lo || g >= a.g_hi) continue;  // rows not used (block-uniform)
+        const int64_t p0 = a.gstart[g], p1 = a.gend[g];
+        const float4 xa = xrel[p0 + hl < p1 ? p0 + hl : p0], xb = xrel[p0 + 16 + hl < p1 ? p0 + 16 + hl : p0];
+        const f2 kappa = cst<f2>(a.kappa);
+        const bool glap = a.lap_body[gb];
+        float UL[2] = {0, 0}, eL[2] = {0, 0}, UY[2] = {0, 0}, eY[2] = {0, 0};
+        // the group's entries go evenly to its items
+        const int64_t i0 = a.fitem_off[g], fo = a.far_off[g], nf = a.far_off[g + 1] - fo;
+        const int64_t per = (nf + a.fitem_off[g + 1] - i0 - 1) / (a.fitem_off[g + 1] - i0);
+        const int64_t fb = fo + (it - i0) * per, f1 = min(fo + nf, fb + per);
+        int64_t e = next_entry<float>(a, fb + 2 * w + half, f1, 2 * NW, dm);
+        float4 q = make_float4(0.f, 0.f, 0.f, 0.f), pm[PRE ? ML : 1];
+        int nb = -1;  // the node's body
+        auto fetch = [&]() {
+            if (e >= f1) return;
+            q = a.far4[e];
+            if (glap) nb = a.nbody[__float_as_int(q.w)];
+            if constexpr (PRE) {
+                const float4* c = farv + (int64_t)__float_as_int(q.w) * NV;
+#pragma unroll
+                for (int k = 0; k < ML; ++k)
+                    if (hl + 16 * k < NV) pm[k] = c[hl + 16 * k];
+            }
+        };
+        float4* sv = reinterpret_cast<float4*>(sM[w][half]);
+        auto put = [&](int k, const float4& c) {
+            sv[2 * k] = make_float4(c.x, c.x, c.y, c.y);
+            sv[2 * k + 1] = make_float4(c.z, c.z, c.w, c.w);
+        };
+        fetch();
+        while (__any_sync(0xffffffffu, e < f1)) {
+            const bool on = e < f1;
+            __syncwarp();
+            if constexpr (PRE) {
+#pragma unroll
+                for (int k = 0; k < ML; ++k)
+                    if (hl + 16 * k < NV) put(hl + 16 * k, pm[k]);
+            } else if (on) {
+                const float4* c = farv + (int64_t)__float_as_int(q.w) * NV;
+                for (int k = hl; k < NV; k += 16) put(k, c[k]);
+            }
+            __syncwarp();
+            const bool lap = on && glap && nb == gb;
+            // a half without a node evaluates what its slots hold at a
+            // harmless place and drops the result
+            const f2 Rx = on ? f2{xa.x - q.x, xb.x - q.x} : f2{1.f, 1.f};
+            const f2 Ry = on ? f2{xa.y - q.y, xb.y - q.y} : f2{0.f, 0.f};
+            const f2 Rz = on ? f2{xa.z - q.z, xb.z - q.z} : f2{0.f, 0.f};
+            if (on) e = next_entry<float>(a, e + 2 * NW, f1, 2 * NW, dm);
+            fetch();  // the next node
+            f2 uL, uY;
+            if (__any_sync(0xffffffffu, lap)) {
+                far_eval<f2, P, true>(Rx, Ry, Rz, kappa, sM[w][half], sM[w][half] + NC, sC, uL, uY);
+                kadd(UL[0], eL[0], lap ? uL.a : 0.f);
+                kadd(UL[1], eL[1], lap ? uL.b : 0.f);
+            } else {
+                far_eval<f2, P, false>(Rx, Ry, Rz, kappa, sM[w][half], sM[w][half] + NC, sC, uL, uY);
+            }
+            kadd(UY[0], eY[0], on ? uY.a : 0.f);
+            kadd(UY[1], eY[1], on ? uY.b : 0.f);
+        }
+        // a lane keeps the target of its own number and gives the other half its other one
+        const int give = 1 - half;
+        const float oL = __shfl_xor_sync(0xffffffffu, give ? UL[1] : UL[0], 16);
+        const float oeL = __shfl_xor_sync(0xffffffffu, give ? eL[1] : eL[0], 16);
+        const float oY = __shfl_xor_sync(0xffffffffu, give ? UY[1] : UY[0], 16);
+        const float oeY = __shfl_xor_sync(0xffffffffu, give ? eY[1] : eY[0], 16);
+        float sL = half ? UL[1] : UL[0], cL = half ? eL[1] : eL[0], sY = half ? UY[1] : UY[0], cY = half ? eY[1] : eY[0];
+        kadd(sL, cL, oL);
+        kadd(sY, cY, oY);
+        store_item<float, NW>(red, w, lane, sL, cL + oeL, sY, cY + oeY, a.Uf + 64 * it);
+    }
+}
+
+// FP64 and double-single: a node per warp and a target per lane (bound by the
+// FP64 and the FMA pipe; the shared loads hide behind them).
 template <typename real, int P, int NW>
 __global__ void __launch_bounds__(NW * 32) k_m2p(EvalArgs a,
                                                  const typename V4<typename Store<real>::S>::t* __restrict__ xrel,
                                                  const real* __restrict__ far) {
-    using S = typename Store<real>::S;  // storage type of the inputs
+    using S = typename Store<real>::S;  // storage type of the targets
     using s4 = typename V4<S>::t;
-    constexpr int TP = n_terms_pad(P);
-    // orders up to 8: the next node's coefficients are prefetched into
-    // registers (MW words per lane) while the current one is evaluated;
-    // above, they are loaded into shared memory when needed
-    constexpr bool BIG = P > 8;
-    constexpr int MW = BIG ? 1 : (2 * TP + 31) / 32;
-    __shared__ __align__(16) real sM[NW][2 * TP];
+    constexpr int NC = n_far_pad(P);
+    extern __shared__ __align__(16) unsigned char m2p_smem[];
+    real* sM = reinterpret_cast<real*>(m2p_smem) + (threadIdx.x >> 5) * 2 * NC;  // this warp's node
+    float4* rad = reinterpret_cast<float4*>(m2p_smem + (size_t)NW * 2 * NC * sizeof(real)) + threadIdx.x;
     __shared__ real red[NW][4][32];
     __shared__ int64_t s_item;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned long long dm = body_mask(a.bmask);
     for (int64_t it = next_item(a.m2p_work, -1, &s_item); it < a.n_fitems; it = next_item(a.m2p_work, it, &s_item)) {
-    const int64_t g = a.fitem_group[it];
-    if (!(((a.tgt_mask & dm) >> a.gbody[g]) & 1ull) || g < a.g_lo || g >= a.g_hi) continue;  // rows not used (block-uniform)
-    const int64_t p0 = a.gstart[g], p1 = a.gend[g];
-    const int64_t p = p0 + lane;
-    const bool active = p < p1;
-    const s4 xr = active ? xrel[p] : xrel[p0];
-    const double gc0 = a.gcenter[3 * g], gc1 = a.gcenter[3 * g + 1], gc2 = a.gcenter[3 * g + 2];
-    const int gb = a.gbody[g];
-    const real kappa = to_c<real>((S)a.kappa);
-    real UL = 0, cL = 0, UY = 0, cY = 0;
-    const int64_t fb = a.far_off[g] + (it - a.fitem_off[g]) * a.m2p_item;
-    const int64_t f1 = min(a.far_off[g + 1], fb + a.m2p_item);
-    auto seek = [&](int64_t ee) -> int64_t {  // next active entry of this warp
-        if (a.all_active) return ee;
-        while (ee < f1) {
-            int nn;
-            S qx, qy, qz;
-            entry_offset<S>(a, ee, true, gc0, gc1, gc2, nn, qx, qy, qz);
-            if (a.src_active[a.nbody[nn]] && ((dm >> a.nbody[nn]) & 1ull)) return ee;
-            ee += NW;
-        }
-        return ee;
-    };
-    real pm[MW];
-    int nd = -1;
-    S ox = 0, oy = 0, oz = 0;
-    int64_t e = seek(fb + w);
-    if (e < f1) {
-        entry_offset<S>(a, e, true, gc0, gc1, gc2, nd, ox, oy, oz);
-        if constexpr (!BIG) {
-#pragma unroll
-            for (int q = 0; q < MW; ++q) {
-                const int k = lane + 32 * q;
-                pm[q] = k < 2 * TP ? far[(int64_t)nd * 2 * TP + k] : real(0);
+        const int64_t g = a.fitem_group[it];
+        const int gb = a.gbody[g];
+        if (!(((a.tgt_mask & dm) >> gb) & 1ull) || g < a.g_lo || g >= a.g_hi) continue;  // rows not used (block-uniform)
+        const int64_t p0 = a.gstart[g], p1 = a.gend[g];
+        const int64_t p = p0 + lane;
+        const s4 xr = xrel[p < p1 ? p : p0];
+        const double gc0 = a.gcenter[3 * g], gc1 = a.gcenter[3 * g + 1], gc2 = a.gcenter[3 * g + 2];
+        const real kappa = to_c<real>((S)a.kappa);
+        real UL = 0, cL = 0, UY = 0, cY = 0;
+        // the group's entries go evenly to its items
+        const int64_t i0 = a.fitem_off[g], fo = a.far_off[g], nf = a.far_off[g + 1] - fo;
+        const int64_t per = (nf + a.fitem_off[g + 1] - i0 - 1) / (a.fitem_off[g + 1] - i0);
+        const int64_t fb = fo + (it - i0) * per, f1 = min(fo + nf, fb + per);
+        for (int64_t e = next_entry<S>(a, fb + w, f1, NW, dm); e < f1; e = next_entry<S>(a, e + NW, f1, NW, dm)) {
+            const int nd = a.far_l[e];
+            __syncwarp();
+            for (int k = lane; k < 2 * NC; k += 32) sM[k] = far[(int64_t)nd * 2 * NC + k];
+            __syncwarp();
+            const bool lap = (a.nbody[nd] == gb) && a.lap_body[gb];
+            const real Rx = to_c<real>(xr.x - (a.ncenter[3 * nd] - gc0));
+            const real Ry = to_c<real>(xr.y - (a.ncenter[3 * nd + 1] - gc1));
+            const real Rz = to_c<real>(xr.z - (a.ncenter[3 * nd + 2] - gc2));
+            real uL, uY;
+            if constexpr (is_ds<real>) {
+                if (lap) far_eval_ds<P, true>(Rx, Ry, Rz, kappa, sM, sM + NC, rad, NW * 32, uL, uY);
+                else far_eval_ds<P, false>(Rx, Ry, Rz, kappa, sM, sM + NC, rad, NW * 32, uL, uY);
+            } else {
+                if (lap) far_eval<real, P, true>(Rx, Ry, Rz, kappa, sM, sM + NC, nullptr, uL, uY);
+                else far_eval<real, P, false>(Rx, Ry, Rz, kappa, sM, sM + NC, nullptr, uL, uY);
             }
+            if (lap) kadd(UL, cL, uL);
+            kadd(UY, cY, uY);
         }
-    }
-    while (e < f1) {
-        __syncwarp();
-        if constexpr (BIG) {
-            for (int k = lane; k < 2 * TP; k += 32) sM[w][k] = far[(int64_t)nd * 2 * TP + k];
-        } else {
-#pragma unroll
-            for (int q = 0; q < MW; ++q) {
-                const int k = lane + 32 * q;
-                if (k < 2 * TP) sM[w][k] = pm[q];
-            }
-        }
-        __syncwarp();
-        const bool lap = (a.nbody[nd] == gb) && a.lap_body[gb];
-        const real Rx = to_c<real>(xr.x - ox), Ry = to_c<real>(xr.y - oy), Rz = to_c<real>(xr.z - oz);
-        e = seek(e + NW);
-        if (e < f1) {  // the next node (its coefficients prefetched up to order 8)
-            entry_offset<S>(a, e, true, gc0, gc1, gc2, nd, ox, oy, oz);
-            if constexpr (!BIG) {
-#pragma unroll
-                for (int q = 0; q < MW; ++q) {
-                    const int k = lane + 32 * q;
-                    pm[q] = k < 2 * TP ? far[(int64_t)nd * 2 * TP + k] : real(0);
-                }
-            }
-        }
-        real uL, uY;
-        if (lap) far_eval<real, P, true>(Rx, Ry, Rz, kappa, sM[w], sM[w] + TP, uL, uY);
-        else far_eval<real, P, false>(Rx, Ry, Rz, kappa, sM[w], sM[w] + TP, uL, uY);
-        kadd(UL, cL, uL);
-        kadd(UY, cY, uY);
-    }
-    store_item<real, NW>(red, w, lane, UL, cL, UY, cY, a.Uf + 64 * it);
+        store_item<real, NW>(red, w, lane, UL, cL, UY, cY, a.Uf + 64 * it);
     }
 }
 
@@ -790,9 +966,9 @@ struct UpArgs {
     int K;
     int64_t lvl_begin, lvl_end;  // node ids of one level (unused by k_upward)
     int p2m_grid;                // > 0: P2M over at most this many blocks (leaves strided)
-    int64_t n_nodes;             // k_far_coef: every node
+    int64_t n_nodes;             // k_far: every node
     const void* far_tab;         // its table (farfield.cu) in the arithmetic type
-    void* far;                   // its output: 2 * n_terms_pad(P) coefficients per node
+    void* far;                   // its output: 2 * n_far_pad(P) coefficients per node
     const int32_t* parent;       // k_upward: parent of every node (-1 at a body's root)
     int* arrive;                 // k_upward: per node, children finished (zero between launches)
 };
@@ -820,195 +996,60 @@ __device__ __constant__ const int kBinom[9][9] = {
     {1, 3, 3, 1, 0, 0, 0, 0, 0},      {1, 4, 6, 4, 1, 0, 0, 0, 0},      {1, 5, 10, 10, 5, 1, 0, 0, 0},
     {1, 6, 15, 20, 15, 6, 1, 0, 0},   {1, 7, 21, 35, 35, 21, 7, 1, 0}, {1, 8, 28, 56, 70, 56, 28, 8, 1}};
 
-// Degree a + b + c of the evaluation-order index j (a, then b, then c).
-__device__ __forceinline__ int eval_degree(int j, int P) {
-    int a = 0;
-    for (;; ++a) {
-        const int n = (P - a + 1) * (P - a + 2) / 2;
-        if (j < n) break;
-        j -= n;
-    }
-    int b = 0;
-    for (;; ++b) {
-        const int n = P - a - b + 1;
-        if (j < n) break;
-        j -= n;
-    }
-    return a + b + j;
-}
-
-// Nonzero entries of one output row of the far-field tables: a Yukawa
-// output of degree p takes the moments of degrees p, p + 2, ..., P, a Laplace
-// output those of degree p.
-__host__ __device__ constexpr int far_row_nnz(int p, int P) {
-    int n = (p + 1) * (p + 2) / 2;  // Laplace
-    for (int q = p; q <= P; q += 2) n += (q + 1) * (q + 2) / 2;
-    return n;
-}
-// Packed table size, and the offset of the first row of degree p (rows in
-// the graded order of the moments).
-__host__ __device__ constexpr int far_pack_offset(int p, int P) {
-    int o = 0;
-    for (int q = 0; q < p; ++q) o += (q + 1) * (q + 2) / 2 * far_row_nnz(q, P);
-    return o;
-}
-
 // Far-field coefficients of every node of an active body from its moments
-// (farfield.cu).  The table comes packed: per output row in the graded order,
-// its Yukawa entries over the moments of degrees p, p + 2, ... then its
-// Laplace entries over degree p (far_pack_offset, far_row_nnz); it is staged
-// in shared memory once per block.  The block then takes nodes in turn: the
-// node's moments go to shared memory, each thread forms outputs (its row of
-// the packed table against the moments) and writes them in the evaluation
-// order of far_eval.  Output per node: Laplace then Yukawa, each padded with
-// zeros.
-template <typename real, int P>
-__global__ void __launch_bounds__(128) k_far_coef(UpArgs a, const real* __restrict__ mom) {
-    constexpr int T = MI<P>::T;
-    constexpr int TP = n_terms_pad(P);
-    constexpr int NNZ = far_pack_offset(P + 1, P);
-    extern __shared__ __align__(16) unsigned char far_smem[];
-    real* tab = reinterpret_cast<real*>(far_smem);
-    real* sm = tab + ((NNZ + 3) & ~3);
-    const real* __restrict__ gtab = (const real*)a.far_tab;
-    for (int k = threadIdx.x; k < NNZ; k += blockDim.x) tab[k] = gtab[k];
-    real* __restrict__ far = (real*)a.far;
-    for (int64_t nd = blockIdx.x; nd < a.n_nodes; nd += gridDim.x) {
-        if (!body_on(a, a.nbody[nd])) continue;  // block-uniform
-        __syncthreads();
-        for (int k = threadIdx.x; k < 2 * T; k += blockDim.x) sm[k] = mom[nd * 2 * T + k];
-        for (int k = T + threadIdx.x; k < TP; k += blockDim.x) {  // padding
-            far[nd * 2 * TP + k] = real(0);
-            far[nd * 2 * TP + TP + k] = real(0);
-        }
-        __syncthreads();
-        for (int j = threadIdx.x; j < T; j += blockDim.x) {
-            int x, y, z;
-            decode_mi(j, x, y, z);
-            const int p = x + y + z;
-            const int g0 = p * (p + 1) * (p + 2) / 6;  // first graded index of degree p
-            const real* row = tab + far_pack_offset(p, P) + (j - g0) * far_row_nnz(p, P);
-            real aY = 0, aL = 0;
-            int e = 0;
-            for (int q = p; q <= P; q += 2) {
-                const int k0 = q * (q + 1) * (q + 2) / 6, k1 = k0 + (q + 1) * (q + 2) / 2;
-                for (int k = k0; k < k1; ++k) aY += row[e++] * sm[T + k];
-            }
-            for (int k = g0; k < g0 + (p + 1) * (p + 2) / 2; ++k) aL += row[e++] * sm[k];
-            // evaluation-order index of (x, y, z): a = x, b = y, c = z
-            int ev = 0;
-            for (int aa = 0; aa < x; ++aa) ev += (P - aa + 1) * (P - aa + 2) / 2;
-            ev += y * (P - x + 1) - y * (y - 1) / 2 + z;
-            far[nd * 2 * TP + ev] = aL;
-            far[nd * 2 * TP + TP + ev] = aY;
-        }
-    }
-}
-
-template <typename real, int P>
-constexpr size_t far_coef_smem() {
-    return sizeof(real) * (((far_pack_offset(P + 1, P) + 3) & ~3) + 2 * MI<P>::T);
-}
-
-// Orders above 8, where the packed table no longer fits shared memory: the
-// table is read from global memory (L2-resident) and each of its entries
-// serves NB nodes, whose moments the block stages in shared memory; a
-// thread forms output rows j (sums in the order of k_far_coef) for all NB
-// nodes.  Inactive nodes in a block get no output.
+// (the tables of farfield.cu): a block takes NB nodes, whose moments it stages
+// side by side in shared memory, and a thread forms one column of the Yukawa
+// or the Laplace table for all of them, so that a table entry (coalesced, from
+// L1 / L2) and NB / 4 shared loads serve NB multiply-adds.  Columns are
+// ordered by degree, and a warp skips the moment degrees that none of its
+// columns takes.  Output per node: Laplace then Yukawa coefficients in the
+// order of far_pos.
 template <typename real, int P, int NB>
-__global__ void __launch_bounds__(128) k_far_big(UpArgs a, const real* __restrict__ mom) {
-    constexpr int T = MI<P>::T;
-    constexpr int TP = n_terms_pad(P);
+__global__ void __launch_bounds__(2 * far_cols(P)) k_far(UpArgs a, const real* __restrict__ mom) {
+    constexpr int T = MI<P>::T, TR = far_cols(P), NC = n_far_pad(P);
     extern __shared__ __align__(16) unsigned char far_smem[];
-    real(*sm)[2 * T] = reinterpret_cast<real(*)[2 * T]>(far_smem);
-    const real* __restrict__ tab = (const real*)a.far_tab;
+    real(*sm)[NB] = reinterpret_cast<real(*)[NB]>(far_smem);  // [2 T][NB]
+    const bool yuk = threadIdx.x < TR;
+    const int j = yuk ? threadIdx.x : threadIdx.x - TR;
+    const real* __restrict__ tab = (const real*)a.far_tab + (yuk ? 0 : (size_t)T * TR) + j;
     real* __restrict__ far = (real*)a.far;
+    int l = 0;
+    while ((l + 1) * (l + 1) <= j) ++l;
+    const int r = j - l * l;
+    const int m = (r + 1) / 2;
+    const int out = (yuk ? NC : 0) + far_pos(P, l, m, r ? (r - 1) & 1 : 0);
     for (int64_t n0 = (int64_t)blockIdx.x * NB; n0 < a.n_nodes; n0 += (int64_t)gridDim.x * NB) {
         const int nn = (int)min((int64_t)NB, a.n_nodes - n0);
         bool act[NB];
 #pragma unroll
         for (int i = 0; i < NB; ++i) act[i] = i < nn && body_on(a, a.nbody[n0 + i]);
         __syncthreads();
-        for (int q = threadIdx.x; q < NB * 2 * T; q += blockDim.x) {
-            const int i = q / (2 * T), k = q - i * 2 * T;
-            sm[i][k] = act[i] ? mom[(n0 + i) * 2 * T + k] : real(0);
-        }
-        if constexpr (TP > T) {
-            for (int q = threadIdx.x; q < NB * (TP - T); q += blockDim.x) {  // padding
-                const int i = q / (TP - T), k = T + q - i * (TP - T);
-                if (act[i]) {
-                    far[(n0 + i) * 2 * TP + k] = real(0);
-                    far[(n0 + i) * 2 * TP + TP + k] = real(0);
-                }
-            }
-        }
+#pragma unroll
+        for (int i = 0; i < NB; ++i)
+            for (int k = threadIdx.x; k < 2 * T; k += blockDim.x)
+                sm[k][i] = act[i] ? mom[(n0 + i) * 2 * T + k] : real(0);
         __syncthreads();
-        for (int j = threadIdx.x; j < T; j += blockDim.x) {
-            int x, y, z;
-            decode_mi(j, x, y, z);
-            const int p = x + y + z;
-            const int g0 = p * (p + 1) * (p + 2) / 6;
-            const real* row = tab + far_pack_offset(p, P) + (int64_t)(j - g0) * far_row_nnz(p, P);
-            real aY[NB], aL[NB];
+        real acc[NB];
 #pragma unroll
-            for (int i = 0; i < NB; ++i) aY[i] = aL[i] = real(0);
-            int e = 0;
-            for (int q = p; q <= P; q += 2) {
-                const int k0 = q * (q + 1) * (q + 2) / 6, k1 = k0 + (q + 1) * (q + 2) / 2;
-                for (int k = k0; k < k1; ++k) {
-                    const real t = row[e++];
+        for (int i = 0; i < NB; ++i) acc[i] = real(0);
+        const real(*sk)[NB] = yuk ? sm + T : sm;
+#pragma unroll 1
+        for (int q = 0; q <= P; ++q) {
+            const bool takes = l <= P && (yuk ? q >= l && !((q - l) & 1) : q == l);
+            if (!__any_sync(0xffffffffu, takes)) continue;
+            const int k0 = q * (q + 1) * (q + 2) / 6, k1 = k0 + (q + 1) * (q + 2) / 2;
+#pragma unroll 4
+            for (int k = k0; k < k1; ++k) {
+                const real v = tab[(size_t)k * TR];  // zero off the pattern
 #pragma unroll
-                    for (int i = 0; i < NB; ++i) aY[i] += t * sm[i][T + k];
-                }
+                for (int i = 0; i < NB; ++i) acc[i] = madd(v, sk[k][i], acc[i]);
             }
-            for (int k = g0; k < g0 + (p + 1) * (p + 2) / 2; ++k) {
-                const real t = row[e++];
-#pragma unroll
-                for (int i = 0; i < NB; ++i) aL[i] += t * sm[i][k];
-            }
-            int ev = 0;
-            for (int aa = 0; aa < x; ++aa) ev += (P - aa + 1) * (P - aa + 2) / 2;
-            ev += y * (P - x + 1) - y * (y - 1) / 2 + z;
+        }
+        if (j < n_far(P))
 #pragma unroll
             for (int i = 0; i < NB; ++i)
-                if (act[i]) {
-                    far[(n0 + i) * 2 * TP + ev] = aL[i];
-                    far[(n0 + i) * 2 * TP + TP + ev] = aY[i];
-                }
-        }
+                if (act[i]) far[(n0 + i) * 2 * NC + out] = acc[i];
     }
-}
-
-// FP32 far-field coefficients: one block per (node, table), one thread per
-// output j of the evaluation order (blockDim = n_terms_pad(P) rounded up to
-// 32), E[j] = sum_k M[k] tab[k][j] over the table transposed and padded
-// (tab[k][j], rows of far_tr(P) columns, Yukawa then Laplace, zeros off the
-// degree pattern): the warp's 32 threads read consecutive entries of a row
-// (L1-resident after first use) against the node's moments broadcast from
-// shared memory.  The problem is small (nodes x 2 T outputs), so the work is
-// spread over as many warps as it has outputs to hide the load latency.
-__host__ __device__ constexpr int far_tr(int P) { return (n_terms_pad(P) + 31) & ~31; }
-template <int P>
-__global__ void __launch_bounds__(256) k_far_f32(UpArgs a, const float* __restrict__ mom) {
-    constexpr int T = MI<P>::T;
-    constexpr int TP = n_terms_pad(P);
-    constexpr int TR = far_tr(P);
-    __shared__ float m[T];
-    const int64_t nd = blockIdx.x;
-    const int t = blockIdx.y;  // 0: Yukawa (moments T .. 2T-1), 1: Laplace
-    if (!body_on(a, a.nbody[nd])) return;  // block-uniform
-    for (int k = threadIdx.x; k < T; k += blockDim.x) m[k] = mom[nd * 2 * T + (t == 0 ? T : 0) + k];
-    __syncthreads();
-    const int j = threadIdx.x;
-    const float* __restrict__ tab = (const float*)a.far_tab + (size_t)t * T * TR + j;
-    float acc0 = 0.f, acc1 = 0.f;
-#pragma unroll 8
-    for (int k = 0; k + 1 < T; k += 2) {
-        acc0 += m[k] * __ldg(tab + (size_t)k * TR);
-        acc1 += m[k + 1] * __ldg(tab + (size_t)(k + 1) * TR);
-    }
-    if (T & 1) acc0 += m[T - 1] * __ldg(tab + (size_t)(T - 1) * TR);
-    if (j < TP) ((float*)a.far)[nd * 2 * TP + (t == 0 ? TP : 0) + j] = acc0 + acc1;
 }
 
 // ---------------------------------------------------------------- fused upward pass
@@ -1018,7 +1059,7 @@ __global__ void __launch_bounds__(256) k_far_f32(UpArgs a, const float* __restri
 // tree is climbed without a launch or a barrier per level and no block waits
 // for another.  Writers fence before their increment; the climbing block
 // fences after it and reads the children's moments from L2 (ld.global.cg).
-// The far-field coefficients follow in k_far_coef.
+// The far-field coefficients follow in k_far.
 // children shifted at once by the moment shift: all eight while their two
 // buffers take at most 64 KB, else half as many per halving
 __host__ __device__ constexpr int up_child_batch(int bytes, int T) {
@@ -1259,23 +1300,47 @@ __global__ void __launch_bounds__(128) k_upward(UpArgs a, const typename V4<real
     }
 }
 
-// M2P warps per block: 8 (FP32) or 4 (8-byte types, for their registers),
-// halved while the per-warp coefficient slices exceed 40 KB of shared memory
+// M2P launch: blocks of 4 warps.
 template <typename real, int P>
-constexpr int m2p_warps() {
-    int nw = sizeof(real) == 8 ? 4 : 8;
-    while (nw > 1 && (size_t)nw * 2 * n_terms_pad(P) * sizeof(real) > 40 * 1024) nw /= 2;
-    return nw;
+void launch_m2p(const EvalArgs& ev, const void* xrel, const void* far, cudaStream_t s) {
+    if (ev.n_fitems <= 0) return;
+    const unsigned grid = (unsigned)(ev.m2p_work ? ev.persist_blocks : ev.n_fitems);
+    if constexpr (sizeof(real) == sizeof(float)) {
+        constexpr int NW = 4;
+        k_m2p_f32<P, NW><<<grid, NW * 32, 0, s>>>(ev, (const float4*)xrel, (const float*)far);
+    } else {
+        constexpr int NW = 4;
+        constexpr size_t smem =
+            NW * 2 * n_far_pad(P) * sizeof(real) + (is_ds<real> ? sizeof(float4) * NW * 32 * (P + 1) : 0);
+        if constexpr (smem > 40 * 1024)
+            PGB_CUDA(cudaFuncSetAttribute(k_m2p<real, P, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        k_m2p<real, P, NW><<<grid, NW * 32, smem, s>>>(
+            ev, (const typename V4<typename Store<real>::S>::t*)xrel, (const real*)far);
+    }
 }
 
-// Nodes per block of k_far_big: 8 in FP32, 4 in the 8-byte types (shared memory).
-template <typename real>
-constexpr int far_big_nb() { return sizeof(real) == sizeof(float) ? 8 : 4; }
+// The far-field coefficients: 8 nodes per block in FP32 and 4 in the 8-byte
+// types (shared memory), where that gives every SM two blocks; with fewer
+// nodes, two and one per block, whose chain of loads is shorter (130 nodes:
+// 8 us less for the whole product).
+template <typename real, int P, int NB>
+void launch_far_nb(const UpArgs& up, const void* mom, cudaStream_t s) {
+    constexpr size_t smem = sizeof(real) * NB * 2 * MI<P>::T;
+    if constexpr (smem > 40 * 1024)
+        PGB_CUDA(cudaFuncSetAttribute(k_far<real, P, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int64_t gf = (up.n_nodes + NB - 1) / NB;
+    if (up.p2m_grid > 0) gf = std::min<int64_t>(gf, up.p2m_grid);
+    k_far<real, P, NB><<<(unsigned)std::max<int64_t>(gf, 1), 2 * far_cols(P), smem, s>>>(up, (const real*)mom);
+}
+template <typename real, int P>
+void launch_far(const UpArgs& up, const void* mom, cudaStream_t s) {
+    constexpr int NB = sizeof(real) == sizeof(float) ? 8 : 4;
+    if (up.n_nodes >= 304 * NB) launch_far_nb<real, P, NB>(up, mom, s);
+    else launch_far_nb<real, P, NB / 4>(up, mom, s);
+}
 
 // The upward pass of one product: P2M and the moment shifts in one launch
-// (k_upward), then the far-field coefficients (orders up to 8: k_far_f32 in
-// FP32, k_far_coef with the packed table in shared memory otherwise; above:
-// k_far_big for every type).
+// (k_upward), then the far-field coefficients (k_far).
 template <typename real, int P>
 void launch_upward(const UpArgs& up, const void* src, void* mom, cudaStream_t s) {
     using v4 = typename V4<real>::t;
@@ -1289,38 +1354,7 @@ void launch_upward(const UpArgs& up, const void* src, void* mom, cudaStream_t s)
     const int64_t grid = up.p2m_grid > 0 ? std::min<int64_t>(up.n_leaves, up.p2m_grid) : up.n_leaves;
     k_upward<real, P><<<(unsigned)grid, 128, up_smem, s>>>(up, (const v4*)src, (real*)mom);
     if (up.n_nodes <= 0) return;
-    int dev = 0, n_sm = 0;
-    PGB_CUDA(cudaGetDevice(&dev));
-    PGB_CUDA(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
-    if constexpr (P > 8) {
-        constexpr int NB = far_big_nb<real>();
-        constexpr size_t smem = sizeof(real) * NB * 2 * MI<P>::T;
-        static bool attr = false;
-        if (!attr) {
-            PGB_CUDA(cudaFuncSetAttribute(k_far_big<real, P, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)smem));
-            attr = true;
-        }
-        int64_t gf = (up.n_nodes + NB - 1) / NB;
-        if (up.p2m_grid > 0) gf = std::min<int64_t>(gf, up.p2m_grid);
-        k_far_big<real, P, NB><<<(unsigned)std::max<int64_t>(gf, 1), 128, smem, s>>>(up, (const real*)mom);
-    } else if constexpr (sizeof(real) == sizeof(float)) {
-        // FP32: a block per (node, table), a thread per output
-        k_far_f32<P><<<dim3((unsigned)up.n_nodes, 2), far_tr(P), 0, s>>>(up, (const float*)mom);
-    } else {
-        // a few blocks per SM, each with the packed table in shared memory,
-        // taking the nodes in turn
-        constexpr size_t smem = far_coef_smem<real, P>();
-        static bool attr = false;
-        if (!attr) {
-            PGB_CUDA(cudaFuncSetAttribute(k_far_coef<real, P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)smem));
-            attr = true;
-        }
-        int64_t gf = std::min<int64_t>(up.n_nodes, 4 * (int64_t)n_sm);
-        if (up.p2m_grid > 0) gf = std::min<int64_t>(gf, up.p2m_grid);
-        k_far_coef<real, P><<<(unsigned)std::max<int64_t>(gf, 1), 128, smem, s>>>(up, (const real*)mom);
-    }
+    launch_far<real, P>(up, mom, s);
 }
 
 }  // namespace pgb
