@@ -6,19 +6,18 @@
 
 namespace pgb {
 
-void treecode_launch_f32(int stage, int P, const UpArgs& up, const std::vector<int64_t>& lv, const EvalArgs& ev,
-                         const void* src, const void* xrel, void* mom, void* far, cudaStream_t s);
-void treecode_launch_f64(int stage, int P, const UpArgs& up, const std::vector<int64_t>& lv, const EvalArgs& ev,
-                         const void* src, const void* xrel, void* mom, void* far, cudaStream_t s);
-void treecode_launch_ds(int stage, int P, const UpArgs& up, const EvalArgs& ev, const void* src, const void* xrel,
-                        void* mom, const void* far, cudaStream_t s);
-void convert_src_ds(const void* src64, void* src_ds, int64_t n, cudaStream_t s);
+void treecode_launch_f32(int stage, int P, const UpArgs& up, const EvalArgs& ev, const void* xrel, void* mom,
+                         const void* far, cudaStream_t s);
+void treecode_launch_f64(int stage, int P, const UpArgs& up, const EvalArgs& ev, const void* xrel, void* mom,
+                         const void* far, cudaStream_t s);
+void treecode_launch_ds(int stage, int P, const UpArgs& up, const EvalArgs& ev, const void* xrel, void* mom,
+                        const void* far, cudaStream_t s);
+void convert_pd_ds(const void* pd64, void* pd_ds, int64_t n, cudaStream_t s);
 
 static inline int nblk(int64_t n, int t) { return (int)std::max<int64_t>(1, (n + t - 1) / t); }
 
 // Panel densities (psi_L, psi_Y, phi) of the combined potential U = S_V - S_K
-// for every sorted panel, and the per-point source terms
-// A = {y - c_leaf, w psi_L}, B = {w phi n, w psi_Y}.
+// for every sorted panel (dens), and the same times the panel's area (pd).
 //   dielectric: psi_L = dphi, psi_Y = (eps_in/eps_out) dphi, phi = phi
 //   imposed potential: psi_Y = u; imposed charge: phi = u
 // pd: the panel densities times the area (and wcorr, far_rule_f32_scale, in FP32).
@@ -29,7 +28,6 @@ static inline int nblk(int64_t n, int t) { return (int)std::max<int64_t>(1, (n +
 // unknowns plus the imposed sigma0 / phi0 of every surface).
 template <typename real>
 __global__ void k_src_prep(Geo g, BodyDev bd, const double* __restrict__ x, int mode,
-                           const typename V4<real>::t* __restrict__ yrel, typename V4<real>::t* __restrict__ src,
                            typename V4<real>::t* __restrict__ pd, real* __restrict__ dens, double eps_out,
                            double wcorr) {
     const bool known = mode == 1;
@@ -59,8 +57,7 @@ __global__ void k_src_prep(Geo g, BodyDev bd, const double* __restrict__ x, int 
         if (kind == PGB_SET_POTENTIAL) phi = bd.bc[b];
         else if (kind == PGB_SET_CHARGE) psiY = -bd.bc[b] / eps_out;
     }
-    // the FP32 product forms its source terms in FP32 (they are stored in
-    // FP32 anyway); the FP64 product in FP64
+    // the FP32 product keeps its densities in FP32, the FP64 product in FP64
     const real rL = (real)psiL, rY = (real)psiY, rp = (real)phi;
     dens[3 * i] = rL;
     dens[3 * i + 1] = rY;
@@ -72,20 +69,6 @@ __global__ void k_src_prep(Geo g, BodyDev bd, const double* __restrict__ x, int 
     pv.z = area * rp;
     pv.w = 0;
     pd[i] = pv;
-    const real nx = (real)g.n[3 * i], ny = (real)g.n[3 * i + 1], nz = (real)g.n[3 * i + 2];
-    for (int m = 0; m < g.K; ++m) {
-        const int64_t p = i * g.K + m;
-        const real w = (real)g.w[p];
-        typename V4<real>::t A = yrel[p], B;
-        const real wp = w * rp;
-        A.w = w * rL;
-        B.x = wp * nx;
-        B.y = wp * ny;
-        B.z = wp * nz;
-        B.w = w * rY;
-        src[2 * p] = A;
-        src[2 * p + 1] = B;
-    }
 }
 
 // U += near-field corrections (FP64), then the rows of Eq. 6 / Eq. 7 in the
@@ -199,7 +182,7 @@ __global__ void k_rows_init(Geo g, BodyDev bd, const double* x, int mode, double
     }
 }
 
-// Source terms of one region's pass: every body on the region's boundary
+// Panel densities of one region's pass: every body on the region's boundary
 // with the densities of its side of the interface and the side's sign folded
 // in, so that the pass sums s [V psi - K phi] (the Yukawa slots, at the
 // region's screening; kappa = 0 is Laplace); all other bodies are zero.
@@ -208,7 +191,6 @@ __global__ void k_rows_init(Geo g, BodyDev bd, const double* x, int mode, double
 //   psi = -sigma0 / eps_R (known).   mode as k_src_prep (x unused for 1).
 template <typename real>
 __global__ void k_src_region(Geo g, BodyDev bd, RegionDev rd, const double* __restrict__ x, int mode,
-                             const typename V4<real>::t* __restrict__ yrel, typename V4<real>::t* __restrict__ src,
                              typename V4<real>::t* __restrict__ pd, real* __restrict__ dens, double wcorr) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= g.n_pan) return;
@@ -246,20 +228,6 @@ __global__ void k_src_region(Geo g, BodyDev bd, RegionDev rd, const double* __re
     pv.z = area * rp;
     pv.w = 0;
     pd[i] = pv;
-    const real nx = (real)g.n[3 * i], ny = (real)g.n[3 * i + 1], nz = (real)g.n[3 * i + 2];
-    for (int m = 0; m < g.K; ++m) {
-        const int64_t p = i * g.K + m;
-        const real w = (real)g.w[p];
-        typename V4<real>::t A = yrel[p], B;
-        const real wp = w * rp;
-        A.w = 0;
-        B.x = wp * nx;
-        B.y = wp * ny;
-        B.z = wp * nz;
-        B.w = w * rY;
-        src[2 * p] = A;
-        src[2 * p + 1] = B;
-    }
 }
 
 // One region's sums into its rows: the pass's item partials (Yukawa slots)
@@ -328,13 +296,59 @@ void apply_operator(pgb_ctx* c, const double* x, double* y, int precision, bool 
 
 void apply_full(pgb_ctx* c, const double* x, double* y, int precision) { apply_mode(c, x, y, precision, 2, nullptr); }
 
+// One stage of the treecode in the arithmetic `kind` (0 FP32, 1 FP64, 2
+// double-single).
+static void launch_stage(pgb_ctx* c, int stage, int kind, const UpArgs& up, const EvalArgs& ev, void* mom,
+                         cudaStream_t s) {
+    if (kind == 0) treecode_launch_f32(stage, c->p.P, up, ev, c->d_x32, mom, up.far, s);
+    else if (kind == 1) treecode_launch_f64(stage, c->p.P, up, ev, c->d_x64, mom, up.far, s);
+    else treecode_launch_ds(stage, c->p.P, up, ev, c->d_x64, mom, up.far, s);
+}
+
+// The panel moments of the current geometry in the arithmetic `kind`: formed on
+// the context's stream the first time a product of that kind meets the
+// geometry, kept until the geometry or the order changes.  nullptr where they
+// would take more than a sixteenth of the device's memory (336 bytes a panel in
+// FP32 at order 6, 3.3 KB at order 15) or cannot be allocated: the P2M then
+// forms them on the spot.
+static const void* panel_moments(pgb_ctx* c, int kind) {
+    auto& pm = c->pan_mom[kind];
+    if (pm.geom_gen == c->geom_gen && pm.P == c->p.P) return pm.have ? (const void*)pm.buf.p : nullptr;
+    if (c->capturing) return nullptr;  // (every product is prepared outside the capture)
+    pm.have = false;
+    pm.geom_gen = c->geom_gen;
+    pm.P = c->p.P;
+    const size_t esz = kind == 0 ? 4 : 8;
+    const size_t bytes = (size_t)c->n_pan * n_terms(c->p.P) * esz;
+    size_t free_b = 0, total_b = 0;
+    PGB_CUDA(cudaMemGetInfo(&free_b, &total_b));
+    if (bytes > total_b / 16) return nullptr;
+    try {
+        pm.buf.resize(bytes);
+    } catch (const Error& e) {
+        if (e.code != PGB_ENOMEM) throw;
+        return nullptr;
+    }
+    UpArgs up = {};
+    up.K = c->p.K;
+    up.rule = far_rule(c->p.K);
+    up.pg = kind == 0 ? (const void*)c->d_pg32.p : kind == 1 ? (const void*)c->d_pg64.p : (const void*)c->d_pg_ds.p;
+    EvalArgs ev = {};
+    ev.n_pan = c->n_pan;
+    launch_stage(c, STAGE_PANEL_MOMENTS, kind, up, ev, pm.buf.p, c->stream);
+    PGB_CUDA(cudaGetLastError());
+    PGB_LAUNCHED(c, 1);
+    pm.have = true;
+    return pm.buf.p;
+}
+
 // Upward pass as a CUDA graph: captured (on a private stream; nothing runs
 // there) the first time a tree / buffer / source-activity combination is
 // used, then one cudaGraphLaunch on the context stream per product.
-static void upward_graph(pgb_ctx* c, int kind, const UpArgs& up, const EvalArgs& ev, const void* src, void* mom,
-                         cudaStream_t on) {  // kind: 0 FP32, 1 FP64, 2 double-single
+static void upward_graph(pgb_ctx* c, int kind, const UpArgs& up, const EvalArgs& ev, void* mom, cudaStream_t on) {
     auto& gr = c->up_graph[kind];
-    bool ok = gr.exec && gr.tree_gen == c->tree_gen && gr.src == src && gr.mom == mom && gr.ncenter == up.ncenter &&
+    bool ok = gr.exec && gr.tree_gen == c->tree_gen && gr.pd == up.pd && gr.pg == up.pg && gr.pmom == up.pmom &&
+              gr.mom == mom && gr.ncenter == up.ncenter &&
               gr.p2m_grid == up.p2m_grid && gr.far == up.far && gr.far_tab == up.far_tab;
     for (int b = 0; ok && b < PGB_MAX_BODIES; ++b) ok = gr.src_active[b] == up.src_active[b];
     if (!ok) {
@@ -346,14 +360,7 @@ static void upward_graph(pgb_ctx* c, int kind, const UpArgs& up, const EvalArgs&
         PGB_CUDA(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
         std::string why;
         try {
-            if (kind == 0)
-                treecode_launch_f32(PGB_STAGE_UPWARD, c->p.P, up, c->level_begin, ev, src, nullptr, mom, up.far,
-                                    c->cap_stream);
-            else if (kind == 1)
-                treecode_launch_f64(PGB_STAGE_UPWARD, c->p.P, up, c->level_begin, ev, src, nullptr, mom, up.far,
-                                    c->cap_stream);
-            else
-                treecode_launch_ds(PGB_STAGE_UPWARD, c->p.P, up, ev, src, nullptr, mom, up.far, c->cap_stream);
+            launch_stage(c, PGB_STAGE_UPWARD, kind, up, ev, mom, c->cap_stream);
         } catch (const Error& e) {
             why = e.msg;
         }
@@ -372,7 +379,9 @@ static void upward_graph(pgb_ctx* c, int kind, const UpArgs& up, const EvalArgs&
         if (ie != cudaSuccess) gr.exec = nullptr;
         PGB_CUDA(ie);
         gr.tree_gen = c->tree_gen;
-        gr.src = src;
+        gr.pd = up.pd;
+        gr.pg = up.pg;
+        gr.pmom = up.pmom;
         gr.mom = mom;
         gr.far = up.far;
         gr.far_tab = up.far_tab;
@@ -400,20 +409,16 @@ static cudaStream_t upward_stream(pgb_ctx* c, int pi) {
 void reserve_product(pgb_ctx* c, int precision) {
     const int pi = precision == PGB_FP32 ? 0 : 1;
     const int T = n_terms(c->p.P);
-    const int64_t nsrc = c->n_pan * c->p.K;
     c->d_dens[pi].resize(3 * c->n_pan);
     c->d_Up[pi].resize(64 * std::max<int64_t>(c->n_pitems, 1));
     c->d_Uf[pi].resize(64 * std::max<int64_t>(c->n_fitems, 1));
     c->d_work.resize(2);
     const int TP = n_far_pad(c->p.P);
     if (pi == 0) {
-        c->d_src32.resize(2 * nsrc);
         c->d_pd32.resize(c->n_pan);
         c->d_mom32.resize((size_t)c->n_nodes * 2 * T);
         c->d_far32.resize((size_t)c->n_nodes * 2 * TP);
     } else {
-        c->d_src64.resize(2 * nsrc);
-        c->d_src_ds.resize(2 * nsrc);
         c->d_pd64.resize(c->n_pan);
         c->d_pd_ds.resize(c->n_pan);
         c->d_mom64.resize((size_t)c->n_nodes * 2 * T);
@@ -421,6 +426,7 @@ void reserve_product(pgb_ctx* c, int precision) {
         c->d_mom_ds.resize((size_t)c->n_nodes * 2 * T);
         c->d_far_ds.resize((size_t)c->n_nodes * 2 * TP);
     }
+    (void)panel_moments(c, precision == PGB_FP32 ? 0 : precision == PGB_FP64_DS ? 2 : 1);
     (void)far_table(c, c->kappa);
     for (const auto& reg : c->regions) (void)far_table(c, reg->dev.kappa);
     if (c->arrive_gen[pi] != c->tree_gen || c->d_arrive[pi].n < (size_t)c->n_nodes) {
@@ -441,7 +447,6 @@ void apply_mode(pgb_ctx* c, const double* x, double* y, int precision, int mode,
             if (!known_mask[b]) bd.bc[b] = 0.0;
     const int P = c->p.P;
     const int T = n_terms(P);
-    const int64_t nsrc = g.n_src;
     // per-precision work buffers: an FP64 product may run on a side stream
     // while FP32 products go on
     const int pi = precision == PGB_FP32 ? 0 : 1;
@@ -456,10 +461,12 @@ void apply_mode(pgb_ctx* c, const double* x, double* y, int precision, int mode,
     up.leaf_node = c->d_leaf_node; up.nstart = c->d_node_start; up.nend = c->d_node_end;
     up.child = c->d_node_child; up.nchild = c->d_node_nchild;
     up.ncenter = c->d_node_center; up.K = c->p.K; up.nbody = c->d_node_body;
-    up.lvl_begin = up.lvl_end = 0;
     up.p2m_grid = 0;
     up.n_nodes = c->n_nodes;
     up.parent = c->d_node_parent;
+    up.n_internal = c->n_nodes - c->n_leaves;
+    up.internal_node = c->d_internal_node;
+    up.n_ichild = c->d_node_nichild;
     {
         const int pi_up = precision == PGB_FP32 ? 0 : 1;
         auto& cnt = c->d_arrive[pi_up];
@@ -474,6 +481,7 @@ void apply_mode(pgb_ctx* c, const double* x, double* y, int precision, int mode,
         up.p2m_grid = 2 * c->persist_blocks;
     EvalArgs ev;
     ev.n_groups = c->n_groups;
+    ev.n_pan = c->n_pan;
     ev.gstart = c->d_group_start; ev.gend = c->d_group_end; ev.gbody = c->d_group_body;
     ev.gcenter = c->d_group_center; ev.near_off = c->d_near_off; ev.far_off = c->d_far_off;
     ev.near_l = c->d_near; ev.far_l = c->d_far; ev.nstart = c->d_node_start; ev.nend = c->d_node_end;
@@ -527,7 +535,6 @@ void apply_mode(pgb_ctx* c, const double* x, double* y, int precision, int mode,
     const double wcorr = f32 ? far_rule_f32_scale(c->p.K) : 1.0;
     const int TP = n_far_pad(P);
     if (f32) {
-        c->d_src32.resize(2 * nsrc);
         c->d_pd32.resize(c->n_pan);
         c->d_mom32.resize((size_t)c->n_nodes * 2 * T);
         c->d_far32.resize((size_t)c->n_nodes * 2 * TP);
@@ -535,7 +542,6 @@ void apply_mode(pgb_ctx* c, const double* x, double* y, int precision, int mode,
         ev.pg = c->d_pg32.p;
         ev.pd = c->d_pd32.p;
     } else {
-        c->d_src64.resize(2 * nsrc);
         c->d_pd64.resize(c->n_pan);
         c->d_mom64.resize((size_t)c->n_nodes * 2 * T);
         c->d_far64.resize((size_t)c->n_nodes * 2 * TP);
@@ -543,8 +549,7 @@ void apply_mode(pgb_ctx* c, const double* x, double* y, int precision, int mode,
         ev.pg = c->d_pg64.p;
         ev.pd = c->d_pd64.p;
         if (precision == PGB_FP64_DS) {
-            c->d_src_ds.resize(2 * nsrc);
-            c->d_pd_ds.resize(c->n_pan);
+                c->d_pd_ds.resize(c->n_pan);
             c->d_mom_ds.resize((size_t)c->n_nodes * 2 * T);
             c->d_far_ds.resize((size_t)c->n_nodes * 2 * TP);
             up.far = c->d_far_ds.p;
@@ -553,6 +558,12 @@ void apply_mode(pgb_ctx* c, const double* x, double* y, int precision, int mode,
         }
     }
     const bool dsp = precision == PGB_FP64_DS;
+    const int kind = f32 ? 0 : dsp ? 2 : 1;
+    void* mom = f32 ? (void*)c->d_mom32.p : dsp ? (void*)c->d_mom_ds.p : (void*)c->d_mom64.p;
+    up.rule = ev.rule;
+    up.pg = ev.pg;
+    up.pd = ev.pd;
+    up.pmom = panel_moments(c, kind);
     auto tab_for = [&](double kappa) -> const void* {
         const FarTab& t = far_table(c, kappa);
         if (f32) return t.t32.p;
@@ -586,30 +597,20 @@ void apply_mode(pgb_ctx* c, const double* x, double* y, int precision, int mode,
             {
                 StageTimer tm(c, PGB_STAGE_SOURCES + (f32 ? 0 : PGB_STAGE_FP64));
                 if (f32)
-                    k_src_region<float><<<nblk(c->n_pan, 128), 128, 0, s>>>(g, bd, rd, x, mode, c->d_y32, c->d_src32, c->d_pd32,
+                    k_src_region<float><<<nblk(c->n_pan, 128), 128, 0, s>>>(g, bd, rd, x, mode, c->d_pd32,
                                                                              (float*)dens.p, wcorr);
                 else
-                    k_src_region<double><<<nblk(c->n_pan, 128), 128, 0, s>>>(g, bd, rd, x, mode, c->d_y64,
-                                                                              c->d_src64, c->d_pd64, dens.p, wcorr);
-                if (precision == PGB_FP64_DS) {
-                    convert_src_ds(c->d_src64, c->d_src_ds, 2 * nsrc, s);
-                    convert_src_ds(c->d_pd64, c->d_pd_ds, c->n_pan, s);
-                }
+                    k_src_region<double><<<nblk(c->n_pan, 128), 128, 0, s>>>(g, bd, rd, x, mode, c->d_pd64,
+                                                                              dens.p, wcorr);
+                if (precision == PGB_FP64_DS) convert_pd_ds(c->d_pd64, c->d_pd_ds, c->n_pan, s);
                 PGB_CUDA(cudaGetLastError());
-                PGB_LAUNCHED(c, precision == PGB_FP64_DS ? 3 : 1);
+                PGB_LAUNCHED(c, precision == PGB_FP64_DS ? 2 : 1);
             }
             for (int stage : {PGB_STAGE_UPWARD, PGB_STAGE_P2P, PGB_STAGE_M2P}) {
                 StageTimer tm(c, stage + (f32 ? 0 : PGB_STAGE_FP64));
-                if (f32)
-                    treecode_launch_f32(stage, P, up, c->level_begin, ev, c->d_src32, c->d_x32, c->d_mom32,
-                                        c->d_far32, s);
-                else if (dsp)
-                    treecode_launch_ds(stage, P, up, ev, c->d_src_ds, c->d_x64, c->d_mom_ds, c->d_far_ds, s);
-                else
-                    treecode_launch_f64(stage, P, up, c->level_begin, ev, c->d_src64, c->d_x64, c->d_mom64,
-                                        c->d_far64, s);
+                launch_stage(c, stage, kind, up, ev, mom, s);
                 PGB_CUDA(cudaGetLastError());
-                PGB_LAUNCHED(c, 1);
+                PGB_LAUNCHED(c, stage == PGB_STAGE_UPWARD ? 3 : 1);
             }
             {
                 StageTimer tm(c, PGB_STAGE_ASSEMBLE + (f32 ? 0 : PGB_STAGE_FP64));
@@ -631,17 +632,14 @@ void apply_mode(pgb_ctx* c, const double* x, double* y, int precision, int mode,
     {
         StageTimer tm(c, PGB_STAGE_SOURCES + (f32 ? 0 : PGB_STAGE_FP64));
         if (f32)
-            k_src_prep<float><<<nblk(c->n_pan, 128), 128, 0, s>>>(g, bd, x, mode, c->d_y32, c->d_src32, c->d_pd32,
+            k_src_prep<float><<<nblk(c->n_pan, 128), 128, 0, s>>>(g, bd, x, mode, c->d_pd32,
                                                                   (float*)dens.p, c->eps_out, wcorr);
         else
-            k_src_prep<double><<<nblk(c->n_pan, 128), 128, 0, s>>>(g, bd, x, mode, c->d_y64, c->d_src64, c->d_pd64,
+            k_src_prep<double><<<nblk(c->n_pan, 128), 128, 0, s>>>(g, bd, x, mode, c->d_pd64,
                                                                    dens.p, c->eps_out, wcorr);
-        if (precision == PGB_FP64_DS) {
-            convert_src_ds(c->d_src64, c->d_src_ds, 2 * nsrc, s);
-            convert_src_ds(c->d_pd64, c->d_pd_ds, c->n_pan, s);
-        }
+        if (precision == PGB_FP64_DS) convert_pd_ds(c->d_pd64, c->d_pd_ds, c->n_pan, s);
         PGB_CUDA(cudaGetLastError());
-        PGB_LAUNCHED(c, precision == PGB_FP64_DS ? 3 : 1);
+        PGB_LAUNCHED(c, precision == PGB_FP64_DS ? 2 : 1);
     }
     // the upward pass on its own stream, beside P2P (which does not read the
     // moments); M2P waits for it
@@ -650,34 +648,21 @@ void apply_mode(pgb_ctx* c, const double* x, double* y, int precision, int mode,
     PGB_CUDA(cudaStreamWaitEvent(us, c->up_fork[pi], 0));
     {
         StageTimer tm(c, PGB_STAGE_UPWARD + (f32 ? 0 : PGB_STAGE_FP64), us);
-        const void* usrc = f32 ? (const void*)c->d_src32.p : dsp ? (const void*)c->d_src_ds.p : (const void*)c->d_src64.p;
-        void* umom = f32 ? (void*)c->d_mom32.p : dsp ? (void*)c->d_mom_ds.p : (void*)c->d_mom64.p;
         if (c->p.graphs && !c->capturing) {
-            upward_graph(c, f32 ? 0 : dsp ? 2 : 1, up, ev, usrc, umom, us);
-            c->graph_kernels += 2;
+            upward_graph(c, kind, up, ev, mom, us);
+            c->graph_kernels += 3;
             ++c->graph_launches;
+        } else {
+            launch_stage(c, PGB_STAGE_UPWARD, kind, up, ev, mom, us);
         }
-        else if (f32)
-            treecode_launch_f32(PGB_STAGE_UPWARD, P, up, c->level_begin, ev, c->d_src32, c->d_x32, c->d_mom32,
-                                c->d_far32, us);
-        else if (dsp)
-            treecode_launch_ds(PGB_STAGE_UPWARD, P, up, ev, c->d_src_ds, c->d_x64, c->d_mom_ds, c->d_far_ds, us);
-        else
-            treecode_launch_f64(PGB_STAGE_UPWARD, P, up, c->level_begin, ev, c->d_src64, c->d_x64, c->d_mom64,
-                                c->d_far64, us);
         PGB_CUDA(cudaGetLastError());
-        PGB_LAUNCHED(c, 2);
+        PGB_LAUNCHED(c, 3);
     }
     PGB_CUDA(cudaEventRecord(c->up_join[pi], us));
     for (int stage : {PGB_STAGE_P2P, PGB_STAGE_M2P}) {
         if (stage == PGB_STAGE_M2P) PGB_CUDA(cudaStreamWaitEvent(s, c->up_join[pi], 0));
         StageTimer tm(c, stage + (f32 ? 0 : PGB_STAGE_FP64));
-        if (f32)
-            treecode_launch_f32(stage, P, up, c->level_begin, ev, c->d_src32, c->d_x32, c->d_mom32, c->d_far32, s);
-        else if (dsp)
-            treecode_launch_ds(stage, P, up, ev, c->d_src_ds, c->d_x64, c->d_mom_ds, c->d_far_ds, s);
-        else
-            treecode_launch_f64(stage, P, up, c->level_begin, ev, c->d_src64, c->d_x64, c->d_mom64, c->d_far64, s);
+        launch_stage(c, stage, kind, up, ev, mom, s);
         PGB_CUDA(cudaGetLastError());
         PGB_LAUNCHED(c, 1);
     }

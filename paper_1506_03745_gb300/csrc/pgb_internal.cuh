@@ -228,7 +228,7 @@ struct pgb_ctx {
     int64_t n_nodes = 0, n_leaves = 0;
     pgb::DBuf<int32_t> d_node_start, d_node_end, d_node_level, d_node_child, d_node_nchild, d_node_body;
     pgb::DBuf<int32_t> d_node_leaf0, d_node_leaf1, d_leaf_node, d_node_parent;
-    pgb::DBuf<unsigned int> d_up_counter;
+    pgb::DBuf<int32_t> d_internal_node, d_node_nichild;  // nodes with children; children with children of every node
     std::vector<int32_t> h_node_level;   // for per-level passes
     std::vector<int64_t> level_begin;    // node id ranges by level
     pgb::DBuf<int32_t> d_pan_leaf;
@@ -299,9 +299,13 @@ struct pgb_ctx {
     pgb::DBuf<double> d_momT64, d_Tout, d_sT, d_lam, d_gx, d_bu;
 
     // matvec work buffers
-    pgb::DBuf<float4> d_src32;           // 2 per point
-    pgb::DBuf<pgb::dbl4> d_src64;
-    pgb::DBuf<pgb::dbl4> d_src_ds;       // the same split into double-single (32 bytes each)
+    // panel moments of the P2M (k_panel_moments) per arithmetic: FP32, FP64, double-single
+    struct PanMom {
+        pgb::DBuf<unsigned char> buf;
+        uint64_t geom_gen = ~0ull;       // the geometry they were formed for
+        int P = -1;
+        bool have = false;
+    } pan_mom[3];
     pgb::DBuf<double> d_dens[2];            // 3 per sorted panel: psiL, psiY, phi
     pgb::DBuf<float> d_mom32;            // 2*T per node
     pgb::DBuf<double> d_mom64;
@@ -340,7 +344,7 @@ struct pgb_ctx {
     struct UpGraph {
         cudaGraphExec_t exec = nullptr;
         uint64_t tree_gen = 0;
-        const void* src = nullptr;
+        const void *pd = nullptr, *pg = nullptr, *pmom = nullptr;
         void* mom = nullptr;
         void* far = nullptr;
         const void* far_tab = nullptr;
@@ -381,6 +385,7 @@ struct pgb_ctx {
     // beside the P2P kernel, which does not need the moments; per precision
     cudaStream_t up_stream[2] = {nullptr, nullptr};
     cudaEvent_t up_fork[2] = {nullptr, nullptr}, up_join[2] = {nullptr, nullptr};
+    uint64_t geom_gen = 0;               // bumped whenever the world geometry is rebuilt
     uint64_t tree_gen = 0;               // bumped whenever the octree structure is rebuilt
     uint64_t config_gen = 0;             // bumped when bodies, charges, boundary values or solvent change
     bool owns_stream = false;            // lane contexts create (and destroy) their stream

@@ -888,7 +888,7 @@ static void overlap_fork(pgb_ctx* c, const double* xs, void* user) {
     double* xfull = c->d_xspec.p;  // overwrite x* in place: x_outer + inner iterate
     k_axpby<<<nblk(n, 256), 256, 0, s>>>(1.0, oa->x_outer, 1.0, xs, xfull, n);
     c->d_r64.resize(n);
-    reserve_product(c, PGB_FP64);
+    reserve_product(c, c->p.residual ? PGB_FP64_DS : PGB_FP64);
     int dev = 0, sms = 0;
     PGB_CUDA(cudaGetDevice(&dev));
     PGB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));

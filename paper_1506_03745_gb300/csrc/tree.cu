@@ -508,6 +508,18 @@ __global__ void k_parents(const int32_t* child, const int32_t* nch, int64_t n, i
     for (int k = 0; k < nch[i]; ++k) parent[child[i] + k] = (int32_t)i;
 }
 
+// The nodes with children, in any order (count in *cnt), and how many children
+// of every node have children themselves.
+__global__ void k_internal(const int32_t* child, const int32_t* nch, int64_t n, int32_t* list, int32_t* nich,
+                           int* cnt) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    int c = 0;
+    for (int k = 0; k < nch[i]; ++k) c += nch[child[i] + k] > 0;
+    nich[i] = c;
+    if (nch[i] > 0) list[atomicAdd(cnt, 1)] = (int32_t)i;
+}
+
 __global__ void k_fill_i32(int32_t* p, int64_t n, int32_t v) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i < n) p[i] = v;
@@ -629,8 +641,12 @@ void build_order(pgb_ctx* c) {
     c->d_node_parent.resize(nn);
     k_fill_i32<<<nblk(nn, 256), 256, 0, s>>>(c->d_node_parent, nn, -1);
     k_parents<<<nblk(nn, 256), 256, 0, s>>>(c->d_node_child, c->d_node_nchild, nn, c->d_node_parent);
-    c->d_up_counter.resize(nn);
-    PGB_CUDA(cudaMemsetAsync(c->d_up_counter.p, 0, 4 * nn, s));
+    c->d_internal_node.resize(nn + 1);
+    c->d_node_nichild.resize(nn);
+    PGB_CUDA(cudaMemsetAsync(c->d_internal_node.p + nn, 0, 4, s));
+    k_internal<<<nblk(nn, 256), 256, 0, s>>>(c->d_node_child, c->d_node_nchild, nn, c->d_internal_node,
+                                             c->d_node_nichild, c->d_internal_node.p + nn);
+    PGB_CUDA(cudaGetLastError());
     // leaves
     DBuf<int64_t> mark, lscan;
     mark.resize(n);
@@ -873,6 +889,7 @@ __global__ void k_panel_geo(const int32_t* pan_leaf, const int32_t* leaf_node, c
 }
 
 void build_geometry(pgb_ctx* c) {
+    ++c->geom_gen;
     cudaStream_t s = c->stream;
     int64_t n = c->n_pan;
     int K = c->p.K;

@@ -278,8 +278,11 @@ __device__ __forceinline__ void decode_mi(int t, int& x, int& y, int& z) {
 // the run-time body mask of a product (all bodies without one)
 __device__ __forceinline__ unsigned long long body_mask(const unsigned long long* m) { return m ? *m : ~0ull; }
 
+// stage code of the panel moments' launch (the others: PGB_STAGE_*)
+#define STAGE_PANEL_MOMENTS (-1)
+
 struct EvalArgs {
-    int64_t n_groups;
+    int64_t n_groups, n_pan;
     const int32_t *gstart, *gend, *gbody;
     const double* gcenter;
     const int64_t *near_off, *far_off;
@@ -964,13 +967,18 @@ struct UpArgs {
     const unsigned long long* bmask = nullptr;  // as EvalArgs::bmask
     const double* ncenter;
     int K;
-    int64_t lvl_begin, lvl_end;  // node ids of one level (unused by k_upward)
     int p2m_grid;                // > 0: P2M over at most this many blocks (leaves strided)
     int64_t n_nodes;             // k_far: every node
     const void* far_tab;         // its table (farfield.cu) in the arithmetic type
     void* far;                   // its output: 2 * n_far_pad(P) coefficients per node
-    const int32_t* parent;       // k_upward: parent of every node (-1 at a body's root)
-    int* arrive;                 // k_upward: per node, children finished (zero between launches)
+    FarRule rule;                // far rule (panel moments)
+    const void* pg;              // panel geometry (PanelGeo) in the arithmetic type
+    const void* pd;              // panel densities x area
+    const void* pmom;            // panel moments (k_panel_moments), nullptr: formed in the P2M
+    const int32_t* parent;       // k_climb: parent of every node (-1 at a body's root)
+    int* arrive;                 // k_climb: per node, internal children finished (zero between launches)
+    int64_t n_internal;          // k_climb: the nodes with children, in any order, and per node its
+    const int32_t *internal_node, *n_ichild;  // children that have children
 };
 // a source body of the upward pass is used (its densities are not all zero
 // and the run-time mask keeps it)
@@ -978,18 +986,6 @@ __device__ __forceinline__ bool body_on(const UpArgs& a, int b) {
     return a.src_active[b] && (!a.bmask || ((*a.bmask >> b) & 1ull));
 }
 
-
-// C(n, m) for n, m <= 15 (0 for m > n), by Pascal's rule at compile time
-struct BinomTable {
-    double v[16][16];
-    __host__ __device__ constexpr BinomTable() : v() {
-        for (int n = 0; n < 16; ++n) {
-            v[n][0] = 1.0;
-            for (int m = 1; m <= n; ++m) v[n][m] = v[n - 1][m - 1] + (m < n ? v[n - 1][m] : 0.0);
-        }
-    }
-};
-__device__ const BinomTable kBinomTable = BinomTable();
 
 __device__ __constant__ const int kBinom[9][9] = {
     {1, 0, 0, 0, 0, 0, 0, 0, 0},      {1, 1, 0, 0, 0, 0, 0, 0, 0},      {1, 2, 1, 0, 0, 0, 0, 0, 0},
@@ -1038,7 +1034,7 @@ __global__ void __launch_bounds__(2 * far_cols(P)) k_far(UpArgs a, const real* _
             const bool takes = l <= P && (yuk ? q >= l && !((q - l) & 1) : q == l);
             if (!__any_sync(0xffffffffu, takes)) continue;
             const int k0 = q * (q + 1) * (q + 2) / 6, k1 = k0 + (q + 1) * (q + 2) / 2;
-#pragma unroll 4
+#pragma unroll 8
             for (int k = k0; k < k1; ++k) {
                 const real v = tab[(size_t)k * TR];  // zero off the pattern
 #pragma unroll
@@ -1052,42 +1048,52 @@ __global__ void __launch_bounds__(2 * far_cols(P)) k_far(UpArgs a, const real* _
     }
 }
 
-// ---------------------------------------------------------------- fused upward pass
-// The upward pass in one launch: each block takes leaves (P2M), and a node's
-// moment shift runs in the block whose child finished last (a counter per
-// node; the last of nchild increments goes on up, the others stop), so the
-// tree is climbed without a launch or a barrier per level and no block waits
-// for another.  Writers fence before their increment; the climbing block
-// fences after it and reads the children's moments from L2 (ld.global.cg).
-// The far-field coefficients follow in k_far.
-// children shifted at once by the moment shift: all eight while their two
-// buffers take at most 64 KB, else half as many per halving
-__host__ __device__ constexpr int up_child_batch(int bytes, int T) {
-    int cb = 8;
-    while (cb > 1 && 2 * cb * 2 * T * bytes > 64 * 1024) cb /= 2;
-    return cb;
+// ---------------------------------------------------------------- upward pass
+// P2M: a block per leaf (k_p2m).  Moment shifts in one launch (k_climb): a block
+// per internal node whose children are all leaves; a node above runs in the
+// block whose internal child finished last (a counter per node; the last of
+// its internal children's increments goes on up, the others stop), so the tree
+// is climbed without a launch or a barrier per level and no block waits for
+// another.  Writers fence before their increment; the climbing block fences
+// after it and reads the children's moments from L2 (ld.global.cg).  The
+// far-field coefficients follow in k_far.  The whole pass is a chain of loads
+// (its arithmetic is a few microseconds of the GPU): small blocks, many of
+// them resident, and few steps in the chain are what it wants.  P2M and shifts
+// in one kernel of 256-thread blocks held four blocks an SM, 65 us for 2968
+// leaves.
+//
+// P2M.  The densities are constant on a panel, so with the panel's moments
+// V_k = sum_m w_m u_m^k (the far rule's points, u = leaf centre - y) the leaf's
+// moments are
+//   M_k = sum_j A_j psi_j V_jk + sum_a k_a D_a[k - e_a],
+//   D_a[k'] = sum_j A_j phi_j n_j,a V_jk':
+// five multiply-adds per panel and k.  The V depend on the geometry alone; they
+// are formed once per geometry (k_panel_moments) and read back coalesced.
+#define UP_THREADS 256  // k_climb: a warp per child
+__host__ __device__ __forceinline__ int mi_index(int x, int y, int z) {  // position in MI's order
+    const int n = x + y + z;
+    return n * (n + 1) * (n + 2) / 6 + (n - x) * (n - x + 1) / 2 + z;
 }
-template <typename real, int P>
-struct UpShared {
-    static constexpr int T = MI<P>::T;
-    static constexpr int TD = P * (P + 1) * (P + 2) / 6 > 0 ? P * (P + 1) * (P + 2) / 6 : 1;
-    static constexpr int CB = up_child_batch((int)sizeof(real), T);
-    struct P2M {
-        real pw[128][3][P + 1];
-        real sq[128][5];
-        real sd[3][TD];
-    };
-    struct M2M {
-        real bufA[CB][2 * T], bufB[CB][2 * T];
-        real cd[CB][3][P + 1];
-    };
-    union {
-        P2M p;
-        M2M m;
-    } u;
-    real binom[P + 1][P + 1];
-    short idx3[P + 1][P + 1][P + 1];
+constexpr int UP_CHUNK = 64;  // panels whose densities are staged at once
+constexpr int UP_FLY = 4;     // panels whose point powers are staged at once (V formed on the spot)
+// threads of a P2M block: one per multi-index, between 64 and 256
+__host__ __device__ constexpr int p2m_threads(int P) {
+    return n_terms(P) >= 256 ? 256 : (n_terms(P) <= 64 ? 64 : (n_terms(P) + 31) & ~31);
+}
+template <typename real, int P, bool STORED>
+struct P2MShared {
+    static constexpr int T = MI<P>::T, BT = p2m_threads(P);
+    static constexpr int NP = T >= BT ? 1 : BT / T;  // shares of a leaf's panels
+    real q[UP_CHUNK][5];                             // psi_L, psi_Y, phi n (all x area)
+    real sum[NP][5][T];
+    real pw[STORED ? 1 : UP_FLY * 7][3][P + 1];
     signed char kk[T][3];
+};
+template <typename real, int P>
+struct ClimbShared {
+    real buf[8][2 * MI<P>::T];
+    real d[8][3];
+    signed char ln[(P + 1) * (P + 2) / 2][2];
     int next;
 };
 
@@ -1099,203 +1105,270 @@ __device__ __forceinline__ ds ld_cg(const ds* p) {
     const float2 v = __ldcg(reinterpret_cast<const float2*>(p));
     return ds(v.x, v.y);
 }
-// P2M of node nd (a leaf) into mom[nd]: the moments about its centre,
-// u = c - y, one thread per multi-index k (two when T > 128).  The
-// double-layer part is split off:
-//   M_k = sum_s q_s u^k + sum_a k_a D_a[k - e_a],  D_a[k'] = sum_s p_{s,a} u^{k'},
-// so each (point, k) costs one monomial (two products of cached powers) and
-// five multiply-adds; the D_a (|k'| <= P - 1) meet the q sums in shared memory.
+
+// Powers of u = leaf centre - y at the far rule's points of panels j0 .. j0 + np - 1.
 template <typename real, int P>
-__device__ __forceinline__ void up_p2m(const UpArgs& a, int nd, const typename V4<real>::t* __restrict__ src,
-                                       real* __restrict__ mom, UpShared<real, P>& sh) {
-    using v4 = typename V4<real>::t;
-    constexpr int T = MI<P>::T;
-    constexpr int H = (T + 127) / 128;  // multi-indices per thread
-    const int tid = threadIdx.x;
-    const int64_t s0 = (int64_t)a.nstart[nd] * a.K, s1 = (int64_t)a.nend[nd] * a.K;
-    int kx[H], ky[H], kz[H];
-    bool on[H], low[H];
-    real qL[H], qY[H], dx[H], dy[H], dz[H];
-#pragma unroll
-    for (int h = 0; h < H; ++h) {
-        const int k = tid + 128 * h;
-        on[h] = k < T;
-        kx[h] = ky[h] = kz[h] = 0;
-        if (on[h]) {
-            kx[h] = sh.kk[k][0];
-            ky[h] = sh.kk[k][1];
-            kz[h] = sh.kk[k][2];
+__device__ __forceinline__ void stage_powers(const UpArgs& a, int64_t j0, int np, real (*pw)[3][P + 1]) {
+    for (int q = threadIdx.x; q < np * a.K * 3; q += blockDim.x) {
+        const int pt = q / 3, ax = q - 3 * pt;
+        const int jj = pt / a.K;
+        const real* g = (const real*)a.pg + 16 * (j0 + jj);
+        int m = pt - jj * a.K;
+        real v = -g[ax];
+        if (a.K != 3) --m;  // the centroid is point 0
+        if (m >= 0) {
+            const int o = m / 3, k = m - 3 * o;
+            const real s0 = g[4 + ax], s1 = g[8 + ax];  // 2 (v_k - c); the third is minus their sum
+            const real s = k == 0 ? s0 : (k == 1 ? s1 : -(s0 + s1));
+            v = madd(from_dbl<real>(0.5 * a.rule.a[o]), s, v);  // y = c - 3 alpha s_k
         }
-        low[h] = on[h] && kx[h] + ky[h] + kz[h] < P;
-        qL[h] = qY[h] = dx[h] = dy[h] = dz[h] = real(0);
-    }
-    for (int64_t t = s0; t < s1; t += 128) {
-        const int cnt = (int)min((int64_t)128, s1 - t);
-        __syncthreads();
-        if (tid < cnt) {
-            const v4 A = src[2 * (t + tid)], B = src[2 * (t + tid) + 1];
-            const real u[3] = {-A.x, -A.y, -A.z};
-            for (int q = 0; q < 3; ++q) {
-                real v = 1;
-                for (int m = 0; m <= P; ++m) {
-                    sh.u.p.pw[tid][q][m] = v;
-                    v = v * u[q];
-                }
-            }
-            sh.u.p.sq[tid][0] = A.w;
-            sh.u.p.sq[tid][1] = B.w;
-            sh.u.p.sq[tid][2] = B.x;
-            sh.u.p.sq[tid][3] = B.y;
-            sh.u.p.sq[tid][4] = B.z;
-        }
-        __syncthreads();
+        real x = real(1);
 #pragma unroll
-        for (int h = 0; h < H; ++h) {
-            if (!on[h]) continue;
-            for (int j = 0; j < cnt; ++j) {
-                const real mono = sh.u.p.pw[j][0][kx[h]] * sh.u.p.pw[j][1][ky[h]] * sh.u.p.pw[j][2][kz[h]];
-                qL[h] += sh.u.p.sq[j][0] * mono;
-                qY[h] += sh.u.p.sq[j][1] * mono;
-                if (low[h]) {
-                    dx[h] += sh.u.p.sq[j][2] * mono;
-                    dy[h] += sh.u.p.sq[j][3] * mono;
-                    dz[h] += sh.u.p.sq[j][4] * mono;
-                }
-            }
+        for (int d = 0; d <= P; ++d) {
+            pw[pt][ax][d] = x;
+            x = x * v;
         }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int h = 0; h < H; ++h)
-        if (low[h]) {
-            const int k = tid + 128 * h;
-            sh.u.p.sd[0][k] = dx[h];
-            sh.u.p.sd[1][k] = dy[h];
-            sh.u.p.sd[2][k] = dz[h];
-        }
-    __syncthreads();
-#pragma unroll
-    for (int h = 0; h < H; ++h) {
-        if (!on[h]) continue;
-        const int k = tid + 128 * h;
-        real dl = 0;
-        if (kx[h]) dl += real(kx[h]) * sh.u.p.sd[0][sh.idx3[kx[h] - 1][ky[h]][kz[h]]];
-        if (ky[h]) dl += real(ky[h]) * sh.u.p.sd[1][sh.idx3[kx[h]][ky[h] - 1][kz[h]]];
-        if (kz[h]) dl += real(kz[h]) * sh.u.p.sd[2][sh.idx3[kx[h]][ky[h]][kz[h] - 1]];
-        mom[(int64_t)nd * 2 * T + k] = qL[h] + dl;
-        mom[(int64_t)nd * 2 * T + T + k] = qY[h] + dl;
     }
 }
-
-// Moment shift of node nd from its (at most eight) children,
-// M_k(c) = sum_{j<=k} C(k,j) (c - c_child)^{k-j} M_j(c_child): the shift is
-// separable, so it is applied as three one-axis passes x, y, z, each output
-// summing at most P+1 terms; CB children are shifted at once, and the results
-// summed in child order.  The children's moments are read from L2.
+// V_k of the staged panel whose points start at pw.
 template <typename real, int P>
-__device__ __forceinline__ void up_m2m(const UpArgs& a, int nd, real* __restrict__ mom, UpShared<real, P>& sh) {
-    constexpr int T = MI<P>::T;
-    constexpr int CB = UpShared<real, P>::CB;
-    constexpr int HO = (2 * T + 127) / 128;  // outputs per thread
-    const int tid = threadIdx.x;
-    const int nc = a.nchild[nd];
-    const int fc = a.child[nd];
-    real acc[HO];
-#pragma unroll
-    for (int h = 0; h < HO; ++h) acc[h] = real(0);
-    for (int c0 = 0; c0 < nc; c0 += CB) {
-        const int nb = min(CB, nc - c0);
-        __syncthreads();
-        for (int q = tid; q < nb * 2 * T; q += blockDim.x) {
-            const int ci = q / (2 * T), k = q - ci * 2 * T;
-            sh.u.m.bufA[ci][k] = ld_cg(mom + (int64_t)(fc + c0 + ci) * 2 * T + k);
-        }
-        if (tid < 3 * nb) {
-            const int ci = tid / 3, ax = tid - 3 * ci;
-            const real d = from_dbl<real>(a.ncenter[3 * nd + ax] - a.ncenter[3 * (fc + c0 + ci) + ax]);
-            real v = 1;
-            for (int m = 0; m <= P; ++m) {
-                sh.u.m.cd[ci][ax][m] = v;
-                v = v * d;
-            }
-        }
-        __syncthreads();
-#pragma unroll 1
-        for (int ax = 0; ax < 3; ++ax) {
-            real(*srcb)[2 * T] = (ax == 1) ? sh.u.m.bufB : sh.u.m.bufA;
-            real(*dstb)[2 * T] = (ax == 1) ? sh.u.m.bufA : sh.u.m.bufB;
-            for (int it = tid; it < nb * T; it += blockDim.x) {
-                const int ci = it / T, k = it - ci * T;
-                const int k0 = sh.kk[k][0], k1 = sh.kk[k][1], k2 = sh.kk[k][2];
-                const int ka = sh.kk[k][ax];
-                real sL = 0, sY = 0;
-                for (int j = 0; j <= ka; ++j) {
-                    const int jx = ax == 0 ? j : k0, jy = ax == 1 ? j : k1, jz = ax == 2 ? j : k2;
-                    const int jj = sh.idx3[jx][jy][jz];
-                    const real coef = sh.binom[ka][j] * sh.u.m.cd[ci][ax][ka - j];
-                    sL += coef * srcb[ci][jj];
-                    sY += coef * srcb[ci][T + jj];
-                }
-                dstb[ci][k] = sL;
-                dstb[ci][T + k] = sY;
-            }
-            __syncthreads();
-        }
-#pragma unroll
-        for (int h = 0; h < HO; ++h) {
-            const int k = tid + 128 * h;
-            if (k < 2 * T)
-                for (int ci = 0; ci < nb; ++ci) acc[h] += sh.u.m.bufB[ci][k];
-        }
+__device__ __forceinline__ real panel_moment(const UpArgs& a, const real (*pw)[3][P + 1], int kx, int ky, int kz) {
+    real s = real(0);
+    for (int m = 0; m < a.K; ++m) {
+        const int o = a.K == 3 ? 1 : (m + 2) / 3;  // weight: centroid, first, second orbit
+        s = madd(from_dbl<real>(a.rule.w[o]), (pw[m][0][kx] * pw[m][1][ky]) * pw[m][2][kz], s);
     }
-#pragma unroll
-    for (int h = 0; h < HO; ++h) {
-        const int k = tid + 128 * h;
-        if (k < 2 * T) mom[(int64_t)nd * 2 * T + k] = acc[h];
-    }
+    return s;
 }
 
+// The panel moments of all panels: out[j T + k].
 template <typename real, int P>
-__global__ void __launch_bounds__(128) k_upward(UpArgs a, const typename V4<real>::t* __restrict__ src,
-                                                real* __restrict__ mom) {
+__global__ void __launch_bounds__(UP_THREADS) k_panel_moments(UpArgs a, int64_t n_pan, real* __restrict__ out) {
     constexpr int T = MI<P>::T;
-    extern __shared__ __align__(16) unsigned char up_smem[];
-    UpShared<real, P>& sh = *reinterpret_cast<UpShared<real, P>*>(up_smem);
-    const int tid = threadIdx.x;
-    for (int k = tid; k < T; k += blockDim.x) {
+    __shared__ real pw[UP_FLY * 7][3][P + 1];
+    __shared__ signed char kk[T][3];
+    for (int k = threadIdx.x; k < T; k += blockDim.x) {
         int x, y, z;
         decode_mi(k, x, y, z);
-        sh.idx3[x][y][z] = (short)k;
+        kk[k][0] = (signed char)x;
+        kk[k][1] = (signed char)y;
+        kk[k][2] = (signed char)z;
+    }
+    for (int64_t j0 = (int64_t)blockIdx.x * UP_FLY; j0 < n_pan; j0 += (int64_t)gridDim.x * UP_FLY) {
+        const int np = (int)min((int64_t)UP_FLY, n_pan - j0);
+        __syncthreads();
+        stage_powers<real, P>(a, j0, np, pw);
+        __syncthreads();
+        for (int q = threadIdx.x; q < np * T; q += blockDim.x) {
+            const int jj = q / T, k = q - jj * T;
+            out[(j0 + jj) * T + k] = panel_moment<real, P>(a, pw + jj * a.K, kk[k][0], kk[k][1], kk[k][2]);
+        }
+    }
+}
+
+// P2M of a leaf into mom: a thread per multi-index, the panels in NP shares
+// where T leaves threads over.
+template <typename real, int P, bool STORED>
+__global__ void __launch_bounds__(p2m_threads(P)) k_p2m(UpArgs a, real* __restrict__ mom) {
+    using SH = P2MShared<real, P, STORED>;
+    constexpr int T = SH::T, NP = SH::NP, BT = SH::BT;
+    constexpr int H = (T + BT - 1) / BT;  // multi-indices per thread
+    extern __shared__ __align__(16) unsigned char p2m_smem[];
+    SH& sh = *reinterpret_cast<SH*>(p2m_smem);
+    const int tid = threadIdx.x;
+    const int part = NP > 1 ? tid / T : 0, k0 = NP > 1 ? tid - part * T : tid;
+    const bool on = part < NP;
+    for (int k = tid; k < T; k += BT) {
+        int x, y, z;
+        decode_mi(k, x, y, z);
         sh.kk[k][0] = (signed char)x;
         sh.kk[k][1] = (signed char)y;
         sh.kk[k][2] = (signed char)z;
     }
-    for (int q = tid; q < (P + 1) * (P + 1); q += blockDim.x) {
-        const int n = q / (P + 1), m = q - n * (P + 1);
-        sh.binom[n][m] = from_dbl<real>(kBinomTable.v[n][m]);
+    for (int64_t leaf = blockIdx.x; leaf < a.n_leaves; leaf += gridDim.x) {
+    const int nd = a.leaf_node[leaf];
+    if (!body_on(a, a.nbody[nd])) continue;  // block-uniform
+    const int64_t j0 = a.nstart[nd], j1 = a.nend[nd];
+    const real* __restrict__ pg = (const real*)a.pg;
+    const real* __restrict__ pd = (const real*)a.pd;
+    const real* __restrict__ pm = (const real*)a.pmom;
+    real acc[H][5];
+#pragma unroll
+    for (int h = 0; h < H; ++h)
+#pragma unroll
+        for (int c = 0; c < 5; ++c) acc[h][c] = real(0);
+    auto add = [&](int h, real v, const real (&q)[5]) {
+#pragma unroll
+        for (int c = 0; c < 5; ++c) acc[h][c] = madd(v, q[c], acc[h][c]);
+    };
+    for (int64_t c0 = j0; c0 < j1; c0 += UP_CHUNK) {
+        const int cnt = (int)min((int64_t)UP_CHUNK, j1 - c0);
+        __syncthreads();
+        if (tid < cnt) {
+            const real* d = pd + 4 * (c0 + tid);
+            const real* g = pg + 16 * (c0 + tid) + 12;
+            sh.q[tid][0] = d[0];
+            sh.q[tid][1] = d[1];
+            for (int c = 0; c < 3; ++c) sh.q[tid][2 + c] = d[2] * g[c];
+        }
+        __syncthreads();
+        if constexpr (STORED) {
+            if (on) {
+#pragma unroll
+                for (int h = 0; h < H; ++h) {
+                    const int k = k0 + h * BT;
+                    if (k >= T) break;
+                    const real* v = pm + c0 * T + k;
+#pragma unroll 8
+                    for (int j = part; j < cnt; j += NP) add(h, v[(int64_t)j * T], sh.q[j]);
+                }
+            }
+        } else {
+            for (int f = 0; f < cnt; f += UP_FLY) {
+                const int np = min(UP_FLY, cnt - f);
+                __syncthreads();
+                stage_powers<real, P>(a, c0 + f, np, sh.pw);
+                __syncthreads();
+                if (part == 0)
+#pragma unroll
+                    for (int h = 0; h < H; ++h) {
+                        const int k = k0 + h * BT;
+                        if (k >= T) break;
+                        for (int j = 0; j < np; ++j)
+                            add(h, panel_moment<real, P>(a, sh.pw + j * a.K, sh.kk[k][0], sh.kk[k][1], sh.kk[k][2]),
+                                sh.q[f + j]);
+                    }
+            }
+        }
     }
     __syncthreads();
-    for (int64_t leaf = blockIdx.x; leaf < a.n_leaves; leaf += gridDim.x) {
-        int nd = a.leaf_node[leaf];
-        if (!body_on(a, a.nbody[nd])) continue;  // block-uniform
-        up_p2m<real, P>(a, nd, src, mom, sh);
-        for (;;) {
-            // publish nd's moments, then count it at its parent
-            __syncthreads();
-            __threadfence();
-            if (tid == 0) {
-                const int par = a.parent[nd];
-                int go = -1;
-                if (par >= 0 && atomicAdd(a.arrive + par, 1) == a.nchild[par] - 1) go = par;
-                sh.next = go;
+    if (on)
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+            const int k = k0 + h * BT;
+            if (k < T)
+#pragma unroll
+                for (int c = 0; c < 5; ++c) sh.sum[part][c][k] = acc[h][c];
+        }
+    __syncthreads();
+    auto total = [&](int c, int k) {
+        real s = sh.sum[0][c][k];
+#pragma unroll
+        for (int p = 1; p < NP; ++p) s = s + sh.sum[p][c][k];
+        return s;
+    };
+    for (int k = tid; k < T; k += BT) {
+        const int x = sh.kk[k][0], y = sh.kk[k][1], z = sh.kk[k][2];
+        real dl = real(0);
+        if (x) dl = madd(real(x), total(2, mi_index(x - 1, y, z)), dl);
+        if (y) dl = madd(real(y), total(3, mi_index(x, y - 1, z)), dl);
+        if (z) dl = madd(real(z), total(4, mi_index(x, y, z - 1)), dl);
+        mom[(int64_t)nd * 2 * T + k] = total(0, k) + dl;
+        mom[(int64_t)nd * 2 * T + T + k] = total(1, k) + dl;
+    }
+    }
+}
+
+// Moment shift of node nd from its (at most eight) children,
+// M_k(c) = sum_{j<=k} C(k,j) (c - c_child)^{k-j} M_j(c_child), one warp per
+// child: the shift is separable, and along an axis each line of moments
+// s_0..s_n (the other two indices fixed) goes to a lane, which applies
+// s_k += d s_{k-1}, k = n..t, for t = 1..n in registers (Pascal's triangle: after
+// it s_k = sum_j C(k,j) d^{k-j} s_j) -- no index tables, no binomials and no
+// block barriers between the axes.  The children's sums follow in child order.
+template <typename real, int P>
+__device__ __forceinline__ void up_m2m(const UpArgs& a, int nd, int nc, int fc, real* __restrict__ mom,
+                                       ClimbShared<real, P>& sh) {
+    constexpr int T = MI<P>::T, NL = (P + 1) * (P + 2) / 2;  // lines per axis and kernel
+    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+    __syncthreads();
+    if (w < nc) {
+        real* b = sh.buf[w];
+        for (int k = lane; k < 2 * T; k += 32) b[k] = ld_cg(mom + (int64_t)(fc + w) * 2 * T + k);
+        if (lane < 3) sh.d[w][lane] = from_dbl<real>(a.ncenter[3 * nd + lane] - a.ncenter[3 * (fc + w) + lane]);
+        __syncwarp();
+#pragma unroll 1
+        for (int ax = 0; ax < 3; ++ax) {
+            const real d = sh.d[w][ax];
+#pragma unroll 1
+            for (int i = lane; i < ((2 * NL + 31) & ~31); i += 32) {
+                // both kernels' lines side by side, the longest first: the
+                // lanes of a round have lines of about one length, and the
+                // steps beyond the longest of them are left out
+                const int li = min(i >> 1, NL - 1);
+                real* q = b + (i & 1) * T;
+                const int e = sh.ln[li][0], f = sh.ln[li][1], n = i < 2 * NL ? P - e - f : -1;
+                const int nm = __reduce_max_sync(0xffffffffu, n);
+                real s[P + 1];
+                int at[P + 1];
+#pragma unroll
+                for (int k = 0; k <= P; ++k) {
+                    at[k] = ax == 0 ? mi_index(k, e, f) : (ax == 1 ? mi_index(e, k, f) : mi_index(e, f, k));
+                    s[k] = k <= n ? q[at[k]] : real(0);
+                }
+#pragma unroll
+                for (int t = 1; t <= P; ++t) {
+                    if (t <= nm) {
+#pragma unroll
+                        for (int k = P; k >= t; --k)
+                            if (k <= nm) s[k] = madd(d, s[k - 1], s[k]);
+                    }
+                }
+#pragma unroll
+                for (int k = 1; k <= P; ++k)
+                    if (k <= n) q[at[k]] = s[k];
             }
-            __syncthreads();
-            const int par = sh.next;
-            if (par < 0) break;
+            __syncwarp();
+        }
+    }
+    __syncthreads();
+    for (int k = tid; k < 2 * T; k += UP_THREADS) {
+        real s = sh.buf[0][k];
+        for (int c = 1; c < nc; ++c) s = s + sh.buf[c][k];
+        mom[(int64_t)nd * 2 * T + k] = s;
+    }
+}
+
+template <typename real, int P>
+__global__ void __launch_bounds__(UP_THREADS) k_climb(UpArgs a, real* __restrict__ mom) {
+    extern __shared__ __align__(16) unsigned char climb_smem[];
+    ClimbShared<real, P>& sh = *reinterpret_cast<ClimbShared<real, P>*>(climb_smem);
+    const int tid = threadIdx.x;
+    bool ready = false;  // the line table is made when a node is shifted
+    for (int64_t i = blockIdx.x; i < a.n_internal; i += gridDim.x) {
+        int nd = a.internal_node[i];
+        if (a.n_ichild[nd] > 0 || !body_on(a, a.nbody[nd])) continue;  // block-uniform
+        if (!ready) {
+            for (int q = tid; q < (P + 1) * (P + 2) / 2; q += UP_THREADS) {  // (e, f) by e + f = 0..P
+                int s = 0, r = q;
+                while (r > s) r -= ++s;
+                sh.ln[q][0] = (signed char)r;
+                sh.ln[q][1] = (signed char)(s - r);
+            }
+            ready = true;  // (a barrier follows in up_m2m)
+        }
+        int nc = a.nchild[nd], fc = a.child[nd];
+        for (;;) {
+            // the parent's entries are fetched while nd is shifted
+            const int par = a.parent[nd];
+            int pic = 0, pnc = 0, pfc = 0;
+            if (par >= 0) {
+                pic = a.n_ichild[par];
+                pnc = a.nchild[par];
+                pfc = a.child[par];
+            }
+            up_m2m<real, P>(a, nd, nc, fc, mom, sh);
+            // publish nd's moments, then count it at its parent
             __threadfence();
-            up_m2m<real, P>(a, par, mom, sh);
-            if (tid == 0) a.arrive[par] = 0;  // every child has arrived: ready for the next launch
+            __syncthreads();
+            if (tid == 0) sh.next = par >= 0 && atomicAdd(a.arrive + par, 1) == pic - 1;
+            __syncthreads();
+            if (!sh.next) break;
+            __threadfence();
+            if (tid == 0) a.arrive[par] = 0;  // every internal child has arrived: ready for the next launch
             nd = par;
+            nc = pnc;
+            fc = pfc;
         }
     }
 }
@@ -1320,9 +1393,10 @@ void launch_m2p(const EvalArgs& ev, const void* xrel, const void* far, cudaStrea
 }
 
 // The far-field coefficients: 8 nodes per block in FP32 and 4 in the 8-byte
-// types (shared memory), where that gives every SM two blocks; with fewer
+// types (shared memory), where that gives every SM eight blocks; with fewer
 // nodes, two and one per block, whose chain of loads is shorter (130 nodes:
-// 8 us less for the whole product).
+// 8 us less for the whole product).  Above order 8 a block reads megabytes of
+// table, and only many nodes per block pay for them.
 template <typename real, int P, int NB>
 void launch_far_nb(const UpArgs& up, const void* mom, cudaStream_t s) {
     constexpr size_t smem = sizeof(real) * NB * 2 * MI<P>::T;
@@ -1335,24 +1409,33 @@ void launch_far_nb(const UpArgs& up, const void* mom, cudaStream_t s) {
 template <typename real, int P>
 void launch_far(const UpArgs& up, const void* mom, cudaStream_t s) {
     constexpr int NB = sizeof(real) == sizeof(float) ? 8 : 4;
-    if (up.n_nodes >= 304 * NB) launch_far_nb<real, P, NB>(up, mom, s);
+    if (P > 8 || up.n_nodes >= 1216 * NB) launch_far_nb<real, P, NB>(up, mom, s);
     else launch_far_nb<real, P, NB / 4>(up, mom, s);
 }
 
-// The upward pass of one product: P2M and the moment shifts in one launch
-// (k_upward), then the far-field coefficients (k_far).
+// The panel moments of the current geometry (UpArgs::pg, rule, K) into out.
 template <typename real, int P>
-void launch_upward(const UpArgs& up, const void* src, void* mom, cudaStream_t s) {
-    using v4 = typename V4<real>::t;
+void launch_panel_moments(const UpArgs& up, int64_t n_pan, void* out, cudaStream_t s) {
+    const int64_t grid = std::min<int64_t>((n_pan + UP_FLY - 1) / UP_FLY, 152 * 8);
+    if (grid > 0) k_panel_moments<real, P><<<(unsigned)grid, UP_THREADS, 0, s>>>(up, n_pan, (real*)out);
+}
+
+// The upward pass of one product: P2M, the moment shifts, the far-field
+// coefficients.
+template <typename real, int P>
+void launch_upward(const UpArgs& up, void* mom, cudaStream_t s) {
     if (up.n_leaves <= 0) return;
-    constexpr size_t up_smem = sizeof(UpShared<real, P>);
-    static bool up_attr = false;  // per instantiation
-    if (!up_attr) {
-        PGB_CUDA(cudaFuncSetAttribute(k_upward<real, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)up_smem));
-        up_attr = true;
+    auto cap = [&](int64_t n) { return (unsigned)(up.p2m_grid > 0 ? std::min<int64_t>(n, up.p2m_grid) : n); };
+    constexpr size_t s1 = sizeof(P2MShared<real, P, true>), s0 = sizeof(P2MShared<real, P, false>);
+    constexpr size_t sc = sizeof(ClimbShared<real, P>);
+    if constexpr (s0 > 40 * 1024 || sc > 40 * 1024) {
+        PGB_CUDA(cudaFuncSetAttribute(k_p2m<real, P, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s1));
+        PGB_CUDA(cudaFuncSetAttribute(k_p2m<real, P, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s0));
+        PGB_CUDA(cudaFuncSetAttribute(k_climb<real, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sc));
     }
-    const int64_t grid = up.p2m_grid > 0 ? std::min<int64_t>(up.n_leaves, up.p2m_grid) : up.n_leaves;
-    k_upward<real, P><<<(unsigned)grid, 128, up_smem, s>>>(up, (const v4*)src, (real*)mom);
+    if (up.pmom) k_p2m<real, P, true><<<cap(up.n_leaves), p2m_threads(P), s1, s>>>(up, (real*)mom);
+    else k_p2m<real, P, false><<<cap(up.n_leaves), p2m_threads(P), s0, s>>>(up, (real*)mom);
+    if (up.n_internal > 0) k_climb<real, P><<<cap(up.n_internal), UP_THREADS, sc, s>>>(up, (real*)mom);
     if (up.n_nodes <= 0) return;
     launch_far<real, P>(up, mom, s);
 }

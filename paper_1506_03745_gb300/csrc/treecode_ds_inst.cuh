@@ -9,11 +9,12 @@
 namespace pgb {
 
 template <int P>
-inline void launch_ds(int stage, const UpArgs& up, const EvalArgs& ev, const void* src, const void* xrel, void* mom,
+inline void launch_ds(int stage, const UpArgs& up, const EvalArgs& ev, const void* xrel, void* mom,
                       const void* far, cudaStream_t s) {
     // P2M and the moment shifts, then the far-field coefficients, all in
     // double-single on the FP32 pipe
-    if (stage == PGB_STAGE_UPWARD) launch_upward<ds, P>(up, src, mom, s);
+    if (stage == PGB_STAGE_UPWARD) launch_upward<ds, P>(up, mom, s);
+    if (stage == STAGE_PANEL_MOMENTS) launch_panel_moments<ds, P>(up, ev.n_pan, mom, s);
     if (stage == PGB_STAGE_P2P) launch_p2p<ds>(ev, ev.K, xrel, s);
     if (stage == PGB_STAGE_M2P) launch_m2p<ds, P>(ev, xrel, far, s);
 }

@@ -7,10 +7,10 @@
 namespace pgb {
 
 template <typename real, int P>
-static void launch_p(int stage, const UpArgs& up, const std::vector<int64_t>& up_levels, const EvalArgs& ev,
-                     const void* src, const void* xrel, void* mom, void* far, cudaStream_t s) {
-    (void)up_levels;
-    if (stage == PGB_STAGE_UPWARD) launch_upward<real, P>(up, src, mom, s);
+static void launch_p(int stage, const UpArgs& up, const EvalArgs& ev, const void* xrel, void* mom, const void* far,
+                     cudaStream_t s) {
+    if (stage == PGB_STAGE_UPWARD) launch_upward<real, P>(up, mom, s);
+    if (stage == STAGE_PANEL_MOMENTS) launch_panel_moments<real, P>(up, ev.n_pan, mom, s);
     if (stage == PGB_STAGE_P2P) launch_p2p<real>(ev, ev.K, xrel, s);
     if (stage == PGB_STAGE_M2P) launch_m2p<real, P>(ev, xrel, far, s);
 }
