@@ -1003,6 +1003,7 @@ __device__ __constant__ const int kBinom[9][9] = {
 template <typename real, int P, int NB>
 __global__ void __launch_bounds__(2 * far_cols(P)) k_far(UpArgs a, const real* __restrict__ mom) {
     constexpr int T = MI<P>::T, TR = far_cols(P), NC = n_far_pad(P);
+    constexpr int U = 8;  // table entries in flight per thread
     extern __shared__ __align__(16) unsigned char far_smem[];
     real(*sm)[NB] = reinterpret_cast<real(*)[NB]>(far_smem);  // [2 T][NB]
     const bool yuk = threadIdx.x < TR;
@@ -1034,11 +1035,17 @@ __global__ void __launch_bounds__(2 * far_cols(P)) k_far(UpArgs a, const real* _
             const bool takes = l <= P && (yuk ? q >= l && !((q - l) & 1) : q == l);
             if (!__any_sync(0xffffffffu, takes)) continue;
             const int k0 = q * (q + 1) * (q + 2) / 6, k1 = k0 + (q + 1) * (q + 2) / 2;
-#pragma unroll 8
-            for (int k = k0; k < k1; ++k) {
-                const real v = tab[(size_t)k * TR];  // zero off the pattern
+#pragma unroll 1
+            for (int k = k0; k < k1; k += U) {  // whole batches of loads, the last one masked
+                real v[U];
 #pragma unroll
-                for (int i = 0; i < NB; ++i) acc[i] = madd(v, sk[k][i], acc[i]);
+                for (int u = 0; u < U; ++u) v[u] = k + u < k1 ? tab[(size_t)(k + u) * TR] : real(0);  // zero off the pattern
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int kk = min(k + u, k1 - 1);
+#pragma unroll
+                    for (int i = 0; i < NB; ++i) acc[i] = madd(v[u], sk[kk][i], acc[i]);
+                }
             }
         }
         if (j < n_far(P))
@@ -1069,7 +1076,10 @@ __global__ void __launch_bounds__(2 * far_cols(P)) k_far(UpArgs a, const real* _
 //   D_a[k'] = sum_j A_j phi_j n_j,a V_jk':
 // five multiply-adds per panel and k.  The V depend on the geometry alone; they
 // are formed once per geometry (k_panel_moments) and read back coalesced.
-#define UP_THREADS 256  // k_climb: a warp per child
+#define UP_THREADS 256
+// warps per child in k_climb: one up to order 8 (28 lines an axis at order 6),
+// above (136 lines at order 15) four, two in the 8-byte types for their registers
+__host__ __device__ constexpr int climb_wpc(int P, int bytes) { return P > 8 ? (bytes == 4 ? 4 : 2) : 1; }
 __host__ __device__ __forceinline__ int mi_index(int x, int y, int z) {  // position in MI's order
     const int n = x + y + z;
     return n * (n + 1) * (n + 2) / 6 + (n - x) * (n - x + 1) / 2 + z;
@@ -1213,14 +1223,14 @@ __global__ void __launch_bounds__(p2m_threads(P)) k_p2m(UpArgs a, real* __restri
         }
         __syncthreads();
         if constexpr (STORED) {
+            // all of a panel's moments at once: 8 to 16 loads in flight per thread
             if (on) {
+                const real* v = pm + c0 * T + k0;
+#pragma unroll(H >= 4 ? 4 : 8 / H)
+                for (int j = part; j < cnt; j += NP) {
 #pragma unroll
-                for (int h = 0; h < H; ++h) {
-                    const int k = k0 + h * BT;
-                    if (k >= T) break;
-                    const real* v = pm + c0 * T + k;
-#pragma unroll 8
-                    for (int j = part; j < cnt; j += NP) add(h, v[(int64_t)j * T], sh.q[j]);
+                    for (int h = 0; h < H; ++h)
+                        if (H == 1 || k0 + h * BT < T) add(h, v[(int64_t)j * T + h * BT], sh.q[j]);
                 }
             }
         } else {
@@ -1270,59 +1280,84 @@ __global__ void __launch_bounds__(p2m_threads(P)) k_p2m(UpArgs a, real* __restri
 }
 
 // Moment shift of node nd from its (at most eight) children,
-// M_k(c) = sum_{j<=k} C(k,j) (c - c_child)^{k-j} M_j(c_child), one warp per
-// child: the shift is separable, and along an axis each line of moments
+// M_k(c) = sum_{j<=k} C(k,j) (c - c_child)^{k-j} M_j(c_child), climb_wpc warps
+// per child: the shift is separable, and along an axis each line of moments
 // s_0..s_n (the other two indices fixed) goes to a lane, which applies
 // s_k += d s_{k-1}, k = n..t, for t = 1..n in registers (Pascal's triangle: after
-// it s_k = sum_j C(k,j) d^{k-j} s_j) -- no index tables, no binomials and no
+// it s_k = sum_j C(k,j) d^{k-j} s_j), the Laplace and the Yukawa moments side by
+// side (in FP32 as packed halves) -- no index tables, no binomials and no
 // block barriers between the axes.  The children's sums follow in child order.
+template <typename real>
+struct PairOf {
+    struct type {
+        real a, b;
+    };
+};
+template <>
+struct PairOf<float> {
+    using type = f2;
+};
+template <typename real>
+using Pair = typename PairOf<real>::type;
+__device__ __forceinline__ f2 pair_fma(f2 x, f2 y, f2 z) { return fma_(x, y, z); }
+template <typename V>
+__device__ __forceinline__ V pair_fma(const V& x, const V& y, const V& z) {
+    return V{madd(x.a, y.a, z.a), madd(x.b, y.b, z.b)};
+}
 template <typename real, int P>
 __device__ __forceinline__ void up_m2m(const UpArgs& a, int nd, int nc, int fc, real* __restrict__ mom,
                                        ClimbShared<real, P>& sh) {
     constexpr int T = MI<P>::T, NL = (P + 1) * (P + 2) / 2;  // lines per axis and kernel
-    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+    constexpr int CW = 32 * climb_wpc(P, sizeof(real));                     // threads per child
+    const int tid = threadIdx.x, w = tid / CW, lane = tid - w * CW;
+    // the threads of child w (a barrier of their own where they are several warps)
+    auto sync_child = [&]() {
+        if constexpr (CW == 32) __syncwarp();
+        else asm volatile("bar.sync %0, %1;" ::"r"(w + 1), "n"(CW) : "memory");
+    };
     __syncthreads();
     if (w < nc) {
         real* b = sh.buf[w];
-        for (int k = lane; k < 2 * T; k += 32) b[k] = ld_cg(mom + (int64_t)(fc + w) * 2 * T + k);
+        for (int k = lane; k < 2 * T; k += CW) b[k] = ld_cg(mom + (int64_t)(fc + w) * 2 * T + k);
         if (lane < 3) sh.d[w][lane] = from_dbl<real>(a.ncenter[3 * nd + lane] - a.ncenter[3 * (fc + w) + lane]);
-        __syncwarp();
+        sync_child();
 #pragma unroll 1
         for (int ax = 0; ax < 3; ++ax) {
-            const real d = sh.d[w][ax];
+            const Pair<real> dd{sh.d[w][ax], sh.d[w][ax]};
 #pragma unroll 1
-            for (int i = lane; i < ((2 * NL + 31) & ~31); i += 32) {
-                // both kernels' lines side by side, the longest first: the
-                // lanes of a round have lines of about one length, and the
-                // steps beyond the longest of them are left out
-                const int li = min(i >> 1, NL - 1);
-                real* q = b + (i & 1) * T;
-                const int e = sh.ln[li][0], f = sh.ln[li][1], n = i < 2 * NL ? P - e - f : -1;
+            for (int i = lane; i < (NL + CW - 1) / CW * CW; i += CW) {
+                // the longest lines first: the lanes of a round have lines of
+                // about one length, and the steps beyond the longest are left out
+                const int li = min(i, NL - 1);
+                const int e = sh.ln[li][0], f = sh.ln[li][1], n = i < NL ? P - e - f : -1;
                 const int nm = __reduce_max_sync(0xffffffffu, n);
-                real s[P + 1];
+                Pair<real> s[P + 1];
                 int at[P + 1];
 #pragma unroll
                 for (int k = 0; k <= P; ++k) {
                     at[k] = ax == 0 ? mi_index(k, e, f) : (ax == 1 ? mi_index(e, k, f) : mi_index(e, f, k));
-                    s[k] = k <= n ? q[at[k]] : real(0);
+                    s[k] = k <= n ? Pair<real>{b[at[k]], b[T + at[k]]} : Pair<real>{real(0), real(0)};
                 }
 #pragma unroll
                 for (int t = 1; t <= P; ++t) {
                     if (t <= nm) {
 #pragma unroll
                         for (int k = P; k >= t; --k)
-                            if (k <= nm) s[k] = madd(d, s[k - 1], s[k]);
+                            if (k <= nm) s[k] = pair_fma(dd, s[k - 1], s[k]);
                     }
                 }
 #pragma unroll
                 for (int k = 1; k <= P; ++k)
-                    if (k <= n) q[at[k]] = s[k];
+                    if (k <= n) {
+                        b[at[k]] = s[k].a;
+                        b[T + at[k]] = s[k].b;
+                    }
             }
-            __syncwarp();
+            sync_child();
         }
     }
     __syncthreads();
-    for (int k = tid; k < 2 * T; k += UP_THREADS) {
+    for (int k = tid; k < 2 * T; k += blockDim.x) {
         real s = sh.buf[0][k];
         for (int c = 1; c < nc; ++c) s = s + sh.buf[c][k];
         mom[(int64_t)nd * 2 * T + k] = s;
@@ -1330,7 +1365,7 @@ __device__ __forceinline__ void up_m2m(const UpArgs& a, int nd, int nc, int fc, 
 }
 
 template <typename real, int P>
-__global__ void __launch_bounds__(UP_THREADS) k_climb(UpArgs a, real* __restrict__ mom) {
+__global__ void __launch_bounds__(256 * climb_wpc(P, sizeof(real))) k_climb(UpArgs a, real* __restrict__ mom) {
     extern __shared__ __align__(16) unsigned char climb_smem[];
     ClimbShared<real, P>& sh = *reinterpret_cast<ClimbShared<real, P>*>(climb_smem);
     const int tid = threadIdx.x;
@@ -1339,7 +1374,7 @@ __global__ void __launch_bounds__(UP_THREADS) k_climb(UpArgs a, real* __restrict
         int nd = a.internal_node[i];
         if (a.n_ichild[nd] > 0 || !body_on(a, a.nbody[nd])) continue;  // block-uniform
         if (!ready) {
-            for (int q = tid; q < (P + 1) * (P + 2) / 2; q += UP_THREADS) {  // (e, f) by e + f = 0..P
+            for (int q = tid; q < (P + 1) * (P + 2) / 2; q += blockDim.x) {  // (e, f) by e + f = 0..P
                 int s = 0, r = q;
                 while (r > s) r -= ++s;
                 sh.ln[q][0] = (signed char)r;
@@ -1395,8 +1430,8 @@ void launch_m2p(const EvalArgs& ev, const void* xrel, const void* far, cudaStrea
 // The far-field coefficients: 8 nodes per block in FP32 and 4 in the 8-byte
 // types (shared memory), where that gives every SM eight blocks; with fewer
 // nodes, two and one per block, whose chain of loads is shorter (130 nodes:
-// 8 us less for the whole product).  Above order 8 a block reads megabytes of
-// table, and only many nodes per block pay for them.
+// 8 us less for the whole product).  Above order 8 a block reads half a
+// megabyte of table: half as many (658 nodes at order 15 make 165 blocks).
 template <typename real, int P, int NB>
 void launch_far_nb(const UpArgs& up, const void* mom, cudaStream_t s) {
     constexpr size_t smem = sizeof(real) * NB * 2 * MI<P>::T;
@@ -1409,7 +1444,8 @@ void launch_far_nb(const UpArgs& up, const void* mom, cudaStream_t s) {
 template <typename real, int P>
 void launch_far(const UpArgs& up, const void* mom, cudaStream_t s) {
     constexpr int NB = sizeof(real) == sizeof(float) ? 8 : 4;
-    if (P > 8 || up.n_nodes >= 1216 * NB) launch_far_nb<real, P, NB>(up, mom, s);
+    if (P > 8) launch_far_nb<real, P, NB / 2>(up, mom, s);
+    else if (up.n_nodes >= 1216 * NB) launch_far_nb<real, P, NB>(up, mom, s);
     else launch_far_nb<real, P, NB / 4>(up, mom, s);
 }
 
@@ -1435,7 +1471,7 @@ void launch_upward(const UpArgs& up, void* mom, cudaStream_t s) {
     }
     if (up.pmom) k_p2m<real, P, true><<<cap(up.n_leaves), p2m_threads(P), s1, s>>>(up, (real*)mom);
     else k_p2m<real, P, false><<<cap(up.n_leaves), p2m_threads(P), s0, s>>>(up, (real*)mom);
-    if (up.n_internal > 0) k_climb<real, P><<<cap(up.n_internal), UP_THREADS, sc, s>>>(up, (real*)mom);
+    if (up.n_internal > 0) k_climb<real, P><<<cap(up.n_internal), 256 * climb_wpc(P, sizeof(real)), sc, s>>>(up, (real*)mom);
     if (up.n_nodes <= 0) return;
     launch_far<real, P>(up, mom, s);
 }
