@@ -74,8 +74,6 @@ void collect_timing(pgb_ctx* c) {
     }
     c->ev_pending.clear();
 }
-void convert_f32_f64(const float* a, double* b, int64_t n, cudaStream_t s);
-void convert_f64_f32(const double* a, float* b, int64_t n, cudaStream_t s);
 }  // namespace pgb
 
 using namespace pgb;
@@ -666,11 +664,7 @@ int pgb_matvec(pgb_ctx* c, const void* x, void* y, int32_t precision) {
         if (precision != PGB_FP32) {
             apply_operator(c, (const double*)x, (double*)y, precision, false);
         } else {
-            c->d_xtmp.resize(c->n_unk);
-            c->d_ytmp.resize(c->n_unk);
-            convert_f32_f64((const float*)x, c->d_xtmp, c->n_unk, c->stream);
-            apply_operator(c, c->d_xtmp, c->d_ytmp, PGB_FP32, false);
-            convert_f64_f32(c->d_ytmp, (float*)y, c->n_unk, c->stream);
+            apply_f32(c, (const float*)x, (float*)y);
         }
         PGB_CUDA(cudaGetLastError());
         return PGB_OK;

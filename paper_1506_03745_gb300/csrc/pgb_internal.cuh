@@ -476,6 +476,7 @@ void apply_transpose(pgb_ctx* c, const double* lam, double* y, int precision);
 // selects the surfaces of mode 1 (nullptr: all)
 void apply_mode(pgb_ctx* c, const double* x, double* y, int precision, int mode, const int* known_mask);
 void apply_full(pgb_ctx* c, const double* x, double* y, int precision);
+void apply_f32(pgb_ctx* c, const float* x, float* y);  // y = A x in FP32, FP32 vectors
 void coulomb_rows(pgb_ctx* c, double* b);
 void grad(pgb_ctx* c, const double* x, int precision, double tol, int max_iter, int restart, double* dq, double* dbc,
           double* dt, pgb_solve_stats* st);
