@@ -12,6 +12,9 @@ void treecode_launch_f64(int stage, int P, const UpArgs& up, const EvalArgs& ev,
                          const void* far, cudaStream_t s);
 void treecode_launch_ds(int stage, int P, const UpArgs& up, const EvalArgs& ev, const void* xrel, void* mom,
                         const void* far, cudaStream_t s);
+void near_build_f32(const EvalArgs& ev, int K, const void* ng, const void* xrel, void* mat, cudaStream_t s);
+void near_build_f64(const EvalArgs& ev, int K, const void* ng, const void* xrel, void* mat, cudaStream_t s);
+int64_t near_groups(pgb_ctx* c, void* out);
 void convert_pd_ds(const void* pd64, void* pd_ds, int64_t n, cudaStream_t s);
 
 static inline int nblk(int64_t n, int t) { return (int)std::max<int64_t>(1, (n + t - 1) / t); }
@@ -367,6 +370,46 @@ static const void* panel_moments(pgb_ctx* c, int kind) {
     return pm.buf.p;
 }
 
+// The stored near field of the current lists for a product of a running solve
+// (NearScope): formed by the solve's first product on the context's stream, at
+// the cost of about one and a half P2Ps, and kept until the lists, the geometry
+// or the screening change.  Not kept (the P2P then forms the sums, as products
+// outside solves do) where it would take more than an eighth of the device's
+// memory or a quarter of what is free, or cannot be allocated.
+static void near_field(pgb_ctx* c, int kind, EvalArgs& ev) {
+    auto& nm = c->near_mat[kind];
+    if (nm.list_gen != c->list_gen || nm.kappa != c->kappa) {
+        if (c->capturing) return;  // (every product is prepared outside the capture)
+        nm.have = false;
+        nm.list_gen = c->list_gen;
+        nm.kappa = c->kappa;
+        if (c->n_groups == 0 || c->n_pitems == 0) return;
+        try {
+            nm.group.resize(16 * c->n_groups);
+            const int64_t units = near_groups(c, nm.group.p);
+            const size_t bytes = (size_t)units * 64 * (kind == 0 ? 4 : 8);
+            if (bytes > nm.buf.n) {
+                nm.buf.release();
+                size_t free_b = 0, total_b = 0;
+                PGB_CUDA(cudaMemGetInfo(&free_b, &total_b));
+                if (bytes > total_b / 8 || bytes > free_b / 4) return;
+                nm.buf.resize(bytes);
+            }
+        } catch (const Error& e) {
+            if (e.code != PGB_ENOMEM) throw;
+            return;
+        }
+        if (kind == 0) near_build_f32(ev, c->p.K, nm.group.p, c->d_x32, nm.buf.p, c->stream);
+        else near_build_f64(ev, c->p.K, nm.group.p, c->d_x64, nm.buf.p, c->stream);
+        PGB_CUDA(cudaGetLastError());
+        PGB_LAUNCHED(c, 1);
+        nm.have = true;
+    }
+    if (!nm.have) return;
+    ev.near_mat = nm.buf.p;
+    ev.near_group = nm.group.p;
+}
+
 // Upward pass as a CUDA graph: captured (on a private stream; nothing runs
 // there) the first time a tree / buffer / source-activity combination is
 // used, then one cudaGraphLaunch on the context stream per product.
@@ -607,6 +650,7 @@ static void apply_vec(pgb_ctx* c, VecIn xv, VecOut yv, int precision, int mode, 
     up.pg = ev.pg;
     up.pd = ev.pd;
     up.pmom = panel_moments(c, kind);
+    if (c->near_on && kind < 2 && !ev.p2p_work && c->shard_g[0] < 0 && !nested(c)) near_field(c, kind, ev);
     auto tab_for = [&](double kappa) -> const void* {
         const FarTab& t = far_table(c, kappa);
         if (f32) return t.t32.p;

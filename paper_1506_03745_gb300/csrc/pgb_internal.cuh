@@ -299,6 +299,16 @@ struct pgb_ctx {
     pgb::DBuf<double> d_momT64, d_Tout, d_sT, d_lam, d_gx, d_bu;
 
     // matvec work buffers
+    // near field kept for the products of a solve (treecode.cuh, stored near
+    // field): FP32 and FP64
+    struct NearMat {
+        pgb::DBuf<unsigned char> buf, group;
+        uint64_t list_gen = ~0ull;       // the lists they were formed for
+        double kappa = 0;
+        bool have = false;
+    } near_mat[2];
+    uint64_t list_gen = 0;               // bumped whenever the lists or the geometry change
+    bool near_on = false;                // a solve is running: its FP32 / FP64 products may keep it
     // panel moments of the P2M (k_panel_moments) per arithmetic: FP32, FP64, double-single
     struct PanMom {
         pgb::DBuf<unsigned char> buf;
@@ -441,6 +451,13 @@ inline bool nested(const pgb_ctx* c) {
         if (b.parent >= 0 || b.kappa_in != 0.0) return true;
     return false;
 }
+// For the duration of a solve: products keep the near field.
+struct NearScope {
+    pgb_ctx* c;
+    bool prev;
+    explicit NearScope(pgb_ctx* ctx) : c(ctx), prev(ctx->near_on) { c->near_on = true; }
+    ~NearScope() { c->near_on = prev; }
+};
 // CUDA-event interval on the context stream around one stage (no-op when
 // timing is off).
 struct StageTimer {

@@ -890,6 +890,7 @@ __global__ void k_panel_geo(const int32_t* pan_leaf, const int32_t* leaf_node, c
 
 void build_geometry(pgb_ctx* c) {
     ++c->geom_gen;
+    ++c->list_gen;
     cudaStream_t s = c->stream;
     int64_t n = c->n_pan;
     int K = c->p.K;
@@ -1136,6 +1137,58 @@ __global__ void k_list_offsets(int64_t ng, const int64_t* off, const int32_t* id
     }
 }
 
+// Units of the stored near field per group (NearGroup, treecode.cuh): the
+// columns of a dielectric group's own body count twice.
+__global__ void k_near_count(int64_t ng, const int64_t* coff, const float4* col, const int32_t* pbody,
+                             const int32_t* gbody, BodyDev bd, int64_t* units, int32_t* l01) {
+    const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (g >= ng) return;
+    const int64_t c0 = coff[g], n = coff[g + 1] - c0;
+    int32_t l0 = 0, l1 = 0;
+    if (bd.kind[gbody[g]] == PGB_DIELECTRIC) {  // columns ascend by body
+        const int b = gbody[g];
+        auto lower = [&](int body) {
+            int64_t lo = 0, hi = n;
+            while (lo < hi) {
+                const int64_t m = (lo + hi) >> 1;
+                if (pbody[__float_as_int(col[c0 + m].w)] < body) lo = m + 1;
+                else hi = m;
+            }
+            return (int32_t)lo;
+        };
+        l0 = lower(b);
+        l1 = lower(b + 1);
+    }
+    units[g] = n + (l1 - l0);
+    l01[2 * g] = l0;
+    l01[2 * g + 1] = l1;
+}
+__global__ void k_near_groups(int64_t ng, const int64_t* off, const int32_t* l01, int64_t* out) {
+    const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (g >= ng) return;
+    out[2 * g] = off[g];
+    reinterpret_cast<int32_t*>(out + 2 * g + 1)[0] = l01[2 * g];
+    reinterpret_cast<int32_t*>(out + 2 * g + 1)[1] = l01[2 * g + 1];
+}
+// The groups' units into out (NearGroup entries, 16 bytes each); the total.
+int64_t near_groups(pgb_ctx* c, void* out) {
+    cudaStream_t s = c->stream;
+    const int64_t ng = c->n_groups;
+    DBuf<int64_t> units, off;
+    DBuf<int32_t> l01;
+    units.resize(ng);
+    off.resize(ng);
+    l01.resize(2 * ng);
+    k_near_count<<<nblk(ng, 128), 128, 0, s>>>(ng, c->d_col_off, c->d_col, c->d_pbody, c->d_group_body, body_dev(c),
+                                               units, l01);
+    int64_t total = 0;
+    exclusive_scan_i64(units, off, ng, s, &total);
+    k_near_groups<<<nblk(ng, 128), 128, 0, s>>>(ng, off, l01, (int64_t*)out);
+    PGB_CUDA(cudaGetLastError());
+    PGB_LAUNCHED(c, 3);
+    return total;
+}
+
 // P2P columns: the panels of a group's near leaves one after another, in list
 // order; descriptor = (panel centroid - group centre, formed in FP64 and
 // rounded once to FP32, panel).  One warp per group; the lanes take its near
@@ -1250,6 +1303,7 @@ void make_lists(pgb_ctx* c, const double* r2, const double* glo, const double* g
 }
 
 void build_lists(pgb_ctx* c) {
+    ++c->list_gen;
     cudaStream_t s = c->stream;
     int64_t ng = c->n_groups;
     unsigned long long h[4];
@@ -1305,6 +1359,7 @@ void build_lists(pgb_ctx* c) {
 // Offsets of the kept list entries and P2P columns after the node and group
 // centres moved (pgb_tree_refresh): entries, columns and work items stay.
 void refresh_lists(pgb_ctx* c) {
+    ++c->list_gen;
     cudaStream_t s = c->stream;
     const int64_t ng = c->n_groups;
     if (ng == 0) return;

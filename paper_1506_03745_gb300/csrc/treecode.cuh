@@ -308,6 +308,7 @@ struct EvalArgs {
     const int32_t* pbody;          // body of a panel
     const void* pg;                // panel geometry (PanelGeo) in the kernel's arithmetic
     const void* pd;                // panel densities x area, same arithmetic: {psiL, psiY, phi, unused}
+    const void *near_mat = nullptr, *near_group = nullptr;  // stored near field (solves), nullptr: formed
     FarRule rule;
     unsigned long long src_mask;   // bit b: src_active[b]
     // work items (a group's columns in even runs, its far entries in runs of m2p_item)
@@ -523,6 +524,14 @@ __device__ __forceinline__ void far_eval_ds(ds Rx, ds Ry, ds Rz, ds kappa, const
     uL = LAP ? ri * ds_norm(sL) : ds(0);
 }
 
+// e^{-kappa r} of the P2P sums as exp2_scaled(exp_scale(kappa), r).
+__device__ __forceinline__ float exp_scale(float kappa) { return -kappa * 1.4426950408889634f; }
+__device__ __forceinline__ double exp_scale(double kappa) { return -kappa * 1.4426950408889634; }
+__device__ __forceinline__ ds exp_scale(ds kappa) { return -kappa * lit<ds>(1.4426950408889634); }
+template <typename real>
+__device__ __forceinline__ real exp2_scaled(real s, real r) {
+    return exp2_(mul_(s, r));
+}
 // 1/sqrt of a squared distance formed with a cancellation: a value rounded
 // below zero is taken by its magnitude (FP32; the others keep 50 bits more
 // than the distances that occur)
@@ -557,19 +566,21 @@ struct __align__(16) PanelS {
 // instead of 14; in double-single 185 operations (320).  The squared distance
 // loses a factor |d|^2 / r^2 of relative accuracy, below ten on shape-regular
 // panels, of the order of what the FP32 coordinates leave.
-template <typename real, int K, bool LAP, bool OWN>
-__device__ __forceinline__ void p2p_panel(const PanelS<real>& q, bool own, real X, real Y, real Z, real kappa,
-                                          real nkl, const real (&ra)[2], const real (&rw)[3], real& UL, real& UY) {
+// panel_sums: V_L, sum w / r^3, V_Y and its counterpart (without n.d), and n.d.
+template <typename real, int K, bool LAP>
+__device__ __forceinline__ void panel_sums(const PanelS<real>& q, real X, real Y, real Z, real kappa, real nkl,
+                                           const real (&ra)[2], const real (&rw)[3], real& VL, real& KL, real& VY,
+                                           real& KY, real& h) {
     const real dx = X - q.cx, dy = Y - q.cy, dz = Z - q.cz;
     const real D2 = norm_(fma_(dz, dz, fma_(dy, dy, mul_(dx, dx))));
-    const real h = fma_(q.nz, dz, fma_(q.ny, dy, mul_(q.nx, dx)));
+    h = fma_(q.nz, dz, fma_(q.ny, dy, mul_(q.nx, dx)));
     const real one = real(1);
-    real VL = real(0), KL = real(0), VY = real(0), KY = real(0);
+    VL = KL = VY = KY = real(0);
     auto point = [&](const real r2, real& sV, real& sK, real& sW, real& sM, bool first) {
         const real ri = rsqrt_abs(r2);
         const real i2 = mul_(ri, ri);
         const real r = mul_(r2, ri);
-        const real e = mul_(exp2_(mul_(nkl, r)), ri);
+        const real e = mul_(exp2_scaled(nkl, r), ri);
         const real gg = fma_(kappa, r, one);
         const real e2 = mul_(e, i2);
         if (first) {
@@ -616,6 +627,12 @@ __device__ __forceinline__ void p2p_panel(const PanelS<real>& q, bool own, real 
             KY = fma_(rw[1 + o], sM, KY);
         }
     }
+}
+template <typename real, int K, bool LAP, bool OWN>
+__device__ __forceinline__ void p2p_panel(const PanelS<real>& q, bool own, real X, real Y, real Z, real kappa,
+                                          real nkl, const real (&ra)[2], const real (&rw)[3], real& UL, real& UY) {
+    real VL, KL, VY, KY, h;
+    panel_sums<real, K, LAP>(q, X, Y, Z, kappa, nkl, ra, rw, VL, KL, VY, KY, h);
     if (OWN && own) VL = KL = VY = KY = real(0);  // the panel's own integral is a near-field correction
     if (LAP) UL = fma_(q.qL, VL, fma_(mul_(-q.pL, h), KL, UL));
     UY = fma_(q.qY, VY, fma_(mul_(-q.pY, h), KY, UY));
@@ -662,6 +679,26 @@ __device__ __forceinline__ void col_centroid(const EvalArgs& a, const float4& c,
     }
 }
 
+// The geometry of panel j (column c of group g) into q.
+template <typename real>
+__device__ __forceinline__ void stage_panel(const EvalArgs& a, const float4& c, int j, int64_t g, PanelS<real>& q) {
+    // the first 15 values of a staged panel, relative to the leaf
+    const PanelS<real>& v = *reinterpret_cast<const PanelS<real>*>((const real*)a.pg + 16 * (int64_t)j);
+    col_centroid<real>(a, c, j, g, &v.cx, q.cx, q.cy, q.cz);
+    q.g0 = v.g0;
+    q.ux = v.ux;
+    q.uy = v.uy;
+    q.uz = v.uz;
+    q.g1 = v.g1;
+    q.vx = v.vx;
+    q.vy = v.vy;
+    q.vz = v.vz;
+    q.g2 = v.g2;
+    q.nx = v.nx;
+    q.ny = v.ny;
+    q.nz = v.nz;
+}
+
 // Panels summed plainly before they join the compensated sums: about the 32
 // points of rounding growth that the FP32 product's accuracy rests on.  (All
 // 32 panels of a stage in one plain sum: 10-20 % more error against FP64.)
@@ -683,10 +720,9 @@ __global__ void __launch_bounds__(NW * 32) k_p2p(EvalArgs a, const typename V4<t
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned long long dm = body_mask(a.bmask), act = a.src_mask & dm;
     const real kappa = to_c<real>((S)a.kappa);
-    const real nkl = -kappa * lit<real>(1.4426950408889634);  // -kappa log2(e)
+    const real nkl = exp_scale(kappa);
     const real ra[2] = {from_dbl<real>(a.rule.a[0]), from_dbl<real>(a.rule.a[1])};
     const real rw[3] = {from_dbl<real>(a.rule.w[0]), from_dbl<real>(a.rule.w[1]), from_dbl<real>(a.rule.w[2])};
-    const real* __restrict__ pg = (const real*)a.pg;
     const real* __restrict__ pd = (const real*)a.pd;
     for (int64_t it = next_item(a.p2p_work, -1, &s_item); it < a.n_pitems; it = next_item(a.p2p_work, it, &s_item)) {
         const int64_t g = a.pitem_group[it];
@@ -717,21 +753,7 @@ __global__ void __launch_bounds__(NW * 32) k_p2p(EvalArgs a, const typename V4<t
                 lap = glap && b == gb;
                 has_own = j >= p0 && j < p1;
                 PanelS<real>& q = sP[w][lane];
-                // the first 15 values of a staged panel, relative to the leaf
-                const PanelS<real>& v = *reinterpret_cast<const PanelS<real>*>(pg + 16 * (int64_t)j);
-                col_centroid<real>(a, c, j, g, &v.cx, q.cx, q.cy, q.cz);
-                q.g0 = v.g0;
-                q.ux = v.ux;
-                q.uy = v.uy;
-                q.uz = v.uz;
-                q.g1 = v.g1;
-                q.vx = v.vx;
-                q.vy = v.vy;
-                q.vz = v.vz;
-                q.g2 = v.g2;
-                q.nx = v.nx;
-                q.ny = v.ny;
-                q.nz = v.nz;
+                stage_panel<real>(a, c, j, g, q);
                 const bool on = (act >> b) & 1ull;  // a body without density in this product adds nothing
                 const real z = real(0);
                 q.qL = on && lap ? pd[4 * (int64_t)j] : z;
@@ -770,12 +792,214 @@ __global__ void __launch_bounds__(NW * 32) k_p2p(EvalArgs a, const typename V4<t
     }
 }
 
+// ---------------------------------------------------------------- stored near field
+// A GMRES solve applies the same near field tens of times, so it keeps the
+// panel sums of every (target, column) pair: V_Y and K_Y = n.d sum.., and on a
+// group's own dielectric body V_L and K_L before them (the own panel: zeros).
+// A product then streams them, 16 or 8 bytes a pair in FP32, instead of
+// forming seven points each.  Layout: per column units of 32 lanes x 2 values,
+// two units {V_L, K_L}, {V_Y, K_Y} where the Laplace pair is kept (lane by lane
+// four values in FP32), else one.  The Laplace columns of a group are one run.
+struct NearGroup {
+    int64_t unit;     // first unit of the group's columns
+    int32_t l0, l1;   // its Laplace columns, counted from its first column
+};
+__host__ __device__ __forceinline__ int64_t near_unit(const NearGroup& n, int64_t c) {
+    const int64_t in = c - n.l0;
+    return n.unit + c + (in < 0 ? 0 : (in < n.l1 - n.l0 ? in : n.l1 - n.l0));
+}
+template <typename real, bool LAP>
+__device__ __forceinline__ void near_store(real* u, int lane, real vl, real kl, real vy, real ky) {
+    if constexpr (!LAP) {
+        u[2 * lane] = vy;
+        u[2 * lane + 1] = ky;
+    } else if constexpr (sizeof(real) == 4) {
+        reinterpret_cast<float4*>(u)[lane] = make_float4(vl, kl, vy, ky);
+    } else {
+        reinterpret_cast<double2*>(u)[lane] = make_double2(vl, kl);
+        reinterpret_cast<double2*>(u)[32 + lane] = make_double2(vy, ky);
+    }
+}
+
+// Forms the matrix: one block per P2P item, as k_p2p.
+template <typename real, int K, int NW>
+__global__ void __launch_bounds__(NW * 32) k_near_build(EvalArgs a, const NearGroup* __restrict__ ng,
+                                                        const typename V4<real>::t* __restrict__ xrel,
+                                                        real* __restrict__ mat) {
+    __shared__ __align__(16) PanelS<real> sP[NW][32];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const real kappa = (real)a.kappa;
+    const real nkl = exp_scale(kappa);
+    const real ra[2] = {from_dbl<real>(a.rule.a[0]), from_dbl<real>(a.rule.a[1])};
+    const real rw[3] = {from_dbl<real>(a.rule.w[0]), from_dbl<real>(a.rule.w[1]), from_dbl<real>(a.rule.w[2])};
+    const int64_t it = blockIdx.x, g = a.pitem_group[it];
+    const int p0 = a.gstart[g], p1 = a.gend[g];
+    const int p = p0 + lane;
+    const typename V4<real>::t xr = xrel[p < p1 ? p : p0];
+    const NearGroup nm = ng[g];
+    const int64_t i0 = a.pitem_off[g], c0 = a.col_off[g], nc = a.col_off[g + 1] - c0;
+    const int64_t per = (nc + a.pitem_off[g + 1] - i0 - 1) / (a.pitem_off[g + 1] - i0);
+    const int64_t b0 = (it - i0) * per, b1 = min(nc, b0 + per);
+    const int64_t wper = b1 > b0 ? (b1 - b0 + NW - 1) / NW : 0;
+    const int64_t w1 = min(b1, b0 + (w + 1) * wper);
+    for (int64_t e = b0 + w * wper; e < w1; e += 32) {
+        const int cnt = (int)min((int64_t)32, w1 - e);
+        __syncwarp();
+        int j = -1;
+        if (lane < cnt) {
+            const float4 c = a.col[c0 + e + lane];
+            j = __float_as_int(c.w);
+            stage_panel<real>(a, c, j, g, sP[w][lane]);
+        }
+        __syncwarp();
+        for (int k = 0; k < cnt; ++k) {
+            const bool own = __shfl_sync(0xffffffffu, j, k) == p;
+            const int64_t c = e + k;
+            real* u = mat + 64 * near_unit(nm, c);
+            real VL, KL, VY, KY, h;
+            if (c >= nm.l0 && c < nm.l1) {
+                panel_sums<real, K, true>(sP[w][k], xr.x, xr.y, xr.z, kappa, nkl, ra, rw, VL, KL, VY, KY, h);
+                const real z = 0;
+                near_store<real, true>(u, lane, own ? z : VL, own ? z : h * KL, own ? z : VY, own ? z : h * KY);
+            } else {
+                panel_sums<real, K, false>(sP[w][k], xr.x, xr.y, xr.z, kappa, nkl, ra, rw, VL, KL, VY, KY, h);
+                const real z = 0;
+                near_store<real, false>(u, lane, z, z, own ? z : VY, own ? z : h * KY);
+            }
+        }
+    }
+}
+
+// The near-field sums of one product from the matrix, items and warps as in
+// k_p2p; a warp keeps the densities of 32 columns in shared memory and eight
+// columns' loads in flight.  Bound by HBM: 2 x 20480 panels hold 294 MB in FP32
+// and take 62 us beside the upward pass (P2P: 114 us alone); 2600 panels in FP64
+// 44 MB, 48 us a product instead of 1.3 ms on the FP64 pipe.
+template <typename real, int NW>
+__global__ void __launch_bounds__(NW * 32) k_near(EvalArgs a, const NearGroup* __restrict__ ng,
+                                                  const real* __restrict__ mat) {
+    using v4 = typename V4<real>::t;
+    constexpr int U = 8;
+    __shared__ v4 sD[NW][32];  // psi_L, psi_Y, phi
+    __shared__ real red[NW][4][32];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned long long dm = body_mask(a.bmask), act = a.src_mask & dm;
+    const v4* __restrict__ pd = (const v4*)a.pd;
+    const int64_t it = blockIdx.x, g = a.pitem_group[it];
+    if (!(((a.tgt_mask & dm) >> a.gbody[g]) & 1ull)) return;  // rows not used (block-uniform)
+    real UL = 0, cL = 0, UY = 0, cY = 0;
+    const NearGroup nm = ng[g];
+    const int64_t i0 = a.pitem_off[g], c0 = a.col_off[g], nc = a.col_off[g + 1] - c0;
+    const int64_t per = (nc + a.pitem_off[g + 1] - i0 - 1) / (a.pitem_off[g + 1] - i0);
+    const int64_t b0 = (it - i0) * per, b1 = min(nc, b0 + per);
+    const int64_t wper = b1 > b0 ? (b1 - b0 + NW - 1) / NW : 0;
+    const int64_t w1 = min(b1, b0 + (w + 1) * wper);
+    for (int64_t e = b0 + w * wper; e < w1; e += 32) {
+        const int cnt = (int)min((int64_t)32, w1 - e);
+        __syncwarp();
+        v4 d;
+        d.x = d.y = d.z = d.w = 0;
+        if (lane < cnt) {
+            const int j = __float_as_int(a.col[c0 + e + lane].w);
+            if ((act >> a.pbody[j]) & 1ull) d = pd[j];
+        }
+        sD[w][lane] = d;
+        __syncwarp();
+        // runs of one kind of column
+        for (int k = 0; k < cnt;) {
+            const int64_t c = e + k;
+            const bool lap = c >= nm.l0 && c < nm.l1;
+            const int64_t lim = c < nm.l0 ? nm.l0 : (lap ? nm.l1 : nc);
+            const int n = (int)min((int64_t)(cnt - k), lim - c);
+            const real* u = mat + 64 * near_unit(nm, c);
+            for (int q = 0; q < n; q += U) {
+                real sL = 0, sY = 0;
+                if (lap) {
+                    real v[U][4];
+#pragma unroll
+                    for (int r = 0; r < U; ++r) {
+                        const real* p = u + 128 * (int64_t)min(q + r, n - 1);
+                        if constexpr (sizeof(real) == 4) {
+                            const float4 x = __ldcs(reinterpret_cast<const float4*>(p) + lane);
+                            v[r][0] = x.x;
+                            v[r][1] = x.y;
+                            v[r][2] = x.z;
+                            v[r][3] = x.w;
+                        } else {
+                            const double2 x = __ldcs(reinterpret_cast<const double2*>(p) + lane);
+                            const double2 y = __ldcs(reinterpret_cast<const double2*>(p) + 32 + lane);
+                            v[r][0] = x.x;
+                            v[r][1] = x.y;
+                            v[r][2] = y.x;
+                            v[r][3] = y.y;
+                        }
+                    }
+#pragma unroll
+                    for (int r = 0; r < U; ++r)
+                        if (q + r < n) {
+                            const v4 s = sD[w][k + q + r];
+                            sL += v[r][0] * s.x - v[r][1] * s.z;
+                            sY += v[r][2] * s.y - v[r][3] * s.z;
+                        }
+                } else {
+                    real v[U][2];
+#pragma unroll
+                    for (int r = 0; r < U; ++r) {
+                        const real* p = u + 64 * (int64_t)min(q + r, n - 1) + 2 * lane;
+                        if constexpr (sizeof(real) == 4) {
+                            const float2 x = __ldcs(reinterpret_cast<const float2*>(p));
+                            v[r][0] = x.x;
+                            v[r][1] = x.y;
+                        } else {
+                            const double2 x = __ldcs(reinterpret_cast<const double2*>(p));
+                            v[r][0] = x.x;
+                            v[r][1] = x.y;
+                        }
+                    }
+#pragma unroll
+                    for (int r = 0; r < U; ++r)
+                        if (q + r < n) {
+                            const v4 s = sD[w][k + q + r];
+                            sY += v[r][0] * s.y - v[r][1] * s.z;
+                        }
+                }
+                if (lap) kadd(UL, cL, sL);
+                kadd(UY, cY, sY);
+            }
+            k += n;
+        }
+    }
+    store_item<real, NW>(red, w, lane, UL, cL, UY, cY, a.Up + 64 * it);
+}
+
+template <typename real>
+void launch_near_build(const EvalArgs& ev, int K, const void* ng, const void* xrel, void* mat, cudaStream_t s) {
+    constexpr int NW = 8;
+    using x4 = typename V4<real>::t;
+    if (ev.n_pitems <= 0) return;
+    const unsigned grid = (unsigned)ev.n_pitems;
+    const NearGroup* n = (const NearGroup*)ng;
+    switch (K) {
+        case 1: k_near_build<real, 1, NW><<<grid, NW * 32, 0, s>>>(ev, n, (const x4*)xrel, (real*)mat); break;
+        case 3: k_near_build<real, 3, NW><<<grid, NW * 32, 0, s>>>(ev, n, (const x4*)xrel, (real*)mat); break;
+        case 4: k_near_build<real, 4, NW><<<grid, NW * 32, 0, s>>>(ev, n, (const x4*)xrel, (real*)mat); break;
+        case 7: k_near_build<real, 7, NW><<<grid, NW * 32, 0, s>>>(ev, n, (const x4*)xrel, (real*)mat); break;
+        default: fail(PGB_EINVAL, "K must be 1, 3, 4 or 7");
+    }
+}
+
 // The P2P launch for the context's far rule.
 template <typename real>
 void launch_p2p(const EvalArgs& ev, int K, const void* xrel, cudaStream_t s) {
     constexpr int NW = 8;  // warps per block
     using x4 = typename V4<typename Store<real>::S>::t;
     if (ev.n_pitems <= 0) return;
+    if constexpr (!is_ds<real>)
+        if (ev.near_mat) {
+            k_near<real, NW><<<(unsigned)ev.n_pitems, NW * 32, 0, s>>>(ev, (const NearGroup*)ev.near_group,
+                                                                       (const real*)ev.near_mat);
+            return;
+        }
     const unsigned grid = (unsigned)(ev.p2p_work ? ev.persist_blocks : ev.n_pitems);
     switch (K) {
         case 1: k_p2p<real, 1, NW><<<grid, NW * 32, 0, s>>>(ev, (const x4*)xrel); break;

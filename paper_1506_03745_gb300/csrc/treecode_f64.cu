@@ -20,4 +20,8 @@ void treecode_launch_f64(int stage, int P, const UpArgs& up, const EvalArgs& ev,
         default: fail(PGB_EINVAL, "P out of range");
     }
 }
+
+void near_build_f64(const EvalArgs& ev, int K, const void* ng, const void* xrel, void* mat, cudaStream_t s) {
+    launch_near_build<double>(ev, K, ng, xrel, mat, s);
+}
 }  // namespace pgb
