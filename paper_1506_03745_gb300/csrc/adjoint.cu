@@ -7,9 +7,11 @@
 #include <algorithm>
 #include <vector>
 
-#include "adjoint.cuh"
+#include "adjoint_h.cuh"
 
 namespace pgb {
+
+void imposed_rows_f32(pgb_ctx* c, int body, double* y);  // imposed_f32.cu
 
 static inline int nblk(int64_t n, int t) { return (int)std::max<int64_t>(1, (n + t - 1) / t); }
 
@@ -164,16 +166,32 @@ static void build_adjoint(pgb_ctx* c) {
 }
 
 // ---------------------------------------------------------------- A^T lam
-// Per panel j: the K nodes' potentials and normal derivatives weighted by w_s
-// (the transposed V and K products), the transposed near-field corrections,
-// then the columns of A^T lam in the caller's layout.
-__global__ void k_assemble_T(Geo g, BodyDev bd, const double* __restrict__ out4, const double* __restrict__ sT,
+// Per panel j: the far field's columns (pan) and the near field's, from the
+// stored matrix (nearp) or as the K nodes' potentials and normal derivatives
+// weighted by w_s (out4; in FP32 the far field with them, pan == nullptr), the
+// transposed near-field corrections, then the columns of A^T lam in the
+// caller's layout.
+__global__ void k_assemble_T(Geo g, BodyDev bd, const double* __restrict__ out4, const double* __restrict__ pan,
+                             const double* __restrict__ nearp, const double* __restrict__ sT,
                              const int64_t* __restrict__ toff, const int32_t* __restrict__ ti,
                              const dbl4* __restrict__ tval, const double* __restrict__ lam, double* __restrict__ y) {
     const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (j >= g.n_pan) return;
+    const double as = g.A[j];
     double vl = 0, kl = 0, vy = 0, ky = 0;
-    for (int m = 0; m < g.K; ++m) {
+    if (pan) {
+        vl = as * pan[4 * j];
+        kl = as * pan[4 * j + 1];
+        vy = as * pan[4 * j + 2];
+        ky = as * pan[4 * j + 3];
+    }
+    if (nearp) {
+        vl += as * nearp[4 * j];
+        kl += as * nearp[4 * j + 1];
+        vy += as * nearp[4 * j + 2];
+        ky += as * nearp[4 * j + 3];
+    }
+    for (int m = 0; !nearp && m < g.K; ++m) {
         const int64_t q = j * g.K + m;
         const double w = g.w[q];
         vl += w * out4[4 * q];
@@ -207,48 +225,77 @@ __global__ void k_assemble_T(Geo g, BodyDev bd, const double* __restrict__ out4,
     }
 }
 
-template <typename real, int P>
-static void launch_T(pgb_ctx* c, const TArgs& ta0, const void* xrel, const void* yrel, const void* nrm, void* L) {
-    using v4 = typename V4<real>::t;
+// FP32: the kernels of adjoint.cuh.
+template <int P>
+static void launch_T32(pgb_ctx* c, const TArgs& ta0, const float4* xrel, const float4* yrel, const float4* nrm, float* L) {
     constexpr int T = MI<P>::T;
     constexpr int NW = 4;
     cudaStream_t s = c->stream;
     TArgs ta = ta0;
-    PGB_CUDA(cudaMemsetAsync(L, 0, sizeof(real) * (size_t)c->n_nodes * 2 * T, s));
-    k_p2p_T<real><<<(unsigned)std::max<int64_t>(ta.n_leaves, 1), 256, 0, s>>>(ta, (const v4*)xrel, c->d_sT,
-                                                                                (const v4*)yrel, (const v4*)nrm);
+    PGB_CUDA(cudaMemsetAsync(L, 0, sizeof(float) * (size_t)c->n_nodes * 2 * T, s));
+    k_p2p_T<float><<<(unsigned)std::max<int64_t>(ta.n_leaves, 1), 256, 0, s>>>(ta, xrel, c->d_sT,
+                                                                                yrel, nrm);
     if (ta.n_fitems > 0)
-        k_m2p_T<real, P, NW><<<(unsigned)ta.n_fitems, NW * 32, 0, s>>>(ta, (const v4*)xrel, c->d_sT, (real*)L);
+        k_m2p_T<float, P, NW><<<(unsigned)ta.n_fitems, NW * 32, 0, s>>>(ta, xrel, c->d_sT, L);
     int launches = 3;
     for (size_t l = 0; l + 2 < c->level_begin.size(); ++l) {  // parents at level l push to level l + 1
         ta.lvl_begin = c->level_begin[l];
         ta.lvl_end = c->level_begin[l + 1];
         if (ta.lvl_end > ta.lvl_begin) {
-            k_l2l_level<real, P><<<(unsigned)(ta.lvl_end - ta.lvl_begin), 256, 0, s>>>(ta, (real*)L);
+            k_l2l_level<float, P><<<(unsigned)(ta.lvl_end - ta.lvl_begin), 256, 0, s>>>(ta, L);
             ++launches;
         }
     }
-    k_l2p<real, P><<<(unsigned)std::max<int64_t>(ta.n_leaves, 1), 128, 0, s>>>(ta, (const v4*)yrel, (const v4*)nrm,
-                                                                               (const real*)L);
+    k_l2p<float, P><<<(unsigned)std::max<int64_t>(ta.n_leaves, 1), 128, 0, s>>>(ta, yrel, nrm,
+                                                                               (const float*)L);
     PGB_CUDA(cudaGetLastError());
     PGB_LAUNCHED(c, launches);
 }
 
-template <typename real>
-static void dispatch_T(pgb_ctx* c, const TArgs& ta, const void* xrel, const void* yrel, const void* nrm, void* L) {
-    switch (c->p.P) {
-        case 0: launch_T<real, 0>(c, ta, xrel, yrel, nrm, L); break;
-        case 1: launch_T<real, 1>(c, ta, xrel, yrel, nrm, L); break;
-        case 2: launch_T<real, 2>(c, ta, xrel, yrel, nrm, L); break;
-        case 3: launch_T<real, 3>(c, ta, xrel, yrel, nrm, L); break;
-        case 4: launch_T<real, 4>(c, ta, xrel, yrel, nrm, L); break;
-        case 5: launch_T<real, 5>(c, ta, xrel, yrel, nrm, L); break;
-        case 6: launch_T<real, 6>(c, ta, xrel, yrel, nrm, L); break;
-        case 7: launch_T<real, 7>(c, ta, xrel, yrel, nrm, L); break;
-        case 8: launch_T<real, 8>(c, ta, xrel, yrel, nrm, L); break;
-        default: fail(PGB_EINVAL, "the transposed treecode takes P in 0..8");
+// FP64: the kernels of adjoint_h.cuh.
+template <int P>
+static void launch_T64(pgb_ctx* c, const TArgs& ta0, const UpArgs& ua, const dbl4* xrel, const dbl4* yrel, const dbl4* nrm,
+                       double* H, double* L) {
+    constexpr int NC = n_far_pad(P);
+    constexpr int NW = 4;
+    cudaStream_t s = c->stream;
+    TArgs ta = ta0;
+    PGB_CUDA(cudaMemsetAsync(H, 0, sizeof(double) * (size_t)c->n_nodes * 2 * NC, s));
+    const unsigned nl = (unsigned)std::max<int64_t>(ta.n_leaves, 1);
+    if (ta.near_mat) k_near_T<8><<<nl, 256, 0, s>>>(ta, c->d_sT);
+    else k_p2p_T<double><<<nl, 256, 0, s>>>(ta, xrel, c->d_sT, yrel, nrm);
+    if (ta.n_fitems > 0)
+        k_m2p_TH<double, P, NW><<<(unsigned)ta.n_fitems, NW * 32, 0, s>>>(ta, xrel, c->d_sT, H);
+    k_far_TH<double, P><<<(unsigned)c->n_nodes, 128, 0, s>>>(ta, c->n_nodes, (const double*)H, L);
+    int launches = 4;
+    for (size_t l = 1; l + 1 < c->level_begin.size(); ++l) {  // into the nodes of level l
+        ta.lvl_begin = c->level_begin[l];
+        ta.lvl_end = c->level_begin[l + 1];
+        if (ta.lvl_end > ta.lvl_begin) {
+            k_l2l_TH<double, P><<<(unsigned)((ta.lvl_end - ta.lvl_begin + 3) / 4), 128, 0, s>>>(ta, c->d_node_parent,
+                                                                                                L);
+            ++launches;
+        }
     }
+    if (ua.pmom) k_l2p_TH<double, P, true><<<nl, 128, 0, s>>>(ta, ua, (const double*)L);
+    else k_l2p_TH<double, P, false><<<nl, 128, 0, s>>>(ta, ua, (const double*)L);
+    PGB_CUDA(cudaGetLastError());
+    PGB_LAUNCHED(c, launches);
 }
+
+#define PGB_T_ORDERS(CALL)                                                                \
+    switch (c->p.P) {                                                                     \
+        case 0: CALL(0); break;                                                           \
+        case 1: CALL(1); break;                                                           \
+        case 2: CALL(2); break;                                                           \
+        case 3: CALL(3); break;                                                           \
+        case 4: CALL(4); break;                                                           \
+        case 5: CALL(5); break;                                                           \
+        case 6: CALL(6); break;                                                           \
+        case 7: CALL(7); break;                                                           \
+        case 8: CALL(8); break;                                                           \
+        default: fail(PGB_EINVAL, "the transposed treecode takes P in 0..8");             \
+    }
 
 // Row weights of the transposed product: s_L = lam of the interior (Laplace)
 // row of a molecule panel, s_Y = lam of its exterior row or of a surface row.
@@ -295,18 +342,45 @@ void apply_transpose(pgb_ctx* c, const double* lam, double* y, int precision) {
     ta.n_leaves = c->n_leaves;
     ta.leaf_node = c->d_leaf_node;
     ta.lvl_begin = ta.lvl_end = 0;
-    c->d_Tout.resize(4 * n * K);
-    ta.out = c->d_Tout;
+    if (c->p.P > 8) fail(PGB_EINVAL, "the transposed treecode takes P in 0..8");
+    ta.near_mat = ta.near_grp = nullptr;
+    ta.pan = ta.nearp = nullptr;
     c->d_sT.resize(2 * n);
     k_sT<<<nblk(n, 128), 128, 0, s>>>(g, bd, lam, c->d_sT);
     if (precision == PGB_FP32) {
+        c->d_Tout.resize(4 * n * K);
+        ta.out = c->d_Tout;
         c->d_momT32.resize((size_t)c->n_nodes * 2 * T);
-        dispatch_T<float>(c, ta, c->d_x32, c->d_y32, c->d_n32, c->d_momT32);
+#define CALL(P) launch_T32<P>(c, ta, c->d_x32, c->d_y32, c->d_n32, c->d_momT32)
+        PGB_T_ORDERS(CALL)
+#undef CALL
     } else {
+        UpArgs ua = {};  // the panel moments' part of it
+        ua.K = c->p.K;
+        ua.rule = far_rule(c->p.K);
+        ua.pg = c->d_pg64.p;
+        ua.pmom = panel_moments(c, 1);
+        ta.far_tr = far_table(c, c->kappa).tr64.p;
+        ta.ent_col = c->d_ent_col;
+        if (c->near_on && near_ready(c, 1)) {
+            ta.near_mat = c->near_mat[1].buf.p;
+            ta.near_grp = c->near_mat[1].group.p;
+        } else {
+            c->d_Tout.resize(4 * n * K);
+        }
+        ta.out = c->d_Tout;
+        c->d_Tpan.resize(4 * n);
+        c->d_Tnearp.resize(4 * n);
+        ta.pan = c->d_Tpan;
+        ta.nearp = c->d_Tnearp;
+        c->d_farT64.resize((size_t)c->n_nodes * 2 * n_far_pad(c->p.P));
         c->d_momT64.resize((size_t)c->n_nodes * 2 * T);
-        dispatch_T<double>(c, ta, c->d_x64, c->d_y64, c->d_n64, c->d_momT64);
+#define CALL(P) launch_T64<P>(c, ta, ua, c->d_x64, c->d_y64, c->d_n64, c->d_farT64, c->d_momT64)
+        PGB_T_ORDERS(CALL)
+#undef CALL
     }
-    k_assemble_T<<<nblk(n, 128), 128, 0, s>>>(g, bd, c->d_Tout, c->d_sT, c->d_ct_off, c->d_ct_i, c->d_ct_val, lam, y);
+    k_assemble_T<<<nblk(n, 128), 128, 0, s>>>(g, bd, c->d_Tout, ta.pan, ta.near_mat ? ta.nearp : nullptr, c->d_sT,
+                                              c->d_ct_off, c->d_ct_i, c->d_ct_val, lam, y);
     PGB_CUDA(cudaGetLastError());
     PGB_LAUNCHED(c, 2);
 }
@@ -496,6 +570,7 @@ __global__ void __launch_bounds__(256) k_cross_grad(Geo g, const float4* __restr
 void grad(pgb_ctx* c, const double* x, int precision, double tol, int max_iter, int restart, double* dq, double* dbc,
           double* dt, pgb_solve_stats* st) {
     if (!c->tree_valid) fail(PGB_ESTATE, "pgb_tree_build has not run");
+    NearScope keep(c);
     if (c->n_xcorr) fail(PGB_EINVAL, "gradients need the bodies farther apart than 2L (cross-body near entries exist)");
     if (precision != PGB_FP32 && precision != PGB_FP64) fail(PGB_EINVAL, "precision must be PGB_FP32 or PGB_FP64");
     cudaStream_t s = c->stream;
@@ -579,7 +654,8 @@ void grad(pgb_ctx* c, const double* x, int precision, double tol, int max_iter, 
             c->d_bu.resize(n);
             PGB_CUDA(cudaMemsetAsync(c->d_bu.p, 0, 8 * n, s));
             try {
-                apply_operator(c, nullptr, c->d_bu, precision, true, mask);
+                if (precision == PGB_FP32) imposed_rows_f32(c, b, c->d_bu);
+                else apply_operator(c, nullptr, c->d_bu, precision, true, mask);
             } catch (...) {
                 c->bodies[b].bc = saved;
                 throw;

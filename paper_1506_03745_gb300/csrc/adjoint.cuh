@@ -40,6 +40,12 @@ struct TArgs {
     const int32_t *far_l, *fitem_group;
     const float4* far4;
     int m2p_item;
+    // FP64 (adjoint_h.cuh)
+    const void* far_tr;             // far-field table, per column its T entries (FarTab::tr64)
+    const int32_t* ent_col;         // stored near field: an entry's first column in its group
+    const void *near_mat, *near_grp;
+    double* pan;                    // 4 per panel: far field / area of the V_L, K_L, V_Y, K_Y columns (no 1/4pi)
+    double* nearp;                  // the near field's, from the stored matrix
     // near: per source leaf (node id), the forward near entries that hold it
     const int64_t *tn_off;          // n_nodes + 1
     const int64_t* tn_e;            // forward near entry ids (group order)
@@ -186,6 +192,11 @@ __global__ void __launch_bounds__(NW * 32) k_m2p_T(TArgs a, const typename V4<re
         }
     }
 }
+
+__device__ __constant__ const int kBinom[9][9] = {
+    {1, 0, 0, 0, 0, 0, 0, 0, 0},      {1, 1, 0, 0, 0, 0, 0, 0, 0},      {1, 2, 1, 0, 0, 0, 0, 0, 0},
+    {1, 3, 3, 1, 0, 0, 0, 0, 0},      {1, 4, 6, 4, 1, 0, 0, 0, 0},      {1, 5, 10, 10, 5, 1, 0, 0, 0},
+    {1, 6, 15, 20, 15, 6, 1, 0, 0},   {1, 7, 21, 35, 35, 21, 7, 1, 0}, {1, 8, 28, 56, 70, 56, 28, 8, 1}};
 
 // Downward shift for every node of one level that has children:
 // L_j(child) += sum_{k >= j} C(k, j) (c - c_child)^{k - j} L_k(c), applied as

@@ -239,6 +239,17 @@ const FarTab& far_table(pgb_ctx* c, double kappa) {
     PGB_CUDA(cudaMemcpyAsync(t->t64.p, h.data(), 8 * h.size(), cudaMemcpyHostToDevice, c->stream));
     PGB_CUDA(cudaMemcpyAsync(t->t32.p, hf.data(), 4 * hf.size(), cudaMemcpyHostToDevice, c->stream));
     PGB_CUDA(cudaMemcpyAsync(t->tds.p, hds.data(), 4 * hds.size(), cudaMemcpyHostToDevice, c->stream));
+    if (c->p.P <= 8) {  // per column j the table's T entries, [Y, L][j][k]
+        const int T = n_terms(c->p.P), TR = far_cols(c->p.P);
+        std::vector<double> hr(h.size());
+        for (int q = 0; q < 2; ++q)
+            for (int k = 0; k < T; ++k)
+                for (int j = 0; j < TR; ++j)
+                    hr[((size_t)q * TR + j) * T + k] = h[((size_t)q * T + k) * TR + j];
+        t->tr64.resize(hr.size());
+        PGB_CUDA(cudaMemcpyAsync(t->tr64.p, hr.data(), 8 * hr.size(), cudaMemcpyHostToDevice, c->stream));
+        PGB_CUDA(cudaStreamSynchronize(c->stream));
+    }
     PGB_CUDA(cudaStreamSynchronize(c->stream));
     c->far_tabs.push_back(std::move(t));
     return *c->far_tabs.back();

@@ -339,7 +339,7 @@ static void launch_stage(pgb_ctx* c, int stage, int kind, const UpArgs& up, cons
 // would take more than a sixteenth of the device's memory (336 bytes a panel in
 // FP32 at order 6, 3.3 KB at order 15) or cannot be allocated: the P2M then
 // forms them on the spot.
-static const void* panel_moments(pgb_ctx* c, int kind) {
+const void* panel_moments(pgb_ctx* c, int kind) {
     auto& pm = c->pan_mom[kind];
     if (pm.geom_gen == c->geom_gen && pm.P == c->p.P) return pm.have ? (const void*)pm.buf.p : nullptr;
     if (c->capturing) return nullptr;  // (every product is prepared outside the capture)
@@ -376,38 +376,49 @@ static const void* panel_moments(pgb_ctx* c, int kind) {
 // or the screening change.  Not kept (the P2P then forms the sums, as products
 // outside solves do) where it would take more than an eighth of the device's
 // memory or a quarter of what is free, or cannot be allocated.
-static void near_field(pgb_ctx* c, int kind, EvalArgs& ev) {
+bool near_ready(pgb_ctx* c, int kind) {
     auto& nm = c->near_mat[kind];
-    if (nm.list_gen != c->list_gen || nm.kappa != c->kappa) {
-        if (c->capturing) return;  // (every product is prepared outside the capture)
-        nm.have = false;
-        nm.list_gen = c->list_gen;
-        nm.kappa = c->kappa;
-        if (c->n_groups == 0 || c->n_pitems == 0) return;
-        try {
-            nm.group.resize(16 * c->n_groups);
-            const int64_t units = near_groups(c, nm.group.p);
-            const size_t bytes = (size_t)units * 64 * (kind == 0 ? 4 : 8);
-            if (bytes > nm.buf.n) {
-                nm.buf.release();
-                size_t free_b = 0, total_b = 0;
-                PGB_CUDA(cudaMemGetInfo(&free_b, &total_b));
-                if (bytes > total_b / 8 || bytes > free_b / 4) return;
-                nm.buf.resize(bytes);
-            }
-        } catch (const Error& e) {
-            if (e.code != PGB_ENOMEM) throw;
-            return;
+    if (nm.list_gen == c->list_gen && nm.kappa == c->kappa) return nm.have;
+    if (c->capturing) return false;  // (every product is prepared outside the capture)
+    nm.have = false;
+    nm.list_gen = c->list_gen;
+    nm.kappa = c->kappa;
+    if (c->n_groups == 0 || c->n_pitems == 0) return false;
+    try {
+        nm.group.resize(16 * c->n_groups);
+        const int64_t units = near_groups(c, nm.group.p);
+        const size_t bytes = (size_t)units * 64 * (kind == 0 ? 4 : 8);
+        if (bytes > nm.buf.n) {
+            nm.buf.release();
+            size_t free_b = 0, total_b = 0;
+            PGB_CUDA(cudaMemGetInfo(&free_b, &total_b));
+            if (bytes > total_b / 8 || bytes > free_b / 4) return false;
+            nm.buf.resize(bytes);
         }
-        if (kind == 0) near_build_f32(ev, c->p.K, nm.group.p, c->d_x32, nm.buf.p, c->stream);
-        else near_build_f64(ev, c->p.K, nm.group.p, c->d_x64, nm.buf.p, c->stream);
-        PGB_CUDA(cudaGetLastError());
-        PGB_LAUNCHED(c, 1);
-        nm.have = true;
+    } catch (const Error& e) {
+        if (e.code != PGB_ENOMEM) throw;
+        return false;
     }
-    if (!nm.have) return;
-    ev.near_mat = nm.buf.p;
-    ev.near_group = nm.group.p;
+    EvalArgs ev = {};
+    ev.gstart = c->d_group_start;
+    ev.gend = c->d_group_end;
+    ev.gcenter = c->d_group_center;
+    ev.ncenter = c->d_node_center;
+    ev.kappa = c->kappa;
+    ev.col_off = c->d_col_off;
+    ev.col = c->d_col;
+    ev.pnode = c->d_pnode;
+    ev.rule = far_rule(c->p.K);
+    ev.n_pitems = c->n_pitems;
+    ev.pitem_off = c->d_pitem_off;
+    ev.pitem_group = c->d_pitem_group;
+    ev.pg = kind == 0 ? (const void*)c->d_pg32.p : (const void*)c->d_pg64.p;
+    if (kind == 0) near_build_f32(ev, c->p.K, nm.group.p, c->d_x32, nm.buf.p, c->stream);
+    else near_build_f64(ev, c->p.K, nm.group.p, c->d_x64, nm.buf.p, c->stream);
+    PGB_CUDA(cudaGetLastError());
+    PGB_LAUNCHED(c, 1);
+    nm.have = true;
+    return true;
 }
 
 // Upward pass as a CUDA graph: captured (on a private stream; nothing runs
@@ -650,7 +661,10 @@ static void apply_vec(pgb_ctx* c, VecIn xv, VecOut yv, int precision, int mode, 
     up.pg = ev.pg;
     up.pd = ev.pd;
     up.pmom = panel_moments(c, kind);
-    if (c->near_on && kind < 2 && !ev.p2p_work && c->shard_g[0] < 0 && !nested(c)) near_field(c, kind, ev);
+    if (c->near_on && kind < 2 && !ev.p2p_work && c->shard_g[0] < 0 && !nested(c) && near_ready(c, kind)) {
+        ev.near_mat = c->near_mat[kind].buf.p;
+        ev.near_group = c->near_mat[kind].group.p;
+    }
     auto tab_for = [&](double kappa) -> const void* {
         const FarTab& t = far_table(c, kappa);
         if (f32) return t.t32.p;

@@ -126,6 +126,7 @@ struct FarTab {
     DBuf<double> t64;
     DBuf<float> t32;
     DBuf<double> tds;  // the FP64 table split into double-single pairs (8 bytes each)
+    DBuf<double> tr64; // transposed rows, per column the T moments (the transposed treecode), P <= 8
 };
 // far-field coefficients per kernel (2p + 1 per degree p), padded to whole
 // 16-byte vectors, and the tables' columns
@@ -254,6 +255,7 @@ struct pgb_ctx {
     int64_t n_cols = 0;                  // P2P columns (panels of a group's near leaves) over all groups
     pgb::DBuf<int64_t> d_col_off;        // per group (+ total)
     pgb::DBuf<float4> d_col;             // panel centroid - group centre, panel
+    pgb::DBuf<int32_t> d_ent_col;        // first column (within its group) of every near entry
     pgb::DBuf<int32_t> d_pnode;          // leaf node of every panel
     pgb::DBuf<float> d_pg32;             // panel geometry of the P2P kernels, 16 values each
     pgb::DBuf<double> d_pg64, d_pg_ds;   // in FP64 and as double-single pairs (8 bytes a value)
@@ -297,6 +299,8 @@ struct pgb_ctx {
     pgb::DBuf<pgb::dbl4> d_srcT64;
     pgb::DBuf<float> d_momT32;
     pgb::DBuf<double> d_momT64, d_Tout, d_sT, d_lam, d_gx, d_bu;
+    // transposed FP64 product: gathered far-field coefficients; far and near sums per panel
+    pgb::DBuf<double> d_farT64, d_Tpan, d_Tnearp;
 
     // matvec work buffers
     // near field kept for the products of a solve (treecode.cuh, stored near
@@ -486,6 +490,8 @@ Geo geo(const pgb_ctx* c);
 // scans (tree.cu)
 void exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, cudaStream_t s, int64_t* total_host);
 // matvec (matvec.cu)
+bool near_ready(pgb_ctx* c, int kind);  // the stored near field (near_mat[kind]) is there for a running solve's product
+const void* panel_moments(pgb_ctx* c, int kind);  // nullptr: not kept
 void apply_operator(pgb_ctx* c, const double* x, double* y, int precision, bool known_only,
                     const int* known_mask = nullptr);
 void apply_transpose(pgb_ctx* c, const double* lam, double* y, int precision);

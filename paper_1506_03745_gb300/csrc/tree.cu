@@ -1203,10 +1203,11 @@ __global__ void k_col_count(int64_t ng, const int64_t* noff, const int32_t* near
     for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
     if (lane == 0) cnt[g] = c;
 }
-// The entries one after another, each entry's panels written by the warp.
+// The entries one after another, each entry's panels written by the warp; ecol:
+// an entry's first column in its group.
 __global__ void k_col_fill(int64_t ng, const int64_t* noff, const int32_t* nearl, const int32_t* nstart,
                            const int32_t* nend, const double* C, const double* gcen, const int64_t* coff,
-                           float4* col) {
+                           float4* col, int32_t* ecol) {
     const int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (g >= ng) return;
@@ -1214,6 +1215,7 @@ __global__ void k_col_fill(int64_t ng, const int64_t* noff, const int32_t* nearl
     int64_t w = coff[g];
     for (int64_t e = noff[g]; e < noff[g + 1]; ++e) {
         const int s = nstart[nearl[e]], n = nend[nearl[e]] - s;
+        if (lane == 0) ecol[e] = (int32_t)(w - coff[g]);
         for (int q = lane; q < n; q += 32) {
             const int64_t j = s + q;
             col[w + q] = make_float4((float)(C[3 * j] - g0), (float)(C[3 * j + 1] - g1), (float)(C[3 * j + 2] - g2),
@@ -1324,9 +1326,10 @@ void build_lists(pgb_ctx* c) {
         PGB_CUDA(cudaMemcpyAsync(c->d_col_off.p + ng, &nt, 8, cudaMemcpyHostToDevice, s));
         c->n_cols = nt;
         c->d_col.resize(nt);
+        c->d_ent_col.resize(std::max<int64_t>(c->n_near, 1));
         k_col_fill<<<nblk(32 * ng, 128), 128, 0, s>>>(ng, c->d_near_off, c->d_near, c->d_node_start,
                                                       c->d_node_end, c->d_c, c->d_group_center, c->d_col_off,
-                                                      c->d_col);
+                                                      c->d_col, c->d_ent_col);
         PGB_CUDA(cudaGetLastError());
     }
     {
@@ -1368,7 +1371,7 @@ void refresh_lists(pgb_ctx* c) {
     k_list_offsets<<<(unsigned)ng, 64, 0, s>>>(ng, c->d_far_off, c->d_far, c->d_node_center, c->d_group_center,
                                                c->d_far4);
     k_col_fill<<<nblk(32 * ng, 128), 128, 0, s>>>(ng, c->d_near_off, c->d_near, c->d_node_start, c->d_node_end,
-                                                  c->d_c, c->d_group_center, c->d_col_off, c->d_col);
+                                                  c->d_c, c->d_group_center, c->d_col_off, c->d_col, c->d_ent_col);
     PGB_CUDA(cudaGetLastError());
     PGB_CUDA(cudaStreamSynchronize(s));
     PGB_LAUNCHED(c, 3);

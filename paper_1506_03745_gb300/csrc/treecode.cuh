@@ -853,7 +853,8 @@ __global__ void __launch_bounds__(NW * 32) k_near_build(EvalArgs a, const NearGr
         }
         __syncwarp();
         for (int k = 0; k < cnt; ++k) {
-            const bool own = __shfl_sync(0xffffffffu, j, k) == p;
+            // zeros for the own panel and for lanes without a target
+            const bool own = __shfl_sync(0xffffffffu, j, k) == p || p >= p1;
             const int64_t c = e + k;
             real* u = mat + 64 * near_unit(nm, c);
             real VL, KL, VY, KY, h;
@@ -1209,12 +1210,6 @@ struct UpArgs {
 __device__ __forceinline__ bool body_on(const UpArgs& a, int b) {
     return a.src_active[b] && (!a.bmask || ((*a.bmask >> b) & 1ull));
 }
-
-
-__device__ __constant__ const int kBinom[9][9] = {
-    {1, 0, 0, 0, 0, 0, 0, 0, 0},      {1, 1, 0, 0, 0, 0, 0, 0, 0},      {1, 2, 1, 0, 0, 0, 0, 0, 0},
-    {1, 3, 3, 1, 0, 0, 0, 0, 0},      {1, 4, 6, 4, 1, 0, 0, 0, 0},      {1, 5, 10, 10, 5, 1, 0, 0, 0},
-    {1, 6, 15, 20, 15, 6, 1, 0, 0},   {1, 7, 21, 35, 35, 21, 7, 1, 0}, {1, 8, 28, 56, 70, 56, 28, 8, 1}};
 
 // Far-field coefficients of every node of an active body from its moments
 // (the tables of farfield.cu): a block takes NB nodes, whose moments it stages
