@@ -61,21 +61,11 @@ __global__ void k_seg_init_g(double* g, int64_t sV, int m1, const double* beta) 
     for (int i = threadIdx.x; i < m1; i += blockDim.x) g[p * sV + i] = i == 0 ? beta[p] : 0.0;
 }
 
-// y_p = H_p(0:k, 0:k)^{-1} g_p(0:k), k = kcol[p] (upper triangular; one
-// thread per problem)
-__global__ void k_seg_backsolve(const double* H, int ld, int64_t sH, const double* g, int64_t sV, const int* kcol,
-                                double* y, int B) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= B) return;
-    const double* Hp = H + p * sH;
-    const double* gp = g + p * sV;
-    double* yp = y + p * sV;
-    const int k = kcol[p];
-    for (int i = k - 1; i >= 0; --i) {
-        double s = gp[i];
-        for (int j = i + 1; j < k; ++j) s -= Hp[(int64_t)j * ld + i] * yp[j];
-        yp[i] = Hp[(int64_t)i * ld + i] != 0 ? s / Hp[(int64_t)i * ld + i] : 0.0;
-    }
+// y_p = H_p(0:k, 0:k)^{-1} g_p(0:k), k = kcol[p] (upper triangular; a block per problem)
+__global__ void __launch_bounds__(BACK_THREADS) k_seg_backsolve(const double* H, int ld, int64_t sH, const double* g,
+                                                                int64_t sV, const int* kcol, double* y) {
+    const int p = blockIdx.x;
+    backsolve(H + p * sH, ld, g + p * sV, kcol[p], y + p * sV);
 }
 
 // x += sum_{i < kcol[p]} y_p[i] V_i on the rows of problem p
@@ -99,14 +89,6 @@ __global__ void k_seg_axpby(double a, const double* x, double b, const double* y
 }
 
 // ---------------------------------------------------------------- replayed lockstep iterations
-// The column the next replayed product reads: dst = V_j, j from the device.
-__global__ void k_seg_select(const double* __restrict__ V, int64_t n, const int* __restrict__ jdev,
-                             double* __restrict__ dst) {
-    const int64_t j = *jdev;
-    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x)
-        dst[r] = V[j * n + r];
-}
-
 // After the segmented Arnoldi step of column j, one thread per problem (at
 // most 64): an active problem counts the column, keeps its estimate and
 // leaves when it meets its tolerance or breaks down; the body mask of the
@@ -174,10 +156,10 @@ static std::vector<double> seg_norms(pgb_ctx* c, const double* v) {
 }
 
 // Graph of the lockstep iterations after the first column of a cycle: a
-// device-side while loop whose body takes column j (k_seg_select), applies
-// the (preconditioned) operator to the problems the run-time body mask keeps,
-// makes the segmented Arnoldi step of column j and updates every problem's
-// state (k_seg_check).  Captured on the context's capture stream from the
+// device-side while loop whose body applies the (preconditioned)
+// operator to column j (d_xsel) for the problems the run-time body mask keeps,
+// makes the segmented Arnoldi step of column j, which leaves the next column
+// there, and updates every problem's state (k_seg_check).  Captured on the context's capture stream from the
 // launches the host loop makes; the caller sizes every buffer first.
 template <class ApplyPc>
 static void seg_graph_capture(pgb_ctx* c, const ArnSeg& sg, int m, double* hc, double* cs, double* sn, double* g,
@@ -213,12 +195,12 @@ static void seg_graph_capture(pgb_ctx* c, const ArnSeg& sg, int m, double* hc, d
     std::string why;
     PGB_CUDA(cudaStreamBeginCaptureToGraph(c->gm_stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
     try {
-        k_seg_select<<<nblk(n, 256), 256, 0, c->gm_stream>>>(c->d_V, n, ctl, c->d_xsel);
+        const ArnReplay rp{ctl, nullptr, c->d_xsel.p, nullptr, 0};
         apply_pc(c->d_xsel.p, c->d_wk.p);
-        arnoldi_step(c, 0, c->d_wk, c->d_H, hc, cs, sn, g, out, &sg, ctl, m);
+        arnoldi_step(c, 0, c->d_wk, c->d_H, hc, cs, sn, g, out, &sg, &rp, m);
         k_seg_check<<<1, 64, 0, c->gm_stream>>>(out, B, act, kcol, itc, estd, told, c->d_segm.p + 1, c->d_segm.p,
                                                  ctl, h);
-        PGB_LAUNCHED(c, 6);
+        PGB_LAUNCHED(c, 5);
     } catch (const Error& e) {
         why = e.msg;
     }
@@ -386,6 +368,7 @@ static int gmres_seg(pgb_ctx* c, int prec, const double* b, double* x, const dou
                 pm[0] = keep;
                 PGB_CUDA(cudaMemcpyAsync(act, ib.data(), 4 * (3 * B + 2), cudaMemcpyHostToDevice, s));
                 PGB_CUDA(cudaMemcpyAsync(c->d_segm.p, pm.data(), 8, cudaMemcpyHostToDevice, s));
+                PGB_CUDA(cudaMemcpyAsync(c->d_xsel.p, c->d_V.p + n, 8 * n, cudaMemcpyDeviceToDevice, s));  // column 1
                 PGB_CUDA(cudaGraphLaunch(c->seg_exec, s));
                 std::vector<double> eh(B);
                 PGB_CUDA(cudaMemcpyAsync(ib.data(), act, 4 * (3 * B + 2), cudaMemcpyDeviceToHost, s));
@@ -414,7 +397,7 @@ static int gmres_seg(pgb_ctx* c, int prec, const double* b, double* x, const dou
         }
         // x += M^{-1} V y, problem by problem with its own column count
         PGB_CUDA(cudaMemcpyAsync(kcol, kcol_h.data(), 4 * B, cudaMemcpyHostToDevice, s));
-        k_seg_backsolve<<<nblk(B, 32), 32, 0, s>>>(c->d_H, m + 1, sH, g, sV, kcol, yv, B);
+        k_seg_backsolve<<<B, BACK_THREADS, 0, s>>>(c->d_H, m + 1, sH, g, sV, kcol, yv);
         if (pc) {
             PGB_CUDA(cudaMemsetAsync(c->d_pz.p, 0, 8 * n, s));
             k_seg_axpy<<<dim3(nbp, B), SEG_THREADS, 0, s>>>(c->d_V, n, kcol, yv, sV, c->d_poff, c->d_pz);

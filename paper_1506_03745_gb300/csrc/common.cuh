@@ -111,4 +111,44 @@ __device__ T block_sum(T v, T* sh) {
     return v;  // valid in thread 0
 }
 
+// y = H(0:k,0:k)^{-1} g(0:k), upper triangular, column-major with ld, k at
+// most BACK_THREADS, by one block of as many threads: column by column from the
+// last, thread r holds row r and eight columns are in flight.  One thread's
+// chain of dependent loads took 0.3 ms for 80 columns.
+#define BACK_THREADS 256
+__device__ __forceinline__ void backsolve(const double* __restrict__ H, int ld, const double* __restrict__ g, int k,
+                                          double* __restrict__ y) {
+    __shared__ double yi[2];
+    const int r = threadIdx.x;
+    double s = r < k ? g[r] : 0.0;
+    const double d = r < k ? H[(int64_t)r * ld + r] : 0.0;
+    double x[8], nx[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        const int i = k - 1 - u;
+        nx[u] = i > r ? H[(int64_t)i * ld + r] : 0.0;
+    }
+    for (int i0 = k - 1; i0 >= 0; i0 -= 8) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            x[u] = nx[u];
+            const int i = i0 - 8 - u;
+            nx[u] = i > r ? H[(int64_t)i * ld + r] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int i = i0 - u;
+            if (i >= 0) {  // block-uniform
+                if (r == i) {
+                    s = d != 0 ? s / d : 0.0;
+                    yi[u & 1] = s;
+                    y[i] = s;
+                }
+                __syncthreads();
+                if (r < i) s -= x[u] * yi[u & 1];
+            }
+        }
+    }
+}
+
 }  // namespace pgb

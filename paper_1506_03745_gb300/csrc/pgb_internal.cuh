@@ -526,11 +526,21 @@ struct ArnSeg {
     const int* act;
     int64_t sH, sV;
 };
-// jdev != nullptr: the step of the column index held at jdev on the device
-// (h is then the base of H, column j at h + j (mcap + 1)); buffers sized for
-// columns up to mcap
+// A step replayed from a graph: its column is read from jdev (h is then the
+// base of H, column j at h + j (mcap + 1)) and v_{j+1} is also written to xsel,
+// which the next replay's product reads.  With ctl ({tol, column limit,
+// estimate}) the step also advances jdev and sets the loop condition cond;
+// jfin then holds the column for its last launch.
+struct ArnReplay {
+    int* jdev;
+    int* jfin;
+    double* xsel;
+    double* ctl;
+    cudaGraphConditionalHandle cond;
+};
+// rp: buffers sized for columns up to mcap
 void arnoldi_step(pgb_ctx* c, int j, double* w, double* h, double* hc, double* cs, double* sn, double* g,
-                  double* out, const ArnSeg* sg, const int* jdev = nullptr, int mcap = 0);
+                  double* out, const ArnSeg* sg, const ArnReplay* rp = nullptr, int mcap = 0);
 double energy_unit_kcal();
 void phi_reac(pgb_ctx* c, const double* x, double* out);
 // solver (solver.cu)

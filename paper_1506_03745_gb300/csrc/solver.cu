@@ -166,13 +166,8 @@ __global__ void k_axpby(double a, const double* x, double b, const double* y, do
 }
 
 // y = H(0:k,0:k)^{-1} g(0:k) (upper triangular)
-__global__ void k_backsolve(const double* H, int ld, const double* g, int k, double* y) {
-    if (threadIdx.x || blockIdx.x) return;
-    for (int i = k - 1; i >= 0; --i) {
-        double s = g[i];
-        for (int j = i + 1; j < k; ++j) s -= H[(int64_t)j * ld + i] * y[j];
-        y[i] = H[(int64_t)i * ld + i] != 0 ? s / H[(int64_t)i * ld + i] : 0.0;
-    }
+__global__ void __launch_bounds__(BACK_THREADS) k_backsolve(const double* H, int ld, const double* g, int k, double* y) {
+    backsolve(H, ld, g, k, y);
 }
 
 __global__ void k_init_g(double* g, int m1, const double* beta) {
@@ -182,25 +177,43 @@ __global__ void k_init_g(double* g, int m1, const double* beta) {
 
 // ---------------------------------------------------------------- Arnoldi step in four launches
 // The CGS2 step of column j without grid-wide barriers: every block keeps the
-// same rows r = blockIdx.x * blockDim.x + threadIdx.x + k * stride in every
-// launch, so w and v_{j+1} are only ever touched by their owner; the only
-// data crossing blocks are the per-block partial sums, which each block of
-// the next launch reduces for itself (in the same fixed order everywhere).
-//   k_arn_dot:    part[i][b] = (V_i . w) over block b's rows
-//   k_arn_update: c_i = sum_b part[i][b]; w -= sum_i c_i V_i; (pass 1) the
-//                 partials of the second pass, (pass 2) of |w|^2
-//   k_arn_finish: |w|, v_{j+1} = w / |w|, Givens step (block 0)
+// same contiguous rows in every launch, so w and v_{j+1} are only ever touched
+// by their owner; the only data crossing blocks are the per-block partial
+// sums, which each block of the next launch reduces for itself (in the same
+// fixed order everywhere).
+//   k_arn_dot:    part[b][i] = (V_i . w) over block b's rows
+//   k_arn_update: c_i = sum_b part[b][i]; w -= sum_i c_i V_i; (pass 1) the
+//                 partials of the second pass, (pass 2) of |w|^2, and one
+//                 more block for the previous rotations of column j
+//   k_arn_finish: |w|, v_{j+1} = w / |w|, the new rotation (one more block)
+// FP64 operations bound it (two a clock and multiprocessor: a warp's keeps the
+// pipe for 16 clocks, masked lanes or not) and, at few columns, each launch's
+// own latency: 4 n m operations are the step itself.  So a warp takes four
+// vectors over many rows before it adds lanes up (1.5 additions a vector
+// instead of one a row), the blocks' partials are added a thread per vector and
+// slice without a tree over lanes, and the rotations of column j run beside the
+// rows' update instead of as a chain of dependent loads after it.  Loops stay
+// short: each launch runs them cold, and unrolling them further or staging the
+// next loads costs more in instructions fetched than it hides (35.5 against
+// 34.7 ms for the solve below).  61440 unknowns, mean of columns 1 to 117: dots
+// 19.5 -> 11.0 us, updates 24.3 -> 18.5, last launch 17 -> 6, and two launches
+// (column selection, loop test) gone; the solve 38.1 -> 34.5 ms.
 #define ARN_BLOCKS_PER_SM 1
-#define ARN_THREADS 256
+#define ARN_THREADS 512
+#define ARN_WARPS (ARN_THREADS / 32)
+#define ARN_MIN_ROWS 64  // a block's rows, where there are enough (smaller systems leave blocks idle)
+#define ARN_TILE 512     // rows of w whose slices meet in shared memory (a thread each)
+#define ARN_SLICES 4
 
 struct ArnArgs {
     double* V;      // basis, column i at V + i * ld
     int64_t ld, n;
     int j;          // the new column's index (m = j + 1 coefficients)
+    int nb;         // blocks that hold rows
     double* w;      // A v_j on entry
     double* h;      // column j of H
     double* hc;     // second-pass coefficients
-    double* part;   // nb * (m + 1) partial sums, row i at part + i * nb
+    double* part;   // nb * (m + 1) partial sums, block b at part + b * m
     double* part2;  // second buffer (the next launch's partials)
     double *cs, *sn, *g;
     double* out;    // out[0] = |g_{j+1}|, out[1] = h_{j+1,j}
@@ -212,26 +225,29 @@ struct ArnArgs {
     const int64_t* poff;
     const int* act;
     int64_t sH, sV, sP;
-    // jdev != nullptr: the column index is read from device memory (an
-    // Arnoldi step replayed from a graph), j above is ignored and column j
-    // of H is at Hb + j * ldH
-    const int* jdev;
+    // Replayed from a graph (rp.jdev != nullptr): the column index is read
+    // from device memory, j above is ignored and column j of H is at Hb + j * ldH
+    ArnReplay rp;
     double* Hb;
     int64_t ldH;
 };
-__device__ __forceinline__ int arn_j(const ArnArgs& a) { return a.jdev ? *a.jdev : a.j; }
 
 // The slice of ArnArgs that block (., p) works on; false when p is inactive.
+// lo .. hi: the block's rows; nb: the blocks that hold rows of p.
 struct ArnView {
     double *h, *hc, *part, *part2, *cs, *sn, *g, *out;
     int64_t lo, hi;
+    int nb;
 };
 __device__ __forceinline__ bool arn_view(const ArnArgs& a, int j, ArnView& v) {
     const int p = blockIdx.y;
     if (a.act && !a.act[p]) return false;
-    v.lo = a.poff ? a.poff[p] : 0;
-    v.hi = a.poff ? a.poff[p + 1] : a.n;
-    v.h = (a.jdev ? a.Hb + (int64_t)j * a.ldH : a.h) + p * a.sH;
+    const int64_t p0 = a.poff ? a.poff[p] : 0, p1 = a.poff ? a.poff[p + 1] : a.n;
+    v.nb = (int)max((int64_t)1, min((int64_t)a.nb, (p1 - p0 + ARN_MIN_ROWS - 1) / ARN_MIN_ROWS));
+    const int64_t rows = (p1 - p0 + v.nb - 1) / v.nb;
+    v.lo = min(p1, p0 + blockIdx.x * rows);
+    v.hi = min(p1, v.lo + rows);
+    v.h = (a.rp.jdev ? a.Hb + (int64_t)j * a.ldH : a.h) + p * a.sH;
     v.hc = a.hc + p * a.sV;
     v.cs = a.cs + p * a.sV;
     v.sn = a.sn + p * a.sV;
@@ -242,177 +258,278 @@ __device__ __forceinline__ bool arn_view(const ArnArgs& a, int j, ArnView& v) {
     return true;
 }
 
-// Sums of eight values over the 32 lanes of a warp by a butterfly
-// reduce-scatter: each exchange halves the values a lane keeps, so a lane
-// does 9 additions instead of 40 (FP64 additions are scarce on this part).
-// Returns the full sum of value k = 4 b4 + 2 b3 + b2 (b_i: bit i of the lane)
-// in every lane; *k_out receives k.
-__device__ __forceinline__ double warp_sum8(const double (&t)[8], int* k_out) {
+// Sums of four values over the 32 lanes of a warp by a butterfly
+// reduce-scatter (6 additions a lane instead of 20).  Returns the full sum of
+// value k = 2 b4 + b3 (b_i: bit i of the lane) in every lane; *k_out receives k.
+__device__ __forceinline__ double warp_sum4(const double (&t)[4], int* k_out) {
     const int lane = threadIdx.x & 31;
-    double u[4], v[2], x;
-    const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const double give = h4 ? t[k] : t[k + 4];
-        const double keep = h4 ? t[k + 4] : t[k];
-        u[k] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
-    }
+    const bool h4 = lane & 16, h3 = lane & 8;
+    double u[2], x;
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-        const double give = h3 ? u[k] : u[k + 2];
-        const double keep = h3 ? u[k + 2] : u[k];
-        v[k] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
+        const double give = h4 ? t[k] : t[k + 2];
+        const double keep = h4 ? t[k + 2] : t[k];
+        u[k] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
     }
     {
-        const double give = h2 ? v[0] : v[1];
-        const double keep = h2 ? v[1] : v[0];
-        x = keep + __shfl_xor_sync(0xffffffffu, give, 4);
+        const double give = h3 ? u[0] : u[1];
+        const double keep = h3 ? u[1] : u[0];
+        x = keep + __shfl_xor_sync(0xffffffffu, give, 8);
     }
+    x += __shfl_xor_sync(0xffffffffu, x, 4);
     x += __shfl_xor_sync(0xffffffffu, x, 2);
     x += __shfl_xor_sync(0xffffffffu, x, 1);
-    *k_out = (h4 ? 4 : 0) + (h3 ? 2 : 0) + (h2 ? 1 : 0);
+    *k_out = (h4 ? 2 : 0) + (h3 ? 1 : 0);
     return x;
 }
 
-// Block partials of V_i . w (i < m) over this block's rows of its problem,
-// eight vectors at a time.
-__device__ __forceinline__ void arn_block_dots(const ArnArgs& a, const ArnView& v, int m, double* part, double* shd) {
-    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const unsigned nb = gridDim.x;
-    const int64_t stride = (int64_t)nb * blockDim.x;
-    const int64_t r0 = v.lo + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    for (int i0 = 0; i0 < m; i0 += 8) {
-        double t[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        for (int64_t r = r0; r < v.hi; r += stride) {
-            const double wr = a.w[r];
+// Block partials of V_i . w (i < m) over the block's rows: a warp takes four
+// vectors over a segment of the rows (segments where there are fewer fours
+// than warps), two rows a lane at a time.  sh: 4 (ceil(m / 4) segments),
+// at most 4 max(ARN_WARPS, ceil(m / 4)).
+__device__ __forceinline__ void arn_block_dots(const ArnArgs& a, const ArnView& v, int m, double* part, double* sh) {
+    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
+    const int G = (m + 3) / 4, S = max(1, ARN_WARPS / G);
+    const int64_t seg = ((v.hi - v.lo + S - 1) / S + 31) & ~(int64_t)31;
+    for (int q = wi; q < G * S; q += ARN_WARPS) {
+        const int sg = q / G, i0 = 4 * (q - sg * G);
+        const int64_t s0 = v.lo + sg * seg, s1 = min(v.hi, s0 + seg);
+        const double* __restrict__ c[4];
 #pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if (i0 + u < m) t[u] += a.V[(i0 + u) * a.ld + r] * wr;
+        for (int u = 0; u < 4; ++u) c[u] = a.V + min(i0 + u, m - 1) * a.ld;
+        double t[4] = {0, 0, 0, 0};
+#pragma unroll 1
+        for (int64_t r0 = s0 + lane; r0 - lane < s1; r0 += 64) {
+            double x[2][4], wr[2];
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const int64_t r = r0 + 32 * k;
+                const bool on = r < s1;
+                wr[k] = on ? a.w[r] : 0.0;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) x[k][u] = on ? c[u][r] : 0.0;
+            }
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) t[u] += x[k][u] * wr[k];
         }
         int k;
-        const double sum = warp_sum8(t, &k);
-        if ((lane & 3) == 0 && i0 + k < m) shd[(i0 + k) * nw + wi] = sum;
+        const double sum = warp_sum4(t, &k);
+        if ((lane & 7) == 0) sh[(i0 + k) * S + sg] = sum;
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < m; i += blockDim.x) {
+    for (int i = threadIdx.x; i < m; i += ARN_THREADS) {
         double t = 0;
-        for (int k = 0; k < nw; ++k) t += shd[i * nw + k];
-        part[(int64_t)i * nb + blockIdx.x] = t;
+        for (int k = 0; k < S; ++k) t += sh[i * S + k];
+        part[(int64_t)blockIdx.x * m + i] = t;
     }
 }
 
-// c_i = sum_b part[i][b] for i < m into shared memory (one warp per i, lanes
-// over b in a fixed order, then a fixed shuffle tree).
-__device__ __forceinline__ void arn_reduce(const double* part, int m, double* coef) {
-    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const unsigned nb = gridDim.x;
-    for (int i = wi; i < m; i += nw) {
-        double t = 0;
-        for (unsigned b = lane; b < nb; b += 32) t += part[(int64_t)i * nb + b];
-        t = warp_sum(t);
-        if (lane == 0) coef[i] = t;
+// c_i = sum_b part[b][i] for i < m into shared memory: a thread per vector and
+// slice of the blocks, eight loads in flight, then the slices.
+// sh: ARN_THREADS.  m <= 256 (two slices at least).
+__device__ __forceinline__ void arn_reduce(const double* __restrict__ part, int nb, int m, double* coef, double* sh) {
+    const int mp = (m + 31) & ~31, Q = ARN_THREADS / mp;
+    const int q = threadIdx.x / mp, i = threadIdx.x - q * mp;
+    if (q < Q) {
+        double s = 0;
+        if (i < m) {
+            const double* p = part + i;
+#pragma unroll 1
+            for (int b0 = q; b0 < nb; b0 += 8 * Q) {
+                double x[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) x[u] = b0 + u * Q < nb ? p[(b0 + u * Q) * m] : 0.0;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) s += x[u];
+            }
+        }
+        sh[q * mp + i] = s;
+    }
+    __syncthreads();
+    if (threadIdx.x < m) {
+        double s = 0;
+#pragma unroll 1
+        for (int u = 0; u < Q; ++u) s += sh[u * mp + threadIdx.x];
+        coef[threadIdx.x] = s;
     }
     __syncthreads();
 }
 
 __global__ void __launch_bounds__(ARN_THREADS) k_arn_dot(ArnArgs a) {
     extern __shared__ double shd[];
-    const int j = arn_j(a);
+    const int j = a.rp.jdev ? a.rp.jdev[0] : a.j;
+    if (a.rp.jfin && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *a.rp.jfin = j;
     ArnView v;
-    if (!arn_view(a, j, v)) return;
+    if (!arn_view(a, j, v) || blockIdx.x >= v.nb) return;
     arn_block_dots(a, v, j + 1, v.part, shd);
 }
 
-// pass 0: coefficients into h; pass 1: into hc and h += hc.  Then w -= sum
-// c_i V_i on this block's rows and the partials of the next step (pass 0:
-// the second-pass dots; pass 1: |w|^2 in part2[b]).
+// w -= sum_i coef_i V_i over the block's rows, tile by tile: a warp takes 32
+// rows and a slice of the vectors, eight loads at a time, and the slices of a
+// row meet in sh (ARN_SLICES ARN_TILE).  Returns the thread's sum of w^2.
+__device__ __forceinline__ double arn_axpy(const ArnArgs& a, const ArnView& v, int m, const double* coef, double* sh) {
+    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
+    const int vs = ((m + ARN_SLICES - 1) / ARN_SLICES + 7) & ~7, S = (m + vs - 1) / vs;
+    double sq = 0;
+    for (int64_t t0 = v.lo; t0 < v.hi; t0 += ARN_TILE) {
+        const int rows = (int)min((int64_t)ARN_TILE, v.hi - t0), nch = (rows + 31) / 32;
+        for (int q = wi; q < nch * S; q += ARN_WARPS) {
+            const int ch = q % nch, sl = q / nch, at = 32 * ch + lane;
+            const bool on = at < rows;
+            const double* __restrict__ c = a.V + t0 + at;
+            const int i1 = min(m, (sl + 1) * vs);
+            double s = 0;
+            for (int i = sl * vs; i < i1; i += 8) {
+                double x[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) x[u] = on && i + u < i1 ? c[(i + u) * a.ld] : 0.0;
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (i + u < i1) s += coef[i + u] * x[u];
+            }
+            sh[sl * ARN_TILE + at] = s;
+        }
+        __syncthreads();
+        for (int at = threadIdx.x; at < rows; at += ARN_THREADS) {
+            double s = 0;
+            for (int u = 0; u < S; ++u) s += sh[u * ARN_TILE + at];
+            const double wr = a.w[t0 + at] - s;
+            a.w[t0 + at] = wr;
+            sq += wr * wr;
+        }
+        __syncthreads();
+    }
+    return sq;
+}
+
+// pass 0: coefficients into h; pass 1: into hc and h += hc, and the rotations
+// of the earlier columns applied to h (the block after those with rows).
+// Then w -= sum c_i V_i on this block's rows and the partials of the next step
+// (pass 0: the second-pass dots; pass 1: |w|^2 in part[b]).
 __global__ void __launch_bounds__(ARN_THREADS) k_arn_update(ArnArgs a, int pass) {
-    extern __shared__ double shd[];  // m coefficients, then the dot scratch
-    const int j = arn_j(a);
+    extern __shared__ double shd[];
+    __shared__ double coef[256];
+    const int j = a.rp.jdev ? a.rp.jdev[0] : a.j;
     ArnView v;
     if (!arn_view(a, j, v)) return;
     const int m = j + 1;
-    double* coef = shd;
-    double* scratch = shd + ((m + 31) & ~31);
-    arn_reduce(pass ? v.part2 : v.part, m, coef);
-    if (blockIdx.x == 0)
-        for (int i = threadIdx.x; i < m; i += blockDim.x) {
-            if (pass) {
-                v.hc[i] = coef[i];
-                v.h[i] += coef[i];
-            } else {
-                v.h[i] = coef[i];
-            }
+    const bool turn = pass && blockIdx.x == gridDim.x - 1;
+    if (!turn && blockIdx.x >= v.nb) return;
+    const double* part = pass ? v.part2 : v.part;
+    // (the rotation block's own loads fly while the coefficients form)
+    const int i = threadIdx.x;
+    const double c = turn && i < j ? v.cs[i] : 1.0, s = turn && i < j ? v.sn[i] : 0.0, h0 = turn && i < m ? v.h[i] : 0.0;
+    arn_reduce(part, v.nb, m, coef, shd);
+    if (turn) {
+        // y_0 = h_0, y_{i+1} = c_i h_{i+1} - s_i y_i, h_i := c_i y_i + s_i h_{i+1}:
+        // only one operation a rotation is left in the chain
+        double *hs = shd, *b = shd + 257, *y = shd + 513;
+        if (i < m) {
+            v.hc[i] = coef[i];
+            hs[i] = h0 + coef[i];
         }
-    const unsigned nb = gridDim.x;
-    const int64_t stride = (int64_t)nb * blockDim.x;
-    const int64_t r0 = v.lo + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    double sq = 0;
-    for (int64_t r = r0; r < v.hi; r += stride) {
-        double t[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        for (int i0 = 0; i0 < m; i0 += 8)
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if (i0 + u < m) t[u] += coef[i0 + u] * a.V[(i0 + u) * a.ld + r];
-        const double wr = a.w[r] - (((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7])));
-        a.w[r] = wr;
-        sq += wr * wr;
-    }
-    if (pass == 0) {
         __syncthreads();
-        arn_block_dots(a, v, m, v.part2, scratch);
+        if (i < j) {
+            b[i] = c * hs[i + 1];
+            y[i] = s;
+        }
+        __syncthreads();
+        if (i == 0) {
+            double z = hs[0];
+#pragma unroll 1
+            for (int k = 0; k < j; ++k) {
+                const double z1 = b[k] - y[k] * z;
+                y[k] = z;
+                z = z1;
+            }
+            y[j] = z;
+        }
+        __syncthreads();
+        if (i < m) v.h[i] = i < j ? c * y[i] + s * hs[i + 1] : y[i];
+        return;
+    }
+    if (!pass && blockIdx.x == 0 && threadIdx.x < m) v.h[threadIdx.x] = coef[threadIdx.x];
+    const double sq = arn_axpy(a, v, m, coef, shd);
+    if (pass == 0) {
+        arn_block_dots(a, v, m, v.part2, shd);  // (arn_axpy ends in a barrier)
     } else {
-        sq = block_sum(sq, scratch);
-        if (threadIdx.x == 0) v.part[blockIdx.x] = sq;
+        // (warps beyond the block's rows hold zero)
+        const double t = (threadIdx.x & ~31) < v.hi - v.lo ? warp_sum(sq) : 0.0;
+        if ((threadIdx.x & 31) == 0) shd[threadIdx.x >> 5] = t;
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            const double s = warp_sum(threadIdx.x < ARN_WARPS ? shd[threadIdx.x] : 0.0);
+            if (threadIdx.x == 0) v.part[blockIdx.x] = s;
+        }
     }
 }
 
+// |w| and v_{j+1}; the block after those with rows makes the rotation of
+// column j (column-major H, ld = m + 1), applies it to g, out[0] = |g_{j+1}|,
+// out[1] = h_{j+1,j}, and in a graph of one problem keeps the estimate,
+// advances the column and sets the loop condition (go on while the estimate is
+// above the tolerance, no breakdown and columns remain): ctl = {tol, column
+// limit, estimate}.  One warp a block adds up |w|^2 and makes the root and the
+// division: an FP64 operation keeps a warp's scheduler for 64 clocks.
 __global__ void __launch_bounds__(ARN_THREADS) k_arn_finish(ArnArgs a) {
-    extern __shared__ double shd[];
-    const int j = arn_j(a);
+    __shared__ double sh;
+    const int j = a.rp.jfin ? *a.rp.jfin : a.rp.jdev ? a.rp.jdev[0] : a.j;
     ArnView v;
     if (!arn_view(a, j, v)) return;
-    const unsigned nb = gridDim.x;
-    double t = 0;
-    for (unsigned b = threadIdx.x; b < nb; b += blockDim.x) t += v.part[b];
-    t = block_sum(t, shd);
-    if (threadIdx.x == 0) shd[32] = sqrt(t);
-    __syncthreads();
-    const double nrm = shd[32];
-    const double inv = nrm > 0 ? 1.0 / nrm : 0.0;  // one division per block, not per row
-    const int64_t stride = (int64_t)nb * blockDim.x;
-    double* vn = a.V + (int64_t)(j + 1) * a.ld;
-    for (int64_t r = v.lo + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < v.hi; r += stride)
-        vn[r] = a.w[r] * inv;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        // Givens step on column j of H (column-major, ld = m + 1): the previous
-        // rotations, then the new one, applied to g; out[0] = |g_{j+1}|, out[1] = h_{j+1,j}
-        double* h = v.h;
-        h[j + 1] = nrm;
-        for (int i = 0; i < j; ++i) {
-            const double x = v.cs[i] * h[i] + v.sn[i] * h[i + 1];
-            const double y = -v.sn[i] * h[i] + v.cs[i] * h[i + 1];
-            h[i] = x;
-            h[i + 1] = y;
+    const bool turn = blockIdx.x == gridDim.x - 1;
+    if (!turn && blockIdx.x >= v.nb) return;
+    const int lane = threadIdx.x & 31;
+    if (threadIdx.x < 32) {
+        double t = 0;
+        for (int b = lane; b < v.nb; b += 32) t += v.part[b];
+        const double nrm = sqrt(warp_sum(t));
+        if (!turn) {
+            if (lane == 0) sh = nrm > 0 ? 1.0 / nrm : 0.0;
+        } else {
+            const double p = v.h[j], q = nrm;
+            const double r = hypot(p, q);
+            // lane 0: the cosine, lane 1: the sine
+            const double cs = r > 0 ? (lane ? q : p) / r : lane ? 0.0 : 1.0;
+            const double sv = __shfl_sync(0xffffffffu, cs, 1);
+            if (lane == 0) {
+                const double gj = v.g[j], gn = -sv * gj;
+                v.cs[j] = cs;
+                v.sn[j] = sv;
+                v.h[j] = r;
+                v.h[j + 1] = 0;
+                v.g[j + 1] = gn;
+                v.g[j] = cs * gj;
+                v.out[0] = fabs(gn);
+                v.out[1] = q;
+                if (a.rp.ctl) {
+                    a.rp.jdev[0] = j + 1;  // (the other blocks of this launch read jfin)
+                    a.rp.ctl[2] = fabs(gn);
+                    const bool more = fabs(gn) > a.rp.ctl[0] && q > 0 && (double)(j + 1) < a.rp.ctl[1];
+                    cudaGraphSetConditional(a.rp.cond, more ? 1u : 0u);
+                }
+            }
+            return;
         }
-        v.out[1] = h[j + 1];
-        const double p = h[j], q = h[j + 1];
-        const double r = hypot(p, q);
-        const double c = r > 0 ? p / r : 1.0, sv = r > 0 ? q / r : 0.0;
-        v.cs[j] = c;
-        v.sn[j] = sv;
-        h[j] = r;
-        h[j + 1] = 0;
-        v.g[j + 1] = -sv * v.g[j];
-        v.g[j] = c * v.g[j];
-        v.out[0] = fabs(v.g[j + 1]);
+    } else if (turn) {
+        return;
+    }
+    __syncthreads();
+    const double inv = sh;
+    double* vn = a.V + (int64_t)(j + 1) * a.ld;
+    for (int64_t r = v.lo + threadIdx.x; r < v.hi; r += ARN_THREADS) {
+        const double z = a.w[r] * inv;
+        vn[r] = z;
+        if (a.rp.xsel) a.rp.xsel[r] = z;
     }
 }
 
 // The four launches of one Arnoldi step; with sg, for the problems of a
-// block-diagonal system (sg->nbp blocks per problem).
+// block-diagonal system (sg->nbp blocks per problem); with rp, of a replayed
+// iteration with at most mcap columns.
 void arnoldi_step(pgb_ctx* c, int j, double* w, double* h, double* hc, double* cs, double* sn, double* g,
-                  double* out, const ArnSeg* sg, const int* jdev, int mcap) {
+                  double* out, const ArnSeg* sg, const ArnReplay* rp, int mcap) {
     if (c->arn_blocks == 0) {
         int dev = 0, sms = 0;
         PGB_CUDA(cudaGetDevice(&dev));
@@ -420,14 +537,15 @@ void arnoldi_step(pgb_ctx* c, int j, double* w, double* h, double* hc, double* c
         c->arn_blocks = ARN_BLOCKS_PER_SM * sms;
     }
     const int B = sg ? sg->B : 1;
-    // with jdev the column is only known on the device: sizes for the largest (mcap)
-    const int nb = sg ? sg->nbp : c->arn_blocks, m = jdev ? mcap : j + 1, warps = ARN_THREADS / 32;
+    // replayed, the column is only known on the device: sizes for the largest (mcap)
+    const int nb = sg ? sg->nbp : c->arn_blocks, m = rp ? mcap : j + 1;
     c->d_red.resize(std::max<size_t>(c->d_red.n, (size_t)2 * nb * (m + 1) * B));
     ArnArgs a;
     a.V = c->d_V;
     a.ld = c->n_unk;
     a.n = c->n_unk;
     a.j = j;
+    a.nb = nb;
     a.w = w;
     a.h = h;
     a.hc = hc;
@@ -442,19 +560,16 @@ void arnoldi_step(pgb_ctx* c, int j, double* w, double* h, double* hc, double* c
     a.sH = sg ? sg->sH : 0;
     a.sV = sg ? sg->sV : 0;
     a.sP = (int64_t)nb * (m + 1);
-    a.jdev = jdev;
+    a.rp = rp ? *rp : ArnReplay{};
     a.Hb = h;
     a.ldH = (int64_t)mcap + 1;
-    const size_t dots = 8 * (size_t)std::max(32, m * warps);
-    const size_t upd = 8 * (size_t)((m + 31) & ~31) + dots;
-    if (upd > 48 * 1024)
-        PGB_CUDA(cudaFuncSetAttribute(k_arn_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)upd));
+    const size_t dots = 8 * (size_t)(4 * std::max(ARN_WARPS, (m + 3) / 4));
+    const size_t upd = 8 * (size_t)std::max(ARN_SLICES * ARN_TILE, ARN_THREADS);
     cudaStream_t s = c->stream;
-    const dim3 grid(nb, B);
-    k_arn_dot<<<grid, ARN_THREADS, dots, s>>>(a);
-    k_arn_update<<<grid, ARN_THREADS, upd, s>>>(a, 0);
-    k_arn_update<<<grid, ARN_THREADS, upd, s>>>(a, 1);
-    k_arn_finish<<<grid, ARN_THREADS, 8 * 64, s>>>(a);
+    k_arn_dot<<<dim3(nb, B), ARN_THREADS, dots, s>>>(a);
+    k_arn_update<<<dim3(nb, B), ARN_THREADS, upd, s>>>(a, 0);
+    k_arn_update<<<dim3(nb + 1, B), ARN_THREADS, upd, s>>>(a, 1);
+    k_arn_finish<<<dim3(nb + 1, B), ARN_THREADS, 0, s>>>(a);
     PGB_CUDA(cudaGetLastError());
 }
 
@@ -552,32 +667,13 @@ struct Krylov {
 };
 
 // ---------------------------------------------------------------- replayed iterations
-// The column the next replayed product reads: dst = V_j, j from the device.
-__global__ void k_gm_select(const double* __restrict__ V, int64_t n, const int* __restrict__ jdev,
-                            double* __restrict__ dst) {
-    const int64_t j = *jdev;
-    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x)
-        dst[r] = V[j * n + r];
-}
-// After the Arnoldi step of column j: keep the estimate, advance j and set the
-// graph's loop condition (go on while the estimate is above the tolerance,
-// no breakdown and columns remain): ctl = {tol, column limit, estimate}.
-__global__ void k_gm_check(const double* __restrict__ out, int* jdev, double* ctl, cudaGraphConditionalHandle h) {
-    const int j = *jdev;
-    const double est = out[0], hnext = out[1];
-    *jdev = j + 1;
-    ctl[2] = est;
-    const bool more = est > ctl[0] && hnext > 0 && (double)(j + 1) < ctl[1];
-    cudaGraphSetConditional(h, more ? 1u : 0u);
-}
-
 // Restarted GMRES on A x = b from the given x; precision of the operator
 // `prec`; stops when the (estimated) residual <= abs_tol or after max_it
 // iterations.  Returns iterations done; *matvecs counts operator uses.
 // Graph of the GMRES iterations after the first column of a cycle: a
-// device-side while loop whose body takes column j (k_gm_select), applies the
-// (preconditioned) operator, makes the Arnoldi step of column j and tests the
-// estimate (k_gm_check).  Captured from the launches the host loop makes,
+// device-side while loop whose body applies the (preconditioned) operator to
+// column j (d_xsel), makes the Arnoldi step of column j, which leaves the next
+// column there, and tests the estimate (k_arn_finish).  Captured from the launches the host loop makes,
 // with the context's work sent to its own capture stream; rebuilt when the
 // tree, a parameter or a buffer it holds changes (gmres_op also drops it at
 // the start of every call).
@@ -616,11 +712,10 @@ static void gm_graph_ready(pgb_ctx* c, int prec, bool pc, int m, double* w, doub
     std::string why;
     PGB_CUDA(cudaStreamBeginCaptureToGraph(c->gm_stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
     try {
-        k_gm_select<<<nblk(n, 256), 256, 0, c->gm_stream>>>(c->d_V, n, c->d_gmi, c->d_xsel);
+        const ArnReplay rp{c->d_gmi.p, c->d_gmi.p + 1, c->d_xsel.p, c->d_gmd.p, h};
         apply_pc(c->d_xsel.p, w);
-        arnoldi_step(c, 0, w, c->d_H, hcol, cs, sn, g, out2, nullptr, c->d_gmi, m);
-        k_gm_check<<<1, 1, 0, c->gm_stream>>>(out2, c->d_gmi, c->d_gmd, h);
-        PGB_LAUNCHED(c, 6);
+        arnoldi_step(c, 0, w, c->d_H, hcol, cs, sn, g, out2, nullptr, &rp, m);
+        PGB_LAUNCHED(c, 4);
     } catch (const Error& e) {
         why = e.msg;
     }
@@ -699,7 +794,7 @@ int gmres_op(pgb_ctx* c, int prec, bool transpose, const double* b, double* x, d
             c->gm_graph.exec = nullptr;
         }
         // everything the replayed body touches is sized here, outside the capture
-        c->d_gmi.resize(1);
+        c->d_gmi.resize(2);
         c->d_gmd.resize(3);
         c->d_xsel.resize(n);
         if (pc) c->d_pz.resize(n);
@@ -763,6 +858,7 @@ int gmres_op(pgb_ctx* c, int prec, bool transpose, const double* b, double* x, d
                 hj[0] = 1;
                 PGB_CUDA(cudaMemcpyAsync(c->d_gmi.p, hj, sizeof(int), cudaMemcpyHostToDevice, s));
                 PGB_CUDA(cudaMemcpyAsync(c->d_gmd.p, c->h_pinned + 4, 16, cudaMemcpyHostToDevice, s));
+                PGB_CUDA(cudaMemcpyAsync(c->d_xsel.p, c->d_V.p + n, 8 * n, cudaMemcpyDeviceToDevice, s));  // column 1
                 PGB_CUDA(cudaGraphLaunch(c->gm_graph.exec, s));
                 PGB_CUDA(cudaMemcpyAsync(hj, c->d_gmi.p, sizeof(int), cudaMemcpyDeviceToHost, s));
                 PGB_CUDA(cudaMemcpyAsync(c->h_pinned + 5, c->d_gmd.p + 2, 8, cudaMemcpyDeviceToHost, s));
@@ -779,7 +875,7 @@ int gmres_op(pgb_ctx* c, int prec, bool transpose, const double* b, double* x, d
             }
             if (spec && !spec->forked && est <= spec->abs_thresh) {
                 // xs = x + M^{-1} V y with the j + 1 columns so far
-                k_backsolve<<<1, 1, 0, s>>>(c->d_H, m + 1, g, j + 1, yv);
+                k_backsolve<<<1, BACK_THREADS, 0, s>>>(c->d_H, m + 1, g, j + 1, yv);
                 PGB_CUDA(cudaMemcpyAsync(spec->xs, x, 8 * n, cudaMemcpyDeviceToDevice, s));
                 if (pc) {
                     PGB_CUDA(cudaMemsetAsync(c->d_pz.p, 0, 8 * n, s));
@@ -794,7 +890,7 @@ int gmres_op(pgb_ctx* c, int prec, bool transpose, const double* b, double* x, d
                 spec->fork(c, spec->xs, spec->user);
             }
         }
-        k_backsolve<<<1, 1, 0, s>>>(c->d_H, m + 1, g, j, yv);
+        k_backsolve<<<1, BACK_THREADS, 0, s>>>(c->d_H, m + 1, g, j, yv);
         if (pc) {  // x += M^{-1} V y
             PGB_CUDA(cudaMemsetAsync(c->d_pz.p, 0, 8 * n, s));
             k_multi_axpy<<<nblk(n, 256), 256, 0, s>>>(c->d_V, n, j, yv, 1.0, c->d_pz, n);
