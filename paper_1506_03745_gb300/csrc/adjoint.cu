@@ -387,57 +387,21 @@ void apply_transpose(pgb_ctx* c, const double* lam, double* y, int precision) {
 
 // ---------------------------------------------------------------- dF/dx
 // g = dF/dx: molecule panel j: -1/2 sum_k q_k K_L,kj on phi, 1/2 sum_k q_k V_L,kj on
-// dphi (the charge rows of Eq. 13, three tiers); surface panel: 1/2 beta A_j,
-// beta = sigma0 or eps_out phi0.  One block per panel.
-__global__ void k_dFdx(Geo g, BodyDev bd, Rules r, const double* qxyz, const double* qv, const int64_t* qoff,
-                       double eps_out, double* gx) {
-    __shared__ double sh[32];
-    const int64_t j = blockIdx.x;
+// dphi (the charge rows of Eq. 13, three tiers: the panel's charge weights,
+// which the energies of the same tree use); surface panel: 1/2 beta A_j,
+// beta = sigma0 or eps_out phi0.
+__global__ void k_dFdx(Geo g, BodyDev bd, const dbl4* __restrict__ qw, double eps_out, double* gx) {
+    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (j >= g.n_pan) return;
     const int b = g.pbody[j];
     const int64_t loc = g.perm[j] - bd.pan_off[b], N = bd.pan_off[b + 1] - bd.pan_off[b], o = bd.unk_off[b];
     if (bd.kind[b] != PGB_DIELECTRIC) {
-        if (threadIdx.x == 0) {
-            const double beta = bd.kind[b] == PGB_SET_CHARGE ? bd.bc[b] : eps_out * bd.bc[b];
-            gx[o + loc] = 0.5 * beta * g.A[j];
-        }
+        const double beta = bd.kind[b] == PGB_SET_CHARGE ? bd.bc[b] : eps_out * bd.bc[b];
+        gx[o + loc] = 0.5 * beta * g.A[j];
         return;
     }
-    const double* cj = g.c + 3 * j;
-    const double* nj = g.n + 3 * j;
-    const double* v = g.v + 9 * j;
-    double sv = 0, sk = 0;
-    for (int64_t k = qoff[b] + threadIdx.x; k < qoff[b + 1]; k += blockDim.x) {
-        const double* xq = qxyz + 3 * k;
-        double dx = xq[0] - cj[0], dy = xq[1] - cj[1], dz = xq[2] - cj[2];
-        double vl = 0, kl = 0;
-        const bool near = dx * dx + dy * dy + dz * dz < 8.0 * g.A[j];
-        const int M = near ? r.Kn : g.K;
-        for (int m = 0; m < M; ++m) {
-            double y[3], w;
-            if (near) {
-                for (int a = 0; a < 3; ++a)
-                    y[a] = cj[a] + ((r.mun[m][0] * (v[a] - cj[a]) + r.mun[m][1] * (v[3 + a] - cj[a])) +
-                                    r.mun[m][2] * (v[6 + a] - cj[a]));
-                w = r.wn[m] * g.A[j];
-            } else {
-                for (int a = 0; a < 3; ++a) y[a] = g.y[3 * (j * g.K + m) + a];
-                w = g.w[j * g.K + m];
-            }
-            double ex = xq[0] - y[0], ey = xq[1] - y[1], ez = xq[2] - y[2];
-            double rr = sqrt(ex * ex + ey * ey + ez * ez), ri = 1.0 / rr;
-            vl += w * ri;
-            kl += w * (nj[0] * ex + nj[1] * ey + nj[2] * ez) * ri * ri * ri;
-        }
-        sv += qv[k] * vl;
-        sk += qv[k] * kl;
-    }
-    sv = block_sum(sv, sh);
-    sk = block_sum(sk, sh);
-    if (threadIdx.x == 0) {
-        gx[o + loc] = -0.5 * sk / PGB_FOUR_PI;
-        gx[o + N + loc] = 0.5 * sv / PGB_FOUR_PI;
-    }
+    gx[o + loc] = qw ? -0.5 * qw[j].y / PGB_FOUR_PI : 0.0;
+    gx[o + N + loc] = qw ? 0.5 * qw[j].x / PGB_FOUR_PI : 0.0;
 }
 
 // dF/dq_k (internal units): Coulomb potential of the body's other charges +
@@ -595,7 +559,8 @@ void grad(pgb_ctx* c, const double* x, int precision, double tol, int max_iter, 
     // adjoint system A^T lam = dF/dx
     c->d_gx.resize(n);
     c->d_lam.resize(n);
-    k_dFdx<<<(unsigned)np, 128, 0, s>>>(g, bd, r, c->d_qxyz, c->d_qval, qoff, c->eps_out, c->d_gx);
+    charge_weights(c, qoff);
+    k_dFdx<<<nblk(np, 128), 128, 0, s>>>(g, bd, c->n_q ? c->d_qw.p : nullptr, c->eps_out, c->d_gx);
     PGB_CUDA(cudaGetLastError());
     PGB_LAUNCHED(c, 1);
     c->d_V.resize((size_t)(restart + 1) * n);

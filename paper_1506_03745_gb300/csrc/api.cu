@@ -28,9 +28,9 @@ __global__ void k_math_check(int64_t n, const double* x, double* y) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     const double v = x[i];
-    y[7 * i] = rsqrt_nr<1>(v);
-    y[7 * i + 1] = rsqrt_nr<2>(v);
-    y[7 * i + 2] = exp2_taylor(v);
+    y[7 * i] = rsqrt_halley(v);
+    y[7 * i + 1] = rsqrt_halley(v);
+    y[7 * i + 2] = exp2_table(v);
     y[7 * i + 3] = rsqrt(v);
     y[7 * i + 4] = exp2(v);
     y[7 * i + 5] = ds_to_double(ds_rsqrt(ds_from_double(v)));

@@ -33,23 +33,17 @@ __device__ __forceinline__ void rigid(const double* P, const double* v, double* 
         out[a] = dadd(dadd(dadd(dmul(P[3 * a + 0], v[0]), dmul(P[3 * a + 1], v[1])), dmul(P[3 * a + 2], v[2])), P[9 + a]);
 }
 
-// FP64 reciprocal square root, for 1e-30 < x < 1e30: the FP32 SFU estimate
-// (relative error below 2^-22) refined by NEWTON steps of Newton's iteration
-// for 1/y^2 = x, written as y <- y + (y/2)(1 - x y^2).  A step maps a relative
-// error d to about 1.5 d^2: one step leaves below 1e-13, two reach FP64
-// rounding.  x = 0 gives a non-finite value; callers mask it.
-template <int NEWTON>
-__device__ __forceinline__ double rsqrt_nr(double x) {
-    const float xf = __double2float_rn(x);
-    float yf;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(xf));
-    double y = (double)yf;
-#pragma unroll
-    for (int i = 0; i < NEWTON; ++i) {
-        const double e = fma(-(x * y), y, 1.0);
-        y = fma(0.5 * y, e, y);
-    }
-    return y;
+// FP64 reciprocal square root to FP64 rounding: the SFU's estimate from the
+// upper half of x (relative error d below 2^-20) refined by one step of
+// Halley's iteration, y <- y + y e (1/2 + 3/8 e) with e = 1 - x y^2, which
+// leaves about (5/2) d^3.  Five FP64 operations; two steps of Newton's iteration
+// on the FP32 estimate take eight and two conversions.  x = 0 gives a
+// non-finite value; callers mask it.
+__device__ __forceinline__ double rsqrt_halley(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-(x * y), y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
 // Coefficients (ln 2)^k / k! of the Taylor series of 2^f = e^{f ln 2}.
@@ -63,31 +57,39 @@ struct Exp2Coef<0> {
     static constexpr double v = 1.0;
 };
 
-// FP64 2^t for -2^30 < t <= 1020.  t = n + f with n = rint(t), found by adding
-// and removing 1.5 * 2^52 (the sum rounds to an integer, whose low word is n),
-// |f| <= 1/2; 2^f from its Taylor series to degree 11 (remainder below
-// 0.347^12 / 12! * sqrt(2) < 1e-14 relative), then n is added to the exponent
-// field.  Results below 2^-1020 are returned as 0.
-__device__ __forceinline__ double exp2_taylor(double t) {
-    const double magic = 6755399441055744.0;  // 1.5 * 2^52
+// 2^(i / 32), rounded from 60 digits
+static __device__ const double kExp2Frac[32] = {
+    0x1.0000000000000p+0, 0x1.059b0d3158574p+0, 0x1.0b5586cf9890fp+0, 0x1.11301d0125b51p+0,
+    0x1.172b83c7d517bp+0, 0x1.1d4873168b9aap+0, 0x1.2387a6e756238p+0, 0x1.29e9df51fdee1p+0,
+    0x1.306fe0a31b715p+0, 0x1.371a7373aa9cbp+0, 0x1.3dea64c123422p+0, 0x1.44e086061892dp+0,
+    0x1.4bfdad5362a27p+0, 0x1.5342b569d4f82p+0, 0x1.5ab07dd485429p+0, 0x1.6247eb03a5585p+0,
+    0x1.6a09e667f3bcdp+0, 0x1.71f75e8ec5f74p+0, 0x1.7a11473eb0187p+0, 0x1.82589994cce13p+0,
+    0x1.8ace5422aa0dbp+0, 0x1.93737b0cdc5e5p+0, 0x1.9c49182a3f090p+0, 0x1.a5503b23e255dp+0,
+    0x1.ae89f995ad3adp+0, 0x1.b7f76f2fb5e47p+0, 0x1.c199bdd85529cp+0, 0x1.cb720dcef9069p+0,
+    0x1.d5818dcfba487p+0, 0x1.dfc97337b9b5fp+0, 0x1.ea4afa2a490dap+0, 0x1.f50765b6e4540p+0,
+};
+
+// FP64 2^t for t <= 1020.  32 t = n + 32 f with n = rint(32 t), found by adding
+// and removing 1.5 * 2^47 (the sum rounds to a 32nd, whose low word is n),
+// |f| <= 1/64; 2^f from its Taylor series to degree 5 (remainder below
+// (ln 2 / 64)^6 / 6! < 3e-15 relative), times 2^((n mod 32) / 32) from a table
+// (256 bytes, two lines of L1) with n / 32 added to its exponent field.
+// Results below 2^-1020 are returned as 0.  Nine FP64 operations; the series to
+// degree 11 without a table takes fourteen.
+__device__ __forceinline__ double exp2_table(double t) {
+    const double magic = 211106232532992.0;  // 1.5 * 2^47
     const double s = t + magic;
     const int n = __double2loint(s);
     const double f = t - (s - magic);
-    double p = Exp2Coef<11>::v;
-    p = fma(p, f, Exp2Coef<10>::v);
-    p = fma(p, f, Exp2Coef<9>::v);
-    p = fma(p, f, Exp2Coef<8>::v);
-    p = fma(p, f, Exp2Coef<7>::v);
-    p = fma(p, f, Exp2Coef<6>::v);
-    p = fma(p, f, Exp2Coef<5>::v);
+    double p = Exp2Coef<5>::v;
     p = fma(p, f, Exp2Coef<4>::v);
     p = fma(p, f, Exp2Coef<3>::v);
     p = fma(p, f, Exp2Coef<2>::v);
     p = fma(p, f, Exp2Coef<1>::v);
     p = fma(p, f, 1.0);
-    const int hi = __double2hiint(p) + (int)((unsigned)n << 20);
-    const double y = __hiloint2double(hi, __double2loint(p));
-    return n < -1020 ? 0.0 : y;
+    const double u = __ldg(kExp2Frac + (n & 31));
+    const double y = p * __hiloint2double(__double2hiint(u) + (int)((unsigned)(n >> 5) << 20), __double2loint(u));
+    return (unsigned)__double2hiint(t) > 0xC08FE000u ? 0.0 : y;  // t < -1020 by its upper word
 }
 
 template <typename T>

@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -11,51 +12,98 @@
 
 namespace pgb {
 
-// V_L and K_L (without the 1/4pi) of panel j (sorted index) at the point xq:
-// the 19-point rule when |xq - c_j| < 2 L_j, else the K-point rule; 1/r by
-// two Newton steps.
-__device__ __forceinline__ void panel_vk(const Geo& g, const Rules& r, const double* xq, int64_t j, double& vl,
-                                         double& kl) {
-    const double* cj = g.c + 3 * j;
-    const double* nj = g.n + 3 * j;
-    double dx = xq[0] - cj[0], dy = xq[1] - cj[1], dz = xq[2] - cj[2];
-    double d2 = dx * dx + dy * dy + dz * dz;
+// A panel for V_L and K_L at points: with s_k = v_k - c, u = 2 s_0, v = 2 s_1,
+// g_k = |s_k|^2.
+struct VkPanel {
+    double c[3], n[3], u[3], v[3], g[3], A;
+};
+__device__ __forceinline__ VkPanel vk_panel(const Geo& g, int64_t j) {
+    VkPanel q;
+    q.A = g.A[j];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) q.g[k] = 0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        q.c[a] = g.c[3 * j + a];
+        q.n[a] = g.n[3 * j + a];
+        double s[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            s[k] = g.v[9 * j + 3 * k + a] - q.c[a];
+            q.g[k] = fma(s[k], s[k], q.g[k]);
+        }
+        q.u[a] = 2.0 * s[0];
+        q.v[a] = 2.0 * s[1];
+    }
+    return q;
+}
+
+// V_L and K_L (without the 1/4pi) of the panel at the point xq: the 19-point
+// rule when |xq - c| < 2 L, else the far rule by its orbits, y = c - 3 alpha
+// s_k: with d = xq - c the squared distance is |d|^2 + a (2 d.s_k + a |s_k|^2)
+// and the normal product n.d, the panel's (treecode.cuh, panel_sums).  FP64
+// operations bound these sums: ten a point and 22 a panel, against 24 a point
+// from its coordinates with two Newton steps (charge weights of 13000 panels
+// and 900 charges 3.83 -> 2.16 ms).
+template <int K>
+__device__ __forceinline__ void panel_vk(const VkPanel& q, const Rules& r, const FarRule& f, const double* xq,
+                                         double& vl, double& kl) {
+    const double dx = xq[0] - q.c[0], dy = xq[1] - q.c[1], dz = xq[2] - q.c[2];
+    const double d2 = dx * dx + dy * dy + dz * dz;
+    const double h = q.n[0] * dx + q.n[1] * dy + q.n[2] * dz;
     vl = 0;
     kl = 0;
-    if (d2 < 8.0 * g.A[j]) {
-        const double* v = g.v + 9 * j;
+    if (d2 < 8.0 * q.A) {
         for (int m = 0; m < r.Kn; ++m) {
-            double y[3];
-            for (int a = 0; a < 3; ++a)
-                y[a] = cj[a] + ((r.mun[m][0] * (v[a] - cj[a]) + r.mun[m][1] * (v[3 + a] - cj[a])) +
-                                r.mun[m][2] * (v[6 + a] - cj[a]));
-            double ex = xq[0] - y[0], ey = xq[1] - y[1], ez = xq[2] - y[2];
-            double ri = rsqrt_nr<2>(ex * ex + ey * ey + ez * ez);
-            double w = r.wn[m] * g.A[j];
-            vl += w * ri;
-            kl += w * (nj[0] * ex + nj[1] * ey + nj[2] * ez) * ri * ri * ri;
+            // (mu_2 = -mu_0 - mu_1 up to rounding, s_2 = -s_0 - s_1)
+            const double b0 = 0.5 * (r.mun[m][0] - r.mun[m][2]), b1 = 0.5 * (r.mun[m][1] - r.mun[m][2]);
+            const double ex = dx - (b0 * q.u[0] + b1 * q.v[0]), ey = dy - (b0 * q.u[1] + b1 * q.v[1]),
+                         ez = dz - (b0 * q.u[2] + b1 * q.v[2]);
+            const double ri = rsqrt_halley(ex * ex + ey * ey + ez * ez);
+            const double w = r.wn[m] * ri;
+            vl += w;
+            kl += w * (ri * ri);
         }
     } else {
-        for (int m = 0; m < g.K; ++m) {
-            const double* y = g.y + 3 * (j * g.K + m);
-            double ex = xq[0] - y[0], ey = xq[1] - y[1], ez = xq[2] - y[2];
-            double ri = rsqrt_nr<2>(ex * ex + ey * ey + ez * ez);
-            double w = g.w[j * g.K + m];
-            vl += w * ri;
-            kl += w * (nj[0] * ex + nj[1] * ey + nj[2] * ez) * ri * ri * ri;
+        auto point = [&](double r2, double& sv, double& sk) {
+            const double ri = rsqrt_halley(r2);
+            sv += ri;
+            sk += ri * (ri * ri);
+        };
+        if (K != 3) {
+            double sv = 0, sk = 0;
+            point(d2, sv, sk);
+            vl = f.w[0] * sv;
+            kl = f.w[0] * sk;
+        }
+        if (K >= 3) {
+            const double p0 = q.u[0] * dx + q.u[1] * dy + q.u[2] * dz, p1 = q.v[0] * dx + q.v[1] * dy + q.v[2] * dz;
+#pragma unroll
+            for (int o = 0; o < (K == 7 ? 2 : 1); ++o) {
+                const double a = f.a[o];
+                double sv = 0, sk = 0;
+                point(fma(a, fma(a, q.g[0], p0), d2), sv, sk);
+                point(fma(a, fma(a, q.g[1], p1), d2), sv, sk);
+                point(fma(a, fma(a, q.g[2], -(p0 + p1)), d2), sv, sk);
+                vl = fma(f.w[1 + o], sv, vl);
+                kl = fma(f.w[1 + o], sk, kl);
+            }
         }
     }
+    vl *= q.A;
+    kl *= q.A * h;
 }
 
 // Contribution of panel j (sorted index) of body b to phi_reac at xq
 // (without the 1/4pi): -K_L phi + V_L dphi.
-__device__ __forceinline__ double phi_panel(const Geo& g, const BodyDev& bd, const Rules& r, const double* xq,
-                                            const double* x, int b, int64_t j) {
+template <int K>
+__device__ __forceinline__ double phi_panel(const Geo& g, const BodyDev& bd, const Rules& r, const FarRule& f,
+                                            const double* xq, const double* x, int b, int64_t j) {
     const int64_t s0 = bd.pan_off[b], N = bd.pan_off[b + 1] - s0, o = bd.unk_off[b];
     const int64_t loc = g.perm[j] - s0;
     const double phi = x[o + loc], dphi = x[o + N + loc];
     double vl, kl;
-    panel_vk(g, r, xq, j, vl, kl);
+    panel_vk<K>(vk_panel(g, j), r, f, xq, vl, kl);
     return vl * dphi - kl * phi;
 }
 
@@ -71,11 +119,13 @@ __device__ __forceinline__ double phi_panel(const Geo& g, const BodyDev& bd, con
 // The same weights with one thread per panel over all its charges in order,
 // for bodies of fewer than 32 charges (a warp per panel would leave most
 // lanes idle, and the FP64 pipe takes whole warps).
-__global__ void k_charge_weights_1t(Geo g, BodyDev bd, Rules r, const double* qxyz, const double* qv,
+template <int K>
+__global__ void k_charge_weights_1t(Geo g, BodyDev bd, Rules r, FarRule f, const double* qxyz, const double* qv,
                                     const int64_t* qoff, dbl4* w) {
     const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (j >= g.n_pan) return;
     const int b = g.pbody[j];
+    const VkPanel q = vk_panel(g, j);
     double sv[2] = {0, 0}, sk[2] = {0, 0};
     for (int side = 0; side < 2; ++side) {
         const int src = side == 0 ? (bd.kind[b] == PGB_DIELECTRIC ? b : -1) : bd.parent[b];
@@ -83,7 +133,7 @@ __global__ void k_charge_weights_1t(Geo g, BodyDev bd, Rules r, const double* qx
         for (int64_t k = qoff[src]; k < qoff[src + 1]; ++k) {
             const double xq[3] = {qxyz[3 * k], qxyz[3 * k + 1], qxyz[3 * k + 2]};
             double vl, kl;
-            panel_vk(g, r, xq, j, vl, kl);
+            panel_vk<K>(q, r, f, xq, vl, kl);
             sv[side] += qv[k] * vl;
             sk[side] += qv[k] * kl;
         }
@@ -91,12 +141,14 @@ __global__ void k_charge_weights_1t(Geo g, BodyDev bd, Rules r, const double* qx
     w[j] = dbl4{sv[0], sk[0], sv[1], sk[1]};
 }
 
-__global__ void k_charge_weights(Geo g, BodyDev bd, Rules r, const double* qxyz, const double* qv,
+template <int K>
+__global__ void k_charge_weights(Geo g, BodyDev bd, Rules r, FarRule f, const double* qxyz, const double* qv,
                                  const int64_t* qoff, dbl4* w) {
     const int64_t j = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (j >= g.n_pan) return;
     const int b = g.pbody[j];
+    const VkPanel q = vk_panel(g, j);
     double sv[2] = {0, 0}, sk[2] = {0, 0};
     for (int side = 0; side < 2; ++side) {
         const int src = side == 0 ? (bd.kind[b] == PGB_DIELECTRIC ? b : -1) : bd.parent[b];
@@ -104,7 +156,7 @@ __global__ void k_charge_weights(Geo g, BodyDev bd, Rules r, const double* qxyz,
         for (int64_t k = qoff[src] + lane; k < qoff[src + 1]; k += 32) {
             const double xq[3] = {qxyz[3 * k], qxyz[3 * k + 1], qxyz[3 * k + 2]};
             double vl, kl;
-            panel_vk(g, r, xq, j, vl, kl);
+            panel_vk<K>(q, r, f, xq, vl, kl);
             sv[side] += qv[k] * vl;
             sk[side] += qv[k] * kl;
         }
@@ -119,7 +171,8 @@ __global__ void k_charge_weights(Geo g, BodyDev bd, Rules r, const double* qxyz,
 // phi_reac(r_k) = -K_L(phi) + V_L(dphi) at each charge of a dielectric body
 // (Eq. 13), three-tier rule with r_k as target: 19-point rule when
 // |r_k - c_j| < 2 L_j, the K-point rule otherwise.  One block per charge.
-__global__ void k_phi_reac(Geo g, BodyDev bd, Rules r, const double* qxyz, const int32_t* qbody, const double* x,
+template <int K>
+__global__ void k_phi_reac(Geo g, BodyDev bd, Rules r, FarRule f, const double* qxyz, const int32_t* qbody, const double* x,
                            double* out) {
     __shared__ double sh[32];
     const int64_t k = blockIdx.x;
@@ -127,16 +180,26 @@ __global__ void k_phi_reac(Geo g, BodyDev bd, Rules r, const double* qxyz, const
     const double xq[3] = {qxyz[3 * k], qxyz[3 * k + 1], qxyz[3 * k + 2]};
     double acc = 0;
     for (int64_t j = bd.pan_off[b] + threadIdx.x; j < bd.pan_off[b + 1]; j += blockDim.x)
-        acc += phi_panel(g, bd, r, xq, x, b, j);
+        acc += phi_panel<K>(g, bd, r, f, xq, x, b, j);
     acc = block_sum(acc, sh);
     if (threadIdx.x == 0) out[k] = acc / PGB_FOUR_PI;
+}
+
+// call(std::integral_constant<int, K>) for the far rule of K points
+template <class F>
+static void far_points(int K, F&& call) {
+    if (K == 1) call(std::integral_constant<int, 1>{});
+    else if (K == 3) call(std::integral_constant<int, 3>{});
+    else if (K == 4) call(std::integral_constant<int, 4>{});
+    else call(std::integral_constant<int, 7>{});
 }
 
 // The same sums split over blocks of PHI_CHUNK panels (grid: chunks x
 // charges) for few charges: part[k * nch + chunk], reduced in chunk order by
 // k_phi_reduce.
 #define PHI_CHUNK 256
-__global__ void __launch_bounds__(PHI_CHUNK) k_phi_reac_part(Geo g, BodyDev bd, Rules r, const double* qxyz,
+template <int K>
+__global__ void __launch_bounds__(PHI_CHUNK) k_phi_reac_part(Geo g, BodyDev bd, Rules r, FarRule f, const double* qxyz,
                                                             const int32_t* qbody, const double* x, int nch,
                                                             double* part) {
     __shared__ double sh[32];
@@ -144,7 +207,7 @@ __global__ void __launch_bounds__(PHI_CHUNK) k_phi_reac_part(Geo g, BodyDev bd, 
     const int b = qbody[k];
     const double xq[3] = {qxyz[3 * k], qxyz[3 * k + 1], qxyz[3 * k + 2]};
     const int64_t j = bd.pan_off[b] + (int64_t)blockIdx.x * PHI_CHUNK + threadIdx.x;
-    double acc = j < bd.pan_off[b + 1] ? phi_panel(g, bd, r, xq, x, b, j) : 0.0;
+    double acc = j < bd.pan_off[b + 1] ? phi_panel<K>(g, bd, r, f, xq, x, b, j) : 0.0;
     acc = block_sum(acc, sh);
     if (threadIdx.x == 0) part[k * nch + blockIdx.x] = acc;
 }
@@ -159,17 +222,23 @@ __global__ void k_phi_reduce(int64_t nq, int nch, const double* part, double* ou
 // phi_reac at every charge into out (device, n_q): the chunked kernels when
 // the charges alone would not fill the GPU, else one block per charge.
 static void launch_phi_reac(pgb_ctx* c, const Rules& r, const double* x, double* out) {
+    const FarRule f = far_rule(c->p.K);
     int64_t nmax = 0;
     for (auto& b : c->bodies) nmax = std::max<int64_t>(nmax, b.N);
     const int nch = (int)std::max<int64_t>(1, (nmax + PHI_CHUNK - 1) / PHI_CHUNK);
     if (c->n_q < 1024 && c->n_q * nch <= ((int64_t)1 << 22)) {
         c->d_phi_part.resize((size_t)c->n_q * nch);
-        k_phi_reac_part<<<dim3((unsigned)nch, (unsigned)c->n_q), PHI_CHUNK, 0, c->stream>>>(
-            geo(c), body_dev(c), r, c->d_qxyz, c->d_q_body, x, nch, c->d_phi_part);
+        far_points(c->p.K, [&](auto k) {
+            k_phi_reac_part<decltype(k)::value><<<dim3((unsigned)nch, (unsigned)c->n_q), PHI_CHUNK, 0, c->stream>>>(
+                geo(c), body_dev(c), r, f, c->d_qxyz, c->d_q_body, x, nch, c->d_phi_part);
+        });
         k_phi_reduce<<<(unsigned)((c->n_q + 127) / 128), 128, 0, c->stream>>>(c->n_q, nch, c->d_phi_part, out);
         PGB_LAUNCHED(c, 1);
     } else {
-        k_phi_reac<<<(unsigned)c->n_q, 128, 0, c->stream>>>(geo(c), body_dev(c), r, c->d_qxyz, c->d_q_body, x, out);
+        far_points(c->p.K, [&](auto k) {
+            k_phi_reac<decltype(k)::value>
+                <<<(unsigned)c->n_q, 128, 0, c->stream>>>(geo(c), body_dev(c), r, f, c->d_qxyz, c->d_q_body, x, out);
+        });
     }
     PGB_CUDA(cudaGetLastError());
 }
@@ -288,6 +357,33 @@ double energy_unit_kcal() {
     return e * e / (eps0 * 1e-10) * NA / 4184.0;
 }
 
+// Charge weights of the panels (d_qw): computed once per tree, charges and
+// rule, then every solution costs one pass over the panels.  qoff: the bodies'
+// charge offsets on the device.
+void charge_weights(pgb_ctx* c, const int64_t* qoff) {
+    if (!c->n_q) return;
+    const uint64_t key[4] = {c->tree_gen, c->config_gen, (uint64_t)c->p.K, (uint64_t)c->p.K_near};
+    if (!memcmp(key, c->qw_key, sizeof(key))) return;
+    cudaStream_t s = c->stream;
+    const Rules r = make_rules(c->p.K, c->p.K_near, c->p.n_edge);
+    const FarRule f = far_rule(c->p.K);
+    c->d_qw.resize(c->n_pan);
+    int64_t qmax = 0;
+    for (const auto& bo : c->bodies) qmax = std::max<int64_t>(qmax, bo.nq);
+    far_points(c->p.K, [&](auto k) {
+        constexpr int K = decltype(k)::value;
+        if (qmax < 32)
+            k_charge_weights_1t<K><<<(unsigned)((c->n_pan + 127) / 128), 128, 0, s>>>(
+                geo(c), body_dev(c), r, f, c->d_qxyz, c->d_qval, qoff, c->d_qw);
+        else
+            k_charge_weights<K><<<(unsigned)((c->n_pan * 32 + 127) / 128), 128, 0, s>>>(
+                geo(c), body_dev(c), r, f, c->d_qxyz, c->d_qval, qoff, c->d_qw);
+    });
+    PGB_CUDA(cudaGetLastError());
+    PGB_LAUNCHED(c, 1);
+    memcpy(c->qw_key, key, sizeof(key));
+}
+
 void energies(pgb_ctx* c, const double* x, pgb_energies* e, pgb_energies* per_body) {
     if (!c->tree_valid) fail(PGB_ESTATE, "pgb_tree_build has not run");
     cudaStream_t s = c->stream;
@@ -301,25 +397,7 @@ void energies(pgb_ctx* c, const double* x, pgb_energies* e, pgb_energies* per_bo
     qoff.resize(nb + 1);
     PGB_CUDA(cudaMemcpyAsync(qoff.p, qo.data(), 8 * (nb + 1), cudaMemcpyHostToDevice, s));
     Rules r = make_rules(c->p.K, c->p.K_near, c->p.n_edge);
-    // charge weights of the panels: computed once per tree, charges and rule,
-    // then every solution costs one pass over the panels
-    if (c->n_q) {
-        const uint64_t key[4] = {c->tree_gen, c->config_gen, (uint64_t)c->p.K, (uint64_t)c->p.K_near};
-        if (memcmp(key, c->qw_key, sizeof(key))) {
-            c->d_qw.resize(c->n_pan);
-            int64_t qmax = 0;
-            for (const auto& bo : c->bodies) qmax = std::max<int64_t>(qmax, bo.nq);
-            if (qmax < 32)
-                k_charge_weights_1t<<<(unsigned)((c->n_pan + 127) / 128), 128, 0, s>>>(
-                    geo(c), body_dev(c), r, c->d_qxyz, c->d_qval, qoff, c->d_qw);
-            else
-                k_charge_weights<<<(unsigned)((c->n_pan * 32 + 127) / 128), 128, 0, s>>>(
-                    geo(c), body_dev(c), r, c->d_qxyz, c->d_qval, qoff, c->d_qw);
-            PGB_CUDA(cudaGetLastError());
-            PGB_LAUNCHED(c, 1);
-            memcpy(c->qw_key, key, sizeof(key));
-        }
-    }
+    charge_weights(c, qoff);
     {
         DBuf<double> part;
         part.resize((size_t)3 * BODY_PARTS * nb);
@@ -432,7 +510,12 @@ void energies_noalloc(pgb_ctx* c, const double* x, pgb_energies* e) {
     int64_t* qoff = reinterpret_cast<int64_t*>(sums + 3 * PGB_MAX_BODIES);
     PGB_CUDA(cudaMemcpyAsync(qoff, qo, 8 * (nb + 1), cudaMemcpyHostToDevice, s));
     Rules r = make_rules(c->p.K, c->p.K_near, c->p.n_edge);
-    if (c->n_q) k_phi_reac<<<(unsigned)c->n_q, 128, 0, s>>>(geo(c), body_dev(c), r, c->d_qxyz, c->d_q_body, x, phir);
+    const FarRule f = far_rule(c->p.K);
+    if (c->n_q)
+        far_points(c->p.K, [&](auto k) {
+            k_phi_reac<decltype(k)::value>
+                <<<(unsigned)c->n_q, 128, 0, s>>>(geo(c), body_dev(c), r, f, c->d_qxyz, c->d_q_body, x, phir);
+        });
     k_body_sums<<<nb, 128, 0, s>>>(geo(c), body_dev(c), c->d_qxyz, c->d_qval, qoff, phir, nullptr, x, sums);
     PGB_CUDA(cudaGetLastError());
     // Coulomb pair sums, one block per charge, accumulated into the scratch

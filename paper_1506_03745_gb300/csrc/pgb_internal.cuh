@@ -543,6 +543,7 @@ void arnoldi_step(pgb_ctx* c, int j, double* w, double* h, double* hc, double* c
                   double* out, const ArnSeg* sg, const ArnReplay* rp = nullptr, int mcap = 0);
 double energy_unit_kcal();
 void phi_reac(pgb_ctx* c, const double* x, double* out);
+void charge_weights(pgb_ctx* c, const int64_t* qoff);
 // solver (solver.cu)
 void build_rhs(pgb_ctx* c, double* b, int precision, const double* bc = nullptr);
 int solve(pgb_ctx* c, int mode, double tol, int max_iter, int restart, double* x, pgb_solve_stats* st);
