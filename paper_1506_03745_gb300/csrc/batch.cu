@@ -575,6 +575,10 @@ static pgb_ctx* ensure_union(pgb_ctx* c, const std::vector<pgb_ctx*>& src) {
     }
     u->prob_first.push_back((int)u->bodies.size());
     u->n_prob = (int)src.size();
+    for (size_t p = 0; p < src.size(); ++p) {
+        const size_t q = std::find(src.begin(), src.end(), src[p]) - src.begin();
+        for (size_t k = 0; k < src[p]->bodies.size(); ++k) u->body_copy.push_back(u->prob_first[q] + (int)k);
+    }
     note_alloc();
     if (cudaStreamCreateWithFlags(&u->stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaMallocHost(&u->h_pinned, 64) != cudaSuccess) {

@@ -120,11 +120,12 @@ __device__ __forceinline__ double phi_panel(const Geo& g, const BodyDev& bd, con
 // for bodies of fewer than 32 charges (a warp per panel would leave most
 // lanes idle, and the FP64 pipe takes whole warps).
 template <int K>
-__global__ void k_charge_weights_1t(Geo g, BodyDev bd, Rules r, FarRule f, const double* qxyz, const double* qv,
-                                    const int64_t* qoff, dbl4* w) {
+__global__ void k_charge_weights_1t(Geo g, BodyDev bd, BodyCopies cp, Rules r, FarRule f, const double* qxyz, const double* qv,
+                                    const int64_t* qoff, dbl4* w, dbl4* worig) {
     const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (j >= g.n_pan) return;
     const int b = g.pbody[j];
+    if (cp.of[b] != b) return;  // k_copy_weights
     const VkPanel q = vk_panel(g, j);
     double sv[2] = {0, 0}, sk[2] = {0, 0};
     for (int side = 0; side < 2; ++side) {
@@ -139,15 +140,17 @@ __global__ void k_charge_weights_1t(Geo g, BodyDev bd, Rules r, FarRule f, const
         }
     }
     w[j] = dbl4{sv[0], sk[0], sv[1], sk[1]};
+    if (worig) worig[g.perm[j]] = w[j];
 }
 
 template <int K>
-__global__ void k_charge_weights(Geo g, BodyDev bd, Rules r, FarRule f, const double* qxyz, const double* qv,
-                                 const int64_t* qoff, dbl4* w) {
+__global__ void k_charge_weights(Geo g, BodyDev bd, BodyCopies cp, Rules r, FarRule f, const double* qxyz, const double* qv,
+                                 const int64_t* qoff, dbl4* w, dbl4* worig) {
     const int64_t j = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (j >= g.n_pan) return;
     const int b = g.pbody[j];
+    if (cp.of[b] != b) return;  // k_copy_weights
     const VkPanel q = vk_panel(g, j);
     double sv[2] = {0, 0}, sk[2] = {0, 0};
     for (int side = 0; side < 2; ++side) {
@@ -165,7 +168,21 @@ __global__ void k_charge_weights(Geo g, BodyDev bd, Rules r, FarRule f, const do
         sv[side] = warp_sum(sv[side]);
         sk[side] = warp_sum(sk[side]);
     }
-    if (lane == 0) w[j] = dbl4{sv[0], sk[0], sv[1], sk[1]};
+    if (lane == 0) {
+        const dbl4 v{sv[0], sk[0], sv[1], sk[1]};
+        w[j] = v;
+        if (worig) worig[g.perm[j]] = v;
+    }
+}
+
+// The weights of bodies that are others' copies, panel by panel in the body's
+// own order (worig: by original panel index): the first pass of a pose batch
+// summed the same weights for every pose, 7.1 of 57 ms.
+__global__ void k_copy_weights(Geo g, BodyDev bd, BodyCopies cp, const dbl4* __restrict__ worig, dbl4* __restrict__ w) {
+    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (j >= g.n_pan) return;
+    const int b = g.pbody[j], o = cp.of[b];
+    if (o != b) w[j] = worig[g.perm[j] - bd.pan_off[b] + bd.pan_off[o]];
 }
 
 // phi_reac(r_k) = -K_L(phi) + V_L(dphi) at each charge of a dielectric body
@@ -357,6 +374,12 @@ double energy_unit_kcal() {
     return e * e / (eps0 * 1e-10) * NA / 4184.0;
 }
 
+BodyCopies body_copies(const pgb_ctx* c) {
+    BodyCopies cp;
+    for (int k = 0; k < PGB_MAX_BODIES; ++k) cp.of[k] = k < (int)c->body_copy.size() ? c->body_copy[k] : k;
+    return cp;
+}
+
 // Charge weights of the panels (d_qw): computed once per tree, charges and
 // rule, then every solution costs one pass over the panels.  qoff: the bodies'
 // charge offsets on the device.
@@ -368,17 +391,25 @@ void charge_weights(pgb_ctx* c, const int64_t* qoff) {
     const Rules r = make_rules(c->p.K, c->p.K_near, c->p.n_edge);
     const FarRule f = far_rule(c->p.K);
     c->d_qw.resize(c->n_pan);
+    const BodyCopies cp = body_copies(c);
+    DBuf<dbl4> ob;
+    if (!c->body_copy.empty()) ob.resize(c->n_pan);
+    dbl4* orig = c->body_copy.empty() ? nullptr : ob.p;
     int64_t qmax = 0;
     for (const auto& bo : c->bodies) qmax = std::max<int64_t>(qmax, bo.nq);
     far_points(c->p.K, [&](auto k) {
         constexpr int K = decltype(k)::value;
         if (qmax < 32)
             k_charge_weights_1t<K><<<(unsigned)((c->n_pan + 127) / 128), 128, 0, s>>>(
-                geo(c), body_dev(c), r, f, c->d_qxyz, c->d_qval, qoff, c->d_qw);
+                geo(c), body_dev(c), cp, r, f, c->d_qxyz, c->d_qval, qoff, c->d_qw, orig);
         else
             k_charge_weights<K><<<(unsigned)((c->n_pan * 32 + 127) / 128), 128, 0, s>>>(
-                geo(c), body_dev(c), r, f, c->d_qxyz, c->d_qval, qoff, c->d_qw);
+                geo(c), body_dev(c), cp, r, f, c->d_qxyz, c->d_qval, qoff, c->d_qw, orig);
     });
+    if (orig) {
+        k_copy_weights<<<(unsigned)((c->n_pan + 127) / 128), 128, 0, s>>>(geo(c), body_dev(c), cp, orig, c->d_qw);
+        PGB_LAUNCHED(c, 1);
+    }
     PGB_CUDA(cudaGetLastError());
     PGB_LAUNCHED(c, 1);
     memcpy(c->qw_key, key, sizeof(key));

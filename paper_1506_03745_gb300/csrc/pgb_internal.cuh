@@ -177,6 +177,12 @@ struct Geo {
     const double* w;           // weight * area
 };
 
+// Per body the first body with the same mesh and charges (itself: none), for
+// kernels whose sums hold for every rigid pose.
+struct BodyCopies {
+    int of[PGB_MAX_BODIES];
+};
+
 struct BodyDev {  // per-body constants for kernels
     int kind[PGB_MAX_BODIES];
     double eps_ratio[PGB_MAX_BODIES];  // eps_in / eps_out (dielectric)
@@ -411,6 +417,9 @@ struct pgb_ctx {
     // it keeps with the sources it was copied from
     int n_prob = 1;
     std::vector<int> prob_first;
+    // the first body with the same mesh and charges (problems made from one
+    // context: bodies that differ by their pose); empty: none
+    std::vector<int> body_copy;
     pgb::DBuf<int64_t> d_poff;
     int seg_nbp = 0;                     // blocks per problem of the segmented kernels
     pgb::DBuf<double> d_seg, d_seg_red;  // per-problem Krylov vectors; segmented partial sums
@@ -544,6 +553,7 @@ void arnoldi_step(pgb_ctx* c, int j, double* w, double* h, double* hc, double* c
 double energy_unit_kcal();
 void phi_reac(pgb_ctx* c, const double* x, double* out);
 void charge_weights(pgb_ctx* c, const int64_t* qoff);
+BodyCopies body_copies(const pgb_ctx* c);
 // solver (solver.cu)
 void build_rhs(pgb_ctx* c, double* b, int precision, const double* bc = nullptr);
 int solve(pgb_ctx* c, int mode, double tol, int max_iter, int restart, double* x, pgb_solve_stats* st);

@@ -22,13 +22,13 @@ static inline int nblk(int64_t n, int t) { return (int)std::max<int64_t>(1, (n +
 // COUL_LANES lanes a row share its charges (FP64 work of whole warps: one lane
 // a row leaves a molecule of 13000 panels on 100 of the multiprocessors).
 #define COUL_LANES 4
-__global__ void k_coulomb_rows(Geo g, BodyDev bd, const double* qxyz, const double* qv, const int64_t* qoff,
+__global__ void k_coulomb_rows(Geo g, BodyDev bd, BodyCopies cp, const double* qxyz, const double* qv, const int64_t* qoff,
                                const double* eps_in, double* b) {
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, i = t / COUL_LANES;
     const int part = (int)(t % COUL_LANES);
-    const bool on = i < g.n_pan && bd.kind[g.pbody[min(i, g.n_pan - 1)]] == PGB_DIELECTRIC;
     const int64_t ii = min(i, g.n_pan - 1);
     const int bi = g.pbody[ii];
+    const bool on = i < g.n_pan && bd.kind[bi] == PGB_DIELECTRIC && cp.of[bi] == bi;  // (copies: k_copy_rows)
     const double x = g.c[3 * ii], y = g.c[3 * ii + 1], z = g.c[3 * ii + 2];
     const int64_t loc = g.perm[ii] - bd.pan_off[bi];
     const int64_t N = bd.pan_off[bi + 1] - bd.pan_off[bi];
@@ -48,6 +48,16 @@ __global__ void k_coulomb_rows(Geo g, BodyDev bd, const double* qxyz, const doub
     }
 }
 
+// The Coulomb rows of bodies that are others' copies.
+__global__ void k_copy_rows(Geo g, BodyDev bd, BodyCopies cp, double* b) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= g.n_pan) return;
+    const int bi = g.pbody[i], o = cp.of[bi];
+    if (o == bi || bd.kind[bi] != PGB_DIELECTRIC) return;
+    const int64_t loc = g.perm[i] - bd.pan_off[bi];
+    b[bd.unk_off[bi] + loc] = b[bd.unk_off[o] + loc];
+}
+
 // b = 0 except the Coulomb rows of the molecules.
 void coulomb_rows(pgb_ctx* c, double* b) {
     cudaStream_t s = c->stream;
@@ -65,7 +75,12 @@ void coulomb_rows(pgb_ctx* c, double* b) {
     de.resize(eps.size());
     PGB_CUDA(cudaMemcpyAsync(dq.p, qoff.data(), 8 * qoff.size(), cudaMemcpyHostToDevice, s));
     PGB_CUDA(cudaMemcpyAsync(de.p, eps.data(), 8 * eps.size(), cudaMemcpyHostToDevice, s));
-    k_coulomb_rows<<<nblk(COUL_LANES * c->n_pan, 128), 128, 0, s>>>(geo(c), body_dev(c), c->d_qxyz, c->d_qval, dq, de, b);
+    const BodyCopies cp = body_copies(c);
+    k_coulomb_rows<<<nblk(COUL_LANES * c->n_pan, 128), 128, 0, s>>>(geo(c), body_dev(c), cp, c->d_qxyz, c->d_qval, dq, de, b);
+    if (!c->body_copy.empty()) {
+        k_copy_rows<<<nblk(c->n_pan, 256), 256, 0, s>>>(geo(c), body_dev(c), cp, b);
+        PGB_LAUNCHED(c, 1);
+    }
     PGB_CUDA(cudaGetLastError());
     PGB_CUDA(cudaStreamSynchronize(s));
     PGB_LAUNCHED(c, 1);
@@ -102,7 +117,12 @@ void build_rhs(pgb_ctx* c, double* b, int precision, const double* bc) {
     de.resize(eps.size());
     PGB_CUDA(cudaMemcpyAsync(dq.p, qoff.data(), 8 * qoff.size(), cudaMemcpyHostToDevice, s));
     PGB_CUDA(cudaMemcpyAsync(de.p, eps.data(), 8 * eps.size(), cudaMemcpyHostToDevice, s));
-    k_coulomb_rows<<<nblk(COUL_LANES * c->n_pan, 128), 128, 0, s>>>(geo(c), body_dev(c), c->d_qxyz, c->d_qval, dq, de, b);
+    const BodyCopies cp = body_copies(c);
+    k_coulomb_rows<<<nblk(COUL_LANES * c->n_pan, 128), 128, 0, s>>>(geo(c), body_dev(c), cp, c->d_qxyz, c->d_qval, dq, de, b);
+    if (!c->body_copy.empty()) {
+        k_copy_rows<<<nblk(c->n_pan, 256), 256, 0, s>>>(geo(c), body_dev(c), cp, b);
+        PGB_LAUNCHED(c, 1);
+    }
     PGB_CUDA(cudaGetLastError());
     PGB_LAUNCHED(c, 2);
     PGB_CUDA(cudaStreamSynchronize(s));
