@@ -238,11 +238,11 @@ static void launch_T32(pgb_ctx* c, const TArgs& ta0, const float4* xrel, const f
     if (ta.n_fitems > 0)
         k_m2p_T<float, P, NW><<<(unsigned)ta.n_fitems, NW * 32, 0, s>>>(ta, xrel, c->d_sT, L);
     int launches = 3;
-    for (size_t l = 0; l + 2 < c->level_begin.size(); ++l) {  // parents at level l push to level l + 1
+    for (size_t l = 1; l + 1 < c->level_begin.size(); ++l) {  // into the nodes of level l
         ta.lvl_begin = c->level_begin[l];
         ta.lvl_end = c->level_begin[l + 1];
         if (ta.lvl_end > ta.lvl_begin) {
-            k_l2l_level<float, P><<<(unsigned)(ta.lvl_end - ta.lvl_begin), 256, 0, s>>>(ta, L);
+            k_l2l_level<float, P><<<(unsigned)(ta.lvl_end - ta.lvl_begin), 256, 0, s>>>(ta, c->d_node_parent, L);
             ++launches;
         }
     }

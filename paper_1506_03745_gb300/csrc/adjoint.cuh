@@ -198,11 +198,15 @@ __device__ __constant__ const int kBinom[9][9] = {
     {1, 3, 3, 1, 0, 0, 0, 0, 0},      {1, 4, 6, 4, 1, 0, 0, 0, 0},      {1, 5, 10, 10, 5, 1, 0, 0, 0},
     {1, 6, 15, 20, 15, 6, 1, 0, 0},   {1, 7, 21, 35, 35, 21, 7, 1, 0}, {1, 8, 28, 56, 70, 56, 28, 8, 1}};
 
-// Downward shift for every node of one level that has children:
+// Downward shift into the nodes of one level:
 // L_j(child) += sum_{k >= j} C(k, j) (c - c_child)^{k - j} L_k(c), applied as
-// three one-axis passes (the transpose of the moment shift of the upward pass, up_m2m).
+// three one-axis passes (the transpose of the moment shift of the upward pass,
+// up_m2m).  A block per child: its passes are a chain of barriers, which a
+// block per parent walked for one child after the other (20.8 -> 8.7 us a
+// level).
 template <typename real, int P>
-__global__ void __launch_bounds__(256) k_l2l_level(TArgs a, real* __restrict__ Lmom) {
+__global__ void __launch_bounds__(256) k_l2l_level(TArgs a, const int32_t* __restrict__ parent,
+                                                   real* __restrict__ Lmom) {
     constexpr int T = MI<P>::T;
     __shared__ real bufA[2 * T], bufB[2 * T];
     __shared__ real cd[3][P + 1];
@@ -210,11 +214,10 @@ __global__ void __launch_bounds__(256) k_l2l_level(TArgs a, real* __restrict__ L
     __shared__ short idx3[P + 1][P + 1][P + 1];
     __shared__ signed char kk[T][3];
     const int tid = threadIdx.x;
-    const int64_t nd = a.lvl_begin + blockIdx.x;
-    if (nd >= a.lvl_end) return;
-    const int nc = a.nchild[nd];
-    if (nc == 0) return;
-    const int fc = a.child[nd];
+    const int64_t ch = a.lvl_begin + blockIdx.x;
+    if (ch >= a.lvl_end) return;
+    const int nd = parent[ch];
+    if (nd < 0) return;
     for (int k = tid; k < T; k += blockDim.x) {
         int x, y, z;
         decode_mi(k, x, y, z);
@@ -227,42 +230,38 @@ __global__ void __launch_bounds__(256) k_l2l_level(TArgs a, real* __restrict__ L
         const int n = q / (P + 1), m = q - n * (P + 1);
         binom[n][m] = (real)kBinom[n][m];
     }
-    for (int ci = 0; ci < nc; ++ci) {
-        const int ch = fc + ci;
-        __syncthreads();
-        for (int k = tid; k < 2 * T; k += blockDim.x) bufA[k] = Lmom[nd * 2 * T + k];
-        if (tid < 3) {
-            const real d = (real)(a.ncenter[3 * nd + tid] - a.ncenter[3 * ch + tid]);
-            real v = 1;
-            for (int m = 0; m <= P; ++m) {
-                cd[tid][m] = v;
-                v *= d;
-            }
+    for (int k = tid; k < 2 * T; k += blockDim.x) bufA[k] = Lmom[(int64_t)nd * 2 * T + k];
+    if (tid < 3) {
+        const real d = (real)(a.ncenter[3 * nd + tid] - a.ncenter[3 * ch + tid]);
+        real v = 1;
+        for (int m = 0; m <= P; ++m) {
+            cd[tid][m] = v;
+            v *= d;
         }
-        __syncthreads();
-#pragma unroll 1
-        for (int ax = 0; ax < 3; ++ax) {
-            real* src = (ax == 1) ? bufB : bufA;
-            real* dst = (ax == 1) ? bufA : bufB;
-            for (int k = tid; k < T; k += blockDim.x) {
-                const int k0 = kk[k][0], k1 = kk[k][1], k2 = kk[k][2];
-                const int ka = kk[k][ax];
-                const int top = P - (k0 + k1 + k2 - ka);  // largest index along ax with |.| <= P
-                real sL = 0, sY = 0;
-                for (int jv = ka; jv <= top; ++jv) {
-                    const int jx = ax == 0 ? jv : k0, jy = ax == 1 ? jv : k1, jz = ax == 2 ? jv : k2;
-                    const int jj = idx3[jx][jy][jz];
-                    const real coef = binom[jv][ka] * cd[ax][jv - ka];
-                    sL += coef * src[jj];
-                    sY += coef * src[T + jj];
-                }
-                dst[k] = sL;
-                dst[T + k] = sY;
-            }
-            __syncthreads();
-        }
-        for (int k = tid; k < 2 * T; k += blockDim.x) Lmom[(int64_t)ch * 2 * T + k] += bufB[k];
     }
+    __syncthreads();
+#pragma unroll 1
+    for (int ax = 0; ax < 3; ++ax) {
+        real* src = (ax == 1) ? bufB : bufA;
+        real* dst = (ax == 1) ? bufA : bufB;
+        for (int k = tid; k < T; k += blockDim.x) {
+            const int k0 = kk[k][0], k1 = kk[k][1], k2 = kk[k][2];
+            const int ka = kk[k][ax];
+            const int top = P - (k0 + k1 + k2 - ka);  // largest index along ax with |.| <= P
+            real sL = 0, sY = 0;
+            for (int jv = ka; jv <= top; ++jv) {
+                const int jx = ax == 0 ? jv : k0, jy = ax == 1 ? jv : k1, jz = ax == 2 ? jv : k2;
+                const int jj = idx3[jx][jy][jz];
+                const real coef = binom[jv][ka] * cd[ax][jv - ka];
+                sL += coef * src[jj];
+                sY += coef * src[T + jj];
+            }
+            dst[k] = sL;
+            dst[T + k] = sY;
+        }
+        __syncthreads();
+    }
+    for (int k = tid; k < 2 * T; k += blockDim.x) Lmom[ch * 2 * T + k] += bufB[k];
 }
 
 // Far field at the quadrature nodes of every leaf (one block per leaf):
@@ -322,42 +321,43 @@ __global__ void __launch_bounds__(128) k_l2p(TArgs a, const typename V4<real>::t
 }
 
 // Near field, transposed: one block per source leaf b; for every forward near
-// entry (g, b) the 32 targets of g (offsets from the leaf centre, weights,
-// panel) are staged in shared memory and every thread sums them at its
-// quadrature node(s) of b, skipping the target's own panel (as the forward
-// P2P does).  Writes out (4 per node, no 1/4pi).
+// entry (g, b) the targets of g (offsets from the leaf centre, weights, panel)
+// are staged in shared memory and every thread sums them at its quadrature
+// node(s) of b, skipping the target's own panel (as the forward P2P does).
+// Writes out (4 per node, no 1/4pi).  The staging's chain of loads (entry,
+// group, targets) bounds it when one warp stages one entry between barriers:
+// each warp stages one of eight (36000 panels: 428 -> 266 us).
 template <typename real>
 __global__ void __launch_bounds__(256) k_p2p_T(TArgs a, const typename V4<real>::t* __restrict__ xrel,
                                                 const double* __restrict__ sT,
                                                 const typename V4<real>::t* __restrict__ yrel,
                                                 const typename V4<real>::t* __restrict__ nrm) {
     using v4 = typename V4<real>::t;
-    __shared__ v4 sX[32];       // target - leaf centre, s_L
-    __shared__ real sYw[32];    // s_Y
-    __shared__ int sPan[32];    // target panel (-1: none)
+    __shared__ v4 sX[8][32];       // target - leaf centre, s_L
+    __shared__ real sYw[8][32];    // s_Y
+    __shared__ int sFirst[8], sCnt[8], sLap[8];  // first target panel, targets, Laplace pair
     const int64_t leaf = blockIdx.x;
     if (leaf >= a.n_leaves) return;
     const int nd = a.leaf_node[leaf];
     const int nb = a.nbody[nd];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const real kappa = (real)a.kappa;
     const real nkl = -kappa * real(1.4426950408889634);
     const int64_t q0 = (int64_t)a.nstart[nd] * a.K, q1 = (int64_t)a.nend[nd] * a.K;
+    const int64_t t0 = a.tn_off[nd], t1 = a.tn_off[nd + 1];
     for (int64_t qb = q0; qb < q1; qb += blockDim.x) {  // chunks of the leaf's nodes
         const int64_t q = qb + threadIdx.x;
         const bool on = q < q1;
         const v4 A = yrel[on ? q : q0];
         const v4 n = nrm[(on ? q : q0) / a.K];
-        const int64_t panel = (on ? q : q0) / a.K;
+        const int panel = (int)((on ? q : q0) / a.K);
         real acc[4] = {0, 0, 0, 0}, cmp[4] = {0, 0, 0, 0};
-        for (int64_t t = a.tn_off[nd]; t < a.tn_off[nd + 1]; ++t) {
-            const int64_t e = a.tn_e[t];
-            const int64_t g = a.near_group[e];
-            const int64_t p0 = a.gstart[g], p1 = a.gend[g];
-            const int gb = a.gbody[g];
-            const bool lap = (nb == gb) && a.lap_body[gb];
+        for (int64_t tb = t0; tb < t1; tb += 8) {
             __syncthreads();
-            if (threadIdx.x < 32) {
-                const int64_t p = p0 + threadIdx.x;
+            if (tb + w < t1) {
+                const int64_t e = a.tn_e[tb + w];
+                const int g = a.near_group[e];
+                const int p0 = a.gstart[g], p1 = a.gend[g];
                 real ox, oy, oz;
                 if (sizeof(real) == sizeof(float)) {
                     const float4 o = a.near4[e];
@@ -369,47 +369,55 @@ __global__ void __launch_bounds__(256) k_p2p_T(TArgs a, const typename V4<real>:
                     oy = (real)(a.ncenter[3 * nd + 1] - a.gcenter[3 * g + 1]);
                     oz = (real)(a.ncenter[3 * nd + 2] - a.gcenter[3 * g + 2]);
                 }
-                v4 X = v4();
-                real sy = 0;
-                int pan = -1;
+                if (lane == 0) {
+                    const int gb = a.gbody[g];
+                    sFirst[w] = p0;
+                    sCnt[w] = p1 - p0;
+                    sLap[w] = nb == gb && a.lap_body[gb];
+                }
+                const int p = p0 + lane;
                 if (p < p1) {
                     const v4 xr = xrel[p];
+                    v4 X;
                     X.x = xr.x - ox;  // target relative to the leaf centre, as the forward r0
                     X.y = xr.y - oy;
                     X.z = xr.z - oz;
                     X.w = (real)sT[2 * p];
-                    sy = (real)sT[2 * p + 1];
-                    pan = (int)p;
+                    sX[w][lane] = X;
+                    sYw[w][lane] = (real)sT[2 * p + 1];
                 }
-                sX[threadIdx.x] = X;
-                sYw[threadIdx.x] = sy;
-                sPan[threadIdx.x] = pan;
             }
             __syncthreads();
             if (!on) continue;
-            real t0 = 0, t1 = 0, t2 = 0, t3 = 0;
-            for (int i = 0; i < 32; ++i) {
-                const v4 X = sX[i];
-                if (sPan[i] < 0) continue;
-                const real dx = X.x - A.x, dy = X.y - A.y, dz = X.z - A.z;  // x_i - y_s
-                const real r2 = dx * dx + dy * dy + dz * dz;
-                real ri = rsqrt_fast(r2);
-                ri = (r2 > real(0) && sPan[i] != panel) ? ri : real(0);
-                const real ri3 = ri * ri * ri;
-                const real pd = n.x * dx + n.y * dy + n.z * dz;  // n_j . (x_i - y_s)
-                if (lap) {
-                    t0 += X.w * ri;
-                    t1 += X.w * pd * ri3;
+            const int ne = (int)min((int64_t)8, t1 - tb);
+            for (int u = 0; u < ne; ++u) {
+                const int cnt = sCnt[u], own = panel - sFirst[u];
+                const bool lap = sLap[u];
+                real s0 = 0, s1 = 0, s2 = 0, s3 = 0;
+#pragma unroll 4
+                for (int i = 0; i < cnt; ++i) {
+                    const v4 X = sX[u][i];
+                    const real dx = X.x - A.x, dy = X.y - A.y, dz = X.z - A.z;  // x_i - y_s
+                    const real r2 = dx * dx + dy * dy + dz * dz;
+                    real ri = rsqrt_fast(r2);
+                    ri = (r2 > real(0) && i != own) ? ri : real(0);
+                    const real ri3 = ri * ri * ri;
+                    const real pd = n.x * dx + n.y * dy + n.z * dz;  // n_j . (x_i - y_s)
+                    if (lap) {
+                        s0 += X.w * ri;
+                        s1 += X.w * pd * ri3;
+                    }
+                    const real r = r2 * ri;
+                    const real ex = exp2_(nkl * r);
+                    const real sy = sYw[u][i];
+                    s2 += sy * ex * ri;
+                    s3 += sy * (kappa * r + real(1)) * ex * pd * ri3;
                 }
-                const real r = r2 * ri;
-                const real ex = exp2_(nkl * r);
-                t2 += sYw[i] * ex * ri;
-                t3 += sYw[i] * (kappa * r + real(1)) * ex * pd * ri3;
+                kadd(acc[0], cmp[0], s0);
+                kadd(acc[1], cmp[1], s1);
+                kadd(acc[2], cmp[2], s2);
+                kadd(acc[3], cmp[3], s3);
             }
-            kadd(acc[0], cmp[0], t0);
-            kadd(acc[1], cmp[1], t1);
-            kadd(acc[2], cmp[2], t2);
-            kadd(acc[3], cmp[3], t3);
         }
         if (on)
             for (int k = 0; k < 4; ++k) a.out[4 * q + k] = (double)acc[k] + (double)cmp[k];
