@@ -613,6 +613,49 @@ __device__ __forceinline__ void panel_sums(const PanelS<real>& q, real X, real Y
         const real p0 = norm_(fma_(q.uz, dz, fma_(q.uy, dy, mul_(q.ux, dx))));
         const real p1 = norm_(fma_(q.vz, dz, fma_(q.vy, dy, mul_(q.vx, dx))));
         const real p2 = -norm_(add_(p0, p1));
+        if constexpr (std::is_same<real, float>::value && K == 7) {
+            // the two orbits side by side as packed halves: with the stage's loop
+            // kept rolled (63 registers, 32 warps an SM) the issue slots no longer
+            // bound the sums: product of 2 x 20480 panels 202 -> 193 us, of 2 x
+            // 81920 2143 -> 2061 us (packed but unrolled by the compiler: 199, 2106)
+            const f2 a2{ra[0], ra[1]}, k2{kappa, kappa}, n2{nkl, nkl}, o2{1.f, 1.f};
+            f2 tV, tK, tW, tM;
+            auto both = [&](const float p, const float g, bool first) {
+                const f2 r2 = fma_(a2, fma_(a2, f2{g, g}, f2{p, p}), f2{D2, D2});
+                const f2 ri{rsqrt_abs(r2.a), rsqrt_abs(r2.b)};
+                const f2 i2 = mul_(ri, ri);
+                const f2 r = mul_(r2, ri);
+                const f2 x = mul_(n2, r);
+                const f2 e = mul_(f2{exp2_(x.a), exp2_(x.b)}, ri);
+                const f2 gg = fma_(k2, r, o2);
+                const f2 e2 = mul_(e, i2);
+                if (first) {
+                    if (LAP) {
+                        tV = ri;
+                        tK = mul_(ri, i2);
+                    }
+                    tW = e;
+                    tM = mul_(e2, gg);
+                } else {
+                    if (LAP) {
+                        tV = add_(tV, ri);
+                        tK = fma_(ri, i2, tK);
+                    }
+                    tW = add_(tW, e);
+                    tM = fma_(e2, gg, tM);
+                }
+            };
+            both(p0, q.g0, true);
+            both(p1, q.g1, false);
+            both(p2, q.g2, false);
+            if (LAP) {
+                VL = fmaf(rw[1], tV.a, fmaf(rw[2], tV.b, VL));
+                KL = fmaf(rw[1], tK.a, fmaf(rw[2], tK.b, KL));
+            }
+            VY = fmaf(rw[1], tW.a, fmaf(rw[2], tW.b, VY));
+            KY = fmaf(rw[1], tM.a, fmaf(rw[2], tM.b, KY));
+            return;
+        }
 #pragma unroll
         for (int o = 0; o < (K == 7 ? 2 : 1); ++o) {
             real sV, sK, sW, sM;
@@ -773,6 +816,7 @@ __global__ void __launch_bounds__(NW * 32) k_p2p(EvalArgs a, const typename V4<t
                 for (int k0 = 0; k0 < cnt; k0 += P2P_RUN) {
                     real sumL = 0, sumY = 0;
                     const int k1 = min(cnt, k0 + P2P_RUN);
+#pragma unroll 1
                     for (int k = k0; k < k1; ++k)
                         p2p_panel<real, K, decltype(LAPc)::value, decltype(OWNc)::value>(
                             sP[w][k], k == own, X, Y, Z, kappa, nkl, ra, rw, sumL, sumY);
