@@ -67,24 +67,34 @@ def workload_bodies(level=5):
 
 
 # ------------------------------------------------------------------ flops
-def p2p_flops(laplace):
-    """FP32 operations per target x source-point pair of the P2P tile loop
-    (rsqrt and exp counted as one each): difference 3, r^2 5, rsqrt 1, n.d 5,
-    1/r^2 and t 2, Yukawa 10, Laplace 3."""
-    return 26 + (3 if laplace else 0)
+def p2p_flops(laplace, K=PARAMS["K"]):
+    """FP32 operations per target x source-point pair of the P2P sums, which go
+    panel by panel (rsqrt and exp counted as one each): per panel difference
+    3, |d|^2 5, n.d 5, the vertex products 11, the weights of the rule's orbits
+    and the densities; per point 12 (Yukawa), 4 more for the squared distance
+    of an orbit point, 3 for Laplace."""
+    orbits = {1: 0, 3: 1, 4: 1, 7: 2}[K]
+    centre = 0 if K == 3 else 1
+    weights = centre + 2 * orbits  # per sum (two a kernel)
+    panel = 13 + (11 if orbits else 0) + 12 * K + 4 * 3 * orbits + 2 * weights + 5
+    if laplace:
+        panel += 3 * K + 2 * weights + 5
+    return panel / K
 
 
 def m2p_flops(P, laplace):
     """Operations per (target, far node) of the far-field evaluation as the
-    kernel runs it (far_eval: monomials of S = R/r^2 in nested order, one
-    product each, summed per degree against the node's coefficients), counted
-    term by term: setup 22 (R 3, r^2 5, rsqrt 1, 1/r^2 1, S 3, r 1, x 1, x^2 1,
-    g_1 1, exp 1, prefactor 2, final product 2), T - 1 monomial products,
-    2 per Yukawa multiply-add, the radial factors g_p (3 each for p >= 2) and
-    their multiply-adds (2 each for p >= 1); Laplace adds 2 per term and 1."""
-    T = (P + 1) * (P + 2) * (P + 3) // 6
-    yuk = 22 + (T - 1) + 2 * T + 2 * min(P, 1) + 5 * max(P - 1, 0)
-    return yuk + ((2 * T + 1) if laplace else 0)
+    kernel runs it (far_eval: harmonic basis, (P + 1)^2 coefficients a kernel),
+    counted term by term: setup 18 (R 3, r^2 5, rsqrt 1, unit vector 3, r 1,
+    exponent 1, exp 1, prefactor 1, kappa^2 1, final product 1), radial factors
+    2 + 4 (P - 1), Legendre recurrences 3 each for l >= m + 2 and their
+    products with the radial factors, 2 per coefficient, 4 per order m >= 1 and
+    6 for its powers; Laplace adds its own radial factors, products and
+    coefficients."""
+    n = (P + 1) ** 2
+    coef = 2 * n - (2 * P + 1) + P * (P + 1) // 2 + 4 * P + 1
+    yuk = 17 + (2 if P else 0) + 4 * max(P - 1, 0) + 3 * (P * (P - 1) // 2) + 6 * max(P - 1, 0) + coef
+    return yuk + (max(P - 1, 0) + coef if laplace else 0)
 
 
 def p2p_kernel_flops(info):
@@ -1278,7 +1288,7 @@ def main():
     ap.add_argument("--leaf", type=int, default=None, help="override leaf_size (parameter sweeps)")
     ap.add_argument("--P", type=int, default=None, help="override the Taylor order (parameter sweeps)")
     ap.add_argument("--theta", type=float, default=None, help="override theta (parameter sweeps)")
-    ap.add_argument("--p2p-item", type=int, default=None, help="override P2P tiles per work item (sweeps)")
+    ap.add_argument("--p2p-item", type=int, default=None, help="override the P2P work-item size, in runs of 32 points (sweeps)")
     ap.add_argument("--m2p-item", type=int, default=None, help="override far nodes per M2P work item (sweeps)")
     ap.add_argument("--precond", type=int, default=None, help="1: block-diagonal GMRES preconditioner")
     ap.add_argument("--graphs", type=int, default=None, help="0: plain launches instead of the upward-pass graph")
