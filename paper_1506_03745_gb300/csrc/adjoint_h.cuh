@@ -8,8 +8,10 @@
 // and sum_s w_s n . grad_y Phi = -A sum_k V_k sum_a n_a (k_a + 1) L_{k + e_a}
 // (k_l2p_TH).  Within a solve the near field is the stored one, read the other
 // way (k_near_T).  5380 panels, one product: gather 1.89 ms with Taylor
-// coefficients, near field 3.88 ms formed anew, nodes 0.26 ms; the whole
-// gradient 606 -> 95 ms.  (The FP32 product keeps the kernels of adjoint.cuh:
+// coefficients, 0.42 in the harmonic basis with both kernels' sums sharing the
+// recurrences (0.48 one after the other), near field 3.88 ms formed anew, 0.06
+// read, nodes 0.26 ms; the whole
+// gradient 606 -> 74 ms.  (The FP32 product keeps the kernels of adjoint.cuh:
 // what a gradient in FP32 returns is theirs to the last rounding.)
 #pragma once
 #include "adjoint.cuh"
@@ -17,20 +19,25 @@
 namespace pgb {
 
 // The harmonic basis values of one pair, s B_j for j = 0 .. n_far(P) - 1 in the
-// order of far_pos, handed to put(std::integral_constant j, value): Yukawa
-// s e^{-x} / r h_l q_{l,m} (Re, Im), else Laplace s / r r^{-l} q_{l,m} (Re, Im).
-template <typename real, int P, bool YUK, class F>
-__device__ __forceinline__ void far_basis(real Rx, real Ry, real Rz, real kappa, real s, F&& put) {
+// order of far_pos, handed to putY / putL (std::integral_constant j, value):
+// Yukawa sY e^{-x} / r h_l q_{l,m} (Re, Im) and, with LAP, Laplace
+// sL / r r^{-l} q_{l,m} (Re, Im), which share the recurrences of q.
+template <typename real, int P, bool LAP, class FY, class FL>
+__device__ __forceinline__ void far_basis(real Rx, real Ry, real Rz, real kappa, real sY, real sL, FY&& putY, FL&& putL) {
     const real r2 = Rx * Rx + Ry * Ry + Rz * Rz;
     const real ri = rsqrt_(r2);
     const real nx = Rx * ri, ny = Ry * ri, nz = Rz * ri;
-    real h[P + 1];
-    h[0] = (YUK ? exp_(-kappa * (r2 * ri)) * ri : ri) * s;
-    if constexpr (P >= 1) h[1] = YUK ? -(ri + kappa) * h[0] : ri * h[0];
+    real h[P + 1], g[P + 1];
+    h[0] = exp_(-kappa * (r2 * ri)) * ri * sY;
+    g[0] = ri * sL;
+    if constexpr (P >= 1) {
+        h[1] = -(ri + kappa) * h[0];
+        g[1] = ri * g[0];
+    }
     static_for<2, P + 1>([&](auto Lc) {
         constexpr int l = decltype(Lc)::value;
-        if constexpr (YUK) h[l] = (kappa * kappa) * h[l - 2] - (real(2 * l - 1) * ri) * h[l - 1];
-        else h[l] = ri * h[l - 1];
+        h[l] = (kappa * kappa) * h[l - 2] - (real(2 * l - 1) * ri) * h[l - 1];
+        if constexpr (LAP) g[l] = ri * g[l - 1];
     });
     real X = real(1), Y = real(0);
     static_for<0, P + 1>([&](auto M) {
@@ -44,11 +51,19 @@ __device__ __forceinline__ void far_basis(real Rx, real Ry, real Rz, real kappa,
                 q0 = q;
             }
             const real w = l > m ? h[l] * q0 : h[l];
+            const real v = !LAP ? real(0) : l > m ? g[l] * q0 : g[l];
+            constexpr std::integral_constant<int, far_pos(P, l, m, 0)> j0{};
             if constexpr (m == 0) {
-                put(std::integral_constant<int, far_pos(P, l, 0, 0)>{}, w);
+                putY(j0, w);
+                if constexpr (LAP) putL(j0, v);
             } else {
-                put(std::integral_constant<int, far_pos(P, l, m, 0)>{}, w * X);
-                put(std::integral_constant<int, far_pos(P, l, m, 1)>{}, w * Y);
+                constexpr std::integral_constant<int, far_pos(P, l, m, 1)> j1{};
+                putY(j0, w * X);
+                putY(j1, w * Y);
+                if constexpr (LAP) {
+                    putL(j0, v * X);
+                    putL(j1, v * Y);
+                }
             }
         });
         if constexpr (m == 0) {
@@ -64,22 +79,25 @@ __device__ __forceinline__ void far_basis(real Rx, real Ry, real Rz, real kappa,
 
 // Sums over the warp of one pair's basis values, added to dst (atomic: the
 // forward pairs (g, b) of one node b are spread over blocks); 32 at a time.
-template <typename real, int P, bool YUK>
-__device__ __forceinline__ void gather_basis(real Rx, real Ry, real Rz, real kappa, real s, real* dst) {
-    constexpr int NC = n_far(P);
+template <typename real, int P, bool LAP>
+__device__ __forceinline__ void gather_basis(real Rx, real Ry, real Rz, real kappa, real sY, real sL, real* dst) {
+    constexpr int NC = n_far(P), PAD = n_far_pad(P);
     const int lane = threadIdx.x & 31;
-    real v[32];
+    real v[32], u[32];
 #pragma unroll
-    for (int u = 0; u < 32; ++u) v[u] = real(0);
-    far_basis<real, P, YUK>(Rx, Ry, Rz, kappa, s, [&](auto J, real x) {
+    for (int k = 0; k < 32; ++k) v[k] = u[k] = real(0);
+    auto put = [&](real (&b)[32], real* d, auto J, real x) {
         constexpr int j = decltype(J)::value;
-        v[j & 31] = x;
+        b[j & 31] = x;
         if constexpr ((j & 31) == 31 || j == NC - 1) {
             constexpr int b0 = j & ~31;
-            const real sum = reduce_scatter32(v);
-            if (b0 + lane <= j) atomicAdd(dst + b0 + lane, sum);
+            const real sum = reduce_scatter32(b);
+            if (b0 + lane <= j) atomicAdd(d + b0 + lane, sum);
         }
-    });
+    };
+    far_basis<real, P, LAP>(
+        Rx, Ry, Rz, kappa, sY, sL, [&](auto J, real x) { put(v, dst + PAD, J, x); },
+        [&](auto J, real x) { put(u, dst, J, x); });
 }
 
 // Far gather: one block of NW warps per forward M2P work item (up to m2p_item
@@ -87,7 +105,7 @@ __device__ __forceinline__ void gather_basis(real Rx, real Ry, real Rz, real kap
 // (s_L, s_Y); per node b the harmonic values of the 32 targets are summed and
 // added to H(b) (n_far_pad(P) Laplace, then as many Yukawa).  In the Cartesian
 // basis a pair's Taylor coefficients cost 2231 operations and 84 sums per
-// kernel; here about 300 and 49.
+// kernel; here about 200 and 49, bound by FP64 operations.
 template <typename real, int P, int NW>
 __global__ void __launch_bounds__(NW * 32) k_m2p_TH(TArgs a, const typename V4<real>::t* __restrict__ xrel,
                                                     const double* __restrict__ sT, real* __restrict__ H) {
@@ -112,8 +130,8 @@ __global__ void __launch_bounds__(NW * 32) k_m2p_TH(TArgs a, const typename V4<r
         const real Rx = xr.x - (real)(a.ncenter[3 * nd] - gc0), Ry = xr.y - (real)(a.ncenter[3 * nd + 1] - gc1),
                    Rz = xr.z - (real)(a.ncenter[3 * nd + 2] - gc2);
         real* h = H + (int64_t)nd * 2 * NC;
-        gather_basis<real, P, true>(Rx, Ry, Rz, kappa, sY, h + NC);
-        if ((a.nbody[nd] == gb) && a.lap_body[gb]) gather_basis<real, P, false>(Rx, Ry, Rz, kappa, sL, h);
+        if ((a.nbody[nd] == gb) && a.lap_body[gb]) gather_basis<real, P, true>(Rx, Ry, Rz, kappa, sY, sL, h);
+        else gather_basis<real, P, false>(Rx, Ry, Rz, kappa, sY, sL, h);
     }
 }
 

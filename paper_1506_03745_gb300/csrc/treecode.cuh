@@ -106,7 +106,7 @@ __device__ __forceinline__ ds inv_int<ds>(int n) {
 }
 
 __device__ __forceinline__ float rsqrt_(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double rsqrt_(double x) { return rsqrt(x); }
+__device__ __forceinline__ double rsqrt_(double x) { return rsqrt_halley(x); }
 __device__ __forceinline__ float exp_(float x) { return __expf(x); }
 __device__ __forceinline__ double exp_(double x) { return exp(x); }
 // 2^x (the P2P loop folds log2(e) into its constant) and 1/sqrt(x) of the
@@ -566,6 +566,10 @@ struct __align__(16) PanelS {
 // instead of 14; in double-single 185 operations (320).  The squared distance
 // loses a factor |d|^2 / r^2 of relative accuracy, below ten on shape-regular
 // panels, of the order of what the FP32 coordinates leave.
+// In double-single |d|^2 and n.d are rounded once for a panel's points instead
+// of once a point, which no longer averages: a product is within 2.6e-15 to
+// 4.5e-15 of the FP64 one (1.2e-15 to 3.5e-15 point by point; one unit of a
+// pair is 3.6e-15).
 // panel_sums: V_L, sum w / r^3, V_Y and its counterpart (without n.d), and n.d.
 template <typename real, int K, bool LAP>
 __device__ __forceinline__ void panel_sums(const PanelS<real>& q, real X, real Y, real Z, real kappa, real nkl,
