@@ -370,8 +370,8 @@ int pgb_tree_export(struct pgb_ctx* ctx, int32_t* perm, int64_t* near_off, int32
 /* Diagnostic: evaluate the device's FP64 elementary functions of the
  * near-field sums at n host points x (no context; the current device, its
  * default stream, synchronous).  out (host, n x 7, row-major) receives per
- * point: the one-step and two-step Newton reciprocal square roots (valid for
- * 1e-30 < x < 1e30), the Taylor 2^x (valid for -2^30 < x <= 1020), the CUDA
+ * point: the reciprocal square root of the near-field sums and that of the
+ * corrections and energies (the same function), their 2^x (x <= 1020), the CUDA
  * library's rsqrt(x) and exp2(x) for comparison, and the double-single
  * reciprocal square root (1e-30 < x < 1e30) and 2^x (-100 < x < 127) of the
  * PGB_FP64_DS product, each converted back to a double.  PGB_EINVAL for n < 0 or a

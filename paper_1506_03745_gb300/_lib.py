@@ -359,8 +359,7 @@ def pgb_tree_export(ctx):
 
 
 def pgb_math_check(x):
-    """Device FP64 functions at the points x (host array): columns one-step
-    and two-step Newton rsqrt, Taylor exp2, library rsqrt, library exp2,
+    """Device FP64 functions at the points x (host array): columns the rsqrt of the near-field sums (twice), their exp2, library rsqrt, library exp2,
     double-single rsqrt, double-single exp2."""
     x = np.ascontiguousarray(x, dtype=np.float64)
     out = np.zeros((len(x), 7), np.float64)

@@ -43,7 +43,7 @@ __device__ __forceinline__ VkPanel vk_panel(const Geo& g, int64_t j) {
 // s_k: with d = xq - c the squared distance is |d|^2 + a (2 d.s_k + a |s_k|^2)
 // and the normal product n.d, the panel's (treecode.cuh, panel_sums).  FP64
 // operations bound these sums: ten a point and 22 a panel, against 24 a point
-// from its coordinates with two Newton steps (charge weights of 13000 panels
+// from its coordinates with two Newton steps (charge weights of 12500 panels
 // and 900 charges 3.83 -> 2.16 ms).
 template <int K>
 __device__ __forceinline__ void panel_vk(const VkPanel& q, const Rules& r, const FarRule& f, const double* xq,

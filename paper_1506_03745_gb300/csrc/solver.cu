@@ -20,7 +20,7 @@ static inline int nblk(int64_t n, int t) { return (int)std::max<int64_t>(1, (n +
 // a molecule) takes the enclosing body's charges the same way (added to the
 // row, which may hold imposed terms already).
 // COUL_LANES lanes a row share its charges (FP64 work of whole warps: one lane
-// a row leaves a molecule of 13000 panels on 100 of the multiprocessors).
+// a row leaves a molecule of 12500 panels on 100 of the multiprocessors).
 #define COUL_LANES 4
 __global__ void k_coulomb_rows(Geo g, BodyDev bd, BodyCopies cp, const double* qxyz, const double* qv, const int64_t* qoff,
                                const double* eps_in, double* b) {

@@ -621,7 +621,7 @@ __device__ __forceinline__ void panel_sums(const PanelS<real>& q, real X, real Y
             // the two orbits side by side as packed halves: with the stage's loop
             // kept rolled (63 registers, 32 warps an SM) the issue slots no longer
             // bound the sums: product of 2 x 20480 panels 202 -> 193 us, of 2 x
-            // 81920 2143 -> 2061 us (packed but unrolled by the compiler: 199, 2106)
+            // 204020 2143 -> 2061 us (packed but unrolled by the compiler: 199, 2106)
             const f2 a2{ra[0], ra[1]}, k2{kappa, kappa}, n2{nkl, nkl}, o2{1.f, 1.f};
             f2 tV, tK, tW, tM;
             auto both = [&](const float p, const float g, bool first) {
