@@ -142,7 +142,7 @@ __device__ __forceinline__ void gather_coeffs(const real (&G)[T], real s, real* 
     }
 }
 
-// Far gather: one block of NW warps per forward M2P work item (up to m2p_item
+// Far gather (FP32): one block of NW warps per forward M2P work item (up to m2p_item
 // far nodes of one target group, as k_m2p); lane = target i with weights
 // (s_L, s_Y); per node b the Yukawa (and, for a same-body dielectric pair,
 // Laplace) coefficients of the 32 targets are summed and added to Lmom(b)
@@ -161,27 +161,14 @@ __global__ void __launch_bounds__(NW * 32) k_m2p_T(TArgs a, const typename V4<re
     const bool active = p < p1;
     const v4 xr = active ? xrel[p] : xrel[p0];
     const real sL = active ? (real)sT[2 * p] : real(0), sY = active ? (real)sT[2 * p + 1] : real(0);
-    const double gc0 = a.gcenter[3 * g], gc1 = a.gcenter[3 * g + 1], gc2 = a.gcenter[3 * g + 2];
     const int gb = a.gbody[g];
     const real kappa = (real)a.kappa;
     const int64_t fb = a.far_off[g] + (it - a.fitem_off[g]) * a.m2p_item;
     const int64_t f1 = min(a.far_off[g + 1], fb + a.m2p_item);
     for (int64_t e = fb + w; e < f1; e += NW) {
-        int nd;
-        real ox, oy, oz;
-        if (sizeof(real) == sizeof(float)) {
-            const float4 q = a.far4[e];
-            nd = __float_as_int(q.w);
-            ox = (real)q.x;
-            oy = (real)q.y;
-            oz = (real)q.z;
-        } else {
-            nd = a.far_l[e];
-            ox = (real)(a.ncenter[3 * nd] - gc0);
-            oy = (real)(a.ncenter[3 * nd + 1] - gc1);
-            oz = (real)(a.ncenter[3 * nd + 2] - gc2);
-        }
-        const real Rx = xr.x - ox, Ry = xr.y - oy, Rz = xr.z - oz;
+        const float4 q = a.far4[e];
+        const int nd = __float_as_int(q.w);
+        const real Rx = xr.x - q.x, Ry = xr.y - q.y, Rz = xr.z - q.z;
         const bool lap = (a.nbody[nd] == gb) && a.lap_body[gb];
         real G[T];
         taylor_coeffs<real, P, true>(Rx, Ry, Rz, kappa, G);
