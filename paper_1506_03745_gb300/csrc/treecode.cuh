@@ -1357,10 +1357,23 @@ constexpr int UP_FLY = 4;     // panels whose point powers are staged at once (V
 __host__ __device__ constexpr int p2m_threads(int P) {
     return n_terms(P) >= 256 ? 256 : (n_terms(P) <= 64 ? 64 : (n_terms(P) + 31) & ~31);
 }
+// Its threads take a leaf's panels in p2m_shares shares: thread tid those of its
+// share p2m_share, and of each panel the moments of the multi-indices p2m_index
+// (h = 0, 1, ..), -1 where it has none: the block is whole warps, so threads are
+// left over at most orders (96 for the 84 multi-indices of order 6), and what
+// they would read lies behind the last panel's moments.
+__host__ __device__ constexpr int p2m_shares(int P) {
+    return n_terms(P) >= p2m_threads(P) ? 1 : p2m_threads(P) / n_terms(P);
+}
+__host__ __device__ constexpr int p2m_share(int P, int tid) { return p2m_shares(P) > 1 ? tid / n_terms(P) : 0; }
+__host__ __device__ constexpr int p2m_index(int P, int tid, int h) {
+    const int k = tid - p2m_share(P, tid) * n_terms(P) + h * p2m_threads(P);
+    return p2m_share(P, tid) < p2m_shares(P) && k < n_terms(P) ? k : -1;
+}
 template <typename real, int P, bool STORED>
 struct P2MShared {
     static constexpr int T = MI<P>::T, BT = p2m_threads(P);
-    static constexpr int NP = T >= BT ? 1 : BT / T;  // shares of a leaf's panels
+    static constexpr int NP = p2m_shares(P);         // shares of a leaf's panels
     real q[UP_CHUNK][5];                             // psi_L, psi_Y, phi n (all x area)
     real sum[NP][5][T];
     real pw[STORED ? 1 : UP_FLY * 7][3][P + 1];
@@ -1453,8 +1466,8 @@ __global__ void __launch_bounds__(p2m_threads(P)) k_p2m(UpArgs a, real* __restri
     extern __shared__ __align__(16) unsigned char p2m_smem[];
     SH& sh = *reinterpret_cast<SH*>(p2m_smem);
     const int tid = threadIdx.x;
-    const int part = NP > 1 ? tid / T : 0, k0 = NP > 1 ? tid - part * T : tid;
-    const bool on = part < NP;
+    const int part = p2m_share(P, tid), k0 = p2m_index(P, tid, 0);
+    const bool on = k0 >= 0;
     for (int k = tid; k < T; k += BT) {
         int x, y, z;
         decode_mi(k, x, y, z);
@@ -1497,7 +1510,7 @@ __global__ void __launch_bounds__(p2m_threads(P)) k_p2m(UpArgs a, real* __restri
                 for (int j = part; j < cnt; j += NP) {
 #pragma unroll
                     for (int h = 0; h < H; ++h)
-                        if (H == 1 || k0 + h * BT < T) add(h, v[(int64_t)j * T + h * BT], sh.q[j]);
+                        if (h == 0 || p2m_index(P, tid, h) >= 0) add(h, v[(int64_t)j * T + h * BT], sh.q[j]);
                 }
             }
         } else {
@@ -1506,11 +1519,11 @@ __global__ void __launch_bounds__(p2m_threads(P)) k_p2m(UpArgs a, real* __restri
                 __syncthreads();
                 stage_powers<real, P>(a, c0 + f, np, sh.pw);
                 __syncthreads();
-                if (part == 0)
+                if (on && part == 0)
 #pragma unroll
                     for (int h = 0; h < H; ++h) {
-                        const int k = k0 + h * BT;
-                        if (k >= T) break;
+                        const int k = p2m_index(P, tid, h);
+                        if (k < 0) break;
                         for (int j = 0; j < np; ++j)
                             add(h, panel_moment<real, P>(a, sh.pw + j * a.K, sh.kk[k][0], sh.kk[k][1], sh.kk[k][2]),
                                 sh.q[f + j]);
@@ -1522,8 +1535,8 @@ __global__ void __launch_bounds__(p2m_threads(P)) k_p2m(UpArgs a, real* __restri
     if (on)
 #pragma unroll
         for (int h = 0; h < H; ++h) {
-            const int k = k0 + h * BT;
-            if (k < T)
+            const int k = p2m_index(P, tid, h);
+            if (k >= 0)
 #pragma unroll
                 for (int c = 0; c < 5; ++c) sh.sum[part][c][k] = acc[h][c];
         }
