@@ -608,6 +608,7 @@ static void apply_vec(pgb_ctx* c, VecIn xv, VecOut yv, int precision, int mode, 
     ev.col = c->d_col;
     ev.pnode = c->d_pnode;
     ev.pbody = c->d_pbody;
+    ev.pts = c->d_y64;
     ev.rule = far_rule(c->p.K);
     ev.src_mask = 0;
     for (size_t b = 0; b < c->bodies.size(); ++b) ev.src_mask |= (unsigned long long)(ev.src_active[b] != 0) << b;
@@ -646,20 +647,18 @@ static void apply_vec(pgb_ctx* c, VecIn xv, VecOut yv, int precision, int mode, 
         ev.pg = c->d_pg64.p;
         ev.pd = c->d_pd64.p;
         if (precision == PGB_FP64_DS) {
-                c->d_pd_ds.resize(c->n_pan);
+            c->d_pd_ds.resize(c->n_pan);
             c->d_mom_ds.resize((size_t)c->n_nodes * 2 * T);
             c->d_far_ds.resize((size_t)c->n_nodes * 2 * TP);
             up.far = c->d_far_ds.p;
-            ev.pg = c->d_pg_ds.p;
-            ev.pd = c->d_pd_ds.p;
         }
     }
     const bool dsp = precision == PGB_FP64_DS;
     const int kind = f32 ? 0 : dsp ? 2 : 1;
     void* mom = f32 ? (void*)c->d_mom32.p : dsp ? (void*)c->d_mom_ds.p : (void*)c->d_mom64.p;
     up.rule = ev.rule;
-    up.pg = ev.pg;
-    up.pd = ev.pd;
+    up.pg = dsp ? (const void*)c->d_pg_ds.p : ev.pg;
+    up.pd = dsp ? (const void*)c->d_pd_ds.p : ev.pd;
     up.pmom = panel_moments(c, kind);
     if (c->near_on && kind < 2 && !ev.p2p_work && c->shard_g[0] < 0 && !nested(c) && near_ready(c, kind)) {
         ev.near_mat = c->near_mat[kind].buf.p;

@@ -154,20 +154,13 @@ constexpr bool is_ds = false;
 template <>
 constexpr bool is_ds<ds> = true;
 
-// Arithmetic of the P2P and M2P sums: fused forms in FP32 and FP64,
-// double-single without renormalisation where no cancellation follows.
+// Arithmetic of the P2P and M2P sums.
 __device__ __forceinline__ float mul_(float a, float b) { return a * b; }
 __device__ __forceinline__ double mul_(double a, double b) { return a * b; }
-__device__ __forceinline__ ds mul_(ds a, ds b) { return ds_mul_u(a, b); }
 __device__ __forceinline__ float add_(float a, float b) { return a + b; }
 __device__ __forceinline__ double add_(double a, double b) { return a + b; }
-__device__ __forceinline__ ds add_(ds a, ds b) { return ds_add_u(a, b); }
 __device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
-__device__ __forceinline__ ds fma_(ds a, ds b, ds c) { return ds_fma_u(a, b, c); }
-__device__ __forceinline__ float norm_(float a) { return a; }
-__device__ __forceinline__ double norm_(double a) { return a; }
-__device__ __forceinline__ ds norm_(ds a) { return ds_norm(a); }
 // Two FP32 values in one 64-bit register pair: Blackwell's packed FP32
 // arithmetic does both with one instruction.  The FMA pipe takes as long as
 // for two scalar ones (measured: 113-118 lane FMAs per clock and SM either
@@ -306,8 +299,9 @@ struct EvalArgs {
     const float4* col;             // per column: panel centroid - group centre (FP32), panel (int bits)
     const int32_t* pnode;          // leaf node of a panel (FP64 and double-single offsets)
     const int32_t* pbody;          // body of a panel
-    const void* pg;                // panel geometry (PanelGeo) in the kernel's arithmetic
+    const void* pg;                // panel geometry (PanelGeo) in the kernel's arithmetic (FP64 for double-single)
     const void* pd;                // panel densities x area, same arithmetic: {psiL, psiY, phi, unused}
+    const dbl4* pts;               // double-single: the far rule's points relative to their leaf's centre
     const void *near_mat = nullptr, *near_group = nullptr;  // stored near field (solves), nullptr: formed
     FarRule rule;
     unsigned long long src_mask;   // bit b: src_active[b]
@@ -533,11 +527,9 @@ __device__ __forceinline__ real exp2_scaled(real s, real r) {
     return exp2_(mul_(s, r));
 }
 // 1/sqrt of a squared distance formed with a cancellation: a value rounded
-// below zero is taken by its magnitude (FP32; the others keep 50 bits more
-// than the distances that occur)
+// below zero is taken by its magnitude (FP32; FP64 keeps 29 bits more)
 __device__ __forceinline__ float rsqrt_abs(float x) { return rsqrt_fast(fabsf(x)); }
 __device__ __forceinline__ double rsqrt_abs(double x) { return rsqrt_fast(x); }
-__device__ __forceinline__ ds rsqrt_abs(ds x) { return ds_rsqrt(x); }
 
 // One panel staged for the P2P sums: the centroid relative to the group's
 // centre (PanelGeo holds it relative to the leaf's), 2 (v_0 - c), 2 (v_1 - c),
@@ -563,20 +555,17 @@ struct __align__(16) PanelS {
 // The densities and the normal product are met once per panel.  In FP32 a
 // point costs 15 FMA-pipe operations with the panel's share (19 point by
 // point) and 2 MUFU (16 cycles a warp), and a panel five 16-byte shared loads
-// instead of 14; in double-single 185 operations (320).  The squared distance
+// instead of 14.  The squared distance
 // loses a factor |d|^2 / r^2 of relative accuracy, below ten on shape-regular
-// panels, of the order of what the FP32 coordinates leave.
-// In double-single |d|^2 and n.d are rounded once for a panel's points instead
-// of once a point, which no longer averages: a product is within 2.6e-15 to
-// 4.5e-15 of the FP64 one (1.2e-15 to 3.5e-15 point by point; one unit of a
-// pair is 3.6e-15).
+// panels, of the order of what the FP32 coordinates leave.  (Double-single
+// sums point by point: p2p_ds.cuh.)
 // panel_sums: V_L, sum w / r^3, V_Y and its counterpart (without n.d), and n.d.
 template <typename real, int K, bool LAP>
 __device__ __forceinline__ void panel_sums(const PanelS<real>& q, real X, real Y, real Z, real kappa, real nkl,
                                            const real (&ra)[2], const real (&rw)[3], real& VL, real& KL, real& VY,
                                            real& KY, real& h) {
     const real dx = X - q.cx, dy = Y - q.cy, dz = Z - q.cz;
-    const real D2 = norm_(fma_(dz, dz, fma_(dy, dy, mul_(dx, dx))));
+    const real D2 = fma_(dz, dz, fma_(dy, dy, mul_(dx, dx)));
     h = fma_(q.nz, dz, fma_(q.ny, dy, mul_(q.nx, dx)));
     const real one = real(1);
     VL = KL = VY = KY = real(0);
@@ -614,9 +603,9 @@ __device__ __forceinline__ void panel_sums(const PanelS<real>& q, real X, real Y
         KY = mul_(rw[0], sM);
     }
     if (K >= 3) {
-        const real p0 = norm_(fma_(q.uz, dz, fma_(q.uy, dy, mul_(q.ux, dx))));
-        const real p1 = norm_(fma_(q.vz, dz, fma_(q.vy, dy, mul_(q.vx, dx))));
-        const real p2 = -norm_(add_(p0, p1));
+        const real p0 = fma_(q.uz, dz, fma_(q.uy, dy, mul_(q.ux, dx)));
+        const real p1 = fma_(q.vz, dz, fma_(q.vy, dy, mul_(q.vx, dx)));
+        const real p2 = -add_(p0, p1);
         if constexpr (std::is_same<real, float>::value && K == 7) {
             // the two orbits side by side as packed halves: with the stage's loop
             // kept rolled (63 registers, 32 warps an SM) the issue slots no longer
@@ -663,9 +652,9 @@ __device__ __forceinline__ void panel_sums(const PanelS<real>& q, real X, real Y
 #pragma unroll
         for (int o = 0; o < (K == 7 ? 2 : 1); ++o) {
             real sV, sK, sW, sM;
-            point(norm_(fma_(ra[o], fma_(ra[o], q.g0, p0), D2)), sV, sK, sW, sM, true);
-            point(norm_(fma_(ra[o], fma_(ra[o], q.g1, p1), D2)), sV, sK, sW, sM, false);
-            point(norm_(fma_(ra[o], fma_(ra[o], q.g2, p2), D2)), sV, sK, sW, sM, false);
+            point(fma_(ra[o], fma_(ra[o], q.g0, p0), D2), sV, sK, sW, sM, true);
+            point(fma_(ra[o], fma_(ra[o], q.g1, p1), D2), sV, sK, sW, sM, false);
+            point(fma_(ra[o], fma_(ra[o], q.g2, p2), D2), sV, sK, sW, sM, false);
             if (LAP) {
                 VL = fma_(rw[1 + o], sV, VL);
                 KL = fma_(rw[1 + o], sK, KL);
@@ -709,8 +698,8 @@ __device__ __forceinline__ void store_item(real (*red)[4][32], int w, int lane, 
 }
 
 // Centroid of a column's panel relative to the group's centre: in FP32 from the
-// column (one rounding of the FP64 difference), otherwise the centroid
-// relative to its leaf's centre plus the FP64 difference of the centres.
+// column (one rounding of the FP64 difference), in FP64 the centroid
+// relative to its leaf's centre plus the difference of the centres.
 template <typename real>
 __device__ __forceinline__ void col_centroid(const EvalArgs& a, const float4& c, int j, int64_t g,
                                              const real* __restrict__ v, real& x, real& y, real& z) {
@@ -759,14 +748,13 @@ __device__ __forceinline__ void stage_panel(const EvalArgs& a, const float4& c, 
 // share a stage, so a warp's steps are full whatever the leaf sizes.  The
 // item's partial sums go to Up.
 template <typename real, int K, int NW>
-__global__ void __launch_bounds__(NW * 32) k_p2p(EvalArgs a, const typename V4<typename Store<real>::S>::t* __restrict__ xrel) {
-    using S = typename Store<real>::S;  // storage type of the targets
+__global__ void __launch_bounds__(NW * 32) k_p2p(EvalArgs a, const typename V4<real>::t* __restrict__ xrel) {
     __shared__ __align__(16) PanelS<real> sP[NW][32];
     __shared__ real red[NW][4][32];
     __shared__ int64_t s_item;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned long long dm = body_mask(a.bmask), act = a.src_mask & dm;
-    const real kappa = to_c<real>((S)a.kappa);
+    const real kappa = (real)a.kappa;
     const real nkl = exp_scale(kappa);
     const real ra[2] = {from_dbl<real>(a.rule.a[0]), from_dbl<real>(a.rule.a[1])};
     const real rw[3] = {from_dbl<real>(a.rule.w[0]), from_dbl<real>(a.rule.w[1]), from_dbl<real>(a.rule.w[2])};
@@ -777,8 +765,8 @@ __global__ void __launch_bounds__(NW * 32) k_p2p(EvalArgs a, const typename V4<t
         if (!(((a.tgt_mask & dm) >> gb) & 1ull) || g < a.g_lo || g >= a.g_hi) continue;  // rows not used (block-uniform)
         const int p0 = a.gstart[g], p1 = a.gend[g];
         const int p = p0 + lane;
-        const typename V4<S>::t xr = xrel[p < p1 ? p : p0];
-        const real X = to_c<real>(xr.x), Y = to_c<real>(xr.y), Z = to_c<real>(xr.z);
+        const typename V4<real>::t xr = xrel[p < p1 ? p : p0];
+        const real X = xr.x, Y = xr.y, Z = xr.z;
         const bool glap = a.lap_body[gb];
         real UL = 0, cL = 0, UY = 0, cY = 0;
         // the item's columns, then this warp's
@@ -1041,14 +1029,13 @@ void launch_near_build(const EvalArgs& ev, int K, const void* ng, const void* xr
 template <typename real>
 void launch_p2p(const EvalArgs& ev, int K, const void* xrel, cudaStream_t s) {
     constexpr int NW = 8;  // warps per block
-    using x4 = typename V4<typename Store<real>::S>::t;
+    using x4 = typename V4<real>::t;
     if (ev.n_pitems <= 0) return;
-    if constexpr (!is_ds<real>)
-        if (ev.near_mat) {
-            k_near<real, NW><<<(unsigned)ev.n_pitems, NW * 32, 0, s>>>(ev, (const NearGroup*)ev.near_group,
-                                                                       (const real*)ev.near_mat);
-            return;
-        }
+    if (ev.near_mat) {
+        k_near<real, NW><<<(unsigned)ev.n_pitems, NW * 32, 0, s>>>(ev, (const NearGroup*)ev.near_group,
+                                                                   (const real*)ev.near_mat);
+        return;
+    }
     const unsigned grid = (unsigned)(ev.p2p_work ? ev.persist_blocks : ev.n_pitems);
     switch (K) {
         case 1: k_p2p<real, 1, NW><<<grid, NW * 32, 0, s>>>(ev, (const x4*)xrel); break;

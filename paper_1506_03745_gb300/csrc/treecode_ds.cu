@@ -1,8 +1,8 @@
 // Double-single kernels of the FP64-class product (upward pass, far-field
 // coefficients, P2P, M2P): they read the panel geometry and moments split
-// once per geometry, the densities split once per product and the FP64 target
-// offsets, and compute
-// in double-single on the FP32 pipe.
+// once per geometry, the densities split once per product (P2P: the FP64
+// points and densities, split as they are staged) and the FP64 target offsets,
+// and compute in double-single on the FP32 pipe.
 #include "treecode_ds_inst.cuh"
 
 namespace pgb {

@@ -4,7 +4,7 @@
 #pragma once
 #include <algorithm>
 
-#include "treecode.cuh"
+#include "p2p_ds.cuh"
 
 namespace pgb {
 
@@ -15,7 +15,7 @@ inline void launch_ds(int stage, const UpArgs& up, const EvalArgs& ev, const voi
     // double-single on the FP32 pipe
     if (stage == PGB_STAGE_UPWARD) launch_upward<ds, P>(up, mom, s);
     if (stage == STAGE_PANEL_MOMENTS) launch_panel_moments<ds, P>(up, ev.n_pan, mom, s);
-    if (stage == PGB_STAGE_P2P) launch_p2p<ds>(ev, ev.K, xrel, s);
+    if (stage == PGB_STAGE_P2P) launch_p2p_ds(ev, ev.K, xrel, s);
     if (stage == PGB_STAGE_M2P) launch_m2p<ds, P>(ev, xrel, far, s);
 }
 
