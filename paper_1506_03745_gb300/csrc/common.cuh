@@ -33,6 +33,18 @@ __device__ __forceinline__ void rigid(const double* P, const double* v, double* 
         out[a] = dadd(dadd(dadd(dmul(P[3 * a + 0], v[0]), dmul(P[3 * a + 1], v[1])), dmul(P[3 * a + 2], v[2])), P[9 + a]);
 }
 
+// A long thin panel, whose points are summed one by one (treecode.cuh,
+// point_sums): its farthest vertex lies more than sqrt(2 area) from the centroid.
+// 0.88 of sqrt(area) on an equilateral triangle and 1.05 on a right isosceles
+// one; sqrt(2) from an aspect ratio (longest edge over the height on it) of 2.3
+// with the apex over one end to 4 over the middle.  Meshes of spheres, smooth
+// molecules and boxes have none; where there are some, they cost what every
+// panel did before the sums went panel by panel.  g: the squared distances of
+// the vertices.
+__host__ __device__ __forceinline__ bool is_sliver(const double (&g)[3], double area) {
+    return g[0] > 2.0 * area || g[1] > 2.0 * area || g[2] > 2.0 * area;
+}
+
 // FP64 reciprocal square root to FP64 rounding: the SFU's estimate from the
 // upper half of x (relative error d below 2^-20) refined by one step of
 // Halley's iteration, y <- y + y e (1/2 + 3/8 e) with e = 1 - x y^2, which

@@ -16,6 +16,7 @@ namespace pgb {
 // g_k = |s_k|^2.
 struct VkPanel {
     double c[3], n[3], u[3], v[3], g[3], A;
+    bool sliver;
 };
 __device__ __forceinline__ VkPanel vk_panel(const Geo& g, int64_t j) {
     VkPanel q;
@@ -35,6 +36,7 @@ __device__ __forceinline__ VkPanel vk_panel(const Geo& g, int64_t j) {
         q.u[a] = 2.0 * s[0];
         q.v[a] = 2.0 * s[1];
     }
+    q.sliver = is_sliver(q.g, q.A);
     return q;
 }
 
@@ -42,6 +44,8 @@ __device__ __forceinline__ VkPanel vk_panel(const Geo& g, int64_t j) {
 // rule when |xq - c| < 2 L, else the far rule by its orbits, y = c - 3 alpha
 // s_k: with d = xq - c the squared distance is |d|^2 + a (2 d.s_k + a |s_k|^2)
 // and the normal product n.d, the panel's (treecode.cuh, panel_sums).  FP64
+// On a sliver every point has its own offset and normal product (point_sums
+// there).  FP64
 // operations bound these sums: ten a point and 22 a panel, against 24 a point
 // from its coordinates with two Newton steps (charge weights of 12500 panels
 // and 900 charges 3.83 -> 2.16 ms).
@@ -53,6 +57,22 @@ __device__ __forceinline__ void panel_vk(const VkPanel& q, const Rules& r, const
     const double h = q.n[0] * dx + q.n[1] * dy + q.n[2] * dz;
     vl = 0;
     kl = 0;
+    if (q.sliver) {
+        const bool near = d2 < 8.0 * q.A;
+        const int M = near ? r.Kn : K;
+#pragma unroll 1
+        for (int m = 0; m < M; ++m) {
+            const double* mu = near ? r.mun[m] : r.mu[m];
+            const double b0 = 0.5 * (mu[0] - mu[2]), b1 = 0.5 * (mu[1] - mu[2]);
+            const double ex = dx - (b0 * q.u[0] + b1 * q.v[0]), ey = dy - (b0 * q.u[1] + b1 * q.v[1]),
+                         ez = dz - (b0 * q.u[2] + b1 * q.v[2]);
+            const double ri = rsqrt_halley(ex * ex + ey * ey + ez * ez);
+            const double w = (near ? r.wn[m] : r.w[m]) * q.A * ri;
+            vl += w;
+            kl += w * (ri * ri) * (q.n[0] * ex + q.n[1] * ey + q.n[2] * ez);
+        }
+        return;
+    }
     if (d2 < 8.0 * q.A) {
         for (int m = 0; m < r.Kn; ++m) {
             // (mu_2 = -mu_0 - mu_1 up to rounding, s_2 = -s_0 - s_1)
@@ -127,20 +147,24 @@ __global__ void k_charge_weights_1t(Geo g, BodyDev bd, BodyCopies cp, Rules r, F
     const int b = g.pbody[j];
     if (cp.of[b] != b) return;  // k_copy_weights
     const VkPanel q = vk_panel(g, j);
-    double sv[2] = {0, 0}, sk[2] = {0, 0};
+    dbl4 v{0, 0, 0, 0};
+#pragma unroll 1
     for (int side = 0; side < 2; ++side) {
         const int src = side == 0 ? (bd.kind[b] == PGB_DIELECTRIC ? b : -1) : bd.parent[b];
         if (src < 0) continue;
+        double sv = 0, sk = 0;
         for (int64_t k = qoff[src]; k < qoff[src + 1]; ++k) {
             const double xq[3] = {qxyz[3 * k], qxyz[3 * k + 1], qxyz[3 * k + 2]};
             double vl, kl;
             panel_vk<K>(q, r, f, xq, vl, kl);
-            sv[side] += qv[k] * vl;
-            sk[side] += qv[k] * kl;
+            sv += qv[k] * vl;
+            sk += qv[k] * kl;
         }
+        if (side == 0) v.x = sv, v.y = sk;
+        else v.z = sv, v.w = sk;
     }
-    w[j] = dbl4{sv[0], sk[0], sv[1], sk[1]};
-    if (worig) worig[g.perm[j]] = w[j];
+    w[j] = v;
+    if (worig) worig[g.perm[j]] = v;
 }
 
 template <int K>
@@ -152,24 +176,25 @@ __global__ void k_charge_weights(Geo g, BodyDev bd, BodyCopies cp, Rules r, FarR
     const int b = g.pbody[j];
     if (cp.of[b] != b) return;  // k_copy_weights
     const VkPanel q = vk_panel(g, j);
-    double sv[2] = {0, 0}, sk[2] = {0, 0};
+    dbl4 v{0, 0, 0, 0};
+#pragma unroll 1
     for (int side = 0; side < 2; ++side) {
         const int src = side == 0 ? (bd.kind[b] == PGB_DIELECTRIC ? b : -1) : bd.parent[b];
         if (src < 0) continue;
+        double sv = 0, sk = 0;
         for (int64_t k = qoff[src] + lane; k < qoff[src + 1]; k += 32) {
             const double xq[3] = {qxyz[3 * k], qxyz[3 * k + 1], qxyz[3 * k + 2]};
             double vl, kl;
             panel_vk<K>(q, r, f, xq, vl, kl);
-            sv[side] += qv[k] * vl;
-            sk[side] += qv[k] * kl;
+            sv += qv[k] * vl;
+            sk += qv[k] * kl;
         }
-    }
-    for (int side = 0; side < 2; ++side) {
-        sv[side] = warp_sum(sv[side]);
-        sk[side] = warp_sum(sk[side]);
+        sv = warp_sum(sv);
+        sk = warp_sum(sk);
+        if (side == 0) v.x = sv, v.y = sk;
+        else v.z = sv, v.w = sk;
     }
     if (lane == 0) {
-        const dbl4 v{sv[0], sk[0], sv[1], sk[1]};
         w[j] = v;
         if (worig) worig[g.perm[j]] = v;
     }

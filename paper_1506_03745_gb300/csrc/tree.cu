@@ -856,10 +856,10 @@ __global__ void k_rel_sources(const int32_t* pan_leaf, const int32_t* leaf_node,
 
 // Panel geometry of the P2P kernels, 16 values per panel relative to its leaf
 // centre (PanelGeo in treecode.cuh): the centroid c, the vectors 2 (v_0 - c)
-// and 2 (v_1 - c), the normal, and g_k = |v_k - c|^2; in FP32, FP64 and split
-// into double-single.
+// and 2 (v_1 - c), the normal, g_k = |v_k - c|^2, and whether it is a sliver; in
+// FP32, FP64 and split into double-single.
 __global__ void k_panel_geo(const int32_t* pan_leaf, const int32_t* leaf_node, const double* ncen, int64_t n,
-                            const double* V, const double* C, const double* Nn, int32_t* pnode, float* g32,
+                            const double* V, const double* C, const double* Nn, const double* A, int32_t* pnode, float* g32,
                             double* g64, ds* gds) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -880,7 +880,7 @@ __global__ void k_panel_geo(const int32_t* pan_leaf, const int32_t* leaf_node, c
         o[12 + a] = Nn[3 * i + a];
         o[3 + 4 * a] = gk[a];
     }
-    o[15] = 0.0;
+    o[15] = is_sliver(gk, A[i]) ? 1.0 : 0.0;
     for (int q = 0; q < 16; ++q) {
         g32[16 * i + q] = (float)o[q];
         g64[16 * i + q] = o[q];
@@ -989,7 +989,7 @@ void build_geometry(pgb_ctx* c) {
     c->d_pg64.resize(16 * n);
     c->d_pg_ds.resize(16 * n);
     k_panel_geo<<<nblk(n, 128), 128, 0, s>>>(c->d_pan_leaf, c->d_leaf_node, c->d_node_center, n, c->d_v, c->d_c,
-                                             c->d_n, c->d_pnode, c->d_pg32, c->d_pg64, (ds*)c->d_pg_ds.p);
+                                             c->d_n, c->d_A, c->d_pnode, c->d_pg32, c->d_pg64, (ds*)c->d_pg_ds.p);
     PGB_CUDA(cudaGetLastError());
     PGB_CUDA(cudaStreamSynchronize(s));
 }

@@ -535,15 +535,54 @@ __device__ __forceinline__ double rsqrt_abs(double x) { return rsqrt_fast(x); }
 // centre (PanelGeo holds it relative to the leaf's), 2 (v_0 - c), 2 (v_1 - c),
 // the unit normal, g_k = |v_k - c|^2, and the densities times the area:
 // {psi_L, psi_Y, phi of the Laplace pair, phi}; the Laplace two are zero
-// unless the panel and the group share a dielectric body.
+// unless the panel and the group share a dielectric body.  sliver: not zero for
+// a long thin panel (is_sliver).
 template <typename real>
 struct __align__(16) PanelS {
     real cx, cy, cz, g0;
     real ux, uy, uz, g1;
     real vx, vy, vz, g2;
-    real nx, ny, nz, qL;
-    real qY, pL, pY, pad;
+    real nx, ny, nz, sliver;
+    real qL, qY, pL, pY;
 };
+
+// The sums of panel_sums point by point, for slivers: every point's own offset
+// e = d + a s_k, squared distance and normal product n.e (h is 1 then), 19
+// FMA-pipe operations a point.  For a triangle of 10 by 0.05 and targets 0.01
+// from its outer points the panel form is off by up to 3e-2 in FP32 and 9e-11 in
+// FP64, this by what the coordinates leave, 7e-4 and 3e-12.  A stage of columns
+// without a sliver does not ask for one: asking panel by panel cost the FP32
+// product 4 %.
+template <typename real, int K, bool LAP>
+__device__ __forceinline__ void point_sums(const PanelS<real>& q, real X, real Y, real Z, real kappa, real nkl,
+                                           const real (&ra)[2], const real (&rw)[3], real& VL, real& KL, real& VY,
+                                           real& KY) {
+    const real dx = X - q.cx, dy = Y - q.cy, dz = Z - q.cz;
+    VL = KL = VY = KY = real(0);
+#pragma unroll 1
+    for (int m = K == 3 ? 1 : 0; m < (K == 3 ? 4 : K); ++m) {
+        const int k = m > 3 ? m - 3 : m;  // vertex 1..3 of the orbit, 0: the centroid
+        const real b = k == 0 ? real(0) : real(0.5) * (m > 3 ? ra[1] : ra[0]);
+        const real w = m == 0 ? rw[0] : (m > 3 ? rw[2] : rw[1]);
+        // b times 2 s_k; the third vertex's is minus the others' sum
+        const real ex = fma_(b, k == 1 ? q.ux : (k == 2 ? q.vx : -(q.ux + q.vx)), dx);
+        const real ey = fma_(b, k == 1 ? q.uy : (k == 2 ? q.vy : -(q.uy + q.vy)), dy);
+        const real ez = fma_(b, k == 1 ? q.uz : (k == 2 ? q.vz : -(q.uz + q.vz)), dz);
+        const real r2 = fma_(ez, ez, fma_(ey, ey, mul_(ex, ex)));
+        const real h = fma_(q.nz, ez, fma_(q.ny, ey, mul_(q.nx, ex)));
+        const real ri = rsqrt_abs(r2);
+        const real t = mul_(h, mul_(ri, ri));
+        const real r = mul_(r2, ri);
+        const real e = mul_(w, mul_(exp2_scaled(nkl, r), ri));
+        if (LAP) {
+            const real v = mul_(w, ri);
+            VL = add_(VL, v);
+            KL = fma_(v, t, KL);
+        }
+        VY = add_(VY, e);
+        KY = fma_(mul_(e, fma_(kappa, r, real(1))), t, KY);
+    }
+}
 
 // Sums over the far rule's points of one panel for one target at X (relative
 // to the group's centre).  The rule's points are c and c - 3 alpha s_k, s_k =
@@ -557,13 +596,21 @@ struct __align__(16) PanelS {
 // point) and 2 MUFU (16 cycles a warp), and a panel five 16-byte shared loads
 // instead of 14.  The squared distance
 // loses a factor |d|^2 / r^2 of relative accuracy, below ten on shape-regular
-// panels, of the order of what the FP32 coordinates leave.  (Double-single
-// sums point by point: p2p_ds.cuh.)
+// panels, of the order of what the FP32 coordinates leave, and n.d rounds at
+// the size of d instead of X - y; on slivers, whose points come close to targets
+// far from the centroid, both show (point_sums).  (Double-single sums point by
+// point throughout: p2p_ds.cuh.)
 // panel_sums: V_L, sum w / r^3, V_Y and its counterpart (without n.d), and n.d.
-template <typename real, int K, bool LAP>
+// SLIVER: the panel may be one.
+template <typename real, int K, bool LAP, bool SLIVER>
 __device__ __forceinline__ void panel_sums(const PanelS<real>& q, real X, real Y, real Z, real kappa, real nkl,
                                            const real (&ra)[2], const real (&rw)[3], real& VL, real& KL, real& VY,
                                            real& KY, real& h) {
+    if (SLIVER && q.sliver != real(0)) {  // (all lanes alike)
+        point_sums<real, K, LAP>(q, X, Y, Z, kappa, nkl, ra, rw, VL, KL, VY, KY);
+        h = real(1);
+        return;
+    }
     const real dx = X - q.cx, dy = Y - q.cy, dz = Z - q.cz;
     const real D2 = fma_(dz, dz, fma_(dy, dy, mul_(dx, dx)));
     h = fma_(q.nz, dz, fma_(q.ny, dy, mul_(q.nx, dx)));
@@ -664,11 +711,11 @@ __device__ __forceinline__ void panel_sums(const PanelS<real>& q, real X, real Y
         }
     }
 }
-template <typename real, int K, bool LAP, bool OWN>
+template <typename real, int K, bool LAP, bool OWN, bool SLIVER>
 __device__ __forceinline__ void p2p_panel(const PanelS<real>& q, bool own, real X, real Y, real Z, real kappa,
                                           real nkl, const real (&ra)[2], const real (&rw)[3], real& UL, real& UY) {
     real VL, KL, VY, KY, h;
-    panel_sums<real, K, LAP>(q, X, Y, Z, kappa, nkl, ra, rw, VL, KL, VY, KY, h);
+    panel_sums<real, K, LAP, SLIVER>(q, X, Y, Z, kappa, nkl, ra, rw, VL, KL, VY, KY, h);
     if (OWN && own) VL = KL = VY = KY = real(0);  // the panel's own integral is a near-field correction
     if (LAP) UL = fma_(q.qL, VL, fma_(mul_(-q.pL, h), KL, UL));
     UY = fma_(q.qY, VY, fma_(mul_(-q.pY, h), KY, UY));
@@ -718,7 +765,7 @@ __device__ __forceinline__ void col_centroid(const EvalArgs& a, const float4& c,
 // The geometry of panel j (column c of group g) into q.
 template <typename real>
 __device__ __forceinline__ void stage_panel(const EvalArgs& a, const float4& c, int j, int64_t g, PanelS<real>& q) {
-    // the first 15 values of a staged panel, relative to the leaf
+    // the first 16 values of a staged panel, relative to the leaf
     const PanelS<real>& v = *reinterpret_cast<const PanelS<real>*>((const real*)a.pg + 16 * (int64_t)j);
     col_centroid<real>(a, c, j, g, &v.cx, q.cx, q.cy, q.cz);
     q.g0 = v.g0;
@@ -733,6 +780,7 @@ __device__ __forceinline__ void stage_panel(const EvalArgs& a, const float4& c, 
     q.nx = v.nx;
     q.ny = v.ny;
     q.nz = v.nz;
+    q.sliver = v.sliver;
 }
 
 // Panels summed plainly before they join the compensated sums: about the 32
@@ -777,7 +825,7 @@ __global__ void __launch_bounds__(NW * 32) k_p2p(EvalArgs a, const typename V4<r
         const int64_t w1 = min(b1, b0 + (w + 1) * wper);
         for (int64_t e = b0 + w * wper; e < w1; e += 32) {
             const int cnt = (int)min((int64_t)32, w1 - e);
-            bool lap = false, has_own = false;
+            bool lap = false, has_own = false, sliver = false;
             int own = -1;  // the stage's slot of this lane's own panel
             __syncwarp();
             int j = -1;
@@ -789,6 +837,7 @@ __global__ void __launch_bounds__(NW * 32) k_p2p(EvalArgs a, const typename V4<r
                 has_own = j >= p0 && j < p1;
                 PanelS<real>& q = sP[w][lane];
                 stage_panel<real>(a, c, j, g, q);
+                sliver = K >= 3 && q.sliver != real(0);
                 const bool on = (act >> b) & 1ull;  // a body without density in this product adds nothing
                 const real z = real(0);
                 q.qL = on && lap ? pd[4 * (int64_t)j] : z;
@@ -799,29 +848,34 @@ __global__ void __launch_bounds__(NW * 32) k_p2p(EvalArgs a, const typename V4<r
             }
             lap = __any_sync(0xffffffffu, lap);
             has_own = __any_sync(0xffffffffu, has_own);
+            sliver = __any_sync(0xffffffffu, sliver);
             if (has_own)
                 for (int k = 0; k < cnt; ++k)
                     if (__shfl_sync(0xffffffffu, j, k) == p) own = k;
             __syncwarp();
             // a few panels in plain sums, then into the compensated ones
-            auto sums = [&](auto LAPc, auto OWNc) {
+            auto sums = [&](auto LAPc, auto OWNc, auto SLVc) {
                 for (int k0 = 0; k0 < cnt; k0 += P2P_RUN) {
                     real sumL = 0, sumY = 0;
                     const int k1 = min(cnt, k0 + P2P_RUN);
 #pragma unroll 1
                     for (int k = k0; k < k1; ++k)
-                        p2p_panel<real, K, decltype(LAPc)::value, decltype(OWNc)::value>(
+                        p2p_panel<real, K, decltype(LAPc)::value, decltype(OWNc)::value, decltype(SLVc)::value>(
                             sP[w][k], k == own, X, Y, Z, kappa, nkl, ra, rw, sumL, sumY);
                     if (decltype(LAPc)::value) kadd(UL, cL, sumL);
                     kadd(UY, cY, sumY);
                 }
             };
-            if (has_own) {
-                if (lap) sums(std::true_type(), std::true_type());
-                else sums(std::false_type(), std::true_type());
+            const std::true_type yes;
+            const std::false_type no;
+            if (sliver) {
+                sums(yes, yes, yes);  // (the Laplace densities are zero where they do not apply)
+            } else if (has_own) {
+                if (lap) sums(yes, yes, no);
+                else sums(no, yes, no);
             } else {
-                if (lap) sums(std::true_type(), std::false_type());
-                else sums(std::false_type(), std::false_type());
+                if (lap) sums(yes, no, no);
+                else sums(no, no, no);
             }
         }
         store_item<real, NW>(red, w, lane, UL, cL, UY, cY, a.Up + 64 * it);
@@ -895,11 +949,11 @@ __global__ void __launch_bounds__(NW * 32) k_near_build(EvalArgs a, const NearGr
             real* u = mat + 64 * near_unit(nm, c);
             real VL, KL, VY, KY, h;
             if (c >= nm.l0 && c < nm.l1) {
-                panel_sums<real, K, true>(sP[w][k], xr.x, xr.y, xr.z, kappa, nkl, ra, rw, VL, KL, VY, KY, h);
+                panel_sums<real, K, true, (K >= 3)>(sP[w][k], xr.x, xr.y, xr.z, kappa, nkl, ra, rw, VL, KL, VY, KY, h);
                 const real z = 0;
                 near_store<real, true>(u, lane, own ? z : VL, own ? z : h * KL, own ? z : VY, own ? z : h * KY);
             } else {
-                panel_sums<real, K, false>(sP[w][k], xr.x, xr.y, xr.z, kappa, nkl, ra, rw, VL, KL, VY, KY, h);
+                panel_sums<real, K, false, (K >= 3)>(sP[w][k], xr.x, xr.y, xr.z, kappa, nkl, ra, rw, VL, KL, VY, KY, h);
                 const real z = 0;
                 near_store<real, false>(u, lane, z, z, own ? z : VY, own ? z : h * KY);
             }
