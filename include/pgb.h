@@ -218,6 +218,18 @@ int pgb_tree_refresh(struct pgb_ctx* ctx);
  * solvent changed). */
 int pgb_tree_reset(struct pgb_ctx* ctx);
 
+/* Memory that a context holds only to form products faster: the column table
+ * of the P2P sums (16 bytes for every panel of every near leaf of a target
+ * group), the panel moments of the upward pass (per arithmetic) and the near
+ * field that a solve's products share (per precision).  bytes >= 0 bounds each
+ * of these buffers; bytes < 0 is the default, a 32nd, a 16th and an 8th of the
+ * device's memory.  What exceeds its bound is not kept: products then take
+ * longer and need that much less; the sums are the same up to the order of
+ * their rounding.  A new bound drops what is held and the tree (call
+ * pgb_tree_build again).  kept (may be NULL) receives the bytes held: columns,
+ * panel moments, near field, with those of the context's pose lanes and batch. */
+int pgb_keep_limit(struct pgb_ctx* ctx, int64_t bytes, int64_t kept[3]);
+
 /* Number of unknowns 2*N_dielectric + N_surface. */
 int pgb_num_unknowns(struct pgb_ctx* ctx, int64_t* n);
 

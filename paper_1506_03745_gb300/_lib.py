@@ -76,6 +76,7 @@ _SIGS = {
     "pgb_tree_build": (c_i32, [c_vp]),
     "pgb_tree_reset": (c_i32, [c_vp]),
     "pgb_tree_refresh": (c_i32, [c_vp]),
+    "pgb_keep_limit": (c_i32, [c_vp, c_i64, c_vp]),
     "pgb_tree_stats": (c_i32, [c_vp, ctypes.POINTER(pgb_tree_info)]),
     "pgb_num_unknowns": (c_i32, [c_vp, ctypes.POINTER(c_i64)]),
     "pgb_matvec": (c_i32, [c_vp, c_vp, c_vp, c_i32]),
@@ -365,6 +366,14 @@ def pgb_math_check(x):
     out = np.zeros((len(x), 7), np.float64)
     _check(None, lib().pgb_math_check(x.ctypes.data_as(c_vp), len(x), out.ctypes.data_as(c_vp)))
     return out
+
+
+def pgb_keep_limit(ctx, nbytes=-1):
+    """Bound on each buffer that ctx keeps only to be faster (-1: the default);
+    dict(columns, moments, near) of the bytes held now."""
+    kept = np.zeros(3, np.int64)
+    _check(ctx, lib().pgb_keep_limit(ctx, int(nbytes), kept.ctypes.data_as(c_vp)))
+    return dict(zip(("columns", "moments", "near"), (int(k) for k in kept)))
 
 
 def pgb_alloc_count():

@@ -240,6 +240,7 @@ static void ensure_lanes(pgb_ctx* c, int L, int32_t body_id) {
             pgb_ctx* l = new pgb_ctx;
             l->p = c->p;
             l->p.lanes = 1;
+            l->keep_limit = c->keep_limit;
             l->eps_out = c->eps_out;
             l->kappa = c->kappa;
             l->bodies = c->bodies;
@@ -621,6 +622,40 @@ int pgb_tree_reset(pgb_ctx* c) {
     c->tree_valid = false;
     c->adj_valid = false;
     return PGB_OK;
+}
+
+int pgb_keep_limit(pgb_ctx* c, int64_t bytes, int64_t kept[3]) {
+    if (!c) return PGB_EINVAL;
+    return guard(c, [&]() -> int {
+        const int64_t limit = bytes < 0 ? -1 : bytes;
+        if (limit != c->keep_limit) {
+            destroy_lanes(c);
+            destroy_union(c);
+            c->keep_limit = limit;
+            c->d_col.release();
+            for (auto& m : c->pan_mom) {
+                m.buf.release();
+                m.geom_gen = ~0ull;
+            }
+            for (auto& m : c->near_mat) {
+                m.buf.release();
+                m.list_gen = ~0ull;
+            }
+            pgb_tree_reset(c);
+        }
+        if (kept) {
+            kept[0] = kept[1] = kept[2] = 0;
+            std::vector<const pgb_ctx*> all(c->lane_ctx.begin(), c->lane_ctx.end());
+            if (c->union_ctx) all.push_back(c->union_ctx);
+            all.push_back(c);
+            for (const pgb_ctx* q : all) {
+                kept[0] += q->d_col.n * sizeof(float4);
+                for (const auto& m : q->pan_mom) kept[1] += m.buf.n;
+                for (const auto& m : q->near_mat) kept[2] += m.buf.n;
+            }
+        }
+        return PGB_OK;
+    });
 }
 
 int pgb_tree_stats(pgb_ctx* c, pgb_tree_info* info) {

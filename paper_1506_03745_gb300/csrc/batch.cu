@@ -564,6 +564,7 @@ static pgb_ctx* ensure_union(pgb_ctx* c, const std::vector<pgb_ctx*>& src) {
     u->p = c->p;
     u->p.lanes = 1;
     u->p.overlap = 0;
+    u->keep_limit = c->keep_limit;
     u->eps_out = c->eps_out;
     u->kappa = c->kappa;
     for (size_t p = 0; p < src.size(); ++p) {

@@ -333,6 +333,15 @@ static void launch_stage(pgb_ctx* c, int stage, int kind, const UpArgs& up, cons
     else treecode_launch_ds(stage, c->p.P, up, ev, c->d_x64, mom, up.far, s);
 }
 
+size_t keep_bound(pgb_ctx* c, int share) {
+    if (c->keep_limit >= 0) return (size_t)c->keep_limit;
+    if (!c->dev_bytes) {
+        size_t free_b = 0;
+        PGB_CUDA(cudaMemGetInfo(&free_b, &c->dev_bytes));
+    }
+    return c->dev_bytes / share;
+}
+
 // The panel moments of the current geometry in the arithmetic `kind`: formed on
 // the context's stream the first time a product of that kind meets the
 // geometry, kept until the geometry or the order changes.  nullptr where they
@@ -348,9 +357,10 @@ const void* panel_moments(pgb_ctx* c, int kind) {
     pm.P = c->p.P;
     const size_t esz = kind == 0 ? 4 : 8;
     const size_t bytes = (size_t)c->n_pan * n_terms(c->p.P) * esz;
-    size_t free_b = 0, total_b = 0;
-    PGB_CUDA(cudaMemGetInfo(&free_b, &total_b));
-    if (bytes > total_b / 16) return nullptr;
+    if (bytes > keep_bound(c, 16)) {
+        pm.buf.release();
+        return nullptr;
+    }
     try {
         pm.buf.resize(bytes);
     } catch (const Error& e) {
@@ -383,7 +393,7 @@ bool near_ready(pgb_ctx* c, int kind) {
     nm.have = false;
     nm.list_gen = c->list_gen;
     nm.kappa = c->kappa;
-    if (c->n_groups == 0 || c->n_pitems == 0) return false;
+    if (c->n_groups == 0 || c->n_pitems == 0 || !c->d_col.p) return false;
     try {
         nm.group.resize(16 * c->n_groups);
         const int64_t units = near_groups(c, nm.group.p);
@@ -392,7 +402,7 @@ bool near_ready(pgb_ctx* c, int kind) {
             nm.buf.release();
             size_t free_b = 0, total_b = 0;
             PGB_CUDA(cudaMemGetInfo(&free_b, &total_b));
-            if (bytes > total_b / 8 || bytes > free_b / 4) return false;
+            if (bytes > keep_bound(c, 8) || bytes > free_b / 4) return false;
             nm.buf.resize(bytes);
         }
     } catch (const Error& e) {
@@ -602,10 +612,11 @@ static void apply_vec(pgb_ctx* c, VecIn xv, VecOut yv, int precision, int mode, 
         if (c->body_off[b]) ev.tgt_mask &= ~(1ull << b);
     ev.g_lo = c->shard_g[0] >= 0 ? c->shard_g[0] : 0;
     ev.g_hi = c->shard_g[0] >= 0 ? c->shard_g[1] : c->n_groups;
-    ev.near4 = c->d_near4;
     ev.far4 = c->d_far4;
     ev.col_off = c->d_col_off;
     ev.col = c->d_col;
+    ev.ent_col = c->d_ent_col;
+    ev.cen = c->d_c;
     ev.pnode = c->d_pnode;
     ev.pbody = c->d_pbody;
     ev.pts = c->d_y64;

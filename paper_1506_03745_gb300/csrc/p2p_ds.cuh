@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(NW * 32) k_p2p_ds(EvalArgs a, const dbl4* __re
             __syncwarp();
             if (lane < cnt) {
                 const int c = (e + lane) / K, m = e + lane - c * K;
-                const int j = __float_as_int(a.col[w0 + c].w);
+                const int j = __float_as_int(column(a, g, c0, w0 - c0 + c).w);
                 const int b = a.pbody[j];
                 lap = glap && b == gb;
                 const bool on = (act >> b) & 1ull;  // a body without density in this product adds nothing

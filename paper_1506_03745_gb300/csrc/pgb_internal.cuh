@@ -260,7 +260,7 @@ struct pgb_ctx {
     pgb::DBuf<int32_t> d_list_tmp;       // entries kept by the counting traversal (fixed rows per group)
     int64_t n_cols = 0;                  // P2P columns (panels of a group's near leaves) over all groups
     pgb::DBuf<int64_t> d_col_off;        // per group (+ total)
-    pgb::DBuf<float4> d_col;             // panel centroid - group centre, panel
+    pgb::DBuf<float4> d_col;             // panel centroid - group centre, panel; empty: not kept
     pgb::DBuf<int32_t> d_ent_col;        // first column (within its group) of every near entry
     pgb::DBuf<int32_t> d_pnode;          // leaf node of every panel
     pgb::DBuf<float> d_pg32;             // panel geometry of the P2P kernels, 16 values each
@@ -317,6 +317,8 @@ struct pgb_ctx {
         double kappa = 0;
         bool have = false;
     } near_mat[2];
+    int64_t keep_limit = -1;             // pgb_keep_limit
+    size_t dev_bytes = 0;                // the device's memory (keep_bound)
     uint64_t list_gen = 0;               // bumped whenever the lists or the geometry change
     bool near_on = false;                // a solve is running: its FP32 / FP64 products may keep it
     // panel moments of the P2M (k_panel_moments) per arithmetic: FP32, FP64, double-single
@@ -499,6 +501,8 @@ Geo geo(const pgb_ctx* c);
 // scans (tree.cu)
 void exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, cudaStream_t s, int64_t* total_host);
 // matvec (matvec.cu)
+// bytes that one kept structure may take: a share of the device's memory or the caller's limit
+size_t keep_bound(pgb_ctx* c, int share);
 bool near_ready(pgb_ctx* c, int kind);  // the stored near field (near_mat[kind]) is there for a running solve's product
 const void* panel_moments(pgb_ctx* c, int kind);  // nullptr: not kept
 void apply_operator(pgb_ctx* c, const double* x, double* y, int precision, bool known_only,

@@ -1190,7 +1190,7 @@ int64_t near_groups(pgb_ctx* c, void* out) {
 }
 
 // P2P columns: the panels of a group's near leaves one after another, in list
-// order; descriptor = (panel centroid - group centre, formed in FP64 and
+// order; descriptor (where they are kept) = (panel centroid - group centre, formed in FP64 and
 // rounded once to FP32, panel).  One warp per group; the lanes take its near
 // entries 32 at a time.
 __global__ void k_col_count(int64_t ng, const int64_t* noff, const int32_t* nearl, const int32_t* nstart,
@@ -1217,6 +1217,7 @@ __global__ void k_col_fill(int64_t ng, const int64_t* noff, const int32_t* nearl
         const int s = nstart[nearl[e]], n = nend[nearl[e]] - s;
         if (lane == 0) ecol[e] = (int32_t)(w - coff[g]);
         for (int q = lane; q < n; q += 32) {
+            if (!col) break;
             const int64_t j = s + q;
             col[w + q] = make_float4((float)(C[3 * j] - g0), (float)(C[3 * j + 1] - g1), (float)(C[3 * j + 2] - g2),
                                      __int_as_float(s + q));
@@ -1325,7 +1326,19 @@ void build_lists(pgb_ctx* c) {
         exclusive_scan_i64(tc, c->d_col_off, ng, s, &nt);
         PGB_CUDA(cudaMemcpyAsync(c->d_col_off.p + ng, &nt, 8, cudaMemcpyHostToDevice, s));
         c->n_cols = nt;
-        c->d_col.resize(nt);
+        // 16 bytes a (group, near panel) pair: kept up to a thirty-second of the
+        // device's memory, which only direct sums of some hundred thousand panels
+        // exceed (0.5 M at theta = 0: 125 GB).  Beyond it a column is found in the
+        // near list when it is staged (column, treecode.cuh), 4 bytes a near leaf.
+        if ((size_t)nt * sizeof(float4) <= keep_bound(c, 32)) {
+            try {
+                c->d_col.resize(nt);
+            } catch (const Error& e) {  // (resize has released what there was)
+                if (e.code != PGB_ENOMEM) throw;
+            }
+        } else {
+            c->d_col.release();
+        }
         c->d_ent_col.resize(std::max<int64_t>(c->n_near, 1));
         k_col_fill<<<nblk(32 * ng, 128), 128, 0, s>>>(ng, c->d_near_off, c->d_near, c->d_node_start,
                                                       c->d_node_end, c->d_c, c->d_group_center, c->d_col_off,

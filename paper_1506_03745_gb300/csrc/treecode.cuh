@@ -293,10 +293,11 @@ struct EvalArgs {
     // lockstep iteration: bit b clear = body b's rows and sources left out);
     // nullptr: none.  With it all_active is 0.
     const unsigned long long* bmask = nullptr;
-    const float4* near4;           // per near entry: leaf centre - group centre, node id bits
     const float4* far4;            // per far entry: node centre - group centre, node id bits
     const int64_t* col_off;        // per group: its P2P columns [col_off[g], col_off[g+1])
-    const float4* col;             // per column: panel centroid - group centre (FP32), panel (int bits)
+    const float4* col;             // per column: panel centroid - group centre (FP32), panel (int bits); nullptr:
+    const int32_t* ent_col;        // not kept, found by each near entry's first column in its group
+    const double* cen;             // panel centroids
     const int32_t* pnode;          // leaf node of a panel (FP64 and double-single offsets)
     const int32_t* pbody;          // body of a panel
     const void* pg;                // panel geometry (PanelGeo) in the kernel's arithmetic (FP64 for double-single)
@@ -315,6 +316,22 @@ struct EvalArgs {
     unsigned long long *p2p_work, *m2p_work;
     int persist_blocks;            // grid of a persistent launch
 };
+
+// Column i of group g, whose columns start at c0 (EvalArgs::col).  Without the
+// table the near entry that holds it is searched for, and the offset formed as
+// the table's is.
+__device__ __forceinline__ float4 column(const EvalArgs& a, int64_t g, int64_t c0, int64_t i) {
+    if (a.col) return a.col[c0 + i];
+    int64_t lo = a.near_off[g], hi = a.near_off[g + 1];
+    while (hi - lo > 1) {
+        const int64_t m = (lo + hi) >> 1;
+        if (a.ent_col[m] <= i) lo = m;
+        else hi = m;
+    }
+    const int64_t j = a.nstart[a.near_l[lo]] + (i - a.ent_col[lo]);
+    return make_float4((float)(a.cen[3 * j] - a.gcenter[3 * g]), (float)(a.cen[3 * j + 1] - a.gcenter[3 * g + 1]),
+                       (float)(a.cen[3 * j + 2] - a.gcenter[3 * g + 2]), __int_as_float((int)j));
+}
 
 // Item loop of a block: one item per block, or (persistent launch) items
 // taken from a counter until none is left.  The barrier also keeps a block
@@ -830,7 +847,7 @@ __global__ void __launch_bounds__(NW * 32) k_p2p(EvalArgs a, const typename V4<r
             __syncwarp();
             int j = -1;
             if (lane < cnt) {
-                const float4 c = a.col[e + lane];
+                const float4 c = column(a, g, c0, e - c0 + lane);
                 j = __float_as_int(c.w);
                 const int b = a.pbody[j];
                 lap = glap && b == gb;
