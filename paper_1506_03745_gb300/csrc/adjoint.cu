@@ -362,7 +362,7 @@ void apply_transpose(pgb_ctx* c, const double* lam, double* y, int precision) {
         ua.pmom = panel_moments(c, 1);
         ta.far_tr = far_table(c, c->kappa).tr64.p;
         ta.ent_col = c->d_ent_col;
-        if (c->near_on && near_ready(c, 1)) {
+        if ((c->near_on & 2) && near_ready(c, 1)) {
             ta.near_mat = c->near_mat[1].buf.p;
             ta.near_grp = c->near_mat[1].group.p;
         } else {
@@ -534,7 +534,7 @@ __global__ void __launch_bounds__(256) k_cross_grad(Geo g, const float4* __restr
 void grad(pgb_ctx* c, const double* x, int precision, double tol, int max_iter, int restart, double* dq, double* dbc,
           double* dt, pgb_solve_stats* st) {
     if (!c->tree_valid) fail(PGB_ESTATE, "pgb_tree_build has not run");
-    NearScope keep(c);
+    NearScope keep(c, precision);
     if (c->n_xcorr) fail(PGB_EINVAL, "gradients need the bodies farther apart than 2L (cross-body near entries exist)");
     if (precision != PGB_FP32 && precision != PGB_FP64) fail(PGB_EINVAL, "precision must be PGB_FP32 or PGB_FP64");
     cudaStream_t s = c->stream;

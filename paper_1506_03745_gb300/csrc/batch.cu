@@ -418,7 +418,7 @@ static int gmres_seg(pgb_ctx* c, int prec, const double* b, double* x, const dou
 // Solve of the c->n_prob problems of the context (modes as solve()); the
 // statistics of problem p into st[p].  PGB_OK when every problem met tol.
 int solve_seg(pgb_ctx* c, int mode, double tol, int max_iter, int restart, double* x, pgb_solve_stats* st) {
-    NearScope keep(c);
+    NearScope keep(c, mode);
     const int B = c->n_prob;
     const int64_t n = c->n_unk;
     cudaStream_t s = c->stream;

@@ -671,7 +671,7 @@ static void apply_vec(pgb_ctx* c, VecIn xv, VecOut yv, int precision, int mode, 
     up.pg = dsp ? (const void*)c->d_pg_ds.p : ev.pg;
     up.pd = dsp ? (const void*)c->d_pd_ds.p : ev.pd;
     up.pmom = panel_moments(c, kind);
-    if (c->near_on && kind < 2 && !ev.p2p_work && c->shard_g[0] < 0 && !nested(c) && near_ready(c, kind)) {
+    if (kind < 2 && ((c->near_on >> kind) & 1) && !ev.p2p_work && c->shard_g[0] < 0 && !nested(c) && near_ready(c, kind)) {
         ev.near_mat = c->near_mat[kind].buf.p;
         ev.near_group = c->near_mat[kind].group.p;
     }

@@ -320,7 +320,7 @@ struct pgb_ctx {
     int64_t keep_limit = -1;             // pgb_keep_limit
     size_t dev_bytes = 0;                // the device's memory (keep_bound)
     uint64_t list_gen = 0;               // bumped whenever the lists or the geometry change
-    bool near_on = false;                // a solve is running: its FP32 / FP64 products may keep it
+    int near_on = 0;                     // a solve is running: bit k, its products of kind k may keep it
     // panel moments of the P2M (k_panel_moments) per arithmetic: FP32, FP64, double-single
     struct PanMom {
         pgb::DBuf<unsigned char> buf;
@@ -466,11 +466,13 @@ inline bool nested(const pgb_ctx* c) {
         if (b.parent >= 0 || b.kappa_in != 0.0) return true;
     return false;
 }
-// For the duration of a solve: products keep the near field.
+// For the duration of a solve: the products of the precision that it iterates in
+// keep the near field.  (Not the one or two FP64 products of a refinement:
+// forming it costs about one and a half P2Ps.)
 struct NearScope {
     pgb_ctx* c;
-    bool prev;
-    explicit NearScope(pgb_ctx* ctx) : c(ctx), prev(ctx->near_on) { c->near_on = true; }
+    int prev;
+    NearScope(pgb_ctx* ctx, int precision) : c(ctx), prev(ctx->near_on) { c->near_on = precision == PGB_FP64 ? 2 : 1; }
     ~NearScope() { c->near_on = prev; }
 };
 // CUDA-event interval on the context stream around one stage (no-op when

@@ -1032,7 +1032,7 @@ static void overlap_fork(pgb_ctx* c, const double* xs, void* user) {
 }
 
 int solve(pgb_ctx* c, int mode, double tol, int max_iter, int restart, double* x, pgb_solve_stats* st) {
-    NearScope keep(c);
+    NearScope keep(c, mode);
     const int64_t n = c->n_unk;
     cudaStream_t s = c->stream;
     c->d_b.resize(n);
