@@ -225,7 +225,12 @@ int pgb_tree_reset(struct pgb_ctx* ctx);
  * of these buffers; bytes < 0 is the default, a 32nd, a 16th and an 8th of the
  * device's memory.  What exceeds its bound is not kept: products then take
  * longer and need that much less; the sums are the same up to the order of
- * their rounding.  A new bound drops what is held and the tree (call
+ * their rounding.  The near field is formed by the first product of a solve, in
+ * the precision that the solve iterates in, unless it would also take more than
+ * a quarter of the memory then free.  It is given back when the lists change
+ * (pgb_tree_build, pgb_tree_refresh, pgb_tree_reset), and at the end of the solve
+ * where it takes more than a 32nd of its bound.  What is given back stays with
+ * the device's memory pool, for this library's next allocations.  A new bound drops what is held and the tree (call
  * pgb_tree_build again).  kept (may be NULL) receives the bytes held: columns,
  * panel moments, near field, with those of the context's pose lanes and batch. */
 int pgb_keep_limit(struct pgb_ctx* ctx, int64_t bytes, int64_t kept[3]);

@@ -616,6 +616,7 @@ int pgb_tree_refresh(pgb_ctx* c) {
 
 int pgb_tree_reset(pgb_ctx* c) {
     if (!c) return PGB_EINVAL;
+    near_release(c, false);
     c->order_valid = false;
     c->lists_valid = false;
     c->intra_valid = false;
@@ -636,10 +637,6 @@ int pgb_keep_limit(pgb_ctx* c, int64_t bytes, int64_t kept[3]) {
             for (auto& m : c->pan_mom) {
                 m.buf.release();
                 m.geom_gen = ~0ull;
-            }
-            for (auto& m : c->near_mat) {
-                m.buf.release();
-                m.list_gen = ~0ull;
             }
             pgb_tree_reset(c);
         }

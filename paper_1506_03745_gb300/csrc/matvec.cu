@@ -380,6 +380,35 @@ const void* panel_moments(pgb_ctx* c, int kind) {
     return pm.buf.p;
 }
 
+// Memory a stream-ordered allocation can have: what the device has free and what
+// the device's pool holds unused.
+static size_t free_bytes() {
+    size_t free_b = 0, total_b = 0;
+    PGB_CUDA(cudaMemGetInfo(&free_b, &total_b));
+    int dev = 0;
+    cudaMemPool_t pool;
+    uint64_t held = 0, used = 0;
+    PGB_CUDA(cudaGetDevice(&dev));
+    PGB_CUDA(cudaDeviceGetDefaultMemPool(&pool, dev));
+    PGB_CUDA(cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held));
+    PGB_CUDA(cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used));
+    return free_b + (held > used ? held - used : 0);
+}
+
+// Gives the stored near fields back to the pool: all of them (the lists change),
+// or those that take more than a 32nd of their bound (a solve has ended; 1.1 GB
+// here, what 150000 panels hold in FP32 -- forming one anew is a few hundredths of
+// the next solve).
+void near_release(pgb_ctx* c, bool large_only) {
+    for (auto& nm : c->near_mat) {
+        const size_t bound = c->keep_limit >= 0 ? (size_t)c->keep_limit : c->dev_bytes / 8;
+        if (!nm.buf.p || (large_only && nm.buf.n <= bound / 32)) continue;
+        if (nm.buf.st != c->stream) cudaStreamSynchronize(c->stream);  // (freed in the order of its own stream)
+        nm.buf.release();
+        nm.list_gen = ~0ull;
+    }
+}
+
 // The stored near field of the current lists for a product of a running solve
 // (NearScope): formed by the solve's first product on the context's stream, at
 // the cost of about one and a half P2Ps, and kept until the lists, the geometry
@@ -400,9 +429,7 @@ bool near_ready(pgb_ctx* c, int kind) {
         const size_t bytes = (size_t)units * 64 * (kind == 0 ? 4 : 8);
         if (bytes > nm.buf.n) {
             nm.buf.release();
-            size_t free_b = 0, total_b = 0;
-            PGB_CUDA(cudaMemGetInfo(&free_b, &total_b));
-            if (bytes > keep_bound(c, 8) || bytes > free_b / 4) return false;
+            if (bytes > keep_bound(c, 8) || bytes > free_bytes() / 4) return false;
             nm.buf.resize(bytes);
         }
     } catch (const Error& e) {

@@ -468,12 +468,18 @@ inline bool nested(const pgb_ctx* c) {
 }
 // For the duration of a solve: the products of the precision that it iterates in
 // keep the near field.  (Not the one or two FP64 products of a refinement:
-// forming it costs about one and a half P2Ps.)
+// forming it costs about one and a half P2Ps.)  At its end a near field of
+// modest size stays for the next solve on the same lists, a large one is given
+// back (near_release).
+void near_release(pgb_ctx* c, bool large_only);
 struct NearScope {
     pgb_ctx* c;
     int prev;
     NearScope(pgb_ctx* ctx, int precision) : c(ctx), prev(ctx->near_on) { c->near_on = precision == PGB_FP64 ? 2 : 1; }
-    ~NearScope() { c->near_on = prev; }
+    ~NearScope() {
+        c->near_on = prev;
+        if (!prev) near_release(c, true);
+    }
 };
 // CUDA-event interval on the context stream around one stage (no-op when
 // timing is off).

@@ -891,6 +891,7 @@ __global__ void k_panel_geo(const int32_t* pan_leaf, const int32_t* leaf_node, c
 void build_geometry(pgb_ctx* c) {
     ++c->geom_gen;
     ++c->list_gen;
+    near_release(c, false);
     cudaStream_t s = c->stream;
     int64_t n = c->n_pan;
     int K = c->p.K;
@@ -1307,6 +1308,7 @@ void make_lists(pgb_ctx* c, const double* r2, const double* glo, const double* g
 
 void build_lists(pgb_ctx* c) {
     ++c->list_gen;
+    near_release(c, false);
     cudaStream_t s = c->stream;
     int64_t ng = c->n_groups;
     unsigned long long h[4];
@@ -1376,6 +1378,7 @@ void build_lists(pgb_ctx* c) {
 // centres moved (pgb_tree_refresh): entries, columns and work items stay.
 void refresh_lists(pgb_ctx* c) {
     ++c->list_gen;
+    near_release(c, false);
     cudaStream_t s = c->stream;
     const int64_t ng = c->n_groups;
     if (ng == 0) return;
