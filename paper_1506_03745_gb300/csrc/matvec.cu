@@ -352,6 +352,11 @@ const void* panel_moments(pgb_ctx* c, int kind) {
     auto& pm = c->pan_mom[kind];
     if (pm.geom_gen == c->geom_gen && pm.P == c->p.P) return pm.have ? (const void*)pm.buf.p : nullptr;
     if (c->capturing) return nullptr;  // (every product is prepared outside the capture)
+    // the caller captures: what is launched now runs when its graph does, and
+    // products before that need moments too
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    PGB_CUDA(cudaStreamIsCapturing(c->stream, &cs));
+    if (cs != cudaStreamCaptureStatusNone) return nullptr;
     pm.have = false;
     pm.geom_gen = c->geom_gen;
     pm.P = c->p.P;
