@@ -11,8 +11,9 @@
 // coefficients, 0.42 in the harmonic basis with both kernels' sums sharing the
 // recurrences (0.48 one after the other), near field 3.88 ms formed anew, 0.06
 // read, nodes 0.26 ms; the whole
-// gradient 606 -> 74 ms.  (The FP32 product keeps the kernels of adjoint.cuh:
-// what a gradient in FP32 returns is theirs to the last rounding.)
+// gradient 606 -> 74 ms.  (The FP32 product keeps the kernels of adjoint.cuh,
+// whose sums, up to the order of their atomic additions, an FP32 gradient's
+// derivatives rest on.)
 #pragma once
 #include "adjoint.cuh"
 

@@ -255,6 +255,24 @@ const FarTab& far_table(pgb_ctx* c, double kappa) {
     return *c->far_tabs.back();
 }
 
+// The Yukawa table of far_tables in FP32, transposed (tab[k mono_cols(P) + j]):
+// formed once per order and screening, as the harmonic ones (0.1 ms of host time
+// at order 6, 0.45 at 8).
+const float* far_monomials_f32(pgb_ctx* c, double kappa) {
+    FarTab& t = const_cast<FarTab&>(far_table(c, kappa));
+    if (t.mono32.p) return t.mono32.p;
+    const int T = n_terms(t.P), TR = mono_cols(t.P);
+    std::vector<double> rows;
+    far_tables(t.P, kappa, rows);
+    std::vector<float> h((size_t)T * TR, 0.f);
+    for (int j = 0; j < T; ++j)
+        for (int k = 0; k < T; ++k) h[(size_t)k * TR + j] = (float)rows[(size_t)j * T + k];
+    t.mono32.resize(h.size());
+    PGB_CUDA(cudaMemcpyAsync(t.mono32.p, h.data(), 4 * h.size(), cudaMemcpyHostToDevice, c->stream));
+    PGB_CUDA(cudaStreamSynchronize(c->stream));
+    return t.mono32.p;
+}
+
 }  // namespace pgb
 
 extern "C" int pgb_far_table(int32_t P, double kappa, double* out, int64_t n) {

@@ -1,14 +1,16 @@
 // The imposed-boundary terms of an FP32 gradient, b_known of one surface with
 // its imposed value set to one (pgb_grad: dF/dsigma0 and dF/dphi0 take
 // lam . b_known).  They are one FP32 product per surface and gradient, and the
-// derivative carries that product's rounding, 3e-9 to 7e-9 of its value against
+// derivative carries that product's rounding, 1e-9 to 4e-9 of its value against
 // the double-single product's.  The sums here are formed point by point, with
-// Cartesian moments and monomials, in one fixed order; forming them in the
-// order of the products of the solve moves the derivative by 1e-9 to 1e-8.  So
-// that an FP32 gradient keeps its value, this path keeps its arithmetic; it is
-// 0.3 ms of a gradient of 36000 panels.  Orders 0..8 (as pgb_grad), Yukawa
-// kernel only: imposed densities live on surfaces, and the Laplace kernel
-// couples a molecule only to itself.
+// Cartesian moments and monomials, in one fixed order; the products of the
+// solve, in another order, or the double-single one move the derivative by that
+// much, ten times and more what two runs of one gradient differ in it (1e-11 to
+// 6e-10, from the atomic additions of the adjoint solve).  So that an FP32
+// gradient's derivative in an imposed value stays what it was, this path keeps
+// its arithmetic; it is 0.3 ms of a gradient of 36000 panels.  Orders 0..8 (as
+// pgb_grad), Yukawa kernel only: imposed densities live on surfaces, and the
+// Laplace kernel couples a molecule only to itself.
 #include <algorithm>
 
 #include "treecode.cuh"
@@ -31,8 +33,6 @@ struct ImpArgs {
     const float* tab;              // far-field table, transposed: tab[k TR + j]
     float *mom, *far;              // T moments, n_pad coefficients per node
 };
-__host__ __device__ constexpr int imp_pad(int P) { return (n_terms(P) + 3) & ~3; }
-__host__ __device__ constexpr int imp_cols(int P) { return (imp_pad(P) + 31) & ~31; }
 
 // Densities of the surface (psi_Y, phi per panel, zero elsewhere) and its point
 // source terms.
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(256) k_imp_m2m(ImpArgs a, int64_t lo) {
 // Monomial far-field coefficients (the table of pgb_far_table) of every node.
 template <int P>
 __global__ void __launch_bounds__(256) k_imp_far(ImpArgs a) {
-    constexpr int T = MI<P>::T, TP = imp_pad(P), TR = imp_cols(P);
+    constexpr int T = MI<P>::T, TP = n_mono_pad(P), TR = mono_cols(P);
     __shared__ float m[T];
     const int64_t nd = blockIdx.x;
     if (a.nbody[nd] != a.body) return;
@@ -310,7 +310,7 @@ template <int P>
 __global__ void __launch_bounds__(256) k_imp_eval(ImpArgs a, const int64_t* toff, const float4* td, const int4* tm,
                                                   int item, const int64_t* foff, const float4* far4, int fitem,
                                                   const float4* xrel, double* U) {
-    constexpr int T = MI<P>::T, TP = imp_pad(P);
+    constexpr int T = MI<P>::T, TP = n_mono_pad(P);
     (void)T;
     __shared__ float4 sA[8][32], sB[8][32];
     __shared__ float sM[8][TP];
@@ -403,14 +403,14 @@ __global__ void k_imp_rows(Geo g, BodyDev bd, int body, const int32_t* pan_group
 
 template <int P>
 void run(pgb_ctx* c, int body, double* y) {
-    constexpr int T = MI<P>::T, TP = imp_pad(P), TR = imp_cols(P);
+    constexpr int T = MI<P>::T, TP = n_mono_pad(P), TR = mono_cols(P);
     cudaStream_t s = c->stream;
     const int64_t n = c->n_pan, ng = c->n_groups, nn = c->n_nodes;
     const Geo g = geo(c);
     const BodyDev bd = body_dev(c);
     DBuf<float4> src, td;
     DBuf<float2> dens;
-    DBuf<float> mom, far, tab;
+    DBuf<float> mom, far;
     DBuf<int64_t> tc, toff;
     DBuf<int4> tm;
     DBuf<double> U;
@@ -418,13 +418,6 @@ void run(pgb_ctx* c, int body, double* y) {
     dens.resize(n);
     mom.resize(nn * T);
     far.resize(nn * TP);
-    std::vector<double> rows;
-    far_tables(P, c->kappa, rows);
-    std::vector<float> ht((size_t)T * TR, 0.f);
-    for (int j = 0; j < T; ++j)
-        for (int k = 0; k < T; ++k) ht[(size_t)k * TR + j] = (float)rows[(size_t)j * T + k];
-    tab.resize(ht.size());
-    PGB_CUDA(cudaMemcpyAsync(tab.p, ht.data(), 4 * ht.size(), cudaMemcpyHostToDevice, s));
     ImpArgs a;
     a.body = body;
     a.K = c->p.K;
@@ -440,7 +433,7 @@ void run(pgb_ctx* c, int body, double* y) {
     a.leaf_node = c->d_leaf_node;
     a.ncenter = c->d_node_center;
     a.src = src;
-    a.tab = tab;
+    a.tab = far_monomials_f32(c, c->kappa);
     a.mom = mom;
     a.far = far;
     k_imp_src<<<nblk(n, 128), 128, 0, s>>>(g, bd, body, c->eps_out, c->d_y32, src, dens);
@@ -467,7 +460,6 @@ void run(pgb_ctx* c, int body, double* y) {
                                             c->d_corr_j, c->d_corr_val32, c->d_xcorr_off, c->d_xcorr_j,
                                             c->d_xcorr_val32, y);
     PGB_CUDA(cudaGetLastError());
-    PGB_CUDA(cudaStreamSynchronize(s));  // (the host table above)
     PGB_LAUNCHED(c, launches);
 }
 

@@ -126,6 +126,7 @@ struct FarTab {
     DBuf<double> t64;
     DBuf<float> t32;
     DBuf<double> tds;  // the FP64 table split into double-single pairs (8 bytes each)
+    DBuf<float> mono32; // the monomial Yukawa table of pgb_far_table, transposed (imposed_f32.cu; formed when first asked for)
     DBuf<double> tr64; // transposed rows, per column the T moments (the transposed treecode), P <= 8
 };
 // far-field coefficients per kernel (2p + 1 per degree p), padded to whole
@@ -134,6 +135,9 @@ __host__ __device__ constexpr int n_far(int P) { return (P + 1) * (P + 1); }
 __host__ __device__ constexpr int n_far_pad(int P) { return (n_far(P) + 3) & ~3; }
 __host__ __device__ constexpr int far_cols(int P) { return (n_far(P) + 31) & ~31; }
 void far_tables(int P, double kappa, std::vector<double>& tab);
+// padded term count of the monomial coefficients, and the columns of their device table
+__host__ __device__ constexpr int n_mono_pad(int P) { return (n_terms(P) + 3) & ~3; }
+__host__ __device__ constexpr int mono_cols(int P) { return (n_mono_pad(P) + 31) & ~31; }
 
 struct Body {
     int kind = PGB_DIELECTRIC;
@@ -499,6 +503,7 @@ void build_order(pgb_ctx* c);
 void build_geometry(pgb_ctx* c);
 void build_lists(pgb_ctx* c);
 const FarTab& far_table(pgb_ctx* c, double kappa);
+const float* far_monomials_f32(pgb_ctx* c, double kappa);
 void refresh_lists(pgb_ctx* c);
 void make_lists(pgb_ctx* c, const double* r2, const double* glo, const double* ghi, DBuf<int64_t>& noff,
                 DBuf<int32_t>& nearl, DBuf<int64_t>& foff, DBuf<int32_t>& farl, DBuf<float4>& near4,
