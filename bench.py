@@ -97,9 +97,17 @@ def m2p_flops(P, laplace):
     return yuk + (max(P - 1, 0) + coef if laplace else 0)
 
 
-def p2p_kernel_flops(info):
+def p2p_point_flops(laplace):
+    """The same point by point, as the double-single product sums: difference 3,
+    |x - y|^2 5, the normal product 5, rsqrt, 1/r^2 and its product 3, r 1,
+    exponent, exp and its product 3, 1 + kappa r 2, the Yukawa term and sum 4;
+    Laplace 3."""
+    return 29 if laplace else 26
+
+
+def p2p_kernel_flops(info, flops=p2p_flops):
     yp = info["p2p_pairs"] - info["p2p_laplace_pairs"]
-    return yp * p2p_flops(False) + info["p2p_laplace_pairs"] * p2p_flops(True)
+    return yp * flops(False) + info["p2p_laplace_pairs"] * flops(True)
 
 
 def m2p_kernel_flops(info, P):
@@ -500,14 +508,39 @@ def run_gpu(args):
     info = pgb.pgb_tree_stats(ctx)
     peaks = device_peaks(dev)
     peak_tflops = peaks["fp32_tflops"]
+    hbm = load_peaks().get("hbm_gbs")
     kern = {}
-    for name, stage, fl in (("k_p2p<float> (P2P, near leaves)", "p2p", p2p_kernel_flops(info)),
-                            ("k_m2p<float,6> (M2P, far nodes)", "m2p", m2p_kernel_flops(info, PARAMS["P"]))):
-        ms, calls = timing[stage]
-        kern[stage] = dict(kernel=name, total_ms=ms, calls=calls, flops=fl,
-                           avg_ms=ms / calls if calls else None,
-                           achieved=fl / (ms / calls / 1e3) / 1e12 if calls else None)
-    dom = max(kern.values(), key=lambda k: k["total_ms"])
+
+    def alu(name, stage, times, fl):
+        ms, calls = times[stage]
+        avg = ms / calls if calls else None
+        ach = fl / (avg / 1e3) / 1e12 if avg else None
+        return dict(kernel=name, total_ms=ms, calls=calls, flops=fl, avg_ms=avg, bound="alu", achieved=ach, unit="TFLOP/s",
+                    peak=peak_tflops, frac=ach / peak_tflops if ach else None)
+
+    # the products of a step, timed in another solve on the same tree, which
+    # finds the near field kept: it streams it (k_near) instead of summing points
+    pgb.pgb_timing(ctx, True, read=True)
+    pgb.pgb_solve(ctx, pgb.PGB_FP32_REFINE, TOL, MAX_ITER, RESTART, x)
+    again = pgb.pgb_timing(ctx, False, read=True)
+    near_bytes = pgb.pgb_keep_limit(ctx)["near"]
+    ms, calls = again["p2p"]
+    if near_bytes and calls:
+        ach = near_bytes / (ms / calls / 1e3) / 1e9
+        kern["near"] = dict(kernel="k_near<float> (near leaves, stored sums)", total_ms=ms, calls=calls, bytes=near_bytes,
+                            avg_ms=ms / calls, bound="hbm", achieved=ach, unit="GB/s", peak=hbm,
+                            frac=ach / hbm if hbm else None, peak_source="MEASURED_PEAKS.json hbm_gbs (of measured)")
+    kern["m2p"] = alu("k_m2p_f32<6> (M2P, far nodes)", "m2p", again, m2p_kernel_flops(info, PARAMS["P"]))
+    # products outside a solve sum the points (k_p2p), beside the upward pass and M2P
+    xf = torch.randn(n, dtype=torch.float32, device=dev)
+    yf = torch.empty_like(xf)
+    pgb.pgb_matvec(ctx, xf, yf, pgb.PGB_FP32)
+    pgb.pgb_timing(ctx, True, read=True)
+    for _ in range(20):
+        pgb.pgb_matvec(ctx, xf, yf, pgb.PGB_FP32)
+    kern["p2p"] = alu("k_p2p<float> (P2P of products outside a solve)", "p2p", pgb.pgb_timing(ctx, False, read=True),
+                      p2p_kernel_flops(info))
+    dom = max((kern[k] for k in ("near", "m2p") if k in kern), key=lambda k: k["avg_ms"] or 0.0)
     traffic = recorded_traffic(dom["kernel"].split(" ")[0])
     # the FP64-class product of the refinement residual: same algorithmic
     # counts.  residual = 1: double-single kernels on the FP32 pipe, set
@@ -517,7 +550,8 @@ def run_gpu(args):
     fp64_peak = peaks["sm_count"] * 2 * 2 * peaks["sm_max_mhz"] * 1e6 / 1e12
     tag = "ds" if PARAMS["residual"] else "double"
     ds_prof = recorded_counters("ds_residual_two_sphere.txt")
-    for name, stage, fl in ((f"k_p2p<{tag}> (P2P, FP64-class residual)", "p2p_fp64", p2p_kernel_flops(info)),
+    residual_flops = p2p_kernel_flops(info, p2p_point_flops if PARAMS["residual"] else p2p_flops)
+    for name, stage, fl in ((f"k_p2p<{tag}> (P2P, FP64-class residual)" if tag != "ds" else "k_p2p_ds (P2P, FP64-class residual)", "p2p_fp64", residual_flops),
                             (f"k_m2p<{tag},6> (M2P, FP64-class residual)", "m2p_fp64",
                              m2p_kernel_flops(info, PARAMS["P"]))):
         ms, calls = timing[stage]
@@ -544,7 +578,6 @@ def run_gpu(args):
     # CSR offset and group data (8 + 4 + 4 + 16 B) and permutation/body
     # (8 B); per unknown x read and y written (16 B); per work item its 64
     # FP64 partial sums (512 B).  The whole working set stays in L2.
-    hbm = load_peaks().get("hbm_gbs")
     ms, calls = timing["assemble"]
     asm_bytes = (20 * info["n_corrections"] + 60 * info["n_panels"] + 16 * info["n_unknowns"] +
                  512 * (info["n_p2p_items"] + info["n_m2p_items"]))
@@ -605,15 +638,15 @@ def run_gpu(args):
         "stage_ms_per_step": {k: v[0] / args.steps for k, v in timing.items() if k not in ("kernel_launches", "host_launches")},
         "gpu_launches": timing["kernel_launches"],
         "host_launch_calls": timing["host_launches"],
-        "roofline": {"kernel": dom["kernel"], "bound": "alu", "achieved": dom["achieved"],
-                     "peak": peak_tflops, "unit": "TFLOP/s",
-                     "frac": (dom["achieved"] / peak_tflops) if dom["achieved"] else None,
-                     "traffic": traffic, "flops_per_launch": dom["flops"], "launches": dom["calls"],
-                     "avg_launch_ms": dom["avg_ms"],
-                     "peak_source": peaks["note"], "sm_count": peaks["sm_count"],
+        "roofline": {"kernel": dom["kernel"], "bound": dom["bound"], "achieved": dom["achieved"],
+                     "peak": dom["peak"], "unit": dom["unit"], "frac": dom["frac"],
+                     "traffic": traffic, "flops_per_launch": dom.get("flops"), "bytes_per_launch": dom.get("bytes"),
+                     "launches": dom["calls"], "avg_launch_ms": dom["avg_ms"],
+                     "peak_source": dom.get("peak_source", peaks["note"]), "sm_count": peaks["sm_count"],
                      "sm_max_mhz": peaks["sm_max_mhz"],
-                     "note": "dominant kernel of the FP32 treecode product (the inner products of a step); "
-                             "the FP64-class residual kernels are in other_kernels, against the FP32 pipe",
+                     "note": "longest kernel of the inner products of a step, timed in a solve that finds its near field "
+                             "kept (beside the other stream's kernels); k_p2p, which products outside a solve run, and "
+                             "the FP64-class residual kernels are in other_kernels",
                      "other_kernels": {k: {kk: vv for kk, vv in v.items() if kk != "kernel"} | {"kernel": v["kernel"]}
                                        for k, v in kern.items() if v is not dom}},
         "tree": info,

@@ -136,8 +136,10 @@ typedef struct pgb_tree_info {
 /* Device time per stage of the hot path, accumulated with CUDA events on
  * the context's stream while timing is enabled (pgb_timing). */
 #define PGB_STAGE_SOURCES 0   /* FP32 matvec: panel densities and per-point source terms */
-#define PGB_STAGE_UPWARD 1    /* FP32 matvec: P2M at the leaves + moment shifts to the root */
-#define PGB_STAGE_P2P 2       /* FP32 matvec: P2P over the near leaves */
+#define PGB_STAGE_UPWARD 1    /* FP32 matvec: P2M at the leaves + moment shifts to the root; the panel
+                                 moments, an interval of their own once per geometry */
+#define PGB_STAGE_P2P 2       /* FP32 matvec: near leaves: P2P, or in a solve the kept near field's stream
+                                 and, an interval of its own once per lists, its formation */
 #define PGB_STAGE_M2P 3       /* FP32 matvec: M2P over the far nodes */
 #define PGB_STAGE_ASSEMBLE 4  /* FP32 matvec: near-field corrections + block rows */
 #define PGB_STAGE_KRYLOV 5    /* Arnoldi (CGS2), Givens, updates */

@@ -378,6 +378,7 @@ const void* panel_moments(pgb_ctx* c, int kind) {
     up.pg = kind == 0 ? (const void*)c->d_pg32.p : kind == 1 ? (const void*)c->d_pg64.p : (const void*)c->d_pg_ds.p;
     EvalArgs ev = {};
     ev.n_pan = c->n_pan;
+    StageTimer tm(c, PGB_STAGE_UPWARD + (kind == 0 ? 0 : PGB_STAGE_FP64));
     launch_stage(c, STAGE_PANEL_MOMENTS, kind, up, ev, pm.buf.p, c->stream);
     PGB_CUDA(cudaGetLastError());
     PGB_LAUNCHED(c, 1);
@@ -455,6 +456,7 @@ bool near_ready(pgb_ctx* c, int kind) {
     ev.pitem_off = c->d_pitem_off;
     ev.pitem_group = c->d_pitem_group;
     ev.pg = kind == 0 ? (const void*)c->d_pg32.p : (const void*)c->d_pg64.p;
+    StageTimer tm(c, PGB_STAGE_P2P + (kind == 0 ? 0 : PGB_STAGE_FP64));
     if (kind == 0) near_build_f32(ev, c->p.K, nm.group.p, c->d_x32, nm.buf.p, c->stream);
     else near_build_f64(ev, c->p.K, nm.group.p, c->d_x64, nm.buf.p, c->stream);
     PGB_CUDA(cudaGetLastError());
