@@ -4,12 +4,12 @@
 // double-single that form rounds |d|^2 and n.d once for all points of a panel,
 // and seven points with one common error no longer average it: products lay
 // 2.7e-15 to 4.9e-15 (relative, 2-norm) from the FP64 ones.  So here every
-// point has its own position, squared distance and normal product, each
-// operation is renormalised, and the target's offset from a leaf's centre is
-// formed in FP64 and split once a leaf: 1.1e-15 to 3.0e-15 over the same six
-// systems (one unit of a pair is 3.6e-15).  Kept from the leaf's centre because
-// the points' rounding is then of the leaf's size; from the group's centre
-// 1.5e-15 to 3.4e-15, with offsets added as pairs 2.2e-15 to 3.9e-15.
+// point has its own position, squared distance and normal product, and the
+// target's offset from a leaf's centre is formed in FP64 and split once a leaf:
+// 1.1e-15 to 3.0e-15 over the same six systems (one unit of a pair is 3.6e-15).
+// Kept from the leaf's centre because the points' rounding is then of the leaf's
+// size; from the group's centre 1.5e-15 to 3.4e-15, with offsets added as pairs
+// 2.2e-15 to 3.9e-15.
 #pragma once
 #include "treecode.cuh"
 
@@ -17,18 +17,22 @@ namespace pgb {
 
 // One point {y, q_L}, {p n, q_Y} for one target at x, both relative to the
 // leaf's centre: U_L += q_L / r - p n.(x - y) / r^3 and the Yukawa counterpart.
+// Differences, the normal product, the exponent's argument and the sums are
+// renormalised; the products between them need not be (1.91 -> 1.81 ms for the
+// product below and the same distances from FP64 to 5 %; with none renormalised
+// 1.3e-15 to 3.1e-15).
 template <bool LAP>
 __device__ __forceinline__ void ds_point(const ds4& A, const ds4& B, bool own, ds x, ds y, ds z, ds kappa, ds nkl,
                                          ds& UL, ds& UY) {
     const ds dx = x - A.x, dy = y - A.y, dz = z - A.z;
-    const ds r2 = ds_fma(dx, dx, ds_fma(dy, dy, dz * dz));
+    const ds r2 = ds_fma(dx, dx, ds_fma_u(dy, dy, ds_mul_u(dz, dz)));
     ds ri = ds_rsqrt(r2);
     if (own) ri = ds(0);  // the panel's own integral is a near-field correction
-    const ds t = ds_fma(B.x, dx, ds_fma(B.y, dy, B.z * dz)) * (ri * ri);
-    const ds r = r2 * ri;
-    const ds e = ds_exp2(nkl * r) * ri;
-    if (LAP) UL = ds_fma(ri, A.w - t, UL);
-    UY = ds_fma(e, ds_fma(-ds_fma(kappa, r, ds(1)), t, B.w), UY);
+    const ds t = ds_mul_u(ds_fma(B.x, dx, ds_fma(B.y, dy, B.z * dz)), ds_mul_u(ri, ri));
+    const ds r = ds_mul_u(r2, ri);
+    const ds e = ds_mul_u(ds_exp2(nkl * r), ri);
+    if (LAP) UL = ds_fma(ri, ds_add_u(A.w, -t), UL);
+    UY = ds_fma(e, ds_fma_u(-ds_fma_u(kappa, r, ds(1)), t, B.w), UY);
 }
 
 // Points summed plainly before they join an item's sums: their additions round
@@ -36,9 +40,9 @@ __device__ __forceinline__ void ds_point(const ds4& A, const ds4& B, bool own, d
 #define P2P_DS_RUN 16
 
 // Work items, columns and warps as k_p2p; a warp stages 32 points at a time,
-// one per lane.  Bound by FP32 operations, about 250 a point with the Laplace
-// kernel: product of 36200 panels 1.91 ms (panel by panel 1.51; before it, with
-// slower functions, 2.55; two points at a time 1.96 -> 1.91).
+// one per lane.  Bound by FP32 operations, about 230 a point with the Laplace
+// kernel: product of 36200 panels 1.81 ms (panel by panel 1.51; before it, with
+// slower functions, 2.55; two points at a time 1.96 -> 1.91 then).
 template <int K, int NW>
 __global__ void __launch_bounds__(NW * 32) k_p2p_ds(EvalArgs a, const dbl4* __restrict__ xrel) {
     __shared__ __align__(16) ds4 sA[NW][32], sB[NW][32];
