@@ -333,6 +333,15 @@ static void launch_stage(pgb_ctx* c, int stage, int kind, const UpArgs& up, cons
     else treecode_launch_ds(stage, c->p.P, up, ev, c->d_x64, mom, up.far, s);
 }
 
+int sm_count(pgb_ctx* c) {
+    if (!c->sms) {
+        int dev = 0;
+        PGB_CUDA(cudaGetDevice(&dev));
+        PGB_CUDA(cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev));
+    }
+    return c->sms;
+}
+
 size_t keep_bound(pgb_ctx* c, int share) {
     if (c->keep_limit >= 0) return (size_t)c->keep_limit;
     if (!c->dev_bytes) {
@@ -373,6 +382,7 @@ const void* panel_moments(pgb_ctx* c, int kind) {
         return nullptr;
     }
     UpArgs up = {};
+    up.sms = sm_count(c);
     up.K = c->p.K;
     up.rule = far_rule(c->p.K);
     up.pg = kind == 0 ? (const void*)c->d_pg32.p : kind == 1 ? (const void*)c->d_pg64.p : (const void*)c->d_pg_ds.p;
@@ -602,6 +612,7 @@ static void apply_vec(pgb_ctx* c, VecIn xv, VecOut yv, int precision, int mode, 
     up.leaf_node = c->d_leaf_node; up.nstart = c->d_node_start; up.nend = c->d_node_end;
     up.child = c->d_node_child; up.nchild = c->d_node_nchild;
     up.ncenter = c->d_node_center; up.K = c->p.K; up.nbody = c->d_node_body;
+    up.sms = sm_count(c);
     up.p2m_grid = 0;
     up.n_nodes = c->n_nodes;
     up.parent = c->d_node_parent;

@@ -356,6 +356,7 @@ struct pgb_ctx {
     pgb::DBuf<pgb::dbl4> d_pc;           // block-diagonal preconditioner, per sorted panel
     pgb::DBuf<double> d_pz;              // its work vector
     bool pc_ready = false;
+    int sms = 0;                         // the device's multiprocessors (sm_count)
     int arn_blocks = 0;                  // grid of the Arnoldi-step kernels (0: not yet set)
     int persist_blocks = 0;              // > 0: products launch P2P/M2P persistently with this grid
     pgb::DBuf<unsigned long long> d_work;  // their item counters
@@ -514,6 +515,7 @@ Geo geo(const pgb_ctx* c);
 // scans (tree.cu)
 void exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, cudaStream_t s, int64_t* total_host);
 // matvec (matvec.cu)
+int sm_count(pgb_ctx* c);
 // bytes that one kept structure may take: a share of the device's memory or the caller's limit
 size_t keep_bound(pgb_ctx* c, int share);
 bool near_ready(pgb_ctx* c, int kind);  // the stored near field (near_mat[kind]) is there for a running solve's product

@@ -557,12 +557,7 @@ __global__ void __launch_bounds__(ARN_THREADS) k_arn_finish(ArnArgs a) {
 // iteration with at most mcap columns.
 void arnoldi_step(pgb_ctx* c, int j, double* w, double* h, double* hc, double* cs, double* sn, double* g,
                   double* out, const ArnSeg* sg, const ArnReplay* rp, int mcap) {
-    if (c->arn_blocks == 0) {
-        int dev = 0, sms = 0;
-        PGB_CUDA(cudaGetDevice(&dev));
-        PGB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        c->arn_blocks = ARN_BLOCKS_PER_SM * sms;
-    }
+    if (c->arn_blocks == 0) c->arn_blocks = ARN_BLOCKS_PER_SM * sm_count(c);
     const int B = sg ? sg->B : 1;
     // replayed, the column is only known on the device: sizes for the largest (mcap)
     const int nb = sg ? sg->nbp : c->arn_blocks, m = rp ? mcap : j + 1;
@@ -826,12 +821,7 @@ int gmres_op(pgb_ctx* c, int prec, bool transpose, const double* b, double* x, d
         c->d_xsel.resize(n);
         if (pc) c->d_pz.resize(n);
         reserve_product(c, prec);
-        if (c->arn_blocks == 0) {
-            int dev = 0, sms = 0;
-            PGB_CUDA(cudaGetDevice(&dev));
-            PGB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-            c->arn_blocks = ARN_BLOCKS_PER_SM * sms;
-        }
+        if (c->arn_blocks == 0) c->arn_blocks = ARN_BLOCKS_PER_SM * sm_count(c);
         c->d_red.resize(std::max<size_t>(c->d_red.n, (size_t)2 * c->arn_blocks * (m + 1)));
     }
     int it = 0;

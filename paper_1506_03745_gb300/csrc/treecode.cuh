@@ -1304,6 +1304,7 @@ struct UpArgs {
     const unsigned long long* bmask = nullptr;  // as EvalArgs::bmask
     const double* ncenter;
     int K;
+    int sms;                     // the device's multiprocessors
     int p2m_grid;                // > 0: P2M over at most this many blocks (leaves strided)
     int64_t n_nodes;             // k_far: every node
     const void* far_tab;         // its table (farfield.cu) in the arithmetic type
@@ -1789,14 +1790,14 @@ template <typename real, int P>
 void launch_far(const UpArgs& up, const void* mom, cudaStream_t s) {
     constexpr int NB = sizeof(real) == sizeof(float) ? 8 : 4;
     if (P > 8) launch_far_nb<real, P, NB / 2>(up, mom, s);
-    else if (up.n_nodes >= 1216 * NB) launch_far_nb<real, P, NB>(up, mom, s);
+    else if (up.n_nodes >= (int64_t)8 * up.sms * NB) launch_far_nb<real, P, NB>(up, mom, s);
     else launch_far_nb<real, P, NB / 4>(up, mom, s);
 }
 
 // The panel moments of the current geometry (UpArgs::pg, rule, K) into out.
 template <typename real, int P>
 void launch_panel_moments(const UpArgs& up, int64_t n_pan, void* out, cudaStream_t s) {
-    const int64_t grid = std::min<int64_t>((n_pan + UP_FLY - 1) / UP_FLY, 152 * 8);
+    const int64_t grid = std::min<int64_t>((n_pan + UP_FLY - 1) / UP_FLY, (int64_t)8 * up.sms);
     if (grid > 0) k_panel_moments<real, P><<<(unsigned)grid, UP_THREADS, 0, s>>>(up, n_pan, (real*)out);
 }
 
