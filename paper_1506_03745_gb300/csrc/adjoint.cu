@@ -324,11 +324,9 @@ void apply_transpose(pgb_ctx* c, const double* lam, double* y, int precision) {
     const int64_t n = c->n_pan, K = c->p.K;
     const int T = n_terms(c->p.P);
     TArgs ta;
-    ta.n_groups = c->n_groups;
     ta.gstart = c->d_group_start; ta.gend = c->d_group_end; ta.gbody = c->d_group_body;
     ta.gcenter = c->d_group_center; ta.ncenter = c->d_node_center;
     ta.nstart = c->d_node_start; ta.nend = c->d_node_end; ta.nbody = c->d_node_body;
-    ta.nchild = c->d_node_nchild; ta.child = c->d_node_child;
     ta.K = (int)K;
     ta.kappa = c->kappa;
     for (int b = 0; b < PGB_MAX_BODIES; ++b) ta.lap_body[b] = 0;
@@ -338,7 +336,6 @@ void apply_transpose(pgb_ctx* c, const double* lam, double* y, int precision) {
     ta.far4 = c->d_far4;
     ta.m2p_item = c->p.m2p_item;
     ta.tn_off = c->d_tn_off; ta.tn_e = c->d_tn_e; ta.near_group = c->d_near_group; ta.near4 = c->d_near4;
-    ta.near_l = c->d_near;
     ta.n_leaves = c->n_leaves;
     ta.leaf_node = c->d_leaf_node;
     ta.lvl_begin = ta.lvl_end = 0;

@@ -27,10 +27,9 @@ namespace pgb {
 
 struct TArgs {
     // the forward target groups and their lists
-    int64_t n_groups;
     const int32_t *gstart, *gend, *gbody;
     const double *gcenter, *ncenter;
-    const int32_t *nstart, *nend, *nbody, *nchild, *child;
+    const int32_t *nstart, *nend, *nbody;
     int K;
     double kappa;
     int lap_body[PGB_MAX_BODIES];
@@ -51,7 +50,6 @@ struct TArgs {
     const int64_t* tn_e;            // forward near entry ids (group order)
     const int32_t* near_group;      // group of each forward near entry
     const float4* near4;            // leaf centre - group centre per forward near entry
-    const int32_t* near_l;          // leaf node of each forward near entry
     int64_t n_leaves;
     const int32_t* leaf_node;
     int64_t lvl_begin, lvl_end;     // node range of one level (k_l2l_level)

@@ -632,7 +632,6 @@ static void apply_vec(pgb_ctx* c, VecIn xv, VecOut yv, int precision, int mode, 
     if (precision != PGB_FP32 && c->persist_blocks > 0)  // side product: P2M on two blocks per SM
         up.p2m_grid = 2 * c->persist_blocks;
     EvalArgs ev;
-    ev.n_groups = c->n_groups;
     ev.n_pan = c->n_pan;
     ev.gstart = c->d_group_start; ev.gend = c->d_group_end; ev.gbody = c->d_group_body;
     ev.gcenter = c->d_group_center; ev.near_off = c->d_near_off; ev.far_off = c->d_far_off;

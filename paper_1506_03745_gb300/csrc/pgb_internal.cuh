@@ -295,18 +295,13 @@ struct pgb_ctx {
     // adjoint (transposed treecode): built on first use after each tree build
     bool adj_valid = false;
     std::vector<int64_t> group_begin;      // first group of each body (+ total)
-    pgb::DBuf<float4> d_yT32, d_n32, d_cT32;
-    pgb::DBuf<pgb::dbl4> d_yT64, d_n64, d_cT64;
-    pgb::DBuf<double> d_rT2, d_gTlo, d_gThi;
-    int64_t n_Tnear = 0, n_Tfar = 0;
-    pgb::DBuf<int64_t> d_Tnear_off, d_Tfar_off, d_ct_off;
-    pgb::DBuf<int32_t> d_Tnear, d_Tfar, d_ct_i;
-    pgb::DBuf<float4> d_Tnear4, d_Tfar4;
+    pgb::DBuf<float4> d_n32, d_cT32;
+    pgb::DBuf<pgb::dbl4> d_n64, d_cT64;
+    pgb::DBuf<int64_t> d_ct_off;
+    pgb::DBuf<int32_t> d_ct_i;
     pgb::DBuf<pgb::dbl4> d_ct_val;
     pgb::DBuf<int32_t> d_near_group;     // group of each forward near entry
     pgb::DBuf<int64_t> d_tn_off, d_tn_e;   // forward near entries by source leaf (CSR over nodes)
-    pgb::DBuf<float4> d_srcT32;
-    pgb::DBuf<pgb::dbl4> d_srcT64;
     pgb::DBuf<float> d_momT32;
     pgb::DBuf<double> d_momT64, d_Tout, d_sT, d_lam, d_gx, d_bu;
     // transposed FP64 product: gathered far-field coefficients; far and near sums per panel
@@ -348,8 +343,6 @@ struct pgb_ctx {
     pgb::DBuf<double> d_Up[2], d_Uf[2];        // P2P / M2P partial sums: 64 per work item (32 L, then 32 Y)
     pgb::DBuf<double> d_xtmp, d_ytmp;    // FP64 staging for FP32 matvec API
     // scratch
-    pgb::DBuf<int64_t> d_scan_tmp;
-    pgb::DBuf<unsigned char> d_scratch;
 
     // solver
     pgb::DBuf<double> d_V, d_H, d_red, d_gv, d_b, d_bc, d_r, d_wk, d_xs, d_small;

@@ -95,15 +95,6 @@ template <>
 __device__ __forceinline__ ds lit<ds>(double d) {
     return ds_const(d);
 }
-// 1/n in the arithmetic type (n a compile-time constant after unrolling)
-template <typename C>
-__device__ __forceinline__ C inv_int(int n) {
-    return C(1) / C(n);
-}
-template <>
-__device__ __forceinline__ ds inv_int<ds>(int n) {
-    return ds_const(1.0 / n);
-}
 
 __device__ __forceinline__ float rsqrt_(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double rsqrt_(double x) { return rsqrt_halley(x); }
@@ -275,7 +266,7 @@ __device__ __forceinline__ unsigned long long body_mask(const unsigned long long
 #define STAGE_PANEL_MOMENTS (-1)
 
 struct EvalArgs {
-    int64_t n_groups, n_pan;
+    int64_t n_pan;
     const int32_t *gstart, *gend, *gbody;
     const double* gcenter;
     const int64_t *near_off, *far_off;
