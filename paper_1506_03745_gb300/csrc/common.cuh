@@ -86,7 +86,8 @@ static __device__ const double kExp2Frac[32] = {
 // |f| <= 1/64; 2^f from its Taylor series to degree 5 (remainder below
 // (ln 2 / 64)^6 / 6! < 3e-15 relative), times 2^((n mod 32) / 32) from a table
 // (256 bytes, two lines of L1) with n / 32 added to its exponent field.
-// Results below 2^-1020 are returned as 0.  Nine FP64 operations; the series to
+// Results from 2^-1020 down are returned as 0 (t beyond -1020 by more than
+// 2^-11, which its upper word tells).  Nine FP64 operations; the series to
 // degree 11 without a table takes fourteen.
 __device__ __forceinline__ double exp2_table(double t) {
     const double magic = 211106232532992.0;  // 1.5 * 2^47
@@ -101,7 +102,7 @@ __device__ __forceinline__ double exp2_table(double t) {
     p = fma(p, f, 1.0);
     const double u = __ldg(kExp2Frac + (n & 31));
     const double y = p * __hiloint2double(__double2hiint(u) + (int)((unsigned)(n >> 5) << 20), __double2loint(u));
-    return (unsigned)__double2hiint(t) > 0xC08FE000u ? 0.0 : y;  // t < -1020 by its upper word
+    return (unsigned)__double2hiint(t) > 0xC08FE000u ? 0.0 : y;  // by the upper word
 }
 
 template <typename T>
