@@ -75,14 +75,18 @@ __global__ void __launch_bounds__(NW * 32) k_p2p_ds(EvalArgs a, const dbl4* __re
         const int np = K * (int)max((int64_t)0, min(b1, w0 + wper) - w0);
         for (int e = 0; e < np; e += 32) {
             const int cnt = min(32, np - e);
-            bool lap = false;
+            bool lap = false, on = false;
+            const int c = (e + lane) / K, m = e + lane - c * K;
+            int j = -1, b = 0;
+            if (lane < cnt) {
+                j = __float_as_int(column(a, g, c0, w0 - c0 + c).w);
+                b = a.pbody[j];
+                on = (act >> b) & 1ull;
+            }
+            if (!__any_sync(0xffffffffu, on)) continue;  // (as k_p2p)
             __syncwarp();
             if (lane < cnt) {
-                const int c = (e + lane) / K, m = e + lane - c * K;
-                const int j = __float_as_int(column(a, g, c0, w0 - c0 + c).w);
-                const int b = a.pbody[j];
                 lap = glap && b == gb;
-                const bool on = (act >> b) & 1ull;  // a body without density in this product adds nothing
                 const double wt = on ? a.rule.w[K == 3 ? 1 : (m + 2) / 3] : 0.0;
                 const dbl4 d = pd[j], v = a.pts[(int64_t)j * K + m];
                 const double* n = pg + 16 * (int64_t)j + 12;

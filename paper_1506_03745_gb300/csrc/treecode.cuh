@@ -838,20 +838,26 @@ __global__ void __launch_bounds__(NW * 32) k_p2p(EvalArgs a, const typename V4<r
         const int64_t w1 = min(b1, b0 + (w + 1) * wper);
         for (int64_t e = b0 + w * wper; e < w1; e += 32) {
             const int cnt = (int)min((int64_t)32, w1 - e);
-            bool lap = false, has_own = false, sliver = false;
+            bool lap = false, has_own = false, sliver = false, on = false;
             int own = -1;  // the stage's slot of this lane's own panel
-            __syncwarp();
-            int j = -1;
+            int j = -1, b = 0;
+            float4 c;
             if (lane < cnt) {
-                const float4 c = column(a, g, c0, e - c0 + lane);
+                c = column(a, g, c0, e - c0 + lane);
                 j = __float_as_int(c.w);
-                const int b = a.pbody[j];
+                b = a.pbody[j];
+                on = (act >> b) & 1ull;
+            }
+            // a body without density in this product adds nothing; a group's
+            // columns ascend by body, so its stages are left out whole
+            if (!__any_sync(0xffffffffu, on)) continue;
+            __syncwarp();
+            if (lane < cnt) {
                 lap = glap && b == gb;
                 has_own = j >= p0 && j < p1;
                 PanelS<real>& q = sP[w][lane];
                 stage_panel<real, K>(a, c, j, g, q);
                 sliver = K >= 3 && q.sliver != real(0);
-                const bool on = (act >> b) & 1ull;  // a body without density in this product adds nothing
                 const real z = real(0);
                 q.qL = on && lap ? pd[4 * (int64_t)j] : z;
                 q.qY = on ? pd[4 * (int64_t)j + 1] : z;
@@ -1004,10 +1010,13 @@ __global__ void __launch_bounds__(NW * 32) k_near(EvalArgs a, const NearGroup* _
         __syncwarp();
         v4 d;
         d.x = d.y = d.z = d.w = 0;
+        bool on = false;
         if (lane < cnt) {
             const int j = __float_as_int(a.col[c0 + e + lane].w);
-            if ((act >> a.pbody[j]) & 1ull) d = pd[j];
+            on = (act >> a.pbody[j]) & 1ull;
+            if (on) d = pd[j];
         }
+        if (!__any_sync(0xffffffffu, on)) continue;  // (as k_p2p)
         sD[w][lane] = d;
         __syncwarp();
         // runs of one kind of column
