@@ -161,10 +161,10 @@ class Clocks:
 # ------------------------------------------------------------------ profile
 def kernel_source_hash():
     """First 16 hex digits of the SHA-256 of the treecode kernels' sources
-    (treecode.cuh, then ds.cuh): the key under which a committed ncu summary
-    records the source it was taken on."""
+    (treecode.cuh, ds.cuh, then p2p_ds.cuh): the key under which a committed ncu
+    summary records the source it was taken on."""
     h = hashlib.sha256()
-    for f in ("treecode.cuh", "ds.cuh"):
+    for f in ("treecode.cuh", "ds.cuh", "p2p_ds.cuh"):
         h.update(open(os.path.join(ROOT, "paper_1506_03745_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 

@@ -251,7 +251,8 @@ int pgb_rhs(struct pgb_ctx* ctx, double* b);
 
 /* GMRES solve of Eq. 6 / Eq. 7 (Section 3.2).  mode PGB_FP64, PGB_FP32_REFINE
  * or PGB_FP32; tol on ||b - A x||/||b|| (measured with the FP64 operator,
- * except in PGB_FP32 mode where the FP32 operator is used); max_iter total inner iterations;
+ * except in PGB_FP32 mode where the FP32 operator is used, and where the iteration goes on to
+ * 0.99 tol so that the residual's own rounding does not miss tol); max_iter total inner iterations;
  * restart = Krylov dimension (1..256).  x_out: device doubles, n_unknowns.
  * Returns PGB_ENOCONV (x_out and stats still written) when tol is not met. */
 int pgb_solve(struct pgb_ctx* ctx, int32_t mode, double tol, int32_t max_iter, int32_t restart,

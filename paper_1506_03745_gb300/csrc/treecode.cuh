@@ -1145,8 +1145,11 @@ __device__ __forceinline__ int64_t next_entry(const EvalArgs& a, int64_t e, int6
 // targets as the halves of packed values.  A target per lane in scalar
 // arithmetic issued 384 instructions per (node, 32 targets) with monomials and
 // 314 in the harmonic basis, at 56-64 % of the issue rate; packed, they halve
-// and the FMA pipe is the bound.  The coefficients lie in shared memory twice
-// over (c, c), ready as packed operands, and so do the recurrence constants.
+// (85 -> 65 us at order 6 for 2 x 20480 panels).  What is left is latency: 126
+// registers hold 23 % of the warps, the issue slots are 53 % and the FMA pipe
+// 31 % busy; fewer registers for more warps cost more than they gave (102: 1 %,
+// 80: 3 % of the product).  The coefficients lie in shared memory twice over
+// (c, c), ready as packed operands, and so do the recurrence constants.
 template <int P, int NW>
 __global__ void __launch_bounds__(NW * 32) k_m2p_f32(EvalArgs a, const float4* __restrict__ xrel,
                                                      const float* __restrict__ far) {
