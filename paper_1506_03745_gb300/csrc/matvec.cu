@@ -427,7 +427,7 @@ void near_release(pgb_ctx* c, bool large_only) {
 
 // The stored near field of the current lists for a product of a running solve
 // (NearScope): formed by the solve's first product on the context's stream, at
-// the cost of about one and a half P2Ps, and kept until the lists, the geometry
+// about the cost of one P2P, and kept until the lists, the geometry
 // or the screening change.  Not kept (the P2P then forms the sums, as products
 // outside solves do) where it would take more than an eighth of the device's
 // memory or a quarter of what is free, or cannot be allocated.

@@ -466,7 +466,7 @@ inline bool nested(const pgb_ctx* c) {
 }
 // For the duration of a solve: the products of the precision that it iterates in
 // keep the near field.  (Not the one or two FP64 products of a refinement:
-// forming it costs about one and a half P2Ps.)  At its end a near field of
+// forming it costs what one P2P does, and twice the FP32 one's memory.)  At its end a near field of
 // modest size stays for the next solve on the same lists, a large one is given
 // back (near_release).
 void near_release(pgb_ctx* c, bool large_only);
