@@ -17,7 +17,9 @@ LIB = os.path.join(OUT, "libpgb.so")
 SOURCES = ["tree.cu", "matvec.cu", "treecode_f32.cu", "treecode_f64.cu", "solver.cu", "energy.cu", "adjoint.cu",
            "imposed_f32.cu", "treecode_ds.cu", "treecode_ds_hi.cu", "batch.cu", "farfield.cu", "shard.cu", "api.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-pthread", "-Xcompiler", "-Wno-deprecated-declarations"]
+# --no-compress: nvcc compresses device code beyond some size, and its first kernel in a process then waits for
+# the expansion (7 ms for the FP64 treecode's)
+FLAGS = ["-O3", "--no-compress", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-pthread", "-Xcompiler", "-Wno-deprecated-declarations"]
 
 
 def nvcc():
