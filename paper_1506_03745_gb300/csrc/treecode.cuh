@@ -983,9 +983,9 @@ __global__ void __launch_bounds__(NW * 32) k_near_build(EvalArgs a, const NearGr
 
 // The near-field sums of one product from the matrix, items and warps as in
 // k_p2p; a warp keeps the densities of 32 columns in shared memory and eight
-// columns' loads in flight.  Bound by HBM: 2 x 20480 panels hold 294 MB in FP32
-// and take 62 us beside the upward pass (P2P: 114 us alone); 2600 panels in FP64
-// 44 MB, 48 us a product instead of 1.3 ms on the FP64 pipe.
+// columns' loads in flight.  Bound by HBM in FP32: 2 x 20480 panels hold 283 MB
+// and take 56 us alone, 60 to 78 beside the upward pass (k_p2p: 101 us alone); by
+// the FP64 pipe in FP64: 565 MB, 346 us (k_p2p: 9.3 ms).
 template <typename real, int NW>
 __global__ void __launch_bounds__(NW * 32) k_near(EvalArgs a, const NearGroup* __restrict__ ng,
                                                   const real* __restrict__ mat) {
