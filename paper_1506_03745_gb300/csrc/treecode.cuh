@@ -808,8 +808,17 @@ __device__ __forceinline__ void stage_panel(const EvalArgs& a, const float4& c, 
 // then sums them for its target (p2p_panel).  The panels of several leaves
 // share a stage, so a warp's steps are full whatever the leaf sizes.  The
 // item's partial sums go to Up.
+//
+// FP64 is compiled for two blocks on an SM (126 registers at seven points).
+// Left to itself the compiler takes 80 registers and spills, three blocks fit,
+// and they keep the upward pass and the M2P, which run beside them, out of the
+// SMs: products of 4240 panels at order 8 1.50 -> 1.27 ms, of 4500 panels with
+// the four-point rule 1.38 -> 1.21 ms.  Where the P2P is most of the product
+// (order 6, seven points) 1.65 ms either way, and 1.67 -> 1.73 ms with the
+// geometry out of cache.  (96 registers: 1.27, 1.27 and 1.69 ms.)  FP32 takes 63
+// or 64 registers by itself; the bound would make it 91.
 template <typename real, int K, int NW>
-__global__ void __launch_bounds__(NW * 32) k_p2p(EvalArgs a, const typename V4<real>::t* __restrict__ xrel) {
+__global__ void __launch_bounds__(NW * 32, sizeof(real) == 8 ? 2 : 0) k_p2p(EvalArgs a, const typename V4<real>::t* __restrict__ xrel) {
     __shared__ __align__(16) PanelS<real> sP[NW][32];
     __shared__ real red[NW][4][32];
     __shared__ int64_t s_item;
